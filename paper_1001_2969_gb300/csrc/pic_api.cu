@@ -351,6 +351,9 @@ __global__ void k_step_begin(StepCtl *c, const double *rf, int nrf, double dt, i
 // nmain1 / nalive1 null: the pass held the ions still (subcycling)
 __global__ void k_step_end(StepCtl *c, DevScalars *ds, int32_t *nmain0, const int32_t *nalive0, int32_t *nmain1,
                            const int32_t *nalive1) {
+    // the barrier of the births numbering this pass's sort may run
+    c->bar = 0;
+    c->bar_timeout = 0;
     if (c->halt) return;
     *nmain0 = *nalive0;
     unsigned long long n = (unsigned long long)(*nalive0);
@@ -363,19 +366,10 @@ __global__ void k_step_end(StepCtl *c, DevScalars *ds, int32_t *nmain0, const in
     c->step += 1;
 }
 
-// sort epilogue: the sorted counts take effect for the next pass
 // a pass that holds the ions: the births its newborn ions join start at
 // the buffer's present count (skipped once the step has failed, so that a
 // dropped pass's newborns can be cut off again)
-// zero what the particle passes accumulate into (null members skipped)
-struct PassReset {
-    double *N[2];
-    int32_t *counts[2];
-    int32_t *nbirths[2];
-    int32_t *nb0;
-    int32_t *chunk_next;  // [2]
-    int ng, ncell;
-};
+// zero what the particle passes accumulate into (a batch's reactors; else k_birth_finish does)
 __global__ void k_pass_reset(PassReset r) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
     for (int s = 0; s < 2; ++s) {
@@ -387,7 +381,6 @@ __global__ void k_pass_reset(PassReset r) {
     if (t == 0) {
         for (int s = 0; s < 2; ++s)
             if (r.nbirths[s]) *r.nbirths[s] = 0;
-        if (r.nb0) *r.nb0 = 0;
         r.chunk_next[0] = r.chunk_next[1] = 0;
     }
 }
@@ -396,14 +389,6 @@ __global__ void k_hold_ions(const StepCtl *c, int32_t *nb0, const int32_t *nb) {
     if (c->halt) return;
     *nb0 = *nb;
 }
-__global__ void k_sort_end(StepCtl *c, int32_t *nalive0, const int32_t *ntotal0, int32_t *nalive1,
-                           const int32_t *ntotal1) {
-    if (sort_skip(c)) return;
-    *nalive0 = *ntotal0;
-    *nalive1 = *ntotal1;
-    c->sort_pending = 0;
-}
-
 // External circuit (Sec. 2.5, end), Vahedi's superposition: the charge on
 // the z = 0 electrode (Gauss's law on the electrode row: displacement flux
 // eps0 c_0j (phi_0j - phi_1j) into row 1 less the half-cell charge
@@ -810,6 +795,24 @@ void fill_step_args(pic_handle *h, StepArgs<T> &a, int s, int src_set, int dst_s
     a.eedf_scale = h->cfg.eedf_bins > 0 ? (T)(h->cfg.eedf_bins / h->cfg.eedf_emax_eV) : (T)0;
 }
 
+// the births of the last pass, whose output are the buffer sets par_e, par_i
+BirthJob birth_job(pic_handle *h, int par_e, int par_i) {
+    BirthJob b{};
+    for (int s = 0; s < 2; ++s) {
+        SpecDev &d = h->sp[s];
+        const int par = s == 1 ? par_i : par_e;
+        b.key[s] = d.bkey[par];
+        b.id[s] = d.births[par].id;
+        b.nb[s] = d.d_nbirths[par];
+        b.nb0[s] = d.d_nb0;
+        b.nalive[s] = d.d_nalive;
+        b.ntotal[s] = d.d_ntotal;
+    }
+    b.ctl = h->sctl;
+    b.tmp = h->rtmp;
+    return b;
+}
+
 // Enqueues one timestep (Sec. 2.1 merged cycle) without a host
 // synchronisation; failures halt the step on the device (StepCtl) and are
 // resolved by pic_step after the last step of the call.
@@ -836,23 +839,18 @@ void sort_branch(pic_handle *h, int par_e, int par_i, bool ions, cudaStream_t st
         launch_rank<T>(view<T>(d.main[par]), d.d_nmain[par], view<T>(d.births[par]), d.d_nbirths[par],
                        d.cursor, d.perm, d.d_ntotal, d.cap, &h->ds->status, h->sctl, h->ncell, st);
     }
-    h->launches += 4 * ns + 1;
+    launch_birth_rank(birth_job(h, par_e, par_i), st);
+    h->launches += 4 * ns + 2;
 }
 
-// the rest of the sort: newborn numbering (a cooperative launch, after the
-// field solve's), then the sorted counts take effect
-void sort_finish(pic_handle *h, int par_e, int par_i, cudaStream_t st) {
-    for (int s = 0; s < 2; ++s) {
-        SpecDev &d = h->sp[s];
-        const int par = s == 1 ? par_i : par_e;
-        // in a batch: at most 8 blocks (a step's births are few; the numbering
-        // is a cooperative launch, and a wide one waits for free SMs)
-        launch_birth_ids(d.bkey[par], d.births[par].id, d.d_nbirths[par], d.d_nb0, h->sctl, s, h->rtmp, st,
-                         h->in_batch ? 1 : 1 << 30);
-    }
-    k_sort_end<<<1, 1, 0, st>>>(h->sctl, h->sp[0].d_nalive, h->sp[0].d_ntotal, h->sp[1].d_nalive,
-                                 h->sp[1].d_ntotal);
-    h->launches += 3;
+// the rest of the sort: many newborns' numbering (a cooperative launch, after
+// the field solve's), then the sorted counts take effect; r (not null): the
+// coming pass's accumulators are cleared by the same launch
+void sort_finish(pic_handle *h, int par_e, int par_i, cudaStream_t st, const PassReset *r) {
+    // in a batch: one block (a step's births are few; the numbering is a
+    // cooperative launch, and a wide one waits for free SMs)
+    launch_birth_finish(birth_job(h, par_e, par_i), r, st, h->in_batch ? 1 : 1 << 30);
+    h->launches += 1;
 }
 
 // Enqueue one timestep (Sec. 2.1, merged cycle) on h->st: the field at the
@@ -927,10 +925,6 @@ void one_step(pic_handle *h, cudaStream_t sb, bool mv, int part = 0, SolveJob *j
     if (sb) cudaStreamWaitEvent(st, h->ev_join, 0);
     }
     {
-        PhaseTimer t(h, 3);
-        sort_finish(h, src, isrc, st);
-    }
-    {
         // the passes' deposit, cell counts, births counters and chunk
         // counters start at zero (one launch for both species)
         PassReset r{};
@@ -943,9 +937,16 @@ void one_step(pic_handle *h, cudaStream_t sb, bool mv, int part = 0, SolveJob *j
             r.counts[s] = d.counts;
             r.nbirths[s] = d.d_nbirths[s == 1 ? idst : dst];
         }
-        if (mv && h->K > 1) r.nb0 = h->sp[1].d_nb0;  // else always 0
-        k_pass_reset<<<std::max(1, std::min(152 * 4, (std::max(h->ng, h->ncell) + 255) / 256)), 256, 0, st>>>(r);
-        h->launches += 1;
+        {
+            PhaseTimer t(h, 3);
+            sort_finish(h, src, isrc, st, h->in_batch ? nullptr : &r);
+        }
+        if (h->in_batch) {  // its births numbering has one block: too few to clear with
+            k_pass_reset<<<std::max(1, std::min(152 * 4, (std::max(h->ng, h->ncell) + 255) / 256)), 256, 0, st>>>(r);
+            h->launches += 1;
+        }
+        // (else always 0)
+        if (mv && h->K > 1) cudaMemsetAsync(h->sp[1].d_nb0, 0, sizeof(int32_t), st);
         if (!mv) {
             // held ions: deposit, counts and births stay; this pass's
             // newborns are numbered from the births already there
@@ -1011,7 +1012,7 @@ template <typename T>
 void sort_tail(pic_handle *h) {
     PhaseTimer t(h, 3);
     sort_branch<T>(h, h->cur, h->cur_i, true, h->st);
-    sort_finish(h, h->cur, h->cur_i, h->st);
+    sort_finish(h, h->cur, h->cur_i, h->st, nullptr);
 }
 
 void drop_graphs(pic_handle *h) {

@@ -283,8 +283,6 @@ template <typename T>
 void launch_rank(PBuf<T> main, const int32_t *n_main, PBuf<T> births, const int32_t *n_births,
                  int32_t *cursor, int32_t *perm, const int32_t *n_alive, int64_t cap,
                  const int32_t *status, const StepCtl *ctl, int ncell, cudaStream_t st);
-// births of species s get ids next_id[s] + rank of their key among the
-// *nb births (one cooperative launch; next_id[s] advances by *nb)
 struct RadixTmp {
     uint64_t *k0, *k1;
     uint32_t *v0, *v1;
@@ -295,10 +293,33 @@ struct RadixTmp {
 // the bounded-wait self-test (sortk.cu): 0 when it ran, *gave_up = 1 when
 // the wait ran out as it must
 int wait_selftest(long long limit, int *gave_up);
-// numbers the births key/id[*nb0 .. *nb) (nb0 nullable: from 0), on at
-// most max_grid blocks
-void launch_birth_ids(const uint64_t *key, uint64_t *id, const int32_t *nb, const int32_t *nb0, StepCtl *ctl,
-                      int s, RadixTmp tmp, cudaStream_t st, int max_grid = 1 << 30);
+// the births of a pass of both species, entries [*nb0, *nb) of their
+// buffers, and where the sorted counts go
+struct BirthJob {
+    const uint64_t *key[2];
+    uint64_t *id[2];
+    const int32_t *nb[2], *nb0[2];
+    int32_t *nalive[2];
+    const int32_t *ntotal[2];
+    StepCtl *ctl;
+    RadixTmp tmp;
+};
+// what the particle passes accumulate into, cleared before them (null
+// members skipped)
+struct PassReset {
+    double *N[2];
+    int32_t *counts[2];
+    int32_t *nbirths[2];
+    int32_t *chunk_next;  // [2]
+    int ng, ncell;
+};
+// births get ids next_id[s] + stride x rank of their key among the pass's
+// births of their species: few births by the first kernel (beside the field
+// solve), many by the second, which also moves the ids on, makes the sorted
+// counts current and (r not null) clears the coming pass's accumulators; on
+// at most max_grid blocks
+void launch_birth_rank(const BirthJob &b, cudaStream_t st);
+void launch_birth_finish(const BirthJob &b, const PassReset *r, cudaStream_t st, int max_grid = 1 << 30);
 
 // ---- multigrid (field.cu) ----
 struct MGLevel {

@@ -9,9 +9,9 @@
 //
 // Newborns are numbered next_id + stride x rank of their key (parent
 // species, parent id, birth slot; the stride is 1 unless the reactor's
-// particles are shared among processes): one block ranks small batches directly, larger batches
-// go through an LSD radix sort of (key, index) pairs, both in one
-// cooperative launch that reads the count on the device.
+// particles are shared among processes): small batches by counting the smaller
+// keys of each, larger ones by an LSD radix sort of (key, index) pairs in one
+// cooperative launch; both read the count on the device.
 #include <limits.h>
 
 #include <algorithm>
@@ -298,57 +298,70 @@ void launch_rank(PBuf<T> mainb, const int32_t *n_main, PBuf<T> births, const int
 
 // ---- newborn numbering ----
 // Births get ids next_id + rank of their key (parent species, parent id,
-// birth index), as in the oracle.  One cooperative launch: up to
-// kSmallBirths keys block 0 ranks each key by counting smaller ones; above
-// that the grid runs an LSD radix sort over 8-bit digits (a digit shared by
-// every key is skipped), tiles of kRadixTile keys, grid barriers between the
-// histogram, scan and scatter phases.
-constexpr int kSmallBirths = 2048;
+// birth index), as in the oracle.  Up to kRankBirths of them k_birth_rank
+// counts the smaller keys of each; above that k_birth_finish runs an LSD
+// radix sort over 8-bit digits (a digit shared by every key is skipped),
+// tiles of kRadixTile keys, grid barriers between the histogram, scan and
+// scatter phases.
 constexpr int kRadixThreads = 1024;
 constexpr int kRadixPer = 2;
 constexpr int kRadixTile = kRadixThreads * kRadixPer;
 
-__global__ void __launch_bounds__(kRadixThreads)
-    k_birth_ids(const uint64_t *key, uint64_t *id, const int32_t *nb_dev, const int32_t *nb0_dev, StepCtl *ctl, int s,
-                RadixTmp t) {
-    // the small path's keys and the scatter's per-warp digit counts share space
-    constexpr int kBuf = kSmallBirths * 8 > (kRadixThreads / 32) * 256 * 4 ? kSmallBirths * 8
-                                                                            : (kRadixThreads / 32) * 256 * 4;
-    __shared__ __align__(16) unsigned char s_buf[kBuf];
-    uint64_t *s_key = reinterpret_cast<uint64_t *>(s_buf);
-    uint32_t (*s_wc)[256] = reinterpret_cast<uint32_t (*)[256]>(s_buf);
+// Rank by counting: a block takes kRankKeys keys at a time, 16 threads each,
+// and passes all keys through shared memory.  No block waits for another, so
+// it runs as an ordinary kernel beside the field solve (ids are first read
+// by the next particle pass).  Bound by issue: the n^2 comparisons are spread
+// over the grid.  One block per species, which made the same comparisons
+// before, held up the pass after the solve for 105 us per species in the
+// first steps of c2 (many births) and 4 us with few; with this kernel beside
+// the solve c2 went from 1107 to 1092 us a step, c1 from 314 to 298, eight
+// batched reactors from 1739 to 1667.  The line to the radix sort is where
+// the comparisons (67M: some 9 us of the whole GPU's issue slots, mostly
+// hidden by the solve) still cost less than its ~20 grid barriers (~1 us
+// each, after the solve).
+constexpr int kRankBirths = 8192;
+constexpr int kRankKeys = 16;
+constexpr int kRankTile = 2048;
+constexpr int kBirthThreads = 256;
+
+__global__ void __launch_bounds__(kBirthThreads) k_birth_rank(BirthJob b) {
+    __shared__ uint64_t s_key[kRankTile];
+    if (sort_skip(b.ctl)) return;
+    const int s = blockIdx.y, first = *b.nb0[s];
+    const int nb = *b.nb[s] - first;
+    if (nb <= 0 || first < 0 || nb > kRankBirths) return;
+    const uint64_t *key = b.key[s] + first;
+    const uint64_t base = b.ctl->next_id[s];
+    const uint64_t stride = b.ctl->id_stride ? b.ctl->id_stride : 1ull;
+    const int q = threadIdx.x & 15;
+    for (int g = blockIdx.x * kRankKeys; g < nb; g += gridDim.x * kRankKeys) {
+        const int k = g + (threadIdx.x >> 4);
+        const uint64_t mine = k < nb ? key[k] : 0ull;
+        int rank = 0;
+        for (int t0 = 0; t0 < nb; t0 += kRankTile) {
+            const int tn = min(kRankTile, nb - t0);
+            __syncthreads();  // the tile before is read
+            for (int e = threadIdx.x; e < tn; e += kBirthThreads) s_key[e] = key[t0 + e];
+            __syncthreads();
+#pragma unroll 4
+            for (int e = q; e < tn; e += 16) rank += s_key[e] < mine;
+        }
+        for (int o = 8; o > 0; o >>= 1) rank += __shfl_xor_sync(0xffffffffu, rank, o);
+        if (q == 0 && k < nb) b.id[s][first + k] = base + stride * (uint64_t)rank;
+    }
+}
+
+// Radix numbering of nb > kRankBirths keys by the whole (co-resident) grid;
+// false when a grid barrier gave up
+__device__ bool radix_births(const uint64_t *key, uint64_t *id, int nb, StepCtl *ctl, uint64_t base,
+                             const RadixTmp &t, unsigned &nbar) {
+    __shared__ uint32_t s_wc[kRadixThreads / 32][256];
     __shared__ uint32_t s_run[256];
     __shared__ int s_warp[32];
     __shared__ int s_carry;
-    if (sort_skip(ctl)) return;
-    // the births of the last pass: the buffer's entries from *nb0_dev on
-    const int first = nb0_dev ? *nb0_dev : 0;
-    const int nb = *nb_dev - first;
-    if (nb <= 0 || first < 0) return;
-    key += first;
-    id += first;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (nb <= kSmallBirths) {
-        if (blockIdx.x != 0) return;
-        const uint64_t base = ctl->next_id[s];
-        const uint64_t stride = ctl->id_stride ? ctl->id_stride : 1ull;
-        for (int k = tid; k < nb; k += blockDim.x) s_key[k] = key[k];
-        __syncthreads();
-        for (int k = tid; k < nb; k += blockDim.x) {
-            const uint64_t mine = s_key[k];
-            int rank = 0;
-            for (int q = 0; q < nb; ++q) rank += s_key[q] < mine;
-            id[k] = base + stride * (uint64_t)rank;
-        }
-        __syncthreads();
-        if (tid == 0) ctl->next_id[s] = base + stride * (uint64_t)nb;
-        return;
-    }
-    // every block reads the base before the first barrier; block 0 moves it on at the end
-    const uint64_t base = ctl->next_id[s];
     const uint64_t stride = ctl->id_stride ? ctl->id_stride : 1ull;
     const int ntiles = (nb + kRadixTile - 1) / kRadixTile;
-    unsigned nbar = 0;
     // a wait that gives up fails the sort (its ids would be wrong)
     auto bar = [&]() {
         if (count_barrier(&ctl->bar, (++nbar) * gridDim.x, &ctl->bar_timeout)) return true;
@@ -359,7 +372,7 @@ __global__ void __launch_bounds__(kRadixThreads)
         t.k0[e] = key[e];
         t.v0[e] = (uint32_t)e;
     }
-    if (!bar()) return;
+    if (!bar()) return false;
     uint64_t *ka = t.k0, *kb = t.k1;
     uint32_t *va = t.v0, *vb = t.v1;
     for (int shift = 0; shift < 64; shift += 8) {
@@ -375,7 +388,7 @@ __global__ void __launch_bounds__(kRadixThreads)
             if (tid < 256) t.hist[tid * ntiles + tile] = s_run[tid];
             __syncthreads();
         }
-        if (!bar()) return;
+        if (!bar()) return false;
         // block 0: exclusive scan in digit-major order; a digit held by all
         // keys leaves the order as it is
         if (blockIdx.x == 0) {
@@ -405,7 +418,7 @@ __global__ void __launch_bounds__(kRadixThreads)
                 }
             }
         }
-        if (!bar()) return;
+        if (!bar()) return false;
         if (*(volatile int *)t.flag) continue;
         // stable scatter of each tile: rounds of kRadixThreads keys in order;
         // inside a round a key's place is (keys of its digit in earlier
@@ -442,7 +455,7 @@ __global__ void __launch_bounds__(kRadixThreads)
                 __syncthreads();
             }
         }
-        if (!bar()) return;
+        if (!bar()) return false;
         uint64_t *tk = ka;
         ka = kb;
         kb = tk;
@@ -451,7 +464,55 @@ __global__ void __launch_bounds__(kRadixThreads)
         vb = tv;
     }
     for (int r = blockIdx.x * blockDim.x + tid; r < nb; r += gridDim.x * blockDim.x) id[va[r]] = base + stride * (uint64_t)r;
-    if (blockIdx.x == 0 && tid == 0) ctl->next_id[s] = base + stride * (uint64_t)nb;
+    return true;
+}
+
+// The end of the pending sort and the start of the pass that reads it: the
+// births k_birth_rank left are numbered, the ids move on, the sorted counts
+// take effect, and (reset) what the coming pass accumulates into is cleared.
+// One launch for what were seven nodes in a row between the field and the
+// pass (two births numberings with their counters' clears, sort end, reset).
+// Cooperative when it has more than one block (the radix sort's barriers).
+__global__ void __launch_bounds__(kRadixThreads) k_birth_finish(BirthJob b, PassReset r, int reset) {
+    const int tid = threadIdx.x, t = blockIdx.x * blockDim.x + tid, all = gridDim.x * blockDim.x;
+    if (reset) {
+        for (int s = 0; s < 2; ++s) {
+            if (r.N[s])
+                for (int k = t; k < r.ng; k += all) r.N[s][k] = 0.0;
+            if (r.counts[s])
+                for (int k = t; k < r.ncell; k += all) r.counts[s][k] = 0;
+        }
+        if (t == 0) {
+            for (int s = 0; s < 2; ++s)
+                if (r.nbirths[s]) *r.nbirths[s] = 0;
+            r.chunk_next[0] = r.chunk_next[1] = 0;
+        }
+    }
+    StepCtl *ctl = b.ctl;
+    if (sort_skip(ctl)) return;
+    // every block reads the counts and the bases before the first barrier;
+    // block 0 moves the bases on at the end
+    int nb[2], first[2];
+    uint64_t base[2];
+    for (int s = 0; s < 2; ++s) {
+        first[s] = *b.nb0[s];
+        nb[s] = first[s] < 0 ? 0 : *b.nb[s] - first[s];
+        base[s] = ctl->next_id[s];
+    }
+    const bool large = nb[0] > kRankBirths || nb[1] > kRankBirths;
+    if (!large && blockIdx.x != 0) return;
+    unsigned nbar = 0;
+    for (int s = 0; s < 2; ++s)
+        if (nb[s] > kRankBirths)
+            if (!radix_births(b.key[s] + first[s], b.id[s] + first[s], nb[s], ctl, base[s], b.tmp, nbar)) return;
+    if (t == 0) {
+        const uint64_t stride = ctl->id_stride ? ctl->id_stride : 1ull;
+        for (int s = 0; s < 2; ++s) {
+            if (nb[s] > 0) ctl->next_id[s] = base[s] + stride * (uint64_t)nb[s];
+            *b.nalive[s] = *b.ntotal[s];
+        }
+        ctl->sort_pending = 0;
+    }
 }
 
 // failure-detection self-test: one block waits at the bounded grid barrier
@@ -474,8 +535,14 @@ int wait_selftest(long long limit, int *gave_up) {
     return 0;
 }
 
-void launch_birth_ids(const uint64_t *key, uint64_t *id, const int32_t *nb, const int32_t *nb0, StepCtl *ctl,
-                      int s, RadixTmp tmp, cudaStream_t st, int max_grid) {
+void launch_birth_rank(const BirthJob &b, cudaStream_t st) {
+    // at most 128 blocks per species, no more than the births can fill; a
+    // block finds out by itself that there is nothing for it to do
+    const int g = std::max(1, std::min(128, (std::min(b.tmp.max_n, kRankBirths) + kRankKeys - 1) / kRankKeys));
+    k_birth_rank<<<dim3(g, 2), kBirthThreads, 0, st>>>(b);
+}
+
+void launch_birth_finish(const BirthJob &b, const PassReset *r, cudaStream_t st, int max_grid) {
     // one block per SM (the launch needs them co-resident), per device
     static int grids[64] = {0};
     int dev = 0;
@@ -484,20 +551,23 @@ void launch_birth_ids(const uint64_t *key, uint64_t *id, const int32_t *nb, cons
     if (grid == 0) {
         int nsm = 0, per = 0;
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_birth_ids, kRadixThreads, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_birth_finish, kRadixThreads, 0);
         grid = std::max(1, std::min(nsm, nsm * per));
     }
-    cudaMemsetAsync(&ctl->bar, 0, sizeof(unsigned) + sizeof(int32_t), st);  // counter and timeout flag
-    void *args[] = {(void *)&key, (void *)&id, (void *)&nb, (void *)&nb0, (void *)&ctl, (void *)&s, (void *)&tmp};
     // no more blocks than tiles of the largest batch of births (a small
     // reactor's numbering does not hold the whole GPU)
     // (max_grid: a reactor of a batch, whose numbering must not wait for
     // many co-resident blocks while the other reactors' kernels hold SMs)
-    const int g = std::max(1, std::min(std::min(grid, max_grid), (tmp.max_n + kRadixTile - 1) / kRadixTile));
-    if (g == 1)  // one block: its barriers wait for itself alone, no co-residency to ask for
-        k_birth_ids<<<1, kRadixThreads, 0, st>>>(key, id, nb, nb0, ctl, s, tmp);
-    else
-        cudaLaunchCooperativeKernel((void *)k_birth_ids, g, kRadixThreads, args, 0, st);
+    const int g = std::max(1, std::min(std::min(grid, max_grid), (b.tmp.max_n + kRadixTile - 1) / kRadixTile));
+    BirthJob job = b;
+    PassReset rs = r ? *r : PassReset{};
+    int reset = r ? 1 : 0;
+    if (g == 1) {  // one block: its barriers wait for itself alone, no co-residency to ask for
+        k_birth_finish<<<1, kRadixThreads, 0, st>>>(job, rs, reset);
+    } else {
+        void *args[] = {(void *)&job, (void *)&rs, (void *)&reset};
+        cudaLaunchCooperativeKernel((void *)k_birth_finish, g, kRadixThreads, args, 0, st);
+    }
 }
 
 template void launch_hist<float>(PBuf<float>, const int32_t *, int32_t *, cudaStream_t);
