@@ -13,7 +13,7 @@
 //  - the whole solve is one cooperative launch: the residual and the
 //    restriction chain run over tiles of columns, convergence is decided on
 //    the device, and a block sweeps one black line with the two red lines
-//    beside it, so one barrier separates two levels;
+//    beside it as soon as the coarse rows above it are there;
 //  - prolongation is folded into the red sweep: red (odd) rows are
 //    recomputed whole by their line solve, so only the injection of the
 //    coarse correction into the black (even) neighbour rows is ever used;
@@ -333,112 +333,177 @@ __global__ void k_rhs_bc(const MGFast *__restrict__ mp, const double *rho, doubl
     } else
         p = phi[k];
     phi[k] = p;
-    // the solve alternates between phi and a copy (both carry the boundary
-    // values); the level-0 correction starts at zero (and stays zero on the
-    // boundary); the solve's control block starts cleared
-    m.phi2[k] = p;
-    if (m.u32[0])
-        m.u32[0][k] = 0.0f;
-    else
-        m.u64[0][k] = 0.0;
+    // the solve's control block starts cleared
     for (int w = k; w < (int)(sizeof(MGCtl) / sizeof(unsigned)); w += nz * nr)
         reinterpret_cast<unsigned *>(m.ctl)[w] = 0u;
 }
 
 // ---------------------------------------------------------------------------
-// The whole solve in one cooperative launch.  Blocks are co-resident (the
-// launch guarantees it), and phases are separated by a grid barrier whose
-// spin is bounded: after kSpinLimit polls a block raises `timeout` and every
-// block leaves.  The V-cycle works on the correction delta of phi in both
-// precisions (FP32 delta and residual for the mixed path).  Per cycle:
-//   1. residual of phi + delta, its norms and the restriction chain down to
-//      the coarsest level, one tile of columns per block (coalesced rows);
-//   2. convergence decision (every block reads the same maxima), then
-//      phi += delta;
-//   3. up the levels, one phase per level: the block owning black line
-//      i = 2q + 2 solves the red lines 2q + 1 and 2q + 3 beside it (two
-//      warps at once), keeps them in shared memory and solves the black
-//      line.  A red line shared by two blocks is computed by both from the
-//      same data, bit for bit, and stored by one.  So one barrier separates
-//      two levels instead of two.
-// The coarsest row is solved by block 0 in the phase of level L-1, which
-// block 0 sweeps alone.  Levels with at most kBarGroup black lines belong to
-// the first kBarGroup blocks, separated by a barrier among those blocks only;
-// the rest of the grid waits at the next full barrier.
+// The whole solve in one cooperative launch (its blocks are co-resident).
+// The V-cycle works on the correction delta of phi in both precisions (FP32
+// delta and residual for the mixed path).  Per cycle:
+//   1. one tile of columns per block: the residual (FP64 path: of phi + delta;
+//      mixed path: by the GCR step), its norm, and the restriction chain down
+//      to the coarsest level;
+//   2. convergence decision: every block reads the same norms;
+//   3. up the levels: the unit of a black line i = 2q + 2 solves the red lines
+//      2q + 1 and 2q + 3 beside it (two warps at once), keeps them in shared
+//      memory and solves the black line.  A red line shared by two units is
+//      computed by both from the same data, bit for bit, and stored by one.
+// The solve is bound by latency: a c2 cycle is a chain of one tile phase, two
+// all-to-all exchanges and seven levels of line solves, each under a
+// microsecond of arithmetic.  So no barrier separates the phases: what one
+// block hands to another (rows of the correction, the restricted right-hand
+// sides, norms, dot products) travels in flagged words that the reader polls
+// (Flag in pic_internal.cuh), and a unit starts when its three coarse rows
+// are there.  Units are dealt coarse to fine, block b taking units b, b + P,
+// ...; a unit waits only for units before it, so the chain cannot lock.  Each
+// unit's line factors stay in shared memory for the whole solve where they
+// fit; operator, Krylov vectors and phi are read and written by the block
+// that owns them, and nothing drops them from L1.
+// Words are reused every cycle under a new tag.  That is safe: a tile phase
+// starts with every row of the cycle's level-0 correction, each of which comes
+// after all its unit's reads and after those of all units above it; and rows
+// of the next correction are written after the exchange of norms that ends
+// the tile phase, to which every block comes with its own reads done.
+// Measured, a whole stand-alone solve (with its set-up launches) against the
+// same phases between grid barriers, which took ~1 us each and cost every
+// phase its L1: 33 x 65 mixed 216 -> 157 us, 65 x 300 mixed 326 -> 228,
+// 257 x 1025 mixed 626 -> 527, 129 x 513 FP64 886 -> 803 (FP64 line solves).
 // ---------------------------------------------------------------------------
-constexpr int kBarGroup = 8;  // blocks that sweep the coarse levels alone
 
 // ---- factor lines into shared memory ----
-// A line's factors move in one bulk copy that completes on the region's
-// mbarrier (thread 0 issues it).  All threads of the block keep the same
-// state: the parity of the next completion and whether a copy is pending.
+// Bulk copies that complete on an mbarrier (thread 0 issues them).  All
+// threads of the block keep the same state: per region the parity of the next
+// completion and whether a copy is pending.
 struct Loader {
-    unsigned mbar;
-    unsigned phase;
-    int pending;
+    unsigned mbar;     // the first region's mbarrier (8 bytes each)
+    unsigned phase, pending;  // bit per region
 };
 
-__device__ __forceinline__ void ld_begin(Loader &q, unsigned bytes) {
+__device__ __forceinline__ void ld_begin(Loader &q, int r, unsigned bytes) {
     if (threadIdx.x == 0) {
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(q.mbar), "r"(bytes) : "memory");
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(q.mbar + 8 * r), "r"(bytes)
+                     : "memory");
     }
-    q.pending = 1;
+    q.pending |= 1u << r;
 }
 
 // sizes and addresses are multiples of 16 bytes
-__device__ __forceinline__ void ld_copy(Loader &q, void *dst, const void *src, unsigned bytes) {
+__device__ __forceinline__ void ld_copy(const Loader &q, int r, void *dst, const void *src, unsigned bytes) {
     if (threadIdx.x == 0)
         asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                     ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src), "r"(bytes), "r"(q.mbar)
+                     ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src), "r"(bytes), "r"(q.mbar + 8 * r)
                      : "memory");
 }
 
-// wait for the region's copy (every thread of the block calls it); false,
-// for the whole block, when the bounded wait gave up
-__device__ __forceinline__ bool ld_wait(Loader &q) {
-    if (!q.pending) return true;
+// wait for region r's copy (every thread of the block calls it); false where
+// the bounded wait gave up
+__device__ __forceinline__ bool ld_wait(Loader &q, int r) {
+    if (!(q.pending >> r & 1u)) return true;
     bool ok = false;
     for (long long it = 0; it < kSpinLimit && !ok; ++it) {
         unsigned done;
         asm volatile(
             "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
             : "=r"(done)
-            : "r"(q.mbar), "r"(q.phase)
+            : "r"(q.mbar + 8 * r), "r"(q.phase >> r & 1u)
             : "memory");
         ok = done != 0;
     }
-    ok = !__syncthreads_or(!ok);
-    if (ok) {
-        q.pending = 0;
-        q.phase ^= 1u;
-    }
+    q.pending &= ~(1u << r);
+    q.phase ^= 1u << r;
     return ok;
 }
 
-// black lines of a level with nz rows (at least one unit of work: nz = 3 has
-// a red line only)
-__device__ __forceinline__ int units_of(int nz) { return max((nz - 3) / 2, 1); }
-
 constexpr int kSolveThreads = 256;
-constexpr int kU = 4;   // elements per thread and batch in the residual phase
-constexpr int kUL = 4;  // unknowns per thread and batch of a level's right-hand sides
+constexpr int kU = 4;  // elements per thread and batch in the residual phase
 
-// MINB: blocks per SM the registers must allow.  One (the compiler then
-// takes ~200 registers) is a little faster for a reactor's solve alone; two
-// (127 registers, no spills) lets the solves of a batch of reactors share
-// SMs, and the batch step runs ~28 % faster with it.
-// One reactor's solve on nbk blocks (bid: this block's index among them).
+// the larger of a over the block's threads (bit patterns), and of b
+__device__ __forceinline__ void block_max2(unsigned long long &a, unsigned long long &b,
+                                           unsigned long long (*s)[kSolveThreads / 32]) {
+    for (int o = 16; o > 0; o >>= 1) {
+        a = max(a, __shfl_xor_sync(0xffffffffu, a, o));
+        b = max(b, __shfl_xor_sync(0xffffffffu, b, o));
+    }
+    if ((threadIdx.x & 31) == 0) {
+        s[0][threadIdx.x >> 5] = a;
+        s[1][threadIdx.x >> 5] = b;
+    }
+    __syncthreads();
+    for (int w = 0; w < kSolveThreads / 32; ++w) {
+        a = max(a, s[0][w]);
+        b = max(b, s[1][w]);
+    }
+}
+
+// nz = 3: one interior row, phi's own, solved exactly in FP64 by one block
+template <int M>
+__device__ __forceinline__ void solve_row(const MGFast &m, double *phi, int nr, double tol, int max_cycles,
+                                          double *B, double *F) {
+    __shared__ unsigned long long s_max[2][kSolveThreads / 32];
+    const int tid = threadIdx.x, n = nr - 1;
+    const double *cz = m.cz[0], *cr = m.cr[0];
+    auto at = [](int j) { return (j % M) * kRow + j / M; };
+    for (int k = tid; k < line_factor_elems(M); k += kSolveThreads) F[k] = m.facc[k];
+    double bn = 0.0;
+    for (int cyc = 0;; ++cyc) {
+        unsigned long long rmax = 0ull, bmax = 0ull;
+        for (int j = tid; j < n; j += kSolveThreads) {
+            const size_t k = (size_t)nr + j;
+            const double below = cz[k - nr] * phi[k - nr], above = cz[k] * phi[k + nr], right = cr[k] * phi[k + 1];
+            const double left = j > 0 ? cr[k - 1] * phi[k - 1] : 0.0;
+            rmax = max(rmax, abs_bits(m.f0[k] - (m.dg0[k] * phi[k] - below - above - right - left)));
+            bmax = max(bmax, abs_bits(m.f0[k] + below + above + (j == n - 1 ? right : 0.0)));
+        }
+        block_max2(rmax, bmax, s_max);
+        const double rn = __longlong_as_double((long long)rmax);
+        if (cyc == 0) bn = __longlong_as_double((long long)bmax);
+        int d = 0;
+        if (bn == 0.0)
+            d = 3;
+        else if (tol > 0.0 && rn <= tol * bn)
+            d = 1;
+        else if (cyc >= max_cycles)
+            d = tol > 0.0 ? 2 : 1;
+        if (tid == 0) {
+            m.ctl->last_res = rn;
+            m.ctl->bnorm = bn;
+            m.ctl->cycles = cyc;
+            if (d == 1) m.ctl->converged = 1;
+            if (d == 3) m.ctl->zero_rhs = 1;
+        }
+        if (d == 3)
+            for (int j = tid; j < n; j += kSolveThreads) phi[nr + j] = 0.0;
+        if (d) return;
+        for (int j = tid; j < kLine * M; j += kSolveThreads) {
+            double rhs = 0.0;
+            if (j < n) {
+                const size_t k = (size_t)nr + j;
+                rhs = m.f0[k] + cz[k - nr] * phi[k - nr] + cz[k] * phi[k + nr];
+                if (j == n - 1) rhs += cr[k] * phi[k + 1];
+            }
+            B[at(j)] = rhs;
+        }
+        __syncthreads();
+        if (tid < 32) warp_line_solve<double, M>(F, B, tid);
+        __syncthreads();
+        for (int j = tid; j < n; j += kSolveThreads) phi[nr + j] = B[at(j)];
+        __syncthreads();
+    }
+}
+
+// One reactor's solve on P blocks (bid: this block's index among them).
 template <typename Tv, int M>
-__device__ __forceinline__ void solve_body(const MGFast *__restrict__ mp, double *phi, int nr, int first_cycle,
+__device__ __forceinline__ void solve_body(const MGFast *__restrict__ mp, double *phi, int nr,
                                            const SolveLayout &lay, double tol, int max_cycles,
-                                           const StepCtl *sctl, const int bid, const int nbk) {
+                                           const StepCtl *sctl, const int bid, const int P) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     if (sctl && sctl->halt) return;  // an earlier failure of this step
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nt = blockDim.x;
-    // the level table in shared memory: every grid barrier's acquire drops
-    // L1, and a table read from L2 before each level's loads would put an L2
-    // round trip in front of every phase
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    constexpr int nt = kSolveThreads;
+    // the level table in shared memory (read in front of every phase's loads)
     __shared__ __align__(16) MGFast s_m;
     {
         static_assert(sizeof(MGFast) % 8 == 0, "the level table is copied in 8-byte words");
@@ -449,275 +514,284 @@ __device__ __forceinline__ void solve_body(const MGFast *__restrict__ mp, double
     }
     const MGFast &m = s_m;
     MGCtl *ctl = m.ctl;
-    const int n = nr - 1, nz0 = m.nz[0], ng = nz0 * nr, L = m.nlev - 1;
+    const int n = nr - 1, nz0 = m.nz[0], L = m.nlev - 1;
     constexpr int NW = kLine * M;  // unknowns of a line with its padding
-    const bool mixed = sizeof(Tv) == 4;
-    Tv *delta = mixed ? (Tv *)m.u32[0] : (Tv *)m.u64[0];  // level-0 correction (zero on the boundary)
     constexpr int LFE = line_factor_elems(M);
-    const unsigned FBv = (unsigned)(LFE * sizeof(Tv)), FBd = (unsigned)(LFE * sizeof(double));
-    // levels whose work fits in G blocks are swept by the first G blocks only
-    const int G = min(kBarGroup, nbk);
-    int lb = L;
-    while (lb > 0 && units_of(m.nz[lb - 1]) <= G) --lb;
-    const bool in_group = bid < G;
-    __shared__ unsigned long long s_r[32], s_b[32];
-    __shared__ double s_dot[4][32];
-    __shared__ double s_sum[4];
+    if (L == 0) {
+        if (bid == 0)
+            solve_row<M>(m, phi, nr, tol, max_cycles, reinterpret_cast<double *>(smem_raw),
+                         reinterpret_cast<double *>(smem_raw + lay.offC));
+        return;
+    }
+    using Fv = Flag<Tv>;
+    using Wv = typename Fv::W;
+    constexpr bool mixed = sizeof(Tv) == 4;  // flexible GCR(1) around the V-cycle; else the plain V(0,1) iteration
+    const unsigned ep = *(volatile unsigned *)m.epoch;  // tags of this solve: ep + 1 + cycle
+    __shared__ unsigned long long s_max[2][2][nt / 32];
+    __shared__ double s_dot[2][4][nt / 32];
     __shared__ double s_ab[3];  // the GCR step's beta, alpha and |q|^2
-    // the mixed path accelerates its refinement by flexible GCR(1) (the
-    // Krylov vectors are allocated for it); the FP64 path runs the paper's
-    // plain V(0,1) iteration
-    const bool kry = mixed && m.kr != nullptr && L > 0;
+    __shared__ __align__(8) unsigned long long s_mbar[kMaxSlots + 1];
     double kc = 0.0;  // |w|^2 of the previous direction's A-image
-    __shared__ __align__(8) unsigned long long s_mbar[3];
-    __shared__ int s_decide;
+    double bn = 0.0;  // max |b|
     if (tid == 0) {
-        for (int b = 0; b < 3; ++b)
+        for (int b = 0; b <= kMaxSlots; ++b)
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"((unsigned)__cvta_generic_to_shared(&s_mbar[b]))
                          : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
-    // red factors; black factors; coarsest-row factors
-    Loader qR{(unsigned)__cvta_generic_to_shared(&s_mbar[0]), 0u, 0};
-    Loader qB{(unsigned)__cvta_generic_to_shared(&s_mbar[1]), 0u, 0};
-    Loader qC{(unsigned)__cvta_generic_to_shared(&s_mbar[2]), 0u, 0};
-    // leave with no copy in flight (bounded waits); fail: a wait gave up
-    auto leave = [&](bool fail) {
-        if (fail && tid == 0) atomicExch(&ctl->timeout, 1);
-        ld_wait(qR);
-        ld_wait(qB);
-        ld_wait(qC);
+    Loader ld{(unsigned)__cvta_generic_to_shared(&s_mbar[0]), 0u, 0u};
+    // ---- this block's units: levels L-1 (one unit) .. 0, coarse to fine ----
+    const int units = (2 << L) - 2 - L, nun = units > bid ? (units - bid + P - 1) / P : 0;
+    const int S = lay.slots;
+    auto unit_at = [&](int u, int &l, int &q) {
+        l = L - 1;
+        for (int w = 1; u >= w; w = 2 * w + 1) {  // units of level l
+            u -= w;
+            --l;
+        }
+        q = u;
     };
-    int first = first_cycle;
-    unsigned ngrid = 0, ngroup = 0;  // barriers of each kind passed
-    // the iterate alternates between phi and its copy (L > 0): the residual
-    // phase reads cur + delta and stores it as nxt, the next cycle's iterate
-    const bool dbuf = L > 0;
-    double *cur = phi, *nxt = m.phi2;
-    // coarsest-row factors in the V-cycle's type (nz = 3: phi's own row, FP64)
-    const Tv *facc_v = mixed ? (const Tv *)m.facc32 : (const Tv *)m.facc;
-    const unsigned FBc = (unsigned)(LFE * sizeof(Tv));
-    Tv *Bf0 = reinterpret_cast<Tv *>(smem_raw + lay.offBuf);
-    Tv *Bf1 = reinterpret_cast<Tv *>(smem_raw + lay.offBuf + M * kRow * 8);
-    Tv *Bf2 = reinterpret_cast<Tv *>(smem_raw + lay.offBuf + 2 * M * kRow * 8);
-    double *BC = reinterpret_cast<double *>(smem_raw + lay.offBuf);
-    Tv *W0 = reinterpret_cast<Tv *>(smem_raw + lay.offW);
-    Tv *W1 = W0 + NW;
-    Tv *R0 = reinterpret_cast<Tv *>(smem_raw + lay.offF);
-    Tv *R1 = R0 + LFE;
-    Tv *FBk = R1 + LFE;
+    Tv *slots = reinterpret_cast<Tv *>(smem_raw + lay.offF);
+    constexpr unsigned FB = (unsigned)(LFE * sizeof(Tv));
+    // request the factors of this block's k-th unit (its k-th modulo nun) into slot r
+    auto request = [&](int k, int r) {
+        int l, q;
+        unit_at(bid + (k % nun) * P, l, q);
+        const Tv *fac = mixed ? (const Tv *)m.fac32[l] : (const Tv *)m.fac64[l];
+        Tv *dst = slots + (size_t)r * 3 * LFE;
+        ld_begin(ld, r, 3 * FB);
+        // lines 2q + 1, 2q + 2, 2q + 3 lie one after another
+        ld_copy(ld, r, dst, fac + (size_t)(2 * q) * LFE, 3 * FB);
+    };
+    for (int k = 0; k < min(nun, S); ++k) request(k, k);
     Tv *FC = reinterpret_cast<Tv *>(smem_raw + lay.offC);
-    double *FC64 = reinterpret_cast<double *>(smem_raw + lay.offC);
+    if (bid == 0) {  // the coarsest row
+        ld_begin(ld, kMaxSlots, FB);
+        ld_copy(ld, kMaxSlots, FC, mixed ? (const Tv *)m.facc32 : (const Tv *)m.facc, FB);
+    }
+    // leave with no copy in flight (bounded waits), the tags used up
+    auto leave = [&](int cyc) {
+        for (int r = 0; r <= kMaxSlots; ++r) ld_wait(ld, r);
+        if (bid == 0 && tid == 0) *m.epoch = ep + (unsigned)cyc + 4u;
+    };
+    Tv *Bf0 = reinterpret_cast<Tv *>(smem_raw), *Bf1 = Bf0 + M * kRow, *Bf2 = Bf1 + M * kRow;
+    Tv *W0 = reinterpret_cast<Tv *>(smem_raw + lay.offW), *W1 = W0 + NW;
+    double *St = reinterpret_cast<double *>(smem_raw);
+    const int tw = lay.tw, sw = tw + 2, ntile = (n + tw - 1) / tw, tn = tw * (nz0 - 2);
+    Tv *T0 = reinterpret_cast<Tv *>(smem_raw + lay.offT), *T1 = T0 + (size_t)tw * nz0;
+    Wv *lu0 = (Wv *)m.lu[0], *lf0 = (Wv *)m.lf[0];
     // position of unknown j in a line buffer
     auto at = [](int j) { return (j % M) * kRow + j / M; };
+    bool fail = false;
+    int g = 0;  // units done
     for (int cyc = 0;; ++cyc) {
-        // ---- residual of phi + delta, its norms, and the restriction chain ----
-        if (bid == 0 && L > 0) {
-            ld_begin(qC, FBc);
-            ld_copy(qC, FC, facc_v, FBc);
-        }
+        const unsigned tag = ep + 1u + (unsigned)cyc;
+        __syncthreads();  // the line buffers are read; the tile takes their place
         // maxima as bit patterns of |x| (ordered like the values; a NaN
         // compares above every number), so the reductions are integer work
         unsigned long long rmax = 0ull, bmax = 0ull;
-        {
-            const double *cz = m.cz[0], *cr = m.cr[0];
-            const int tw = lay.tw, sw = tw + 2;
-            // phi + delta of the tile and its two neighbour columns, all rows
-            double *S = reinterpret_cast<double *>(smem_raw + lay.offBuf);
-            // the restriction chain runs in the V-cycle's type
-            Tv *T0 = reinterpret_cast<Tv *>(smem_raw + lay.offF);
-            Tv *T1 = T0 + (size_t)tw * nz0;
-            Tv *f0v = mixed ? (Tv *)m.f32[0] : (Tv *)m.f64[0];
-            const int ntile = (n + tw - 1) / tw;
-            // the restriction chain of the residual tile T0 (columns j0 ..)
-            // down to the coarsest level, in the V-cycle's type
-            auto chain = [&](int j0) {
-        Tv *src = T0, *dst = T1;
-        int nzp = nz0;
-        for (int l = 1; l <= L; ++l) {
-            const int nzc = m.nz[l];
-            Tv *fl = mixed ? (Tv *)m.f32[l] : (Tv *)m.f64[l];
-            for (int e = tid; e < tw * (nzc - 2); e += nt) {
-                const int c = e % tw, I = 1 + e / tw, j = j0 + c;
-                const Tv *s = src + (size_t)c * nzp;
-                const Tv v = (Tv)0.5 * s[2 * I - 1] + s[2 * I] + (Tv)0.5 * s[2 * I + 1];
-                dst[(size_t)c * nzc + I] = v;
-                if (j < n) {
-                    const size_t k = (size_t)I * nr + j;
-                    if (l == L)
-                        m.fc64[k] = (double)v;
-                    else
-                        fl[k] = v;
+        const double *cz = m.cz[0], *cr = m.cr[0];
+        // the level-0 correction of the cycle before at the tile's nodes and
+        // its neighbour columns' (zero on the boundary), a batch per thread
+        auto delta_batch = [&](int e0, int j0, Tv (&dv)[kU]) {
+            const Wv *p[kU];
+#pragma unroll
+            for (int u = 0; u < kU; ++u) {
+                const int e = e0 + u * nt, c = e % sw - 1, i = e / sw, j = j0 + c;
+                p[u] = (e < sw * nz0 && j >= 0 && j < n && i > 0 && i < nz0 - 1) ? lu0 + (size_t)i * nr + j : nullptr;
+            }
+            flag_wait<Tv, kU>(p, dv, tag - 1u, &ctl->timeout, fail);
+        };
+        // the restriction chain of the residual tile T0 (columns j0 ..) down
+        // to the coarsest level, in the V-cycle's type: a warp per column
+        auto chain = [&](int j0) {
+            for (int c = warp; c < tw; c += nt / 32) {
+                const int j = j0 + c;
+                if (j >= n) break;
+                Tv *src = T0 + (size_t)c * nz0, *dst = T1 + (size_t)c * nz0;
+                for (int l = 1; l <= L; ++l) {
+                    const int nzc = m.nz[l];
+                    Wv *fl = (Wv *)m.lf[l];
+                    for (int I = 1 + lane; I < nzc - 1; I += 32) {
+                        const Tv v = (Tv)0.5 * src[2 * I - 1] + src[2 * I] + (Tv)0.5 * src[2 * I + 1];
+                        dst[I] = v;
+                        Fv::store(fl + (size_t)I * nr + j, v, tag);
+                    }
+                    __syncwarp();
+                    Tv *tmp = src;
+                    src = dst;
+                    dst = tmp;
                 }
             }
-            __syncthreads();
-            Tv *tmp = src;
-            src = dst;
-            dst = tmp;
-            nzp = nzc;
-        }
-            };
-            if (kry && cyc > 0) {
-                // ---- flexible GCR(1) step (mixed path) ----
-                // z: the V-cycle's correction of the last cycle; w = A z;
-                // the direction is z less its projection on the previous
-                // one (in the A-image), the step length minimises |r|_2
-                double a[4] = {0.0, 0.0, 0.0, 0.0};  // r.w, w.w, w.wp, r.wp
-                for (int t = bid; t < ntile; t += nbk) {
-                    const int j0 = t * tw;
-                    for (int e0 = tid; e0 < sw * nz0; e0 += kU * nt) {
-                        Tv dv[kU];
+        };
+        if (mixed && cyc > 0) {
+            // ---- flexible GCR(1) step (mixed path) ----
+            // z: the V-cycle's correction of the last cycle; w = A z; the
+            // direction is z less its projection on the previous one (in the
+            // A-image), the step length minimises |r|_2
+            double a[4] = {0.0, 0.0, 0.0, 0.0};  // r.w, w.w, w.wp, r.wp
+            for (int t = bid; t < ntile; t += P) {
+                const int j0 = t * tw;
+                for (int e0 = tid; e0 < sw * nz0; e0 += kU * nt) {
+                    Tv dv[kU];
+                    delta_batch(e0, j0, dv);
 #pragma unroll
-                        for (int u = 0; u < kU; ++u) {
-                            const int e = e0 + u * nt, c = e % sw - 1, i = e / sw, j = j0 + c;
-                            dv[u] = (e < sw * nz0 && j >= 0 && j < nr) ? delta[(size_t)i * nr + j] : (Tv)0;
-                        }
-#pragma unroll
-                        for (int u = 0; u < kU; ++u) {
-                            const int e = e0 + u * nt, c = e % sw - 1, i = e / sw;
-                            if (e < sw * nz0) S[(size_t)(c + 1) * nz0 + i] = (double)dv[u];
-                        }
+                    for (int u = 0; u < kU; ++u) {
+                        const int e = e0 + u * nt, c = e % sw - 1, i = e / sw;
+                        if (e < sw * nz0) St[(size_t)(c + 1) * nz0 + i] = (double)dv[u];
                     }
-                    __syncthreads();
-                    // batches of kU nodes per thread, loads first
-                    for (int e0 = tid; e0 < tw * (nz0 - 2); e0 += kU * nt) {
-                        double ca[kU], cb[kU], ce[kU], cd[kU], dgv[kU], rv[kU], wpv[kU];
-#pragma unroll
-                        for (int u = 0; u < kU; ++u) {
-                            const int e = e0 + u * nt, c = e % tw, i = 1 + e / tw, j = j0 + c;
-                            ca[u] = cb[u] = ce[u] = cd[u] = dgv[u] = rv[u] = wpv[u] = 0.0;
-                            if (e < tw * (nz0 - 2) && j < n) {
-                                const size_t k = (size_t)i * nr + j;
-                                ca[u] = cz[k - nr];
-                                cb[u] = cz[k];
-                                ce[u] = cr[k];
-                                cd[u] = j > 0 ? cr[k - 1] : 0.0;
-                                dgv[u] = m.dg0[k];
-                                rv[u] = m.kr[k];
-                                wpv[u] = m.kwp[k];
-                            }
-                        }
-#pragma unroll
-                        for (int u = 0; u < kU; ++u) {
-                            const int e = e0 + u * nt, c = e % tw, i = 1 + e / tw, j = j0 + c;
-                            if (e >= tw * (nz0 - 2) || j >= n) continue;
-                            const size_t k = (size_t)i * nr + j;
-                            const double *Sc = S + (size_t)(c + 1) * nz0 + i;
-                            const double w = dgv[u] * Sc[0] - ca[u] * Sc[-1] - cb[u] * Sc[1] - ce[u] * Sc[nz0] -
-                                             cd[u] * Sc[-nz0];
-                            m.kw[k] = w;
-                            a[0] += rv[u] * w;
-                            a[1] += w * w;
-                            a[2] += w * wpv[u];
-                            a[3] += rv[u] * wpv[u];
-                        }
-                    }
-                    __syncthreads();  // S is reused by the next tile
-                }
-                // the warp's four sums with few FP64 additions (the pipe is
-                // narrow): halves of the warp trade the products they do not
-                // keep (16 apart: 0, 1 stay low, 2, 3 high; 8 apart: one
-                // product per quarter), then each quarter sums its own;
-                // product 2 (lane >> 4) + ((lane >> 3) & 1) ends in the
-                // quarter's lanes
-                {
-                    const bool hi = lane >= 16, q1 = (lane & 8) != 0;
-                    const double s0 = __shfl_xor_sync(0xffffffffu, hi ? a[0] : a[2], 16);
-                    const double s1 = __shfl_xor_sync(0xffffffffu, hi ? a[1] : a[3], 16);
-                    const double b0 = (hi ? a[2] : a[0]) + s0, b1 = (hi ? a[3] : a[1]) + s1;
-                    double c = (q1 ? b1 : b0) + __shfl_xor_sync(0xffffffffu, q1 ? b0 : b1, 8);
-                    for (int o = 4; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-                    if ((lane & 7) == 0) s_dot[2 * (lane >> 4) + ((lane >> 3) & 1)][warp] = c;
                 }
                 __syncthreads();
-                if (tid < 4) {
-                    double v = 0.0;
-                    for (int q = 0; q < (nt >> 5); ++q) v += s_dot[tid][q];
-                    m.kpart[(size_t)bid * 4 + tid] = v;
+                const size_t q0 = (size_t)t * tn;
+                // batches of kU nodes per thread, loads first
+                for (int e0 = tid; e0 < tn; e0 += kU * nt) {
+                    double ca[kU], cb[kU], ce[kU], cd[kU], dgv[kU], rv[kU], wpv[kU];
+#pragma unroll
+                    for (int u = 0; u < kU; ++u) {
+                        const int e = e0 + u * nt, c = e % tw, i = 1 + e / tw, j = j0 + c;
+                        ca[u] = cb[u] = ce[u] = cd[u] = dgv[u] = rv[u] = wpv[u] = 0.0;
+                        if (e < tn && j < n) {
+                            const size_t k = (size_t)i * nr + j;
+                            ca[u] = cz[k - nr];
+                            cb[u] = cz[k];
+                            ce[u] = cr[k];
+                            cd[u] = j > 0 ? cr[k - 1] : 0.0;
+                            dgv[u] = m.dg0[k];
+                            rv[u] = m.kr[q0 + e];
+                            wpv[u] = m.kwp[q0 + e];
+                        }
+                    }
+#pragma unroll
+                    for (int u = 0; u < kU; ++u) {
+                        const int e = e0 + u * nt, c = e % tw, i = 1 + e / tw, j = j0 + c;
+                        if (e >= tn || j >= n) continue;
+                        const double *Sc = St + (size_t)(c + 1) * nz0 + i;
+                        const double w = dgv[u] * Sc[0] - ca[u] * Sc[-1] - cb[u] * Sc[1] - ce[u] * Sc[nz0] -
+                                         cd[u] * Sc[-nz0];
+                        m.kw[q0 + e] = w;
+                        a[0] += rv[u] * w;
+                        a[1] += w * w;
+                        a[2] += w * wpv[u];
+                        a[3] += rv[u] * wpv[u];
+                    }
                 }
-                if (!count_barrier(&ctl->bar_count.v, (++ngrid) * nbk, &ctl->timeout)) {
-                    leave(false);
+                if (t + P < ntile) __syncthreads();  // the tile is rewritten by the next
+            }
+            // the warp's four sums with few FP64 additions (the pipe is
+            // narrow): halves of the warp trade the products they do not
+            // keep (16 apart: 0, 1 stay low, 2, 3 high; 8 apart: one
+            // product per quarter), then each quarter sums its own;
+            // product 2 (lane >> 4) + ((lane >> 3) & 1) ends in the
+            // quarter's lanes
+            {
+                const bool hi = lane >= 16, q1 = (lane & 8) != 0;
+                const double s0 = __shfl_xor_sync(0xffffffffu, hi ? a[0] : a[2], 16);
+                const double s1 = __shfl_xor_sync(0xffffffffu, hi ? a[1] : a[3], 16);
+                const double b0 = (hi ? a[2] : a[0]) + s0, b1 = (hi ? a[3] : a[1]) + s1;
+                double c = (q1 ? b1 : b0) + __shfl_xor_sync(0xffffffffu, q1 ? b0 : b1, 8);
+                for (int o = 4; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+                if ((lane & 7) == 0) s_dot[0][2 * (lane >> 4) + ((lane >> 3) & 1)][warp] = c;
+            }
+            if (__syncthreads_or(fail)) {
+                leave(cyc);
+                return;
+            }
+            if (tid < 4) {
+                double v = 0.0;
+                for (int q = 0; q < nt / 32; ++q) v += s_dot[0][tid][q];
+                Flag<double>::store(m.xd + (size_t)bid * 4 + tid, v, tag);
+            }
+            // every block sums the partial products in the same fixed order
+            // (the same step length everywhere): thread t takes entries t,
+            // t + nt, ... of product t % 4 (nt is a multiple of 32)
+            {
+                double v = 0.0;
+                for (int e0 = tid; e0 < 4 * P; e0 += 2 * nt) {
+                    const ulonglong2 *p[2] = {m.xd + e0, e0 + nt < 4 * P ? m.xd + e0 + nt : nullptr};
+                    double x[2];
+                    flag_wait<double, 2>(p, x, tag, &ctl->timeout, fail);
+                    v += x[0];
+                    v += x[1];
+                }
+                for (int o = 4; o < 32; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+                if (lane < 4) s_dot[1][lane][warp] = v;
+                if (__syncthreads_or(fail)) {
+                    leave(cyc);
                     return;
                 }
-                // every block sums the partial products in the same fixed
-                // order (the same step length everywhere), all its threads
-                // loading at once: thread t takes entries t, t + nt, ... of
-                // product t % 4 (nt is a multiple of 32)
-                {
-                    double v = 0.0;
-#pragma unroll 4
-                    for (int e = tid; e < 4 * nbk; e += nt) v += m.kpart[e];
-                    for (int o = 4; o < 32; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-                    if (lane < 4) s_dot[lane][warp] = v;
-                    __syncthreads();
-                    if (tid < 4) {
-                        double t = 0.0;
-                        for (int q = 0; q < (nt >> 5); ++q) t += s_dot[tid][q];
-                        s_sum[tid] = t;
-                    }
-                    __syncthreads();
-                    // the step's scalars by one thread: GB300's FP64 pipe is
-                    // narrow, and every thread dividing cost microseconds
-                    if (tid == 0) {
-                        const double beta = kc > 0.0 ? s_sum[2] / kc : 0.0;
-                        const double den = s_sum[1] - beta * s_sum[2];
+                // the step's scalars by one thread: GB300's FP64 pipe is
+                // narrow, and every thread dividing cost microseconds
+                if (warp == 0) {
+                    double t = 0.0;
+                    if (lane < 4)
+                        for (int q = 0; q < nt / 32; ++q) t += s_dot[1][lane][q];
+                    const double rw = __shfl_sync(0xffffffffu, t, 0), ww = __shfl_sync(0xffffffffu, t, 1),
+                                 wwp = __shfl_sync(0xffffffffu, t, 2), rwp = __shfl_sync(0xffffffffu, t, 3);
+                    if (lane == 0) {
+                        const double beta = kc > 0.0 ? wwp / kc : 0.0;
+                        const double den = ww - beta * wwp;
                         s_ab[0] = beta;
-                        s_ab[1] = den > 0.0 ? (s_sum[0] - beta * s_sum[3]) / den : 1.0;
+                        s_ab[1] = den > 0.0 ? (rw - beta * rwp) / den : 1.0;
                         s_ab[2] = den > 0.0 ? den : 0.0;
                     }
-                    __syncthreads();
                 }
-                const double beta = s_ab[0], alpha = s_ab[1];
-                kc = s_ab[2];
-                __syncthreads();  // s_sum and s_ab are rewritten by the next cycle
-                for (int t = bid; t < ntile; t += nbk) {
-                    const int j0 = t * tw;
-                    for (int e0 = tid; e0 < tw * (nz0 - 2); e0 += kU * nt) {
-                        double pz[kU], qw[kU], zp[kU], wpv[kU], xv[kU], rv[kU];
+                __syncthreads();
+            }
+            const double beta = s_ab[0], alpha = s_ab[1];
+            kc = s_ab[2];
+            const bool one = bid + P >= ntile;  // the block's only tile: z is still in St
+            for (int t = bid; t < ntile; t += P) {
+                const int j0 = t * tw;
+                const size_t q0 = (size_t)t * tn;
+                for (int e0 = tid; e0 < tn; e0 += kU * nt) {
+                    double pz[kU], qw[kU], zp[kU], wpv[kU], xv[kU], rv[kU];
 #pragma unroll
-                        for (int u = 0; u < kU; ++u) {
-                            const int e = e0 + u * nt, c = e % tw, i = 1 + e / tw, j = j0 + c;
-                            pz[u] = qw[u] = zp[u] = wpv[u] = xv[u] = rv[u] = 0.0;
-                            if (e < tw * (nz0 - 2) && j < n) {
-                                const size_t k = (size_t)i * nr + j;
-                                pz[u] = (double)delta[k];
-                                qw[u] = m.kw[k];
-                                if (beta != 0.0) {
-                                    zp[u] = m.kzp[k];
-                                    wpv[u] = m.kwp[k];
-                                }
-                                xv[u] = cur[k];
-                                rv[u] = m.kr[k];
+                    for (int u = 0; u < kU; ++u) {
+                        const int e = e0 + u * nt, c = e % tw, i = 1 + e / tw, j = j0 + c;
+                        pz[u] = qw[u] = zp[u] = wpv[u] = xv[u] = rv[u] = 0.0;
+                        if (e < tn && j < n) {
+                            const size_t k = (size_t)i * nr + j;
+                            pz[u] = one ? St[(size_t)(c + 1) * nz0 + i] : (double)Fv::value(Fv::load(lu0 + k));
+                            qw[u] = m.kw[q0 + e];
+                            if (beta != 0.0) {
+                                zp[u] = m.kzp[q0 + e];
+                                wpv[u] = m.kwp[q0 + e];
                             }
-                        }
-#pragma unroll
-                        for (int u = 0; u < kU; ++u) {
-                            const int e = e0 + u * nt, c = e % tw, i = 1 + e / tw, j = j0 + c;
-                            if (e >= tw * (nz0 - 2)) break;
-                            double rn = 0.0;
-                            if (j < n) {
-                                const size_t k = (size_t)i * nr + j;
-                                const double p = pz[u] - beta * zp[u], q = qw[u] - beta * wpv[u];
-                                nxt[k] = xv[u] + alpha * p;
-                                rn = rv[u] - alpha * q;
-                                m.kr[k] = rn;
-                                m.kzp[k] = p;
-                                m.kwp[k] = q;
-                                rmax = max(rmax, abs_bits(rn));
-                                f0v[k] = (Tv)rn;
-                            }
-                            T0[(size_t)c * nz0 + i] = (Tv)rn;
+                            xv[u] = phi[k];
+                            rv[u] = m.kr[q0 + e];
                         }
                     }
-                    __syncthreads();
-                    chain(j0);
+#pragma unroll
+                    for (int u = 0; u < kU; ++u) {
+                        const int e = e0 + u * nt, c = e % tw, i = 1 + e / tw, j = j0 + c;
+                        if (e >= tn) break;
+                        double rn = 0.0;
+                        if (j < n) {
+                            const size_t k = (size_t)i * nr + j;
+                            const double p = pz[u] - beta * zp[u], q = qw[u] - beta * wpv[u];
+                            phi[k] = xv[u] + alpha * p;
+                            rn = rv[u] - alpha * q;
+                            m.kr[q0 + e] = rn;
+                            m.kzp[q0 + e] = p;
+                            m.kwp[q0 + e] = q;
+                            rmax = max(rmax, abs_bits(rn));
+                            Fv::store(lf0 + k, (Tv)rn, tag);
+                        }
+                        T0[(size_t)c * nz0 + i] = (Tv)rn;
+                    }
                 }
-            } else
-            for (int t = bid; t < ntile; t += nbk) {
+                __syncthreads();
+                chain(j0);
+                if (t + P < ntile) __syncthreads();
+            }
+        } else {
+            for (int t = bid; t < ntile; t += P) {
                 const int j0 = t * tw;
-                // batches of kU elements per thread: all loads first (stores to
-                // global memory would otherwise hold back the next loads)
+                // phi of the tile and its two neighbour columns, all rows: the
+                // iterate at first, then (FP64 path) the tile's own copy plus
+                // the correction; batches of kU elements per thread, loads first
+                double *own = m.ps + (size_t)t * sw * nz0;
                 for (int e0 = tid; e0 < sw * nz0; e0 += kU * nt) {
                     double pv[kU];
                     Tv dv[kU];
@@ -726,31 +800,30 @@ __device__ __forceinline__ void solve_body(const MGFast *__restrict__ mp, double
                         const int e = e0 + u * nt, c = e % sw - 1, i = e / sw, j = j0 + c;
                         pv[u] = 0.0;
                         dv[u] = 0;
-                        if (e < sw * nz0 && j >= 0 && j < nr) {
-                            const size_t k = (size_t)i * nr + j;
-                            pv[u] = cur[k];
-                            dv[u] = delta[k];
-                        }
+                        if (e < sw * nz0 && j >= 0 && j < nr) pv[u] = cyc > 0 ? own[e] : phi[(size_t)i * nr + j];
                     }
+                    if (cyc > 0) delta_batch(e0, j0, dv);
 #pragma unroll
                     for (int u = 0; u < kU; ++u) {
                         const int e = e0 + u * nt, c = e % sw - 1, i = e / sw, j = j0 + c;
                         if (e >= sw * nz0) break;
                         const double v = pv[u] + (double)dv[u];
-                        // the iterate of the next cycle, stored by the tile that owns the node
-                        if (dbuf && c >= 0 && c < tw && j < n && i > 0 && i < nz0 - 1) nxt[(size_t)i * nr + j] = v;
-                        S[(size_t)(c + 1) * nz0 + i] = v;
+                        if (!mixed) own[e] = v;
+                        // the iterate, stored by the tile that owns the node
+                        if (cyc > 0 && c >= 0 && c < tw && j < n && i > 0 && i < nz0 - 1) phi[(size_t)i * nr + j] = v;
+                        St[(size_t)(c + 1) * nz0 + i] = v;
                     }
                 }
                 __syncthreads();
+                const size_t q0 = (size_t)t * tn;
                 // interior rows only: the chain never reads a level's boundary rows
-                for (int e0 = tid; e0 < tw * (nz0 - 2); e0 += kU * nt) {
+                for (int e0 = tid; e0 < tn; e0 += kU * nt) {
                     double ca[kU], cb[kU], ce[kU], cd[kU], dgv[kU], fv[kU];
 #pragma unroll
                     for (int u = 0; u < kU; ++u) {
                         const int e = e0 + u * nt, c = e % tw, i = 1 + e / tw, j = j0 + c;
                         ca[u] = cb[u] = ce[u] = cd[u] = dgv[u] = fv[u] = 0.0;
-                        if (e < tw * (nz0 - 2) && j < n) {
+                        if (e < tn && j < n) {
                             const size_t k = (size_t)i * nr + j;
                             ca[u] = cz[k - nr];
                             cb[u] = cz[k];
@@ -762,297 +835,210 @@ __device__ __forceinline__ void solve_body(const MGFast *__restrict__ mp, double
                     }
 #pragma unroll
                     for (int u = 0; u < kU; ++u) {
-                    const int e = e0 + u * nt, c = e % tw, i = 1 + e / tw, j = j0 + c;
-                    if (e >= tw * (nz0 - 2)) break;
-                    double r = 0.0;
-                    if (j < n) {
-                        const size_t k = (size_t)i * nr + j;
-                        const double *Sc = S + (size_t)(c + 1) * nz0 + i;
-                        const double a = ca[u], cc = cb[u], ee = ce[u], d = cd[u];
-                        const double Au = dgv[u] * Sc[0] - a * Sc[-1] - cc * Sc[1] - ee * Sc[nz0] - d * Sc[-nz0];
-                        const double f = fv[u];
-                        r = f - Au;
-                        rmax = max(rmax, abs_bits(r));
-                        if (first) {
-                            double bb = f;
-                            if (i == 1) bb += a * Sc[-1];
-                            if (i == nz0 - 2) bb += cc * Sc[1];
-                            if (j == nr - 2) bb += ee * Sc[nz0];
-                            bmax = max(bmax, abs_bits(bb));
+                        const int e = e0 + u * nt, c = e % tw, i = 1 + e / tw, j = j0 + c;
+                        if (e >= tn) break;
+                        double r = 0.0;
+                        if (j < n) {
+                            const size_t k = (size_t)i * nr + j;
+                            const double *Sc = St + (size_t)(c + 1) * nz0 + i;
+                            const double a = ca[u], cc = cb[u], ee = ce[u], d = cd[u];
+                            const double Au = dgv[u] * Sc[0] - a * Sc[-1] - cc * Sc[1] - ee * Sc[nz0] - d * Sc[-nz0];
+                            const double f = fv[u];
+                            r = f - Au;
+                            rmax = max(rmax, abs_bits(r));
+                            if (cyc == 0) {
+                                double bb = f;
+                                if (i == 1) bb += a * Sc[-1];
+                                if (i == nz0 - 2) bb += cc * Sc[1];
+                                if (j == nr - 2) bb += ee * Sc[nz0];
+                                bmax = max(bmax, abs_bits(bb));
+                            }
+                            Fv::store(lf0 + k, (Tv)r, tag);
+                            if (mixed) m.kr[q0 + e] = r;
                         }
-                        if (L > 0) f0v[k] = (Tv)r;
-                        if (kry) m.kr[k] = r;
-                    }
-                    T0[(size_t)c * nz0 + i] = (Tv)r;
+                        T0[(size_t)c * nz0 + i] = (Tv)r;
                     }
                 }
                 __syncthreads();
                 chain(j0);
-            }
-            for (int o = 16; o > 0; o >>= 1) {
-                rmax = max(rmax, __shfl_xor_sync(0xffffffffu, rmax, o));
-                bmax = max(bmax, __shfl_xor_sync(0xffffffffu, bmax, o));
-            }
-            if (lane == 0) {
-                s_r[warp] = rmax;
-                s_b[warp] = bmax;
-            }
-            __syncthreads();
-            if (tid < 32) {
-                unsigned long long r = tid < (nt >> 5) ? s_r[tid] : 0ull;
-                unsigned long long b = tid < (nt >> 5) ? s_b[tid] : 0ull;
-                for (int o = 16; o > 0; o >>= 1) {
-                    r = max(r, __shfl_xor_sync(0xffffffffu, r, o));
-                    b = max(b, __shfl_xor_sync(0xffffffffu, b, o));
-                }
-                if (tid == 0) {
-                    atomicMax(&ctl->rb[cyc & 1], r);
-                    if (first) atomicMax(&ctl->b_bits, b);
-                }
+                if (t + P < ntile) __syncthreads();
             }
         }
-        if (!count_barrier(&ctl->bar_count.v, (++ngrid) * nbk, &ctl->timeout)) {
-            leave(false);
-            return;
-        }
-        // ---- decision: every block reads the same maxima ----
+        // ---- decision: every block reads every block's maxima ----
+        block_max2(rmax, bmax, s_max[0]);
+        // (two sets in turn: a block that owns no unit may still be reading the
+        // norms of the cycle before)
+        ulonglong2 *xr = m.xr + (size_t)(cyc & 1) * 2 * kMaxSolveBlocks;
         if (tid == 0) {
-            const double rn = __longlong_as_double((long long)*(volatile unsigned long long *)&ctl->rb[cyc & 1]);
-            const double bn = __longlong_as_double((long long)*(volatile unsigned long long *)&ctl->b_bits);
-            int d = 0;  // 0 continue, 1 converged, 2 out of cycles, 3 zero right-hand side
-            if (bn == 0.0)
-                d = 3;
-            else if (tol > 0.0 && rn <= tol * bn)
-                d = 1;
-            else if (cyc >= max_cycles)
-                d = tol > 0.0 ? 2 : 1;
-            s_decide = d;
-            if (bid == 0) {
-                ctl->last_res = rn;
-                ctl->bnorm = bn;
-                ctl->cycles = cyc;
-                ctl->rb[(cyc + 1) & 1] = 0ull;  // read by all blocks one cycle ago
-                if (d == 1) ctl->converged = 1;
-                if (d == 3) ctl->zero_rhs = 1;
-            }
+            Flag<double>::store(xr + 2 * bid, __longlong_as_double((long long)rmax), tag);
+            if (cyc == 0) Flag<double>::store(xr + 2 * bid + 1, __longlong_as_double((long long)bmax), tag);
         }
-        __syncthreads();
-        const int decide = s_decide;
-        first = 0;
-        if (decide == 3) {
-            for (int k = bid * nt + tid; k < ng; k += nbk * nt) {
-                const int i = k / nr, j = k % nr;
-                if (i > 0 && i < nz0 - 1 && j < nr - 1) phi[k] = 0.0;
-            }
-            leave(false);
+        rmax = bmax = 0ull;
+        for (int e = tid; e < P; e += nt) {
+            const ulonglong2 *p[2] = {xr + 2 * e, cyc == 0 ? xr + 2 * e + 1 : nullptr};
+            double x[2];
+            flag_wait<double, 2>(p, x, tag, &ctl->timeout, fail);
+            rmax = max(rmax, (unsigned long long)__double_as_longlong(x[0]));
+            bmax = max(bmax, (unsigned long long)__double_as_longlong(x[1]));
+        }
+        block_max2(rmax, bmax, s_max[1]);
+        if (__syncthreads_or(fail)) {
+            leave(cyc);
             return;
         }
-        if (decide != 0) {
-            // the answer is the iterate the residual phase just stored
-            if (dbuf && nxt != phi)
-                for (int k = bid * nt + tid; k < ng; k += nbk * nt) {
-                    const int i = k / nr, j = k % nr;
-                    if (i > 0 && i < nz0 - 1 && j < nr - 1) phi[k] = nxt[k];
+        const double rn = __longlong_as_double((long long)rmax);
+        if (cyc == 0) bn = __longlong_as_double((long long)bmax);
+        int decide = 0;  // 0 continue, 1 converged, 2 out of cycles, 3 zero right-hand side
+        if (bn == 0.0)
+            decide = 3;
+        else if (tol > 0.0 && rn <= tol * bn)
+            decide = 1;
+        else if (cyc >= max_cycles)
+            decide = tol > 0.0 ? 2 : 1;
+        if (bid == 0 && tid == 0) {
+            ctl->last_res = rn;
+            ctl->bnorm = bn;
+            ctl->cycles = cyc;
+            if (decide == 1) ctl->converged = 1;
+            if (decide == 3) ctl->zero_rhs = 1;
+        }
+        if (decide == 3)
+            for (int t = bid; t < ntile; t += P)
+                for (int e = tid; e < tn; e += nt) {
+                    const int j = t * tw + e % tw;
+                    if (j < n) phi[(size_t)(1 + e / tw) * nr + j] = 0.0;
                 }
-            leave(false);
+        if (decide != 0) {  // phi holds the iterate of this residual
+            leave(cyc);
             return;
         }
-        if (dbuf) {
-            double *t = cur;
-            cur = nxt;
-            nxt = t;
-        }
-        if (L == 0) {
-            // nz = 3: the single interior row of phi, exactly
-            if (bid == 0) {
-                ld_begin(qC, FBd);
-                ld_copy(qC, FC64, m.facc, FBd);
-                const double *cz = m.cz[0], *cr = m.cr[0];
-                for (int j = tid; j < NW; j += nt) {
-                    double rhs = 0.0;
-                    if (j < n) {
-                        const size_t k = (size_t)nr + j;
-                        rhs = m.f0[k] + cz[k - nr] * phi[k - nr] + cz[k] * phi[k + nr];
-                        if (j == n - 1) rhs += cr[k] * phi[k + 1];
-                    }
-                    BC[at(j)] = rhs;
-                }
-                __syncthreads();
-                if (!ld_wait(qC)) {
-                    leave(true);
+        // ---- up: per unit, a black line with the two red lines beside it ----
+        constexpr int kE = (NW + nt - 1) / nt;  // unknowns of a line per thread
+        for (int k = 0; k < nun; ++k, ++g) {
+            int l, q;
+            unit_at(bid + k * P, l, q);
+            const int nzl = m.nz[l], nzc = m.nz[l + 1], slot = nun <= S ? k : g % S;
+            const int ra = 2 * q + 1, rb = 2 * q + 3, ib = 2 * q + 2;
+            Wv *u = (Wv *)m.lu[l];
+            const Wv *uc = (const Wv *)m.lu[l + 1], *f = (const Wv *)m.lf[l];
+            const Tv *czl = mixed ? (const Tv *)m.cz32[l] : (const Tv *)m.cz[l];
+            // coarse rows below ra, between (row ib) and above rb; the level's
+            // ends are zero
+            const int Ia = q, Im = q + 1, Ib = q + 2;
+            const bool va = Ia > 0, vb = Ib < nzc - 1;
+            Tv um0[kE];  // level L-1: the coarsest row, solved here
+            if (l == L - 1) {
+                const Wv *fc = (const Wv *)m.lf[L];
+                const Wv *p[kE];
+                Tv x[kE];
+#pragma unroll
+                for (int s = 0; s < kE; ++s) p[s] = tid + s * nt < n ? fc + nr + tid + s * nt : nullptr;
+                flag_wait<Tv, kE>(p, x, tag, &ctl->timeout, fail);
+#pragma unroll
+                for (int s = 0; s < kE; ++s)
+                    if (tid + s * nt < NW) Bf0[at(tid + s * nt)] = x[s];
+                if (!ld_wait(ld, kMaxSlots)) fail = true;
+                if (__syncthreads_or(fail)) {
+                    if (tid == 0) atomicExch(&ctl->timeout, 1);
+                    leave(cyc);
                     return;
                 }
-                if (warp == 0) warp_line_solve<double, M>(FC64, BC, lane);
+                if (warp == 0) warp_line_solve<Tv, M>(FC, Bf0, lane);
                 __syncthreads();
-                for (int j = tid; j < n; j += nt) phi[(size_t)nr + j] = BC[at(j)];
-            }
-            if (!count_barrier(&ctl->bar_count.v, (++ngrid) * nbk, &ctl->timeout)) {
-                leave(false);
-                return;
-            }
-            continue;
-        }
-        // level 0's sweeps rewrite delta: when they run in the group alone,
-        // every block's update of phi has to be in first
-        if (lb == 0)
-            if (!count_barrier(&ctl->bar_count.v, (++ngrid) * nbk, &ctl->timeout)) {
-                leave(false);
-                return;
-            }
-        // ---- up: per level, each black line with the two red lines beside it ----
-        bool have = false;  // this block's first red factors of the level are requested
-        for (int l = L - 1; l >= 0; --l) {
-            const bool grp = l >= lb;
-            const int P = grp ? G : nbk;
-            const int nzl = m.nz[l], nzc = m.nz[l + 1];
-            const int NB = (nzl - 3) / 2;  // black lines (>= 1: nzl >= 5 here)
-            Tv *u = mixed ? (Tv *)m.u32[l] : (Tv *)m.u64[l];
-            const Tv *uc = mixed ? (const Tv *)m.u32[l + 1] : (const Tv *)m.u64[l + 1];
-            const Tv *f = mixed ? (const Tv *)m.f32[l] : (const Tv *)m.f64[l];
-            const Tv *cz = mixed ? (const Tv *)m.cz32[l] : (const Tv *)m.cz[l];
-            const Tv *fac = mixed ? (const Tv *)m.fac32[l] : (const Tv *)m.fac64[l];
-            bool fail = false;
-            if (bid < P) {
-                if (l == L - 1 && bid == 0) {
-                    // the coarsest row (FP64 factors, requested with the residual),
-                    // then level L-1 in this block alone
-                    for (int j = tid; j < NW; j += nt) Bf0[at(j)] = j < n ? (Tv)m.fc64[(size_t)nr + j] : (Tv)0;
-                    __syncthreads();
-                    if (!ld_wait(qC)) {
-                        leave(true);
-                        return;
-                    }
-                    if (warp == 0) warp_line_solve<Tv, M>(FC, Bf0, lane);
-                    __syncthreads();
-                    Tv *ucw = mixed ? (Tv *)m.u32[L] : (Tv *)m.u64[L];
-                    for (int j = tid; j < n; j += nt) ucw[(size_t)nr + j] = Bf0[at(j)];
-                    __syncthreads();
-                    have = false;
-                }
-                for (int q = bid; q < NB; q += P) {
-                    const int ra = 2 * q + 1, rb = 2 * q + 3, ib = 2 * q + 2;
-                    // factor requests: the reds (unless already in), then the black
-                    if (!(have && q == bid)) {
-                        ld_begin(qR, 2 * FBv);
-                        ld_copy(qR, R0, fac + (size_t)(ra - 1) * LFE, FBv);
-                        ld_copy(qR, R1, fac + (size_t)(rb - 1) * LFE, FBv);
-                    }
-                    ld_begin(qB, FBv);
-                    ld_copy(qB, FBk, fac + (size_t)(ib - 1) * LFE, FBv);
-                    have = false;
-                    // right-hand sides: reds get f plus the coarse correction
-                    // injected at rows i -/+ 1; the black line keeps its own f
-                    // and couplings for later
-                    const int Ia = (ra - 1) / 2, Ib = (rb + 1) / 2;  // coarse rows below ra, above rb
-                    const int Im = (ra + 1) / 2;                     // coarse row between (= row ib)
-                    const bool va = Ia > 0 && Ia < nzc - 1, vm = Im > 0 && Im < nzc - 1, vb = Ib > 0 && Ib < nzc - 1;
-                    for (int j0 = tid; j0 < NW; j0 += kUL * nt) {
-                        // rows ra, ib = ra + 1, rb = ra + 2: cz[ib - 1] = cz[ra], cz[ib] = cz[rb - 1]
-                        Tv ua[kUL], um[kUL], ub[kUL], fa[kUL], fbv[kUL], fk[kUL], z0[kUL], z1[kUL], z2[kUL], z3[kUL];
 #pragma unroll
-                        for (int u = 0; u < kUL; ++u) {
-                            const int j = j0 + u * nt;
-                            ua[u] = um[u] = ub[u] = fa[u] = fbv[u] = fk[u] = z0[u] = z1[u] = z2[u] = z3[u] = 0;
-                            if (j < n) {
-                                const size_t ka = (size_t)ra * nr + j;
-                                if (va) ua[u] = uc[(size_t)Ia * nr + j];
-                                if (vm) um[u] = uc[(size_t)Im * nr + j];
-                                if (vb) ub[u] = uc[(size_t)Ib * nr + j];
-                                fa[u] = f[ka];
-                                fk[u] = f[ka + nr];
-                                fbv[u] = f[ka + 2 * nr];
-                                z0[u] = cz[ka - nr];
-                                z1[u] = cz[ka];
-                                z2[u] = cz[ka + nr];
-                                z3[u] = cz[ka + 2 * nr];
-                            }
-                        }
+                for (int s = 0; s < kE; ++s) um0[s] = tid + s * nt < NW ? Bf0[at(tid + s * nt)] : (Tv)0;
+            }
+            // rows ra, ib = ra + 1, rb = ra + 2: cz[ib - 1] = cz[ra], cz[ib] = cz[rb - 1]
+            Tv z[4][kE], fx[3 * kE], ux[3 * kE];
+            {
+                const Wv *p[3 * kE];
 #pragma unroll
-                        for (int u = 0; u < kUL; ++u) {
-                            const int j = j0 + u * nt;
-                            if (j >= NW) break;
-                            const int pj = at(j);
-                            Bf0[pj] = fa[u] + z0[u] * ua[u] + z1[u] * um[u];
-                            Bf1[pj] = fbv[u] + z2[u] * um[u] + z3[u] * ub[u];
-                            Bf2[pj] = fk[u];
-                            W0[j] = z1[u];
-                            W1[j] = z2[u];
-                        }
-                    }
-                    __syncthreads();
-                    if (!ld_wait(qR)) {
-                        fail = true;
-                        break;
-                    }
-                    if (warp == 0)
-                        warp_line_solve<Tv, M>(R0, Bf0, lane);
-                    else if (warp == 1)
-                        warp_line_solve<Tv, M>(R1, Bf1, lane);
-                    __syncthreads();
-                    for (int j = tid; j < NW; j += nt) {
-                        const int pj = at(j);
-                        const Tv x0 = Bf0[pj], x1 = Bf1[pj];
-                        if (j < n) {
-                            u[(size_t)ra * nr + j] = x0;
-                            // red rb is also the next black's red ra: one block stores it
-                            if (q == NB - 1) u[(size_t)rb * nr + j] = x1;
-                            Bf2[pj] = Bf2[pj] + W0[j] * x0 + W1[j] * x1;
-                        }
-                    }
-                    __syncthreads();
-                    if (!ld_wait(qB)) {
-                        fail = true;
-                        break;
-                    }
-                    if (warp == 0) warp_line_solve<Tv, M>(FBk, Bf2, lane);
-                    __syncthreads();
-                    for (int j = tid; j < n; j += nt) u[(size_t)ib * nr + j] = Bf2[at(j)];
-                    __syncthreads();  // buffers and factor regions are reused
+                for (int s = 0; s < kE; ++s) {
+                    const int j = tid + s * nt;
+#pragma unroll
+                    for (int w = 0; w < 4; ++w) z[w][s] = j < n ? czl[(size_t)(2 * q + w) * nr + j] : (Tv)0;
+#pragma unroll
+                    for (int w = 0; w < 3; ++w) p[3 * s + w] = j < n ? f + (size_t)(ra + w) * nr + j : nullptr;
                 }
-                // request the next level's first red factors of this block
-                if (!fail && l > 0) {
-                    const int ln = l - 1;
-                    const int Pn = ln >= lb ? G : nbk;
-                    const int nbn = (m.nz[ln] - 3) / 2;
-                    if (bid < Pn && bid < nbn) {
-                        const Tv *facn = mixed ? (const Tv *)m.fac32[ln] : (const Tv *)m.fac64[ln];
-                        const int q = bid;
-                        ld_begin(qR, 2 * FBv);
-                        ld_copy(qR, R0, facn + (size_t)(2 * q) * LFE, FBv);
-                        ld_copy(qR, R1, facn + (size_t)(2 * q + 2) * LFE, FBv);
-                        have = true;
+                flag_wait<Tv, 3 * kE>(p, fx, tag, &ctl->timeout, fail);
+                if (l < L - 1) {
+#pragma unroll
+                    for (int s = 0; s < kE; ++s) {
+                        const int j = tid + s * nt;
+                        p[3 * s] = j < n && va ? uc + (size_t)Ia * nr + j : nullptr;
+                        p[3 * s + 1] = j < n ? uc + (size_t)Im * nr + j : nullptr;
+                        p[3 * s + 2] = j < n && vb ? uc + (size_t)Ib * nr + j : nullptr;
+                    }
+                    flag_wait<Tv, 3 * kE>(p, ux, tag, &ctl->timeout, fail);
+                } else {
+#pragma unroll
+                    for (int s = 0; s < kE; ++s) {
+                        ux[3 * s] = ux[3 * s + 2] = 0;
+                        ux[3 * s + 1] = um0[s];
                     }
                 }
             }
-            if (fail) {
-                leave(true);
+            // right-hand sides: reds get f plus the coarse correction injected
+            // at rows i -/+ 1; the black line keeps its own f and couplings
+#pragma unroll
+            for (int s = 0; s < kE; ++s) {
+                const int j = tid + s * nt;
+                if (j >= NW) break;
+                const int pj = at(j);
+                Bf0[pj] = fx[3 * s] + z[0][s] * ux[3 * s] + z[1][s] * ux[3 * s + 1];
+                Bf1[pj] = fx[3 * s + 2] + z[2][s] * ux[3 * s + 1] + z[3][s] * ux[3 * s + 2];
+                Bf2[pj] = fx[3 * s + 1];
+                W0[j] = z[1][s];
+                W1[j] = z[2][s];
+            }
+            if (!ld_wait(ld, slot)) fail = true;
+            if (__syncthreads_or(fail)) {
+                if (tid == 0) atomicExch(&ctl->timeout, 1);
+                leave(cyc);
                 return;
             }
-            // levels in the group alone are separated by the group barrier;
-            // every other level boundary is a grid barrier
-            bool ok;
-            if (l > 0 && grp && l - 1 >= lb)
-                ok = in_group ? count_barrier(&ctl->gbar_count.v, (++ngroup) * G, &ctl->timeout) : true;
-            else
-                ok = count_barrier(&ctl->bar_count.v, (++ngrid) * nbk, &ctl->timeout);
-            if (!ok) {
-                leave(false);
-                return;
+            const Tv *F = slots + (size_t)slot * 3 * LFE;
+            if (warp == 0)
+                warp_line_solve<Tv, M>(F, Bf0, lane);
+            else if (warp == 1)
+                warp_line_solve<Tv, M>(F + 2 * LFE, Bf1, lane);
+            __syncthreads();
+#pragma unroll
+            for (int s = 0; s < kE; ++s) {
+                const int j = tid + s * nt;
+                if (j >= n) break;
+                const int pj = at(j);
+                const Tv x0 = Bf0[pj], x1 = Bf1[pj];
+                Fv::store(u + (size_t)ra * nr + j, x0, tag);
+                // red rb is also the next black's red ra: one unit stores it
+                if (rb == nzl - 2) Fv::store(u + (size_t)rb * nr + j, x1, tag);
+                Bf2[pj] = Bf2[pj] + W0[j] * x0 + W1[j] * x1;
+            }
+            __syncthreads();
+            if (warp == 0) warp_line_solve<Tv, M>(F + LFE, Bf2, lane);
+            __syncthreads();
+            if (nun > S) request(g + S, slot);
+#pragma unroll
+            for (int s = 0; s < kE; ++s) {
+                const int j = tid + s * nt;
+                if (j < n) Fv::store(u + (size_t)ib * nr + j, Bf2[at(j)], tag);
             }
         }
     }
 }
 
+// MINB: blocks per SM the registers must allow: one for a reactor's solve
+// alone, two for the solves of a batch of reactors, which share SMs.
 template <typename Tv, int M, int MINB>
 __global__ void __launch_bounds__(kSolveThreads, MINB)
-    k_solve_persistent(const MGFast *__restrict__ mp, double *phi, int nr, int first_cycle, SolveLayout lay,
-                       double tol, int max_cycles, const StepCtl *sctl) {
-    solve_body<Tv, M>(mp, phi, nr, first_cycle, lay, tol, max_cycles, sctl, blockIdx.x, gridDim.x);
+    k_solve_persistent(const MGFast *__restrict__ mp, double *phi, int nr, SolveLayout lay, double tol,
+                       int max_cycles, const StepCtl *sctl) {
+    solve_body<Tv, M>(mp, phi, nr, lay, tol, max_cycles, sctl, blockIdx.x, gridDim.x);
 }
 
 // The solves of several reactors (one line chunk M, one precision) in one
-// cooperative launch: job k takes blocks [block0, block0 + nblocks) and its
-// barriers count its own blocks only, so the reactors proceed side by side.
+// cooperative launch: job k takes blocks [block0, block0 + nblocks) and hands
+// its words to its own blocks only, so the reactors proceed side by side.
 template <typename Tv, int M, int MINB>
 __global__ void __launch_bounds__(kSolveThreads, MINB) k_solve_multi(const SolveJob *__restrict__ jobs, int njobs) {
     int lo = 0, hi = njobs - 1;  // the job whose block range holds this block
@@ -1066,12 +1052,15 @@ __global__ void __launch_bounds__(kSolveThreads, MINB) k_solve_multi(const Solve
     const SolveJob &j = jobs[lo];
     const int bid = (int)blockIdx.x - j.block0;
     if (bid >= j.nblocks) return;
-    solve_body<Tv, M>(j.mp, j.phi, j.nr, j.first_cycle, j.lay, j.tol, j.max_cycles, j.sctl, bid, j.nblocks);
+    solve_body<Tv, M>(j.mp, j.phi, j.nr, j.lay, j.tol, j.max_cycles, j.sctl, bid, j.nblocks);
 }
 
 }  // namespace
 
 size_t mg_line_factor_elems(int nr) { return (size_t)line_factor_elems(line_chunk(nr - 1)); }
+
+// tiles of one to eight columns, the last one whole, with two neighbour columns each
+size_t mg_tile_elems(int nz, int nr) { return (size_t)nz * (nr + 8) * 3; }
 
 int mg_line_chunk(int nr) { return line_chunk(nr - 1); }
 
@@ -1201,41 +1190,59 @@ bool solve_job(const FieldDims &fd, MGFast &m, double *phi, bool mixed, double t
     const size_t es = mixed ? sizeof(float) : sizeof(double);
     const size_t LFE = (size_t)line_factor_elems(M);
     SolveLayout lay{};
-    // wide: residual tiles of 4 columns over two blocks per black line: the
-    // residual phase (FP64 stencil, restriction chain) runs on twice the SMs
-    // the line phases need; the remaining SMs stay free for the cell sort
-    // that runs beside the solve in a timestep (measured on c2: 0.551 ->
-    // 0.518 ms per solve; three blocks per line leave the sort too few SMs).
-    // Narrow (one block per black line, tiles of 8): many reactors solving
-    // side by side each take fewer SMs.
-    lay.tw = wide ? 4 : 8;
+    const int L = m.nlev - 1;
     size_t off = 0;
     auto take = [&](size_t b) {
         const size_t o = off;
         off += (b + 127) & ~(size_t)127;
         return (int)o;
     };
-    // line buffers and couplings; during the residual phase the same space
-    // holds phi + delta of a tile of columns with its two neighbours
-    const size_t bufw = (size_t)3 * M * kRow * sizeof(double) + (size_t)2 * kLine * M * sizeof(double);
-    const size_t stage = (size_t)(lay.tw + 2) * nz * sizeof(double);
-    lay.offBuf = take(std::max(bufw, stage) - (size_t)2 * kLine * M * sizeof(double));
-    lay.offW = take((size_t)2 * kLine * M * sizeof(double));
-    lay.offF = take(std::max((size_t)3 * LFE * es, (size_t)2 * lay.tw * nz * es));
-    lay.offC = take(LFE * sizeof(double));
-    const size_t sp = off;
-    // a wide solve (one reactor alone) takes the one-block-per-SM build; a
-    // narrow one (a reactor of a batch) the two-block build
+    int grid = 1;
     const int minb = wide ? 1 : 2;
+    if (L == 0) {
+        take((size_t)M * kRow * sizeof(double));
+        lay.offC = take(LFE * sizeof(double));
+        lay.tw = 4;
+    } else {
+        // residual tiles of 4 columns (a 32-byte sector of flagged words per
+        // row) while there are as many SMs, and on the FP64 path, whose factor
+        // lines leave no room for more; else 8
+        lay.tw = mixed && (!wide || n > 4 * nsm) ? 8 : 4;
+        // the line buffers and couplings of the line phases share their space
+        // with the residual phase's tile (with its two neighbour columns) and
+        // restriction buffers (very tall meshes: narrower tiles)
+        const size_t buf = ((size_t)3 * M * kRow * es + 127) & ~(size_t)127, line = buf + (size_t)2 * kLine * M * es;
+        const size_t fac = LFE * es + (size_t)3 * LFE * es + 512;
+        size_t tile = 0, both = 0;
+        for (;; lay.tw /= 2) {
+            tile = ((size_t)(lay.tw + 2) * nz * sizeof(double) + 127) & ~(size_t)127;
+            both = std::max(line, tile + (size_t)2 * lay.tw * nz * es);
+            if (lay.tw == 1 || both + fac <= kSolveSmemLimit) break;
+        }
+        lay.offW = (int)buf;
+        lay.offT = (int)tile;
+        take(both);
+        lay.offC = take(LFE * es);
+        // a block per tile and per unit of the line phases
+        const int units = (2 << L) - 2 - L, ntile = (n + lay.tw - 1) / lay.tw;
+        grid = wide ? std::min(nsm, std::max(units, ntile)) : std::max(1, (nz - 1) / 2);
+        // factor slots: all of a block's units, as far as they fit (a batch's
+        // blocks: two to an SM)
+        const size_t room = wide ? kSolveSmemLimit : kSolveSmemLimit / 2;
+        const int want = std::min(kMaxSlots, (units + grid - 1) / grid);
+        lay.slots = 1;
+        while (lay.slots < want && off + (size_t)(lay.slots + 1) * 3 * LFE * es <= room) ++lay.slots;
+        lay.offF = take((size_t)lay.slots * 3 * LFE * es);
+    }
+    const size_t sp = off;
     void *fn = mixed ? solve_kernel<float>(M, minb) : solve_kernel<double>(M, minb);
     int per_sm = 0;
     if (sp <= kSolveSmemLimit) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kSolveThreads, sp);
     if (per_sm < 1) return false;
-    const int grid = std::max(1, std::min(nsm * per_sm, std::min(nsm, (wide ? 2 : 1) * ((nz - 1) / 2))));
+    grid = std::min(std::min(grid, nsm * per_sm), kMaxSolveBlocks);
     job.mp = m.self;
     job.phi = phi;
     job.nr = nr;
-    job.first_cycle = 1;
     job.lay = lay;
     job.tol = tol;
     job.max_cycles = max_cycles;
@@ -1294,8 +1301,7 @@ int mg_fast_solve(const FieldDims &fd, MGFast &m, const double *rho, const doubl
     k_rhs_bc<<<(ng + 255) / 256, 256, 0, st>>>(mp, rho, phi, phi_zL, V, nz, nr, warm ? 0 : 1, sctl,
                                                v_from_ctl ? 1 : 0, warm ? phi_prev : nullptr);
     ++L;
-    // (k_rhs_bc also copies phi to its alternate, clears the level-0
-    // correction and the solve's control block)
+    // (k_rhs_bc also clears the solve's control block)
     // all cycles in one cooperative launch
     SolveJob job;
     if (!solve_job(fd, m, phi, mixed, tol, max_cycles, sctl, wide, job)) {
@@ -1313,11 +1319,10 @@ int mg_fast_solve(const FieldDims &fd, MGFast &m, const double *rho, const doubl
     const size_t sp = job.smem;
     void *fn = job.fn;
     const int grid = job.nblocks;
-    int first_cycle = 1, nrv = nr, mc = max_cycles;
+    int nrv = nr, mc = max_cycles;
     double tv = tol;
     const StepCtl *sc = sctl;
-    void *args[] = {(void *)&mp, (void *)&phi, (void *)&nrv, (void *)&first_cycle, (void *)&lay,
-                    (void *)&tv, (void *)&mc, (void *)&sc};
+    void *args[] = {(void *)&mp, (void *)&phi, (void *)&nrv, (void *)&lay, (void *)&tv, (void *)&mc, (void *)&sc};
     // the highest stream priority: when a step sorts beside the solve, the
     // solve's blocks take SMs as soon as the sort's short blocks retire
     static int prio = 1;

@@ -9,18 +9,8 @@ namespace pic {
 
 // device-side control of one solve (the one-launch V-cycles)
 struct MGCtl {
-    unsigned long long b_bits;  // max |b| (first cycle), bits of a positive double
-    unsigned long long rb[2];   // per-cycle max |r| (alternating)
     int converged, zero_rhs, cycles, timeout;
     double last_res, bnorm;
-    // barrier counters of the one-launch solve (whole grid; the coarse
-    // levels' group of blocks), each on its own cache line
-    struct alignas(128) Line {
-        unsigned int v;
-        unsigned int pad[31];
-    };
-    Line bar_count;
-    Line gbar_count;
 };
 
 // returned by mg_fast_solve when a bounded device wait gave up, and when
@@ -43,33 +33,38 @@ struct MGFast {
     double *gz[kMaxLevels], *gr[kMaxLevels];
     double *ga;
     // V-cycle correction and right-hand side per level (level 0: the
-    // correction of phi and the residual), FP64 path / FP32 (mixed) path
-    double *u64[kMaxLevels], *f64[kMaxLevels];
-    float *u32[kMaxLevels], *f32[kMaxLevels];
+    // correction of phi and the residual) in flagged words, [nz_l][nr]:
+    // Flag<float>::W on the mixed path, Flag<double>::W on the FP64 path
+    void *lu[kMaxLevels], *lf[kMaxLevels];
     double *fac64[kMaxLevels];                  // line factors, FP64 path
     float *fac32[kMaxLevels];                   // line factors, FP32 V-cycle
     double *facc;                               // coarsest level's line factors (FP64)
     float *facc32;                              // coarsest level's line factors, FP32 V-cycle
-    double *fc64;                               // coarsest level's right-hand side
     double *f0;                                 // fine right-hand side
     double *dg0;                                // fine operator's diagonal
-    double *phi2;                               // second copy of phi (the solve alternates)
-    // flexible GCR(1) of the mixed path (null on the FP64 path): the FP64
-    // residual, A z of the last correction z, the previous direction and
-    // its A-image, and per-block partial dot products (4 per block)
-    double *kr, *kw, *kzp, *kwp, *kpart;
+    // per residual tile, node by node (mg_tile_elems): flexible GCR(1) of the
+    // mixed path -- the FP64 residual, A z of the last correction z, the
+    // previous direction and its A-image; FP64 path: phi of the tile and its
+    // two neighbour columns
+    double *kr, *kw, *kzp, *kwp, *ps;
+    // what the blocks tell one another each cycle, in flagged words: the
+    // norms {max |r|, max |b|} and the GCR step's four partial dot products
+    ulonglong2 *xr, *xd;
+    unsigned *epoch;  // the last solve's tags end below it
     MGCtl *ctl;
     MGFast *self;  // device copy of this struct (kernels read it through a pointer)
 };
 
 // Shared-memory layout of the one-launch solve (byte offsets), set on the host.
 struct SolveLayout {
-    int offBuf;  // three line buffers (right-hand side in, solution out), M * 33 values of 8 bytes each
-    int offW;    // the black line's two coupling coefficients, 32 M values of 8 bytes each
-    int offF;    // factors of the two red lines and the black line; the residual tile lies over them
-    int offC;    // factors of the coarsest row (FP64)
-    int tw;      // columns per residual tile
+    int offW;   // (from 0: three line buffers, M * 33 values each) the black line's two coupling coefficients, 32 M each
+    int offT;   // from 0 in the residual phase: the tile with its neighbour columns; at offT: two restriction buffers
+    int offF;   // factor slots: each two red lines and the black line
+    int offC;   // factors of the coarsest row
+    int slots;  // factor slots
+    int tw;     // columns per residual tile
 };
+constexpr int kMaxSlots = 4;
 
 // One reactor's one-launch solve, as the kernel takes it (a table of these
 // drives the solves of several reactors in one cooperative launch), with its
@@ -77,7 +72,7 @@ struct SolveLayout {
 struct SolveJob {
     const MGFast *mp;
     double *phi;
-    int nr, first_cycle;
+    int nr;
     SolveLayout lay;
     double tol;
     int max_cycles;
@@ -92,6 +87,10 @@ struct SolveJob {
 // line-factor elements of one r-line of a mesh with nr nodes per row
 // (the same count in FP32 and FP64)
 size_t mg_line_factor_elems(int nr);
+// doubles of each tile-wise array (kr, kw, kzp, kwp, ps), and the most blocks
+// a solve takes (entries of xr and xd)
+size_t mg_tile_elems(int nz, int nr);
+constexpr int kMaxSolveBlocks = 512;
 
 // copy the level table to the device (once: its pointers do not change)
 void mg_fast_upload(MGFast &m, cudaStream_t st);

@@ -620,11 +620,11 @@ void setup_device(pic_handle *h) {
         if (h->mixed) {
             m.cz32[l] = (float *)dalloc(h, g * sizeof(float));
             m.cr32[l] = (float *)dalloc(h, g * sizeof(float));
-            m.u32[l] = (float *)dalloc(h, g * sizeof(float));
-            m.f32[l] = (float *)dalloc(h, g * sizeof(float));
-        } else {
-            m.u64[l] = (double *)dalloc(h, g * sizeof(double));
-            m.f64[l] = (double *)dalloc(h, g * sizeof(double));
+        }
+        const size_t fw = g * (h->mixed ? sizeof(Flag<float>::W) : sizeof(Flag<double>::W));
+        for (void **w : {&m.lu[l], &m.lf[l]}) {
+            *w = dalloc(h, fw);
+            cudaMemsetAsync(*w, 0, fw, h->st);
         }
         const size_t fe = (size_t)(z - 2) * line_fe;
         if (z == 3) {
@@ -649,18 +649,24 @@ void setup_device(pic_handle *h) {
         m.ga = g + (size_t)2 * nl * h->nr;
         cudaStreamSynchronize(h->st);  // geo is a local
     }
-    m.fc64 = (double *)dalloc(h, (size_t)3 * h->nr * sizeof(double));
     m.f0 = (double *)dalloc(h, gb);
     m.dg0 = (double *)dalloc(h, gb);
-    m.phi2 = (double *)dalloc(h, gb);
+    const size_t tb = mg_tile_elems(h->nz, h->nr) * sizeof(double);
     if (h->mixed) {
-        m.kr = (double *)dalloc(h, gb);
-        m.kw = (double *)dalloc(h, gb);
-        m.kzp = (double *)dalloc(h, gb);
-        m.kwp = (double *)dalloc(h, gb);
-        m.kpart = (double *)dalloc(h, (size_t)4 * 1024 * sizeof(double));
-        for (double *z : {m.kr, m.kw, m.kzp, m.kwp}) cudaMemsetAsync(z, 0, gb, h->st);
+        for (double **z : {&m.kr, &m.kw, &m.kzp, &m.kwp}) {
+            *z = (double *)dalloc(h, tb);
+            cudaMemsetAsync(*z, 0, tb, h->st);
+        }
+    } else {
+        m.ps = (double *)dalloc(h, tb);
     }
+    // flagged words and their epoch start at zero: tag 0 is never waited for
+    const size_t xb = (size_t)kMaxSolveBlocks * 8 * sizeof(ulonglong2);
+    m.xr = (ulonglong2 *)dalloc(h, xb);
+    m.xd = m.xr + 4 * kMaxSolveBlocks;
+    m.epoch = (unsigned *)dalloc(h, sizeof(unsigned));
+    cudaMemsetAsync(m.xr, 0, xb, h->st);
+    cudaMemsetAsync(m.epoch, 0, sizeof(unsigned), h->st);
     m.ctl = (MGCtl *)dalloc(h, sizeof(MGCtl));
     m.self = (MGFast *)dalloc(h, sizeof(MGFast));
     mg_fast_upload(m, h->st);

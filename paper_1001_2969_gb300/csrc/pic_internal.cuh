@@ -121,6 +121,77 @@ __device__ __forceinline__ bool count_barrier(unsigned *count, unsigned target, 
     return s_ok != 0;
 }
 
+// ---- flagged words: data that blocks of one launch hand to one another ----
+// A value and a 32-bit tag in one 8-byte word (a double: its two halves in two
+// such words), stored and loaded with relaxed gpu-scope accesses, which are
+// single-copy atomic per 8 bytes.  The reader polls the word itself until it
+// carries the tag it waits for, so a hand-over costs one trip to L2 each way:
+// no fence, no separate flag, and L1 keeps what else the block uses (an
+// acquire would drop it).  Tags must not recur while an old word can be read.
+template <typename T>
+struct Flag;
+template <>
+struct Flag<float> {
+    using W = unsigned long long;
+    static __device__ __forceinline__ W load(const W *p) {
+        W w;
+        asm volatile("ld.relaxed.gpu.global.b64 %0, [%1];" : "=l"(w) : "l"(p) : "memory");
+        return w;
+    }
+    static __device__ __forceinline__ void store(W *p, float v, unsigned tag) {
+        const W w = ((W)tag << 32) | __float_as_uint(v);
+        asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(p), "l"(w) : "memory");
+    }
+    static __device__ __forceinline__ bool ready(const W &w, unsigned tag) { return (unsigned)(w >> 32) == tag; }
+    static __device__ __forceinline__ float value(const W &w) { return __uint_as_float((unsigned)w); }
+};
+template <>
+struct Flag<double> {
+    using W = ulonglong2;
+    static __device__ __forceinline__ W load(const W *p) {
+        W w;
+        asm volatile("ld.relaxed.gpu.global.v2.b64 {%0, %1}, [%2];" : "=l"(w.x), "=l"(w.y) : "l"(p) : "memory");
+        return w;
+    }
+    static __device__ __forceinline__ void store(W *p, double v, unsigned tag) {
+        const unsigned long long b = (unsigned long long)__double_as_longlong(v), t = (unsigned long long)tag << 32;
+        asm volatile("st.relaxed.gpu.global.v2.b64 [%0], {%1, %2};" ::"l"(p), "l"(t | (b & 0xffffffffull)),
+                     "l"(t | (b >> 32))
+                     : "memory");
+    }
+    static __device__ __forceinline__ bool ready(const W &w, unsigned tag) {
+        return (unsigned)(w.x >> 32) == tag && (unsigned)(w.y >> 32) == tag;
+    }
+    static __device__ __forceinline__ double value(const W &w) {
+        return __longlong_as_double((long long)((w.x & 0xffffffffull) | (w.y << 32)));
+    }
+};
+
+// Poll N flagged words (null: none, value 0) until all carry `tag`.  Bounded
+// like count_barrier: after `limit` rounds, or once another block gave up,
+// *timeout is raised and `fail` set.  A call with fail set returns at once.
+template <typename T, int N>
+__device__ __forceinline__ void flag_wait(const typename Flag<T>::W *const (&p)[N], T (&v)[N], unsigned tag,
+                                          int *timeout, bool &fail, long long limit = kSpinLimit) {
+    typename Flag<T>::W w[N];
+    for (long long it = 0; !fail;) {
+#pragma unroll
+        for (int k = 0; k < N; ++k)
+            if (p[k]) w[k] = Flag<T>::load(p[k]);
+        bool all = true;
+#pragma unroll
+        for (int k = 0; k < N; ++k)
+            if (p[k]) all = all && Flag<T>::ready(w[k], tag);
+        if (all) break;
+        if ((++it & 255) == 0 && (it > limit || *(volatile int *)timeout)) {
+            atomicExch(timeout, 1);
+            fail = true;
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < N; ++k) v[k] = p[k] && !fail ? Flag<T>::value(w[k]) : (T)0;
+}
+
 // four-wide vectors: float4 for the mixed path, two 16-byte halves for FP64
 struct alignas(16) dbl4 {
     double x, y, z, w;

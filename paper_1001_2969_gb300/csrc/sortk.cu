@@ -516,17 +516,28 @@ __global__ void __launch_bounds__(kRadixThreads) k_birth_finish(BirthJob b, Pass
 }
 
 // failure-detection self-test: one block waits at the bounded grid barrier
-// for a second participant that is never launched; the wait must give up
-__global__ void k_wait_selftest(unsigned *count, int *timeout, long long limit, int *gave_up) {
+// for a second participant that is never launched, then for a flagged word
+// that nothing writes; both waits must give up
+__global__ void k_wait_selftest(unsigned *count, int *timeout, long long limit, int *gave_up,
+                                const Flag<float>::W *word) {
     const bool ok = count_barrier(count, 2u, timeout, limit);
-    if (threadIdx.x == 0) *gave_up = ok ? 0 : 1;
+    const bool said = *(volatile int *)timeout != 0;
+    __syncthreads();
+    if (threadIdx.x == 0) *timeout = 0;
+    __syncthreads();
+    const Flag<float>::W *p[1] = {word};
+    float v[1];
+    bool fail = false;
+    flag_wait<float, 1>(p, v, 1u, timeout, fail, limit);
+    if (threadIdx.x == 0) *gave_up = !ok && said && fail ? 1 : 0;
 }
 
 int wait_selftest(long long limit, int *gave_up) {
-    int *buf = nullptr;  // count, timeout, result
-    if (cudaMalloc(&buf, 3 * sizeof(int)) != cudaSuccess) return -1;
-    cudaMemset(buf, 0, 3 * sizeof(int));
-    k_wait_selftest<<<1, 32>>>(reinterpret_cast<unsigned *>(buf), buf + 1, limit, buf + 2);
+    int *buf = nullptr;  // count, timeout, result; a flagged word
+    if (cudaMalloc(&buf, 6 * sizeof(int)) != cudaSuccess) return -1;
+    cudaMemset(buf, 0, 6 * sizeof(int));
+    k_wait_selftest<<<1, 32>>>(reinterpret_cast<unsigned *>(buf), buf + 1, limit, buf + 2,
+                               reinterpret_cast<const Flag<float>::W *>(buf + 4));
     int out[3] = {0, 0, 0};
     const cudaError_t e = cudaMemcpy(out, buf, sizeof(out), cudaMemcpyDeviceToHost);
     cudaFree(buf);
