@@ -251,50 +251,95 @@ __global__ void k_factor_lines(const MGFast *__restrict__ mp, int l0, int l1, in
     Gf[12 * kLine + p] = recip(B);
 }
 
-// Warp solve of one line with factors F (shared memory): right-hand side in
-// Bs and solution out to the same place, both [k * 33 + p] (lane-minor with
-// a pad against bank conflicts).  All 32 lanes take part.
+// Warp solve of one line: right-hand side in Bs and solution out to the same
+// place, both [k * 33 + p] (lane-minor with a pad against bank conflicts).
+// All 32 lanes take part.  A line is one chain of dependent operations, so the
+// chain is kept to one fused multiply-add per unknown and sweep (the products
+// that do not depend on it are taken out of it) and the factors come in
+// registers where they fit (LineFactors::load, before the right-hand side is
+// there): FP32, M = 16, 635 -> 474 cycles, M = 8, 443 -> 363; the five
+// shuffled reduction steps are ~170 of them.  In FP64 a line is bound by
+// GB300's narrow FP64 pipe (~70 cycles per warp instruction) instead.
 constexpr int kRow = 33;
 
+__device__ __forceinline__ float fma_(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ double fma_(double a, double b, double c) { return fma(a, b, c); }
+
+// a line's factors, lane p's share: in registers (REG), or read from shared
+// memory as they are used
+template <typename Ts, int M, bool REG>
+struct LineFactors;
 template <typename Ts, int M>
-__device__ __forceinline__ void warp_line_solve(const Ts *__restrict__ F, Ts *Bs, int p) {
+struct LineFactors<Ts, M, false> {
+    const Ts *F;
+    int p;
+    __device__ __forceinline__ void load(const Ts *f, int lane) {
+        F = f;
+        p = lane;
+    }
+    template <int ARR>
+    __device__ __forceinline__ Ts at(int k) const {
+        return F[(ARR * M + k) * kLine + p];
+    }
+    __device__ __forceinline__ Ts tail(int k) const { return F[(5 * M + k) * kLine + p]; }
+};
+template <typename Ts, int M>
+struct LineFactors<Ts, M, true> {
+    Ts a[5][M > 1 ? M - 1 : 1], t[13];
+    __device__ __forceinline__ void load(const Ts *F, int p) {
+#pragma unroll
+        for (int r = 0; r < 5; ++r)
+#pragma unroll
+            for (int k = 0; k < M - 1; ++k) a[r][k] = F[(r * M + k) * kLine + p];
+#pragma unroll
+        for (int k = 0; k < 13; ++k) t[k] = F[(5 * M + k) * kLine + p];
+    }
+    template <int ARR>
+    __device__ __forceinline__ Ts at(int k) const {
+        return a[ARR][k];
+    }
+    __device__ __forceinline__ Ts tail(int k) const { return t[k]; }
+};
+
+template <typename Ts, int M, bool REG>
+__device__ __forceinline__ void warp_line_solve(const LineFactors<Ts, M, REG> &q, Ts *Bs, int p) {
     constexpr int MI = M - 1;
-    const Ts *Gf = F + 5 * M * kLine;
-    Ts r;
-    Ts z[MI > 0 ? MI : 1];
+    Ts z[M];
+#pragma unroll
+    for (int k = 0; k < M; ++k) z[k] = Bs[k * kRow + p];
+    Ts r = z[M - 1];
     if constexpr (MI > 0) {
-        Ts zp = Bs[p];
-        z[0] = zp;
 #pragma unroll
-        for (int k = 1; k < MI; ++k) {
-            zp = Bs[k * kRow + p] - F[(0 * M + k) * kLine + p] * zp;
-            z[k] = zp;
-        }
-        Ts zn = z[MI - 1] * F[(1 * M + MI - 1) * kLine + p];
-        z[MI - 1] = zn;
+        for (int k = 1; k < MI; ++k) z[k] = fma_(-q.template at<0>(k), z[k - 1], z[k]);
 #pragma unroll
-        for (int k = MI - 2; k >= 0; --k) {
-            zn = z[k] * F[(1 * M + k) * kLine + p] - F[(2 * M + k) * kLine + p] * zn;
-            z[k] = zn;
-        }
+        for (int k = 0; k < MI; ++k) z[k] *= q.template at<1>(k);
+#pragma unroll
+        for (int k = MI - 2; k >= 0; --k) z[k] = fma_(-q.template at<2>(k), z[k + 1], z[k]);
         const Ts z0n = __shfl_down_sync(0xffffffffu, z[0], 1);
-        r = Bs[(M - 1) * kRow + p] - Gf[p] * z[MI - 1] - Gf[kLine + p] * (p < kLine - 1 ? z0n : (Ts)0);
-    } else {
-        r = Bs[p];
+        r = fma_(-q.tail(0), z[MI - 1], r);
+        if (p < kLine - 1) r = fma_(-q.tail(1), z0n, r);
     }
 #pragma unroll
     for (int st = 0; st < 5; ++st) {
         const int s = 1 << st;
         const Ts rm = __shfl_up_sync(0xffffffffu, r, s), rp = __shfl_down_sync(0xffffffffu, r, s);
-        r = r + Gf[(2 + st) * kLine + p] * rm + Gf[(7 + st) * kLine + p] * rp;
+        r = fma_(q.tail(7 + st), rp, fma_(q.tail(2 + st), rm, r));
     }
-    const Ts I = r * Gf[12 * kLine + p];
+    const Ts I = r * q.tail(12);
     if constexpr (MI > 0) {
         const Ts Ip = __shfl_up_sync(0xffffffffu, I, 1);  // lane 0: v is zero there
 #pragma unroll
-        for (int k = 0; k < MI; ++k) Bs[k * kRow + p] = z[k] + F[(3 * M + k) * kLine + p] * Ip + F[(4 * M + k) * kLine + p] * I;
+        for (int k = 0; k < MI; ++k)
+            Bs[k * kRow + p] = fma_(q.template at<4>(k), I, fma_(q.template at<3>(k), Ip, z[k]));
     }
     Bs[(M - 1) * kRow + p] = I;
+}
+
+template <typename Ts, int M>
+__device__ __forceinline__ void warp_line_solve(const Ts *F, Ts *Bs, int p) {
+    LineFactors<Ts, M, false> q;
+    q.load(F, p);
+    warp_line_solve<Ts, M, false>(q, Bs, p);
 }
 
 // right-hand side rho A_j dz / eps0 and the Dirichlet data of phi; with
@@ -370,6 +415,11 @@ __global__ void k_rhs_bc(const MGFast *__restrict__ mp, const double *rho, doubl
 // same phases between grid barriers, which took ~1 us each and cost every
 // phase its L1: 33 x 65 mixed 216 -> 157 us, 65 x 300 mixed 326 -> 228,
 // 257 x 1025 mixed 626 -> 527, 129 x 513 FP64 886 -> 803 (FP64 line solves).
+// What is exchanged all-to-all is kept in kCopies copies (with one, 128 blocks
+// polling the same few lines of L2 took 3 us for the norms, now 1.8), sums and
+// maxima take few FP64 and 64-bit operations, a tile's restricted levels are
+// stored by rows, and the lines' factors wait in registers: 157 -> 147 us,
+// 228 -> 202, 527 -> 508.
 // ---------------------------------------------------------------------------
 
 // ---- factor lines into shared memory ----
@@ -418,29 +468,33 @@ __device__ __forceinline__ bool ld_wait(Loader &q, int r) {
 }
 
 constexpr int kSolveThreads = 256;
-constexpr int kU = 4;  // elements per thread and batch in the residual phase
 
-// the larger of a over the block's threads (bit patterns), and of b
+// the warp's largest of 64-bit words: high halves first, then the low halves
+// of those that have it (two integer reductions)
+__device__ __forceinline__ unsigned long long warp_max(unsigned long long x) {
+    const unsigned hi = __reduce_max_sync(0xffffffffu, (unsigned)(x >> 32));
+    const unsigned lo = __reduce_max_sync(0xffffffffu, (unsigned)(x >> 32) == hi ? (unsigned)x : 0u);
+    return ((unsigned long long)hi << 32) | lo;
+}
+
+// the largest of a over the block's threads (bit patterns), and of b
 __device__ __forceinline__ void block_max2(unsigned long long &a, unsigned long long &b,
                                            unsigned long long (*s)[kSolveThreads / 32]) {
-    for (int o = 16; o > 0; o >>= 1) {
-        a = max(a, __shfl_xor_sync(0xffffffffu, a, o));
-        b = max(b, __shfl_xor_sync(0xffffffffu, b, o));
-    }
-    if ((threadIdx.x & 31) == 0) {
+    a = warp_max(a);
+    b = warp_max(b);
+    const int lane = threadIdx.x & 31;
+    if (lane == 0) {
         s[0][threadIdx.x >> 5] = a;
         s[1][threadIdx.x >> 5] = b;
     }
     __syncthreads();
-    for (int w = 0; w < kSolveThreads / 32; ++w) {
-        a = max(a, s[0][w]);
-        b = max(b, s[1][w]);
-    }
+    a = warp_max(lane < kSolveThreads / 32 ? s[0][lane] : 0ull);
+    b = warp_max(lane < kSolveThreads / 32 ? s[1][lane] : 0ull);
 }
 
 // nz = 3: one interior row, phi's own, solved exactly in FP64 by one block
 template <int M>
-__device__ __forceinline__ void solve_row(const MGFast &m, double *phi, int nr, double tol, int max_cycles,
+__device__ __noinline__ void solve_row(const MGFast &m, double *phi, int nr, double tol, int max_cycles,
                                           double *B, double *F) {
     __shared__ unsigned long long s_max[2][kSolveThreads / 32];
     const int tid = threadIdx.x, n = nr - 1;
@@ -495,7 +549,8 @@ __device__ __forceinline__ void solve_row(const MGFast &m, double *phi, int nr, 
 }
 
 // One reactor's solve on P blocks (bid: this block's index among them).
-template <typename Tv, int M>
+// WIDE: a block per SM; else two, with half the registers.
+template <typename Tv, int M, bool WIDE>
 __device__ __forceinline__ void solve_body(const MGFast *__restrict__ mp, double *phi, int nr,
                                            const SolveLayout &lay, double tol, int max_cycles,
                                            const StepCtl *sctl, const int bid, const int P) {
@@ -503,6 +558,7 @@ __device__ __forceinline__ void solve_body(const MGFast *__restrict__ mp, double
     if (sctl && sctl->halt) return;  // an earlier failure of this step
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     constexpr int nt = kSolveThreads;
+    constexpr int kU = WIDE ? 4 : 2;  // elements per thread and batch in the residual phase
     // the level table in shared memory (read in front of every phase's loads)
     __shared__ __align__(16) MGFast s_m;
     {
@@ -529,11 +585,11 @@ __device__ __forceinline__ void solve_body(const MGFast *__restrict__ mp, double
     const unsigned ep = *(volatile unsigned *)m.epoch;  // tags of this solve: ep + 1 + cycle
     __shared__ unsigned long long s_max[2][2][nt / 32];
     __shared__ double s_dot[2][4][nt / 32];
-    __shared__ double s_ab[3];  // the GCR step's beta, alpha and |q|^2
+    __shared__ double s_ab[4];  // the GCR step's beta, alpha, |q|^2 and the inverse of that
     __shared__ __align__(8) unsigned long long s_mbar[kMaxSlots + 1];
-    double kc = 0.0;  // |w|^2 of the previous direction's A-image
     double bn = 0.0;  // max |b|
     if (tid == 0) {
+        s_ab[3] = 0.0;
         for (int b = 0; b <= kMaxSlots; ++b)
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"((unsigned)__cvta_generic_to_shared(&s_mbar[b]))
                          : "memory");
@@ -570,22 +626,22 @@ __device__ __forceinline__ void solve_body(const MGFast *__restrict__ mp, double
         ld_begin(ld, kMaxSlots, FB);
         ld_copy(ld, kMaxSlots, FC, mixed ? (const Tv *)m.facc32 : (const Tv *)m.facc, FB);
     }
-    // leave with no copy in flight (bounded waits), the tags used up
-    auto leave = [&](int cyc) {
-        for (int r = 0; r <= kMaxSlots; ++r) ld_wait(ld, r);
-        if (bid == 0 && tid == 0) *m.epoch = ep + (unsigned)cyc + 4u;
-    };
-    Tv *Bf0 = reinterpret_cast<Tv *>(smem_raw), *Bf1 = Bf0 + M * kRow, *Bf2 = Bf1 + M * kRow;
-    Tv *W0 = reinterpret_cast<Tv *>(smem_raw + lay.offW), *W1 = W0 + NW;
+    // line buffers: the two reds, the black line
+    Tv *const Bf = reinterpret_cast<Tv *>(smem_raw);
+    constexpr int BL = M * kRow;
     double *St = reinterpret_cast<double *>(smem_raw);
-    const int tw = lay.tw, sw = tw + 2, ntile = (n + tw - 1) / tw, tn = tw * (nz0 - 2);
+    const int tw = lay.tw, ltw = __ffs(tw) - 1, sw = tw + 2, ntile = (n + tw - 1) >> ltw, tn = tw * (nz0 - 2);
+    // e / sw for e < sw * nz0 (< 2^17): e * ceil(2^32 / sw) >> 32
+    const unsigned sw_inv = 0xffffffffu / (unsigned)sw + 1u;
+    auto div_sw = [&](int e) { return (int)__umulhi((unsigned)e, sw_inv); };
     Tv *T0 = reinterpret_cast<Tv *>(smem_raw + lay.offT), *T1 = T0 + (size_t)tw * nz0;
     Wv *lu0 = (Wv *)m.lu[0], *lf0 = (Wv *)m.lf[0];
     // position of unknown j in a line buffer
     auto at = [](int j) { return (j % M) * kRow + j / M; };
     bool fail = false;
     int g = 0;  // units done
-    for (int cyc = 0;; ++cyc) {
+    int cyc = 0;
+    for (;; ++cyc) {
         const unsigned tag = ep + 1u + (unsigned)cyc;
         __syncthreads();  // the line buffers are read; the tile takes their place
         // maxima as bit patterns of |x| (ordered like the values; a NaN
@@ -598,31 +654,40 @@ __device__ __forceinline__ void solve_body(const MGFast *__restrict__ mp, double
             const Wv *p[kU];
 #pragma unroll
             for (int u = 0; u < kU; ++u) {
-                const int e = e0 + u * nt, c = e % sw - 1, i = e / sw, j = j0 + c;
+                const int e = e0 + u * nt, i = div_sw(e), c = e - i * sw - 1, j = j0 + c;
                 p[u] = (e < sw * nz0 && j >= 0 && j < n && i > 0 && i < nz0 - 1) ? lu0 + (size_t)i * nr + j : nullptr;
             }
             flag_wait<Tv, kU>(p, dv, tag - 1u, &ctl->timeout, fail);
         };
         // the restriction chain of the residual tile T0 (columns j0 ..) down
-        // to the coarsest level, in the V-cycle's type: a warp per column
+        // to the coarsest level, in the V-cycle's type: a warp per column, the
+        // levels one after another in T1; then all of it stored by rows (a
+        // warp's words in few sectors), the coarsest level first, which the
+        // line phases start with
         auto chain = [&](int j0) {
             for (int c = warp; c < tw; c += nt / 32) {
-                const int j = j0 + c;
-                if (j >= n) break;
-                Tv *src = T0 + (size_t)c * nz0, *dst = T1 + (size_t)c * nz0;
+                const Tv *src = T0 + (size_t)c * nz0;
+                Tv *dst = T1 + (size_t)c * (nz0 + kMaxLevels);
                 for (int l = 1; l <= L; ++l) {
                     const int nzc = m.nz[l];
-                    Wv *fl = (Wv *)m.lf[l];
-                    for (int I = 1 + lane; I < nzc - 1; I += 32) {
-                        const Tv v = (Tv)0.5 * src[2 * I - 1] + src[2 * I] + (Tv)0.5 * src[2 * I + 1];
-                        dst[I] = v;
-                        Fv::store(fl + (size_t)I * nr + j, v, tag);
-                    }
+                    for (int I = 1 + lane; I < nzc - 1; I += 32)
+                        dst[I] = (Tv)0.5 * src[2 * I - 1] + src[2 * I] + (Tv)0.5 * src[2 * I + 1];
                     __syncwarp();
-                    Tv *tmp = src;
                     src = dst;
-                    dst = tmp;
+                    dst += nzc;
                 }
+            }
+            __syncthreads();
+            int at_l = 0;  // level l's place in a column
+            for (int l = 1; l < L; ++l) at_l += m.nz[l];
+            for (int l = L; l > 0; --l) {
+                const int nzc = m.nz[l];
+                Wv *fl = (Wv *)m.lf[l];
+                for (int e = tid; e < (nzc - 2) << ltw; e += nt) {
+                    const int c = e & (tw - 1), I = 1 + (e >> ltw), j = j0 + c;
+                    if (j < n) Fv::store(fl + (size_t)I * nr + j, T1[(size_t)c * (nz0 + kMaxLevels) + at_l + I], tag);
+                }
+                if (l > 1) at_l -= m.nz[l - 1];
             }
         };
         if (mixed && cyc > 0) {
@@ -638,7 +703,7 @@ __device__ __forceinline__ void solve_body(const MGFast *__restrict__ mp, double
                     delta_batch(e0, j0, dv);
 #pragma unroll
                     for (int u = 0; u < kU; ++u) {
-                        const int e = e0 + u * nt, c = e % sw - 1, i = e / sw;
+                        const int e = e0 + u * nt, i = div_sw(e), c = e - i * sw - 1;
                         if (e < sw * nz0) St[(size_t)(c + 1) * nz0 + i] = (double)dv[u];
                     }
                 }
@@ -649,7 +714,7 @@ __device__ __forceinline__ void solve_body(const MGFast *__restrict__ mp, double
                     double ca[kU], cb[kU], ce[kU], cd[kU], dgv[kU], rv[kU], wpv[kU];
 #pragma unroll
                     for (int u = 0; u < kU; ++u) {
-                        const int e = e0 + u * nt, c = e % tw, i = 1 + e / tw, j = j0 + c;
+                        const int e = e0 + u * nt, c = e & (tw - 1), i = 1 + (e >> ltw), j = j0 + c;
                         ca[u] = cb[u] = ce[u] = cd[u] = dgv[u] = rv[u] = wpv[u] = 0.0;
                         if (e < tn && j < n) {
                             const size_t k = (size_t)i * nr + j;
@@ -664,7 +729,7 @@ __device__ __forceinline__ void solve_body(const MGFast *__restrict__ mp, double
                     }
 #pragma unroll
                     for (int u = 0; u < kU; ++u) {
-                        const int e = e0 + u * nt, c = e % tw, i = 1 + e / tw, j = j0 + c;
+                        const int e = e0 + u * nt, c = e & (tw - 1), i = 1 + (e >> ltw), j = j0 + c;
                         if (e >= tn || j >= n) continue;
                         const double *Sc = St + (size_t)(c + 1) * nz0 + i;
                         const double w = dgv[u] * Sc[0] - ca[u] * Sc[-1] - cb[u] * Sc[1] - ce[u] * Sc[nz0] -
@@ -693,43 +758,43 @@ __device__ __forceinline__ void solve_body(const MGFast *__restrict__ mp, double
                 for (int o = 4; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
                 if ((lane & 7) == 0) s_dot[0][2 * (lane >> 4) + ((lane >> 3) & 1)][warp] = c;
             }
-            if (__syncthreads_or(fail)) {
-                leave(cyc);
-                return;
-            }
-            if (tid < 4) {
-                double v = 0.0;
-                for (int q = 0; q < nt / 32; ++q) v += s_dot[0][tid][q];
-                Flag<double>::store(m.xd + (size_t)bid * 4 + tid, v, tag);
+            if (__syncthreads_or(fail)) break;
+            // (lane 4 w + k of a warp takes product k of warp w: three additions)
+            auto over_warps = [&](int set) {
+                double v = s_dot[set][lane & 3][lane >> 2];
+                for (int o = 4; o < 32; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+                return v;
+            };
+            static_assert(nt / 32 == 8, "a lane for each product of each warp");
+            if (warp == 0) {
+                const double v = over_warps(0);
+                // one copy for each kCopies-th reader: lane 4 c + k the copy c of product k
+                Flag<double>::store(m.xd + ((size_t)(lane >> 2) * kMaxSolveBlocks + bid) * 4 + (lane & 3), v, tag);
             }
             // every block sums the partial products in the same fixed order
             // (the same step length everywhere): thread t takes entries t,
             // t + nt, ... of product t % 4 (nt is a multiple of 32)
             {
+                const ulonglong2 *xd = m.xd + (size_t)(bid % kCopies) * kMaxSolveBlocks * 4;
                 double v = 0.0;
                 for (int e0 = tid; e0 < 4 * P; e0 += 2 * nt) {
-                    const ulonglong2 *p[2] = {m.xd + e0, e0 + nt < 4 * P ? m.xd + e0 + nt : nullptr};
+                    const ulonglong2 *p[2] = {xd + e0, e0 + nt < 4 * P ? xd + e0 + nt : nullptr};
                     double x[2];
                     flag_wait<double, 2>(p, x, tag, &ctl->timeout, fail);
                     v += x[0];
-                    v += x[1];
+                    if (p[1]) v += x[1];
                 }
                 for (int o = 4; o < 32; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
                 if (lane < 4) s_dot[1][lane][warp] = v;
-                if (__syncthreads_or(fail)) {
-                    leave(cyc);
-                    return;
-                }
+                if (__syncthreads_or(fail)) break;
                 // the step's scalars by one thread: GB300's FP64 pipe is
                 // narrow, and every thread dividing cost microseconds
                 if (warp == 0) {
-                    double t = 0.0;
-                    if (lane < 4)
-                        for (int q = 0; q < nt / 32; ++q) t += s_dot[1][lane][q];
+                    const double t = over_warps(1);
                     const double rw = __shfl_sync(0xffffffffu, t, 0), ww = __shfl_sync(0xffffffffu, t, 1),
                                  wwp = __shfl_sync(0xffffffffu, t, 2), rwp = __shfl_sync(0xffffffffu, t, 3);
                     if (lane == 0) {
-                        const double beta = kc > 0.0 ? wwp / kc : 0.0;
+                        const double beta = wwp * s_ab[3];
                         const double den = ww - beta * wwp;
                         s_ab[0] = beta;
                         s_ab[1] = den > 0.0 ? (rw - beta * rwp) / den : 1.0;
@@ -739,7 +804,8 @@ __device__ __forceinline__ void solve_body(const MGFast *__restrict__ mp, double
                 __syncthreads();
             }
             const double beta = s_ab[0], alpha = s_ab[1];
-            kc = s_ab[2];
+            // 1 / |q|^2 for the next step's beta, off this one's path
+            if (tid == nt - 1) s_ab[3] = s_ab[2] > 0.0 ? 1.0 / s_ab[2] : 0.0;
             const bool one = bid + P >= ntile;  // the block's only tile: z is still in St
             for (int t = bid; t < ntile; t += P) {
                 const int j0 = t * tw;
@@ -748,7 +814,7 @@ __device__ __forceinline__ void solve_body(const MGFast *__restrict__ mp, double
                     double pz[kU], qw[kU], zp[kU], wpv[kU], xv[kU], rv[kU];
 #pragma unroll
                     for (int u = 0; u < kU; ++u) {
-                        const int e = e0 + u * nt, c = e % tw, i = 1 + e / tw, j = j0 + c;
+                        const int e = e0 + u * nt, c = e & (tw - 1), i = 1 + (e >> ltw), j = j0 + c;
                         pz[u] = qw[u] = zp[u] = wpv[u] = xv[u] = rv[u] = 0.0;
                         if (e < tn && j < n) {
                             const size_t k = (size_t)i * nr + j;
@@ -764,7 +830,7 @@ __device__ __forceinline__ void solve_body(const MGFast *__restrict__ mp, double
                     }
 #pragma unroll
                     for (int u = 0; u < kU; ++u) {
-                        const int e = e0 + u * nt, c = e % tw, i = 1 + e / tw, j = j0 + c;
+                        const int e = e0 + u * nt, c = e & (tw - 1), i = 1 + (e >> ltw), j = j0 + c;
                         if (e >= tn) break;
                         double rn = 0.0;
                         if (j < n) {
@@ -797,20 +863,21 @@ __device__ __forceinline__ void solve_body(const MGFast *__restrict__ mp, double
                     Tv dv[kU];
 #pragma unroll
                     for (int u = 0; u < kU; ++u) {
-                        const int e = e0 + u * nt, c = e % sw - 1, i = e / sw, j = j0 + c;
+                        const int e = e0 + u * nt, i = div_sw(e), c = e - i * sw - 1, j = j0 + c;
                         pv[u] = 0.0;
                         dv[u] = 0;
-                        if (e < sw * nz0 && j >= 0 && j < nr) pv[u] = cyc > 0 ? own[e] : phi[(size_t)i * nr + j];
+                        if (e < sw * nz0 && j >= 0 && j < nr) pv[u] = !mixed && cyc > 0 ? own[e] : phi[(size_t)i * nr + j];
                     }
-                    if (cyc > 0) delta_batch(e0, j0, dv);
+                    if (!mixed && cyc > 0) delta_batch(e0, j0, dv);
 #pragma unroll
                     for (int u = 0; u < kU; ++u) {
-                        const int e = e0 + u * nt, c = e % sw - 1, i = e / sw, j = j0 + c;
+                        const int e = e0 + u * nt, i = div_sw(e), c = e - i * sw - 1, j = j0 + c;
                         if (e >= sw * nz0) break;
                         const double v = pv[u] + (double)dv[u];
                         if (!mixed) own[e] = v;
                         // the iterate, stored by the tile that owns the node
-                        if (cyc > 0 && c >= 0 && c < tw && j < n && i > 0 && i < nz0 - 1) phi[(size_t)i * nr + j] = v;
+                        if (!mixed && cyc > 0 && c >= 0 && c < tw && j < n && i > 0 && i < nz0 - 1)
+                            phi[(size_t)i * nr + j] = v;
                         St[(size_t)(c + 1) * nz0 + i] = v;
                     }
                 }
@@ -821,7 +888,7 @@ __device__ __forceinline__ void solve_body(const MGFast *__restrict__ mp, double
                     double ca[kU], cb[kU], ce[kU], cd[kU], dgv[kU], fv[kU];
 #pragma unroll
                     for (int u = 0; u < kU; ++u) {
-                        const int e = e0 + u * nt, c = e % tw, i = 1 + e / tw, j = j0 + c;
+                        const int e = e0 + u * nt, c = e & (tw - 1), i = 1 + (e >> ltw), j = j0 + c;
                         ca[u] = cb[u] = ce[u] = cd[u] = dgv[u] = fv[u] = 0.0;
                         if (e < tn && j < n) {
                             const size_t k = (size_t)i * nr + j;
@@ -835,7 +902,7 @@ __device__ __forceinline__ void solve_body(const MGFast *__restrict__ mp, double
                     }
 #pragma unroll
                     for (int u = 0; u < kU; ++u) {
-                        const int e = e0 + u * nt, c = e % tw, i = 1 + e / tw, j = j0 + c;
+                        const int e = e0 + u * nt, c = e & (tw - 1), i = 1 + (e >> ltw), j = j0 + c;
                         if (e >= tn) break;
                         double r = 0.0;
                         if (j < n) {
@@ -868,11 +935,13 @@ __device__ __forceinline__ void solve_body(const MGFast *__restrict__ mp, double
         block_max2(rmax, bmax, s_max[0]);
         // (two sets in turn: a block that owns no unit may still be reading the
         // norms of the cycle before)
-        ulonglong2 *xr = m.xr + (size_t)(cyc & 1) * 2 * kMaxSolveBlocks;
-        if (tid == 0) {
-            Flag<double>::store(xr + 2 * bid, __longlong_as_double((long long)rmax), tag);
-            if (cyc == 0) Flag<double>::store(xr + 2 * bid + 1, __longlong_as_double((long long)bmax), tag);
+        ulonglong2 *xr = m.xr + (size_t)(cyc & 1) * kCopies * 2 * kMaxSolveBlocks;
+        if (tid < kCopies) {
+            ulonglong2 *to = xr + (size_t)tid * 2 * kMaxSolveBlocks + 2 * bid;
+            Flag<double>::store(to, __longlong_as_double((long long)rmax), tag);
+            if (cyc == 0) Flag<double>::store(to + 1, __longlong_as_double((long long)bmax), tag);
         }
+        xr += (size_t)(bid % kCopies) * 2 * kMaxSolveBlocks;
         rmax = bmax = 0ull;
         for (int e = tid; e < P; e += nt) {
             const ulonglong2 *p[2] = {xr + 2 * e, cyc == 0 ? xr + 2 * e + 1 : nullptr};
@@ -882,10 +951,7 @@ __device__ __forceinline__ void solve_body(const MGFast *__restrict__ mp, double
             bmax = max(bmax, (unsigned long long)__double_as_longlong(x[1]));
         }
         block_max2(rmax, bmax, s_max[1]);
-        if (__syncthreads_or(fail)) {
-            leave(cyc);
-            return;
-        }
+        if (__syncthreads_or(fail)) break;
         const double rn = __longlong_as_double((long long)rmax);
         if (cyc == 0) bn = __longlong_as_double((long long)bmax);
         int decide = 0;  // 0 continue, 1 converged, 2 out of cycles, 3 zero right-hand side
@@ -905,69 +971,68 @@ __device__ __forceinline__ void solve_body(const MGFast *__restrict__ mp, double
         if (decide == 3)
             for (int t = bid; t < ntile; t += P)
                 for (int e = tid; e < tn; e += nt) {
-                    const int j = t * tw + e % tw;
-                    if (j < n) phi[(size_t)(1 + e / tw) * nr + j] = 0.0;
+                    const int j = t * tw + (e & (tw - 1));
+                    if (j < n) phi[(size_t)(1 + (e >> ltw)) * nr + j] = 0.0;
                 }
-        if (decide != 0) {  // phi holds the iterate of this residual
-            leave(cyc);
-            return;
-        }
+        if (decide != 0) break;  // phi holds the iterate of this residual
         // ---- up: per unit, a black line with the two red lines beside it ----
         constexpr int kE = (NW + nt - 1) / nt;  // unknowns of a line per thread
-        for (int k = 0; k < nun; ++k, ++g) {
+        for (int k = 0; k < nun && !fail; ++k, ++g) {
             int l, q;
             unit_at(bid + k * P, l, q);
-            const int nzl = m.nz[l], nzc = m.nz[l + 1], slot = nun <= S ? k : g % S;
-            const int ra = 2 * q + 1, rb = 2 * q + 3, ib = 2 * q + 2;
-            Wv *u = (Wv *)m.lu[l];
-            const Wv *uc = (const Wv *)m.lu[l + 1], *f = (const Wv *)m.lf[l];
-            const Tv *czl = mixed ? (const Tv *)m.cz32[l] : (const Tv *)m.cz[l];
-            // coarse rows below ra, between (row ib) and above rb; the level's
-            // ends are zero
-            const int Ia = q, Im = q + 1, Ib = q + 2;
-            const bool va = Ia > 0, vb = Ib < nzc - 1;
-            Tv um0[kE];  // level L-1: the coarsest row, solved here
-            if (l == L - 1) {
-                const Wv *fc = (const Wv *)m.lf[L];
+            const int nzc = m.nz[l + 1], slot = nun <= S ? k : g % S;
+            const bool deep = l == L - 1;  // the coarsest row is solved here first
+            const int ra = 2 * q + 1;      // rows ra and ra + 2 red, ra + 1 black
+            Wv *u = (Wv *)m.lu[l] + (size_t)ra * nr;
+            const Tv *czl = (mixed ? (const Tv *)m.cz32[l] : (const Tv *)m.cz[l]) + (size_t)2 * q * nr;
+            // warps 0 and 1 solve the reds, warp 2 the black line: their factors
+            // come into registers while the coarse rows are on their way
+            if (!ld_wait(ld, slot) || (deep && !ld_wait(ld, kMaxSlots))) fail = true;
+            constexpr bool kReg = WIDE && sizeof(Tv) == 4 && M <= 16;
+            LineFactors<Tv, M, kReg> lf;
+            if (warp < 3) lf.load(slots + (size_t)(slot * 3 + (warp == 0 ? 0 : 3 - warp)) * LFE, lane);
+            Tv um0[kE];  // deep: the coarsest row
+            if (deep) {
                 const Wv *p[kE];
                 Tv x[kE];
 #pragma unroll
-                for (int s = 0; s < kE; ++s) p[s] = tid + s * nt < n ? fc + nr + tid + s * nt : nullptr;
+                for (int s = 0; s < kE; ++s) p[s] = tid + s * nt < n ? (const Wv *)m.lf[L] + nr + tid + s * nt : nullptr;
                 flag_wait<Tv, kE>(p, x, tag, &ctl->timeout, fail);
 #pragma unroll
                 for (int s = 0; s < kE; ++s)
-                    if (tid + s * nt < NW) Bf0[at(tid + s * nt)] = x[s];
-                if (!ld_wait(ld, kMaxSlots)) fail = true;
+                    if (tid + s * nt < NW) Bf[at(tid + s * nt)] = x[s];
                 if (__syncthreads_or(fail)) {
-                    if (tid == 0) atomicExch(&ctl->timeout, 1);
-                    leave(cyc);
-                    return;
+                    fail = true;
+                    break;
                 }
-                if (warp == 0) warp_line_solve<Tv, M>(FC, Bf0, lane);
+                if (warp == 0) warp_line_solve<Tv, M>(FC, Bf, lane);
                 __syncthreads();
 #pragma unroll
-                for (int s = 0; s < kE; ++s) um0[s] = tid + s * nt < NW ? Bf0[at(tid + s * nt)] : (Tv)0;
+                for (int s = 0; s < kE; ++s) um0[s] = tid + s * nt < NW ? Bf[at(tid + s * nt)] : (Tv)0;
             }
-            // rows ra, ib = ra + 1, rb = ra + 2: cz[ib - 1] = cz[ra], cz[ib] = cz[rb - 1]
-            Tv z[4][kE], fx[3 * kE], ux[3 * kE];
+            Tv z[4][kE], fx[3 * kE], ux[3 * kE];  // z: cz below ra, ra + 1, ra + 2 and above it
             {
                 const Wv *p[3 * kE];
+                const Wv *f = (const Wv *)m.lf[l] + (size_t)ra * nr, *uc = (const Wv *)m.lu[l + 1] + (size_t)q * nr;
 #pragma unroll
                 for (int s = 0; s < kE; ++s) {
                     const int j = tid + s * nt;
 #pragma unroll
-                    for (int w = 0; w < 4; ++w) z[w][s] = j < n ? czl[(size_t)(2 * q + w) * nr + j] : (Tv)0;
+                    for (int w = 0; w < 4; ++w) z[w][s] = j < n ? czl[(size_t)w * nr + j] : (Tv)0;
 #pragma unroll
-                    for (int w = 0; w < 3; ++w) p[3 * s + w] = j < n ? f + (size_t)(ra + w) * nr + j : nullptr;
+                    for (int w = 0; w < 3; ++w) p[3 * s + w] = j < n ? f + (size_t)w * nr + j : nullptr;
                 }
                 flag_wait<Tv, 3 * kE>(p, fx, tag, &ctl->timeout, fail);
-                if (l < L - 1) {
+                if (!deep) {
+                    // coarse rows below ra, between (row ra + 1) and above
+                    // ra + 2: q, q + 1, q + 2, zero at the level's ends
+                    const bool lo = q > 0, hi = q + 2 < nzc - 1;
 #pragma unroll
                     for (int s = 0; s < kE; ++s) {
                         const int j = tid + s * nt;
-                        p[3 * s] = j < n && va ? uc + (size_t)Ia * nr + j : nullptr;
-                        p[3 * s + 1] = j < n ? uc + (size_t)Im * nr + j : nullptr;
-                        p[3 * s + 2] = j < n && vb ? uc + (size_t)Ib * nr + j : nullptr;
+                        p[3 * s] = j < n && lo ? uc + j : nullptr;
+                        p[3 * s + 1] = j < n ? uc + nr + j : nullptr;
+                        p[3 * s + 2] = j < n && hi ? uc + (size_t)2 * nr + j : nullptr;
                     }
                     flag_wait<Tv, 3 * kE>(p, ux, tag, &ctl->timeout, fail);
                 } else {
@@ -978,53 +1043,52 @@ __device__ __forceinline__ void solve_body(const MGFast *__restrict__ mp, double
                     }
                 }
             }
-            // right-hand sides: reds get f plus the coarse correction injected
-            // at rows i -/+ 1; the black line keeps its own f and couplings
+            // right-hand sides: the reds get f plus the coarse correction
+            // injected at the rows beside them; the black line its own f
 #pragma unroll
             for (int s = 0; s < kE; ++s) {
                 const int j = tid + s * nt;
                 if (j >= NW) break;
-                const int pj = at(j);
-                Bf0[pj] = fx[3 * s] + z[0][s] * ux[3 * s] + z[1][s] * ux[3 * s + 1];
-                Bf1[pj] = fx[3 * s + 2] + z[2][s] * ux[3 * s + 1] + z[3][s] * ux[3 * s + 2];
-                Bf2[pj] = fx[3 * s + 1];
-                W0[j] = z[1][s];
-                W1[j] = z[2][s];
+                Tv *B = Bf + at(j);
+                B[0] = fx[3 * s] + z[0][s] * ux[3 * s] + z[1][s] * ux[3 * s + 1];
+                B[BL] = fx[3 * s + 2] + z[2][s] * ux[3 * s + 1] + z[3][s] * ux[3 * s + 2];
             }
-            if (!ld_wait(ld, slot)) fail = true;
             if (__syncthreads_or(fail)) {
-                if (tid == 0) atomicExch(&ctl->timeout, 1);
-                leave(cyc);
-                return;
+                fail = true;
+                break;
             }
-            const Tv *F = slots + (size_t)slot * 3 * LFE;
-            if (warp == 0)
-                warp_line_solve<Tv, M>(F, Bf0, lane);
-            else if (warp == 1)
-                warp_line_solve<Tv, M>(F + 2 * LFE, Bf1, lane);
+            if (warp < 2) warp_line_solve<Tv, M, kReg>(lf, Bf + warp * BL, lane);
             __syncthreads();
 #pragma unroll
             for (int s = 0; s < kE; ++s) {
                 const int j = tid + s * nt;
-                if (j >= n) break;
-                const int pj = at(j);
-                const Tv x0 = Bf0[pj], x1 = Bf1[pj];
-                Fv::store(u + (size_t)ra * nr + j, x0, tag);
-                // red rb is also the next black's red ra: one unit stores it
-                if (rb == nzl - 2) Fv::store(u + (size_t)rb * nr + j, x1, tag);
-                Bf2[pj] = Bf2[pj] + W0[j] * x0 + W1[j] * x1;
+                if (j >= NW) break;
+                Tv *B = Bf + at(j);
+                const Tv x0 = B[0], x1 = B[BL];
+                B[2 * BL] = fx[3 * s + 1] + z[1][s] * x0 + z[2][s] * x1;
+                if (j < n) {
+                    Fv::store(u + j, x0, tag);
+                    // red ra + 2 is also the next unit's ra: one stores it
+                    if (ra + 2 == m.nz[l] - 2) Fv::store(u + (size_t)2 * nr + j, x1, tag);
+                }
             }
             __syncthreads();
-            if (warp == 0) warp_line_solve<Tv, M>(F + LFE, Bf2, lane);
+            if (warp == 2) warp_line_solve<Tv, M, kReg>(lf, Bf + 2 * BL, lane);
             __syncthreads();
             if (nun > S) request(g + S, slot);
 #pragma unroll
             for (int s = 0; s < kE; ++s) {
                 const int j = tid + s * nt;
-                if (j < n) Fv::store(u + (size_t)ib * nr + j, Bf2[at(j)], tag);
+                if (j < n) Fv::store(u + nr + j, Bf[2 * BL + at(j)], tag);
             }
         }
+        if (fail) break;
     }
+    // leave with no copy in flight (bounded waits), the tags used up
+    if (fail && tid == 0) atomicExch(&ctl->timeout, 1);
+#pragma unroll 1
+    for (int r = 0; r <= kMaxSlots; ++r) ld_wait(ld, r);
+    if (bid == 0 && tid == 0) *m.epoch = ep + (unsigned)cyc + 4u;
 }
 
 // MINB: blocks per SM the registers must allow: one for a reactor's solve
@@ -1033,7 +1097,7 @@ template <typename Tv, int M, int MINB>
 __global__ void __launch_bounds__(kSolveThreads, MINB)
     k_solve_persistent(const MGFast *__restrict__ mp, double *phi, int nr, SolveLayout lay, double tol,
                        int max_cycles, const StepCtl *sctl) {
-    solve_body<Tv, M>(mp, phi, nr, lay, tol, max_cycles, sctl, blockIdx.x, gridDim.x);
+    solve_body<Tv, M, MINB == 1>(mp, phi, nr, lay, tol, max_cycles, sctl, blockIdx.x, gridDim.x);
 }
 
 // The solves of several reactors (one line chunk M, one precision) in one
@@ -1052,7 +1116,7 @@ __global__ void __launch_bounds__(kSolveThreads, MINB) k_solve_multi(const Solve
     const SolveJob &j = jobs[lo];
     const int bid = (int)blockIdx.x - j.block0;
     if (bid >= j.nblocks) return;
-    solve_body<Tv, M>(j.mp, j.phi, j.nr, j.lay, j.tol, j.max_cycles, j.sctl, bid, j.nblocks);
+    solve_body<Tv, M, MINB == 1>(j.mp, j.phi, j.nr, j.lay, j.tol, j.max_cycles, j.sctl, bid, j.nblocks);
 }
 
 }  // namespace
@@ -1208,18 +1272,16 @@ bool solve_job(const FieldDims &fd, MGFast &m, double *phi, bool mixed, double t
         // row) while there are as many SMs, and on the FP64 path, whose factor
         // lines leave no room for more; else 8
         lay.tw = mixed && (!wide || n > 4 * nsm) ? 8 : 4;
-        // the line buffers and couplings of the line phases share their space
-        // with the residual phase's tile (with its two neighbour columns) and
+        // the line buffers of the line phases share their space with the residual phase's tile (with its two neighbour columns) and
         // restriction buffers (very tall meshes: narrower tiles)
-        const size_t buf = ((size_t)3 * M * kRow * es + 127) & ~(size_t)127, line = buf + (size_t)2 * kLine * M * es;
+        const size_t line = (size_t)3 * M * kRow * es;
         const size_t fac = LFE * es + (size_t)3 * LFE * es + 512;
         size_t tile = 0, both = 0;
         for (;; lay.tw /= 2) {
             tile = ((size_t)(lay.tw + 2) * nz * sizeof(double) + 127) & ~(size_t)127;
-            both = std::max(line, tile + (size_t)2 * lay.tw * nz * es);
+            both = std::max(line, tile + (size_t)lay.tw * (2 * nz + kMaxLevels) * es);
             if (lay.tw == 1 || both + fac <= kSolveSmemLimit) break;
         }
-        lay.offW = (int)buf;
         lay.offT = (int)tile;
         take(both);
         lay.offC = take(LFE * es);

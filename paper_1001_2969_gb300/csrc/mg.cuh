@@ -57,7 +57,7 @@ struct MGFast {
 
 // Shared-memory layout of the one-launch solve (byte offsets), set on the host.
 struct SolveLayout {
-    int offW;   // (from 0: three line buffers, M * 33 values each) the black line's two coupling coefficients, 32 M each
+    // from 0 in the line phases: three line buffers, M * 33 values each
     int offT;   // from 0 in the residual phase: the tile with its neighbour columns; at offT: two restriction buffers
     int offF;   // factor slots: each two red lines and the black line
     int offC;   // factors of the coarsest row
@@ -91,6 +91,8 @@ size_t mg_line_factor_elems(int nr);
 // a solve takes (entries of xr and xd)
 size_t mg_tile_elems(int nz, int nr);
 constexpr int kMaxSolveBlocks = 512;
+// copies of them, so that not every block reads the same few lines of L2
+constexpr int kCopies = 8;
 
 // copy the level table to the device (once: its pointers do not change)
 void mg_fast_upload(MGFast &m, cudaStream_t st);

@@ -661,9 +661,9 @@ void setup_device(pic_handle *h) {
         m.ps = (double *)dalloc(h, tb);
     }
     // flagged words and their epoch start at zero: tag 0 is never waited for
-    const size_t xb = (size_t)kMaxSolveBlocks * 8 * sizeof(ulonglong2);
+    const size_t xb = (size_t)kMaxSolveBlocks * 8 * kCopies * sizeof(ulonglong2);
     m.xr = (ulonglong2 *)dalloc(h, xb);
-    m.xd = m.xr + 4 * kMaxSolveBlocks;
+    m.xd = m.xr + 4 * kCopies * kMaxSolveBlocks;
     m.epoch = (unsigned *)dalloc(h, sizeof(unsigned));
     cudaMemsetAsync(m.xr, 0, xb, h->st);
     cudaMemsetAsync(m.epoch, 0, sizeof(unsigned), h->st);
