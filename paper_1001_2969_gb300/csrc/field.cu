@@ -21,7 +21,7 @@
 #include <math.h>
 #include <string.h>
 
-#include "pic_internal.cuh"
+#include "mg.cuh"
 
 namespace pic {
 
@@ -414,10 +414,13 @@ int mg_solve(const FieldDims &fd, MGWork &mg, const double *rho, const double *c
 
 // E = -grad phi: central inside, one-sided first order on the boundary rows
 // and on r = R, E_r = 0 on the axis
+// (solved not null: one thread reports the solve before it to ctl; should
+// that halt the step, what the others still write is not read)
 template <typename T>
 __global__ void k_efield(const double *phi, double *Ez, double *Er, typename V2<T>::type *E2,
-                         int nz, int nr, double dz, double dr, const StepCtl *ctl) {
+                         int nz, int nr, double dz, double dr, StepCtl *ctl, const MGCtl *solved) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (solved && k == 0) solve_report(solved, ctl, 0);
     if (k >= nz * nr || (ctl && ctl->halt)) return;
     const int i = k / nr, j = k % nr;
     double ez, er;
@@ -443,19 +446,36 @@ __global__ void k_efield(const double *phi, double *Ez, double *Er, typename V2<
 
 template <typename T>
 void launch_efield(const double *phi, double *Ez, double *Er, typename V2<T>::type *E2, int nz,
-                   int nr, double dz, double dr, const StepCtl *ctl, cudaStream_t st) {
-    k_efield<T><<<nblk(nz * nr), 256, 0, st>>>(phi, Ez, Er, E2, nz, nr, dz, dr, ctl);
+                   int nr, double dz, double dr, StepCtl *ctl, const MGCtl *solved, cudaStream_t st) {
+    k_efield<T><<<nblk(nz * nr), 256, 0, st>>>(phi, Ez, Er, E2, nz, nr, dz, dr, ctl, solved);
 }
 template void launch_efield<float>(const double *, double *, double *, float2 *, int, int, double,
-                                   double, const StepCtl *, cudaStream_t);
+                                   double, StepCtl *, const MGCtl *, cudaStream_t);
 template void launch_efield<double>(const double *, double *, double *, double2 *, int, int,
-                                    double, double, const StepCtl *, cudaStream_t);
+                                    double, double, StepCtl *, const MGCtl *, cudaStream_t);
 
 __global__ void k_moments(const double *Ne, const double *Ni, const double *V, const double *phi,
                           const double *Ez, const double *Er, double *m_ne, double *m_ni,
-                          double *m_phi, double *m_ez, double *m_er, int ng, const StepCtl *ctl) {
+                          double *m_phi, double *m_ez, double *m_er, int ng, StepCtl *c, StepEnd e) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= ng || (ctl && ctl->halt)) return;
+    // the step's end by one thread (nothing it writes is read by the others)
+    if (k == 0) {
+        // the barrier of the births numbering this pass's sort may run
+        c->bar = 0;
+        c->bar_timeout = 0;
+        if (!c->halt) {
+            *e.nmain0 = *e.nalive0;
+            unsigned long long n = (unsigned long long)(*e.nalive0);
+            if (e.nmain1) {
+                *e.nmain1 = *e.nalive1;
+                n += (unsigned long long)(*e.nalive1);
+            }
+            e.ds->cnt[PIC_C_PSTEPS] += n;
+            c->sort_pending = 1;
+            c->step += 1;
+        }
+    }
+    if (k >= ng || c->halt) return;
     m_ne[k] += Ne[k] / V[k];
     m_ni[k] += Ni[k] / V[k];
     m_phi[k] += phi[k];
@@ -463,10 +483,10 @@ __global__ void k_moments(const double *Ne, const double *Ni, const double *V, c
     m_er[k] += Er[k];
 }
 
-void launch_moments(const double *Ne, const double *Ni, const double *V, const double *phi,
-                    const double *Ez, const double *Er, double *m_ne, double *m_ni, double *m_phi,
-                    double *m_ez, double *m_er, int ng, const StepCtl *ctl, cudaStream_t st) {
-    k_moments<<<nblk(ng), 256, 0, st>>>(Ne, Ni, V, phi, Ez, Er, m_ne, m_ni, m_phi, m_ez, m_er, ng, ctl);
+void launch_moments(const double *Ne, const double *Ni, const double *V, const double *phi, const double *Ez,
+                    const double *Er, double *m_ne, double *m_ni, double *m_phi, double *m_ez,
+                    double *m_er, int ng, StepCtl *ctl, const StepEnd &e, cudaStream_t st) {
+    k_moments<<<nblk(ng), 256, 0, st>>>(Ne, Ni, V, phi, Ez, Er, m_ne, m_ni, m_phi, m_ez, m_er, ng, ctl, e);
 }
 
 }  // namespace pic

@@ -1187,31 +1187,7 @@ void raise_smem_limits() {
 
 namespace {
 
-// a timestep's solve reports to the step control instead of the host: V-cycle
-// count, residual, an unconverged flag, and a halt on a timed-out wait
-// `cont`: a second solve with the previous one's operator (the external
-// circuit's charge-free part) adds its cycles to the step's last report and
-// keeps the larger residual
-__global__ void k_solve_done(const MGCtl *c, StepCtl *s, int cont) {
-    if (s->halt) return;
-    if (c->timeout) {
-        s->halt = 1;
-        s->halt_status = ST_TIMEOUT;
-        s->halt_step = s->step;
-        return;
-    }
-    const int cyc = c->zero_rhs ? 0 : c->cycles;
-    s->mg_cycles += (unsigned long long)cyc;
-    const double res = (c->zero_rhs || !(c->bnorm > 0.0)) ? 0.0 : c->last_res / c->bnorm;
-    if (cont) {
-        s->mg_last_cycles += cyc;
-        s->mg_last_res = fmax(s->mg_last_res, res);
-    } else {
-        s->mg_last_cycles = cyc;
-        s->mg_last_res = res;
-    }
-    if (!c->zero_rhs && !c->converged) s->mg_flags |= 1;
-}
+__global__ void k_solve_done(const MGCtl *c, StepCtl *s, int cont) { solve_report(c, s, cont); }
 
 }  // namespace
 
@@ -1323,7 +1299,7 @@ int mg_fast_solve(const FieldDims &fd, MGFast &m, const double *rho, const doubl
                   const double *phi_zL, double *phi, bool warm, bool mixed, double tol,
                   int max_cycles, double *rel_res, int *launches, StepCtl *sctl, cudaStream_t st,
                   bool v_from_ctl, bool setup, cudaEvent_t at_solve, bool wide, SolveJob *defer,
-                  double *phi_prev) {
+                  double *phi_prev, bool report) {
     const int nz = fd.nz, nr = fd.nr, n = nr - 1, ng = nz * nr;
     const int M = line_chunk(n);
     const int nlev = m.nlev;
@@ -1414,8 +1390,10 @@ int mg_fast_solve(const FieldDims &fd, MGFast &m, const double *rho, const doubl
     }
     if (sctl) {
         // inside a timestep: the result stays on the device
-        k_solve_done<<<1, 1, 0, st>>>(m.ctl, sctl, setup ? 0 : 1);
-        ++L;
+        if (report) {
+            k_solve_done<<<1, 1, 0, st>>>(m.ctl, sctl, setup ? 0 : 1);
+            ++L;
+        }
         if (launches) *launches += L;
         return 0;
     }
@@ -1538,10 +1516,6 @@ int mg_multi_launch(const std::vector<SolveJob> &jobs, int j0, int j1, const Sol
     lc.attrs = at;
     lc.numAttrs = 1;
     return cudaLaunchKernelExC(&lc, jobs[j0].fn, args) == cudaSuccess ? 0 : kSolveNoLaunch;
-}
-
-void mg_solve_done(MGFast &m, StepCtl *sctl, bool first_of_step, cudaStream_t st) {
-    k_solve_done<<<1, 1, 0, st>>>(m.ctl, sctl, first_of_step ? 0 : 1);
 }
 
 }  // namespace pic

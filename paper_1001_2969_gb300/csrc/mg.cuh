@@ -13,6 +13,32 @@ struct MGCtl {
     double last_res, bnorm;
 };
 
+// a timestep's solve reports to the step control instead of the host: V-cycle
+// count, residual, an unconverged flag, and a halt on a timed-out wait (one
+// thread calls it).  `cont`: a second solve with the previous one's operator
+// (the external circuit's charge-free part) adds its cycles to the step's last
+// report and keeps the larger residual
+__device__ __forceinline__ void solve_report(const MGCtl *c, StepCtl *s, int cont) {
+    if (s->halt) return;
+    if (c->timeout) {
+        s->halt = 1;
+        s->halt_status = ST_TIMEOUT;
+        s->halt_step = s->step;
+        return;
+    }
+    const int cyc = c->zero_rhs ? 0 : c->cycles;
+    s->mg_cycles += (unsigned long long)cyc;
+    const double res = (c->zero_rhs || !(c->bnorm > 0.0)) ? 0.0 : c->last_res / c->bnorm;
+    if (cont) {
+        s->mg_last_cycles += cyc;
+        s->mg_last_res = fmax(s->mg_last_res, res);
+    } else {
+        s->mg_last_cycles = cyc;
+        s->mg_last_res = res;
+    }
+    if (!c->zero_rhs && !c->converged) s->mg_flags |= 1;
+}
+
 // returned by mg_fast_solve when a bounded device wait gave up, and when
 // the one-launch solve cannot be launched (shared memory, co-residency)
 constexpr int kSolveTimeout = -1000000;
@@ -109,8 +135,9 @@ void mg_fast_geometry(const MGFast &m, int nr, double dr, std::vector<double> &o
 // beside the solve.  wide: two blocks per black line (a reactor alone on the
 // GPU); else one (many reactors solving side by side).
 // defer (narrow solves of a batch): the set-up is enqueued, the solve itself
-// is described in *defer and left to mg_multi_launch; its end (the report to
-// sctl) is then mg_solve_done's.
+// is described in *defer and left to mg_multi_launch; the report to sctl is
+// then the caller's.
+// report false: the report to sctl is left to the caller (launch_efield).
 // phi_prev (warm solves only, optional): the potential of the step before
 // phi's; the V-cycles then start from 2 phi - phi_prev on the interior, and
 // phi_prev takes phi's values (the starting value w_0 of Algorithm 1,
@@ -119,7 +146,7 @@ int mg_fast_solve(const FieldDims &fd, MGFast &m, const double *rho, const doubl
                   const double *phi_zL, double *phi, bool warm, bool mixed, double tol,
                   int max_cycles, double *rel_res, int *launches, StepCtl *sctl, cudaStream_t st,
                   bool v_from_ctl = true, bool setup = true, cudaEvent_t at_solve = nullptr,
-                  bool wide = true, SolveJob *defer = nullptr, double *phi_prev = nullptr);
+                  bool wide = true, SolveJob *defer = nullptr, double *phi_prev = nullptr, bool report = true);
 
 // the launch shape of one reactor's solve (host only); false: not launchable
 bool solve_job(const FieldDims &fd, MGFast &m, double *phi, bool mixed, double tol, int max_cycles,
@@ -138,7 +165,4 @@ std::vector<std::pair<int, int>> mg_multi_plan(std::vector<SolveJob> &jobs, bool
 // launch the planned range [j0, j1) of the device copy of the table
 int mg_multi_launch(const std::vector<SolveJob> &jobs, int j0, int j1, const SolveJob *jobs_dev,
                     cudaStream_t st);
-// a deferred solve's report to its step control (k_solve_done)
-void mg_solve_done(MGFast &m, StepCtl *sctl, bool first_of_step, cudaStream_t st);
-
 }  // namespace pic

@@ -99,10 +99,11 @@ struct pic_handle {
     double *eedf = nullptr;
     double *tmp_grid[3] = {nullptr, nullptr, nullptr};
     double *mom_stage = nullptr;  // the scaled time averages on their way to host buffers
-    // pinned host copy of the step control and the status word, read once per call
-    struct HostCtl {
-        StepCtl c;
-        int32_t status;
+    // pinned host memory the device reports to: the step control and the status
+    // word once per call
+    struct HostCtl : CallReport {
+        unsigned long long cnt[PIC_NCOUNT];  // pic_moments' counters and absorbed charge
+        double qabs[3];
     } *host_ctl = nullptr;
     MGFast mgf;
     RadixTmp rtmp;
@@ -120,7 +121,6 @@ struct pic_handle {
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_fork2 = nullptr, ev_join2 = nullptr;
     StepGraph graphs[8];       // per (cur, cur_i, the pass moves the ions)
     StepGraph sort_graphs[4];  // the last pass's cell sort at the end of a call, per (cur, cur_i)
-    StepGraph check_graphs[4];  // its capacity check alone (the rest deferred), per (cur, cur_i)
     bool sort_deferred = false;  // the last pass's rank and births numbering are still to run
     bool in_batch = false;     // stepped with other reactors (pic_batch): narrow solves
     double ngas = 0.0, nu_max[2] = {0, 0}, p_null[2] = {0, 0};
@@ -330,9 +330,38 @@ __global__ void k_iota(int32_t *p, int n) {
     if (k < n) p[k] = k;
 }
 
-__global__ void k_scale(const double *src, double *dst, int n, double f) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k < n) dst[k] = src[k] * f;
+// pic_moments in one launch: the five averages and the EEDF scaled into their
+// buffers (null: skipped), the counters and the absorbed charge to pinned host
+// memory, and (reset) all of them cleared behind it.  blockIdx.y: the array.
+struct MomentsOut {
+    double *src[6], *dst[6];
+    int ng, nb, reset;
+    double f;
+    DevScalars *ds;
+    StepCtl *ctl;
+    unsigned long long *cnt;
+    double *qabs;
+};
+__global__ void k_moments_out(MomentsOut m) {
+    const int a = blockIdx.y, n = a == 5 ? m.nb : m.ng;
+    double *src = m.src[a], *dst = m.dst[a];
+    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
+        if (dst) dst[k] = src[k] * m.f;
+        if (m.reset) src[k] = 0.0;
+    }
+    if (a == 5 && blockIdx.x == 0) {
+        const int t = threadIdx.x;
+        if (t < PIC_NCOUNT) {
+            m.cnt[t] = m.ds->cnt[t];
+            if (m.reset) m.ds->cnt[t] = 0ull;
+        } else if (t >= 32 && t < 35) {
+            m.qabs[t - 32] = m.ds->qabs[t - 32];
+            if (m.reset) m.ds->qabs[t - 32] = 0.0;
+        } else if (t == 64 && m.reset) {
+            m.ctl->mg_cycles = 0ull;
+        }
+        __threadfence_system();
+    }
 }
 
 // step prologue: the field time's electrode voltage (Sec. 2.5 boundary data)
@@ -344,26 +373,6 @@ __global__ void k_step_begin(StepCtl *c, const double *rf, int nrf, double dt, i
     for (int k = 0; k < nrf; ++k) v += rf[k] * sin(2.0 * kPi * rf[nrf + k] * t + rf[2 * nrf + k]);
     c->V = v;
     c->do_split = split_every > 0 && (c->step % split_every) == split_every - 1;
-}
-
-// step epilogue: the pass wrote *nalive entries into the destination main
-// buffers; their cell sort is pending, and the step advances
-// nmain1 / nalive1 null: the pass held the ions still (subcycling)
-__global__ void k_step_end(StepCtl *c, DevScalars *ds, int32_t *nmain0, const int32_t *nalive0, int32_t *nmain1,
-                           const int32_t *nalive1) {
-    // the barrier of the births numbering this pass's sort may run
-    c->bar = 0;
-    c->bar_timeout = 0;
-    if (c->halt) return;
-    *nmain0 = *nalive0;
-    unsigned long long n = (unsigned long long)(*nalive0);
-    if (nmain1) {
-        *nmain1 = *nalive1;
-        n += (unsigned long long)(*nalive1);
-    }
-    ds->cnt[PIC_C_PSTEPS] += n;
-    c->sort_pending = 1;
-    c->step += 1;
 }
 
 // a pass that holds the ions: the births its newborn ions join start at
@@ -875,10 +884,9 @@ void one_step(pic_handle *h, cudaStream_t sb, bool mv, int part = 0, SolveJob *j
     const int src = h->cur, dst = 1 - h->cur;
     const int isrc = h->cur_i, idst = mv ? 1 - h->cur_i : h->cur_i;
     if (part == 2) {
-        mg_solve_done(h->mgf, h->sctl, true, st);
         launch_efield<T>(h->phi, h->Ez, h->Er, (typename V2<T>::type *)h->E2, h->nz, h->nr, h->dz,
-                         h->dr, h->sctl, st);
-        h->launches += 3;  // the shared solve's share, its report, E
+                         h->dr, h->sctl, h->mgf.ctl, st);
+        h->launches += 2;  // the shared solve's share, E
     } else {
     k_step_begin<<<1, 1, 0, st>>>(h->sctl, h->rf_d, h->cfg.rf.n, h->cfg.dt, h->cfg.split_every);
     h->launches += 1;
@@ -913,7 +921,7 @@ void one_step(pic_handle *h, cudaStream_t sb, bool mv, int part = 0, SolveJob *j
             mg_fast_solve(fd, h->mgf, h->rho, h->chi, 0.0, h->has_phiL ? h->phiL_d : nullptr, h->phi,
                           true, h->mixed, h->cfg.mg_tol, h->cfg.mg_max_cycles, nullptr, &L, h->sctl, st, true,
                           true, fork, !h->in_batch, part == 1 ? job : nullptr,
-                          h->cfg.mg_guess == PIC_GUESS_LINEAR ? h->phi_prev : nullptr);
+                          h->cfg.mg_guess == PIC_GUESS_LINEAR ? h->phi_prev : nullptr, false);
             if (part == 1) {
                 h->launches += L;
                 return;
@@ -925,7 +933,7 @@ void one_step(pic_handle *h, cudaStream_t sb, bool mv, int part = 0, SolveJob *j
             cudaEventRecord(h->ev_join, sb);
         }
         launch_efield<T>(h->phi, h->Ez, h->Er, (typename V2<T>::type *)h->E2, h->nz, h->nr, h->dz,
-                         h->dr, h->sctl, st);
+                         h->dr, h->sctl, h->cfg.circuit_C > 0.0 ? nullptr : h->mgf.ctl, st);
         h->launches += L + 2;
     }
     if (sb) cudaStreamWaitEvent(st, h->ev_join, 0);
@@ -988,29 +996,29 @@ void one_step(pic_handle *h, cudaStream_t sb, bool mv, int part = 0, SolveJob *j
     }
     {
         PhaseTimer t(h, 4);
+        const StepEnd e{h->ds, h->sp[0].d_nmain[dst], mv ? h->sp[1].d_nmain[idst] : nullptr, h->sp[0].d_nalive,
+                        mv ? h->sp[1].d_nalive : nullptr};
         launch_moments(h->N[0], h->N[1], h->V, h->phi, h->Ez, h->Er, h->m_acc[0], h->m_acc[1],
-                       h->m_acc[2], h->m_acc[3], h->m_acc[4], h->ng, h->sctl, st);
-        k_step_end<<<1, 1, 0, st>>>(h->sctl, h->ds, h->sp[0].d_nmain[dst], h->sp[0].d_nalive,
-                                     mv ? h->sp[1].d_nmain[idst] : nullptr, mv ? h->sp[1].d_nalive : nullptr);
-        h->launches += 2;
+                       h->m_acc[2], h->m_acc[3], h->m_acc[4], h->ng, h->sctl, e, st);
+        h->launches += 1;
     }
     h->cur = dst;
     h->cur_i = idst;
 }
 
-// the capacity check of the last pass's sort alone (end of a call): the
-// scans of the cell counts and the check.  Rank, births numbering and the
-// sorted counts stay pending; the next step's graph runs them beside its
-// solve, or complete_sort() before the state is read.  Scans and check are
-// idempotent on unchanged counts, so running them again there is harmless.
-void check_tail(pic_handle *h) {
-    PhaseTimer t(h, 3);
-    for (int s = 0; s < 2; ++s) {
-        SpecDev &d = h->sp[s];
-        launch_scan(d.counts, d.cursor, h->ncell, d.block_sums, d.d_ntotal, d.cap, h->ds, h->sctl, h->st);
+// the end of a call on stream `on`: the capacity check of the last pass's sort
+// and the report to pinned memory.  Rank, births numbering and the sorted
+// counts stay pending; the next step's graph runs them beside its solve, or
+// complete_sort() before the state is read.
+void call_tail(pic_handle *h, cudaStream_t on) {
+    if (!h->host_ctl && cudaMallocHost((void **)&h->host_ctl, sizeof(*h->host_ctl)) != cudaSuccess) {
+        h->host_ctl = nullptr;
+        cudaGetLastError();
     }
-    launch_step_check(h->ds, h->sctl, h->st);
-    h->launches += 7;
+    const int32_t *counts[2] = {h->sp[0].counts, h->sp[1].counts};
+    const int64_t cap[2] = {h->sp[0].cap, h->sp[1].cap};
+    launch_call_tail(counts, h->ncell, cap, h->ds, h->sctl, h->host_ctl, on);
+    h->launches += 1;
 }
 
 // the pending sort of the last pass (end of a call), on h->st
@@ -1027,10 +1035,6 @@ void drop_graphs(pic_handle *h) {
         g = StepGraph();
     }
     for (StepGraph &g : h->sort_graphs) {
-        if (g.exec) cudaGraphExecDestroy(g.exec);
-        g = StepGraph();
-    }
-    for (StepGraph &g : h->check_graphs) {
         if (g.exec) cudaGraphExecDestroy(g.exec);
         g = StepGraph();
     }
@@ -1074,20 +1078,16 @@ void capture_step(pic_handle *h, StepGraph &g, bool mv) {
     }
 }
 
-// capture the pending sort of the current parity (the end of a call), or
-// its capacity check alone
+// capture the pending sort of the current parity
 template <typename T>
-void capture_sort(pic_handle *h, StepGraph &g, bool check_only) {
+void capture_sort(pic_handle *h, StepGraph &g) {
     const int64_t L0 = h->launches;
     cudaStream_t keep = h->st;
     h->st = h->gst;
     cudaGraph_t graph = nullptr;
     cudaError_t e = cudaStreamBeginCapture(h->gst, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
-        if (check_only)
-            check_tail(h);
-        else
-            sort_tail<T>(h);
+        sort_tail<T>(h);
         e = cudaStreamEndCapture(h->gst, &graph);
     }
     h->st = keep;
@@ -1102,15 +1102,14 @@ void capture_sort(pic_handle *h, StepGraph &g, bool check_only) {
     }
 }
 
-// enqueue the pending sort, or its capacity check alone, on stream `on`
-// (private stream: as a graph)
-void enqueue_sort_tail(pic_handle *h, cudaStream_t on, bool check_only = false) {
-    StepGraph &g = (check_only ? h->check_graphs : h->sort_graphs)[h->cur + 2 * h->cur_i];
+// enqueue the pending sort on stream `on` (private stream: as a graph)
+void enqueue_sort_tail(pic_handle *h, cudaStream_t on) {
+    StepGraph &g = h->sort_graphs[h->cur + 2 * h->cur_i];
     if (on == h->gst && !g.exec && !g.failed) {
         if (h->mixed)
-            capture_sort<float>(h, g, check_only);
+            capture_sort<float>(h, g);
         else
-            capture_sort<double>(h, g, check_only);
+            capture_sort<double>(h, g);
     }
     if (on == h->gst && g.exec) {
         cudaGraphLaunch(g.exec, h->gst);
@@ -1119,9 +1118,7 @@ void enqueue_sort_tail(pic_handle *h, cudaStream_t on, bool check_only = false) 
     }
     cudaStream_t keep = h->st;
     h->st = on;
-    if (check_only)
-        check_tail(h);
-    else if (h->mixed)
+    if (h->mixed)
         sort_tail<float>(h);
     else
         sort_tail<double>(h);
@@ -1420,21 +1417,17 @@ void resync_ions(pic_handle *h, bool cut_births) {
     h->launches += 6;
 }
 
-pic_status finish_call(pic_handle *h, int64_t step0, int cur0, int cur_i0, int32_t nsteps) {
-    // the one synchronisation of a call: both words into pinned memory
-    if (!h->host_ctl && cudaMallocHost((void **)&h->host_ctl, sizeof(*h->host_ctl)) != cudaSuccess) {
-        h->host_ctl = nullptr;
-        cudaGetLastError();
+// reported: call_tail has written the report
+pic_status finish_call(pic_handle *h, int64_t step0, int cur0, int cur_i0, int32_t nsteps, bool reported) {
+    CallReport local;
+    CallReport *rp = h->host_ctl ? h->host_ctl : &local;
+    if (!reported || !h->host_ctl) {
+        cudaMemcpyAsync(&rp->c, h->sctl, sizeof(StepCtl), cudaMemcpyDeviceToHost, h->st);
+        cudaMemcpyAsync(&rp->status, &h->ds->status, sizeof(int32_t), cudaMemcpyDeviceToHost, h->st);
     }
-    StepCtl local_c;
-    int32_t local_status = 0;
-    StepCtl *cp = h->host_ctl ? &h->host_ctl->c : &local_c;
-    int32_t *sp = h->host_ctl ? &h->host_ctl->status : &local_status;
-    cudaMemcpyAsync(cp, h->sctl, sizeof(StepCtl), cudaMemcpyDeviceToHost, h->st);
-    cudaMemcpyAsync(sp, &h->ds->status, sizeof(int32_t), cudaMemcpyDeviceToHost, h->st);
     cudaStreamSynchronize(h->st);
-    const StepCtl c = *cp;
-    const int32_t status = *sp;
+    const StepCtl c = rp->c;
+    const int32_t status = rp->status;
     pic_status ce = cuda_check(h, "step");
     if (ce != PIC_OK) return ce;
     // a failed sort ends the call at the pass it sorts, before any later failure
@@ -1506,7 +1499,7 @@ pic_status complete_sort(pic_handle *h) {
     if (!h->sort_deferred) return PIC_OK;
     h->sort_deferred = false;
     enqueue_sort_tail(h, h->st);
-    return finish_call(h, h->step, h->cur, h->cur_i, 0);
+    return finish_call(h, h->step, h->cur, h->cur_i, 0, false);
 }
 
 }  // namespace
@@ -1657,12 +1650,12 @@ pic_status pic_step(pic_handle *h, int32_t nsteps) {
     // the last pass's sort: its capacity check now (a failure is this
     // call's); its rank and births numbering run beside the next step's
     // solve, or before the particle state is read (complete_sort)
-    enqueue_sort_tail(h, on_gst ? h->gst : h->st, true);
+    call_tail(h, on_gst ? h->gst : h->st);
     if (on_gst) {
         cudaEventRecord(h->ev_out, h->gst);
         cudaStreamWaitEvent(h->st, h->ev_out, 0);
     }
-    const pic_status r = finish_call(h, step0, cur0, cur_i0, nsteps);
+    const pic_status r = finish_call(h, step0, cur0, cur_i0, nsteps, true);
     // a failed step leaves the state at the last completed step, sorted
     h->sort_deferred = r == PIC_OK || r == PIC_ERR_NOT_CONVERGED || r == PIC_ERR_NUMERIC;
     return r;
@@ -1784,21 +1777,14 @@ pic_status pic_batch_step(pic_batch *b, int32_t nsteps, pic_status *statuses) {
         }
     }
     if (nsteps > 0) {
-        // every reactor's last sort, side by side on the reactors' streams
-        for (pic_handle *h : b->hs) {
-            StepGraph &g = h->sort_graphs[h->cur + 2 * h->cur_i];
-            if (!g.exec && !g.failed) {
-                if (h->mixed)
-                    capture_sort<float>(h, g, false);
-                else
-                    capture_sort<double>(h, g, false);
-            }
-        }
+        // every reactor's capacity check and report, side by side on the
+        // reactors' streams; the rest of their last sorts waits for the next
+        // step or for the state to be read, as in pic_step
         cudaEventRecord(b->ev_fork, b->origin);
         for (size_t k = 0; k < nh; ++k) {
             pic_handle *h = b->hs[k];
             cudaStreamWaitEvent(h->gst, b->ev_fork, 0);
-            enqueue_sort_tail(h, h->gst);
+            call_tail(h, h->gst);
             cudaEventRecord(b->ev_join[k], h->gst);
             cudaStreamWaitEvent(b->origin, b->ev_join[k], 0);
         }
@@ -1809,8 +1795,8 @@ pic_status pic_batch_step(pic_batch *b, int32_t nsteps, pic_status *statuses) {
     cudaStreamSynchronize(b->st);
     pic_status first = PIC_OK;
     for (size_t k = 0; k < nh; ++k) {
-        const pic_status r = nsteps > 0 ? finish_call(b->hs[k], step0[k], cur0[k], cur0[k], nsteps) : PIC_OK;
-        if (nsteps > 0) b->hs[k]->sort_deferred = false;  // the batch ends with the whole sort
+        const pic_status r = nsteps > 0 ? finish_call(b->hs[k], step0[k], cur0[k], cur0[k], nsteps, true) : PIC_OK;
+        if (nsteps > 0) b->hs[k]->sort_deferred = r == PIC_OK || r == PIC_ERR_NOT_CONVERGED || r == PIC_ERR_NUMERIC;
         if (statuses) statuses[k] = r;
         if (first == PIC_OK && r != PIC_OK) first = r;
     }
@@ -1876,43 +1862,52 @@ pic_status pic_moments(pic_handle *h, pic_moments_out *out, int32_t reset) {
             return fail(h, PIC_ERR_CUDA, "moments: staging allocation failed");
         }
     }
+    MomentsOut mo{};
     for (int k = 0; k < 5; ++k) {
-        if (!dst[k]) continue;
-        double *to = out->on_device ? dst[k] : h->mom_stage + (size_t)k * h->ng;
-        k_scale<<<(h->ng + 255) / 256, 256, 0, h->st>>>(h->m_acc[k], to, h->ng, f);
-        if (!out->on_device) cudaMemcpyAsync(dst[k], to, gb, cudaMemcpyDeviceToHost, h->st);
-        h->launches += 1;
+        mo.src[k] = h->m_acc[k];
+        if (dst[k]) mo.dst[k] = out->on_device ? dst[k] : h->mom_stage + (size_t)k * h->ng;
     }
-    if (out->eedf && h->cfg.eedf_bins > 0) {
-        double *to = out->on_device ? out->eedf : h->mom_stage + 5 * (size_t)h->ng;
-        k_scale<<<(h->cfg.eedf_bins + 255) / 256, 256, 0, h->st>>>(h->eedf, to, h->cfg.eedf_bins, f);
-        if (!out->on_device)
-            cudaMemcpyAsync(out->eedf, to, (size_t)h->cfg.eedf_bins * sizeof(double), cudaMemcpyDeviceToHost, h->st);
-        h->launches += 1;
+    mo.src[5] = h->eedf;
+    if (out->eedf && h->cfg.eedf_bins > 0) mo.dst[5] = out->on_device ? out->eedf : h->mom_stage + 5 * (size_t)h->ng;
+    mo.ng = h->ng;
+    mo.nb = h->cfg.eedf_bins;
+    mo.f = f;
+    mo.reset = reset ? 1 : 0;
+    mo.ds = h->ds;
+    mo.ctl = h->sctl;
+    if (!h->host_ctl && cudaMallocHost((void **)&h->host_ctl, sizeof(*h->host_ctl)) != cudaSuccess) {
+        h->host_ctl = nullptr;
+        cudaGetLastError();
+        return fail(h, PIC_ERR_CUDA, "moments: pinned memory");
     }
-    DevScalars ds;
-    cudaMemcpyAsync(&ds, h->ds, sizeof(ds), cudaMemcpyDeviceToHost, h->st);
+    mo.cnt = h->host_ctl->cnt;
+    mo.qabs = h->host_ctl->qabs;
+    k_moments_out<<<dim3(std::max(1, std::min(64, (h->ng + 255) / 256)), 6), 256, 0, h->st>>>(mo);
+    h->launches += 1;
+    if (!out->on_device) {
+        for (int k = 0; k < 5; ++k)
+            if (dst[k]) cudaMemcpyAsync(dst[k], mo.dst[k], gb, cudaMemcpyDeviceToHost, h->st);
+        if (mo.dst[5])
+            cudaMemcpyAsync(out->eedf, mo.dst[5], (size_t)h->cfg.eedf_bins * sizeof(double), cudaMemcpyDeviceToHost,
+                            h->st);
+    }
     cudaStreamSynchronize(h->st);
+    const pic_status ce = cuda_check(h, "moments");
+    if (ce != PIC_OK) return ce;
     if (out->counters) {
-        for (int k = 0; k < PIC_NCOUNT; ++k) out->counters[k] = (int64_t)ds.cnt[k];
+        for (int k = 0; k < PIC_NCOUNT; ++k) out->counters[k] = (int64_t)h->host_ctl->cnt[k];
         out->counters[PIC_C_MGCYC] = h->mg_cycles_total;
         out->counters[PIC_C_STEPS] = h->steps_total;
     }
     if (out->charge)
-        for (int k = 0; k < 3; ++k) out->charge[k] = ds.qabs[k];
+        for (int k = 0; k < 3; ++k) out->charge[k] = h->host_ctl->qabs[k];
     out->nsamples = h->nsamples;
     if (reset) {
-        for (int k = 0; k < 5; ++k) cudaMemsetAsync(h->m_acc[k], 0, gb, h->st);
-        cudaMemsetAsync(h->eedf, 0, (size_t)std::max(1, h->cfg.eedf_bins) * 8, h->st);
-        cudaMemsetAsync(h->ds->cnt, 0, sizeof(ds.cnt), h->st);
-        cudaMemsetAsync(h->ds->qabs, 0, sizeof(ds.qabs), h->st);
         h->nsamples = 0;
         h->mg_cycles_total = 0;
-        cudaMemsetAsync(&h->sctl->mg_cycles, 0, sizeof(unsigned long long), h->st);
         h->steps_total = 0;
-        cudaStreamSynchronize(h->st);
     }
-    return cuda_check(h, "moments");
+    return PIC_OK;
 }
 
 pic_status pic_get_particles(pic_handle *h, int32_t s, pic_particles_view *view_, int64_t capacity) {

@@ -244,6 +244,13 @@ struct DevScalars {
     unsigned long long mg_res_bits;  // max |residual| of the last residual kernel
     unsigned long long mg_aux_bits;
     int32_t chunk_next[2];  // the particle pass's next unclaimed chunk, per species
+    int32_t tail_total[2], tail_blocks;  // k_call_tail's sums and finished blocks, zero between calls
+};
+
+// what a call reads back at its end (pinned host memory)
+struct CallReport {
+    StepCtl c;
+    int32_t status;
 };
 
 template <typename T>
@@ -348,6 +355,10 @@ void launch_hist(PBuf<T> buf, const int32_t *n_dev, int32_t *counts, cudaStream_
 void launch_scan(const int32_t *counts, int32_t *cursor, int ncell, int32_t *block_sums,
                  int32_t *n_alive, int64_t capacity, DevScalars *ds, const StepCtl *ctl,
                  cudaStream_t st);
+// the end of a call: the capacity check of the pending sort's pass, and the
+// step control and status word written to *report (nullable)
+void launch_call_tail(const int32_t *const counts[2], int ncell, const int64_t cap[2], DevScalars *ds, StepCtl *ctl,
+                      CallReport *report, cudaStream_t st);
 // a failed check of the pending sort's pass (capacity, births overflow)
 void launch_step_check(const DevScalars *ds, StepCtl *ctl, cudaStream_t st);
 template <typename T>
@@ -419,12 +430,23 @@ void launch_finalize(const double *Ne, const double *Ni, const double *V, double
 int mg_solve(const FieldDims &fd, MGWork &mg, const double *rho, const double *chi, double V,
              const double *phi_zL, double *phi, bool warm, bool mixed, double tol, int max_cycles,
              double *rel_res, int *launches, cudaStream_t st);
+// solved (nullable): the report of the solve before it to ctl is made by the
+// same launch
+struct MGCtl;
 template <typename T>
 void launch_efield(const double *phi, double *Ez, double *Er, typename V2<T>::type *E2, int nz,
-                   int nr, double dz, double dr, const StepCtl *ctl, cudaStream_t st);
+                   int nr, double dz, double dr, StepCtl *ctl, const MGCtl *solved, cudaStream_t st);
+// the step's averages, and its end: the pass wrote *nalive entries into the
+// destination main buffers (nmain1, nalive1 null: it held the ions still),
+// their cell sort is pending, and the step advances
+struct StepEnd {
+    DevScalars *ds;
+    int32_t *nmain0, *nmain1;
+    const int32_t *nalive0, *nalive1;
+};
 void launch_moments(const double *Ne, const double *Ni, const double *V, const double *phi,
                     const double *Ez, const double *Er, double *m_ne, double *m_ni,
-                    double *m_phi, double *m_ez, double *m_er, int ng, const StepCtl *ctl,
+                    double *m_phi, double *m_ez, double *m_er, int ng, StepCtl *ctl, const StepEnd &e,
                     cudaStream_t st);
 
 }  // namespace pic

@@ -119,30 +119,51 @@ __global__ void k_scan_apply(const int32_t *counts, int ncell, const int32_t *bl
     }
 }
 
-// the whole scan in one block (meshes of at most kScanOne cells, a batch's
-// small reactors): each thread sums a run of consecutive cells, one block
-// scan, then each thread writes its run's cursors.  Larger meshes take the
-// three tile kernels, whose loads coalesce.
+// the whole scan in one block (meshes of at most kScanOne cells): tiles of
+// 4 x 1024 cells, each thread's four loaded as one vector (the arrays are
+// 256-byte aligned), all tiles' loads before the first block scan.  Larger
+// meshes take the three tile kernels.  (A run of consecutive cells per thread,
+// loaded one by one, took 18 us for 16384 cells.)
 constexpr int kScanOne = 16384;
 __global__ void __launch_bounds__(kScanThreads)
     k_scan_one(const int32_t *counts, int ncell, int32_t *cursor, int32_t *n_alive, int64_t capacity,
                DevScalars *ds, const StepCtl *ctl) {
     __shared__ int s_warp[32];
     if (sort_skip(ctl)) return;
-    const int per = (ncell + kScanThreads - 1) / kScanThreads;
-    const int c0 = min(ncell, threadIdx.x * per), c1 = min(ncell, c0 + per);
-    int v = 0;
-    for (int c = c0; c < c1; ++c) v += counts[c];
-    int tot;
-    int ex = block_exclusive_scan(v, s_warp, &tot);
-    for (int c = c0; c < c1; ++c) {
-        const int x = counts[c];
-        cursor[c] = ex;
-        ex += x;
+    constexpr int kTiles = kScanOne / kScanTile;
+    int c[kTiles][4];
+#pragma unroll
+    for (int t = 0; t < kTiles; ++t) {
+        const int base = t * kScanTile + threadIdx.x * 4;
+        if (base + 3 < ncell) {
+            const int4 v = *reinterpret_cast<const int4 *>(counts + base);
+            c[t][0] = v.x;
+            c[t][1] = v.y;
+            c[t][2] = v.z;
+            c[t][3] = v.w;
+        } else {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) c[t][q] = base + q < ncell ? counts[base + q] : 0;
+        }
+    }
+    int carry = 0;
+#pragma unroll
+    for (int t = 0; t < kTiles; ++t) {
+        const int base = t * kScanTile + threadIdx.x * 4;
+        if (t * kScanTile >= ncell) break;
+        int tot;
+        int ex = carry + block_exclusive_scan(c[t][0] + c[t][1] + c[t][2] + c[t][3], s_warp, &tot);
+        __syncthreads();  // s_warp is rewritten by the next tile
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            if (base + q < ncell) cursor[base + q] = ex;
+            ex += c[t][q];
+        }
+        carry += tot;
     }
     if (threadIdx.x == 0) {
-        *n_alive = tot;
-        if ((int64_t)tot > capacity) atomicOr(&ds->status, ST_CAPACITY);
+        *n_alive = carry;
+        if ((int64_t)carry > capacity) atomicOr(&ds->status, ST_CAPACITY);
     }
 }
 
@@ -167,6 +188,71 @@ __global__ void k_step_check(const DevScalars *ds, StepCtl *ctl) {
 
 void launch_step_check(const DevScalars *ds, StepCtl *ctl, cudaStream_t st) {
     k_step_check<<<1, 1, 0, st>>>(ds, ctl);
+}
+
+// The end of a call: the capacity check of the last pass's pending sort and
+// the call's report, in one launch.  The sort's totals are the sums of the
+// cell counts (its scans, run here before, took seven launches, 15-40 us at
+// the end of every call); blocks of both species add their parts, the last
+// block to finish checks the totals against the capacities, fails the sort if
+// one is over, and writes the step control and the status word to `report`
+// (pinned host memory; null: none).
+constexpr int kTailThreads = 512;
+__global__ void __launch_bounds__(kTailThreads)
+    k_call_tail(const int32_t *c0, const int32_t *c1, int ncell, int64_t cap0, int64_t cap1, DevScalars *ds,
+                StepCtl *ctl, CallReport *report) {
+    __shared__ int s_sum[kTailThreads / 32];
+    __shared__ int s_last;
+    const int32_t *counts = blockIdx.y == 0 ? c0 : c1;
+    const bool skip = sort_skip(ctl);
+    const int n4 = ncell >> 2;
+    int v = 0;
+    if (!skip) {
+        for (int k = blockIdx.x * kTailThreads + threadIdx.x; k < n4; k += gridDim.x * kTailThreads) {
+            const int4 x = reinterpret_cast<const int4 *>(counts)[k];
+            v += x.x + x.y + x.z + x.w;
+        }
+        if (blockIdx.x == 0 && (int)threadIdx.x < (ncell & 3)) v += counts[4 * n4 + threadIdx.x];
+    }
+    v = __reduce_add_sync(0xffffffffu, v);
+    if ((threadIdx.x & 31) == 0) s_sum[threadIdx.x >> 5] = v;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int t = 0;
+        for (int w = 0; w < kTailThreads / 32; ++w) t += s_sum[w];
+        atomicAdd(&ds->tail_total[blockIdx.y], t);
+        __threadfence();
+        s_last = atomicAdd(&ds->tail_blocks, 1) == (int)(gridDim.x * gridDim.y) - 1;
+    }
+    __syncthreads();
+    if (!s_last) return;
+    if (threadIdx.x == 0) {
+        __threadfence();
+        if (!skip) {
+            int st = *(volatile int32_t *)&ds->status;
+            if ((int64_t)atomicAdd(&ds->tail_total[0], 0) > cap0 || (int64_t)atomicAdd(&ds->tail_total[1], 0) > cap1) {
+                st |= ST_CAPACITY;
+                atomicOr(&ds->status, ST_CAPACITY);
+            }
+            if (st & (ST_CAPACITY | ST_BIRTH_OVERFLOW)) sort_failed(ctl, st & (ST_CAPACITY | ST_BIRTH_OVERFLOW));
+        }
+        ds->tail_total[0] = ds->tail_total[1] = ds->tail_blocks = 0;
+    }
+    __syncthreads();
+    if (report) {
+        const unsigned *src = reinterpret_cast<const unsigned *>(ctl);
+        unsigned *dst = reinterpret_cast<unsigned *>(&report->c);
+        for (int k = threadIdx.x; k < (int)(sizeof(StepCtl) / 4); k += kTailThreads)
+            dst[k] = *(volatile const unsigned *)(src + k);
+        if (threadIdx.x == 0) report->status = *(volatile int32_t *)&ds->status;
+        __threadfence_system();
+    }
+}
+
+void launch_call_tail(const int32_t *const counts[2], int ncell, const int64_t cap[2], DevScalars *ds, StepCtl *ctl,
+                      CallReport *report, cudaStream_t st) {
+    const int g = std::max(1, std::min(32, ncell / (kTailThreads * 8)));
+    k_call_tail<<<dim3(g, 2), kTailThreads, 0, st>>>(counts[0], counts[1], ncell, cap[0], cap[1], ds, ctl, report);
 }
 
 // ---- rank: perm[cursor[cell]++] = element (main first, then births) ----

@@ -529,7 +529,7 @@ int window_run(const WindowIn<T> &in, int K, int ckpt, const double *w_host, dou
                     throw 1;
                 if (grad) cudaMemcpyAsync(phi_all[n], phi, (size_t)ng * sizeof(double), cudaMemcpyDeviceToDevice, st);
             }
-            launch_efield<T>(phi, Ez, Er, E2, nz, nr, in.dz, in.dr, nullptr, st);
+            launch_efield<T>(phi, Ez, Er, E2, nz, nr, in.dz, in.dr, nullptr, nullptr, st);
             for (int s = 0; s < 2; ++s) {
                 cudaMemsetAsync(Nout[s], 0, (size_t)ng * sizeof(double), st);
                 if (in.n[s] > 0)
