@@ -38,64 +38,61 @@ __device__ __forceinline__ unsigned long long abs_bits(double x) {
 
 // ---- set-up ----
 
-// nodal chi of every coarse level: full weighting in z, injection on the
-// boundary rows; one warp per column, lanes over rows, levels in shared memory
-__global__ void k_chi_levels(const MGFast *__restrict__ mp, int nr, const StepCtl *ctl) {
+// Set-up, first launch: rho and chi from the particles' deposit (a timestep;
+// else chi is given), and nodal chi of every coarse level: full weighting in z,
+// injection on the boundary rows.  A block takes 2^lc columns: rows loaded side
+// by side, a warp per column down the levels in shared memory, levels stored
+// by rows.  Bound by launch latency and one trip to L2 each way.
+__global__ void __launch_bounds__(256) k_setup_levels(const MGFast *__restrict__ mp, int nr, int lc, FieldSource f,
+                                                      const StepCtl *ctl) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const MGFast &m = *mp;
     if (ctl && ctl->halt) return;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nz0 = m.nz[0];
-    const int j = blockIdx.x * (blockDim.x >> 5) + warp;
-    if (j >= nr) return;
-    double *src = reinterpret_cast<double *>(smem_raw) + (size_t)warp * 2 * nz0;
-    double *dst = src + nz0;
-    for (int i = lane; i < nz0; i += 32) src[i] = m.chi[0][(size_t)i * nr + j];
-    __syncwarp();
-    for (int l = 1; l < m.nlev; ++l) {
-        const int nzc = m.nz[l];
-        for (int I = lane; I < nzc; I += 32) {
-            const double v = (I == 0 || I == nzc - 1)
-                                 ? src[2 * I]
-                                 : 0.25 * src[2 * I - 1] + 0.5 * src[2 * I] + 0.25 * src[2 * I + 1];
-            dst[I] = v;
-            m.chi[l][(size_t)I * nr + j] = v;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nz0 = m.nz[0], nlev = m.nlev;
+    const int cols = 1 << lc, j0 = blockIdx.x << lc, st = 2 * nz0 + kMaxLevels;
+    double *s = reinterpret_cast<double *>(smem_raw);
+    for (int e = threadIdx.x; e < nz0 << lc; e += blockDim.x) {
+        const int c = e & (cols - 1), i = e >> lc, j = j0 + c;
+        if (j >= nr) continue;
+        const size_t k = (size_t)i * nr + j;
+        double x;
+        if (f.Ne) {
+            const double ne = f.Ne[k] / f.V[k], ni = f.Ni[k] / f.V[k];
+            f.rho[k] = f.q0 * ne + f.q1 * ni;
+            // chi = dt^2/(2 eps0) sum_s q_s^2 n_s / m_s ; c_s = q_s^2 dt^2 / (2 eps0 m_s)
+            x = f.c0 * ne + f.c1 * ni;
+            f.chi[k] = x;
+        } else {
+            x = f.chi[k];
         }
-        __syncwarp();
-        double *t = src;
-        src = dst;
-        dst = t;
+        s[(size_t)c * st + i] = x;
     }
-}
-
-// face coefficients of every level (flat index over all levels' nodes)
-__global__ void k_coefs_levels(const MGFast *__restrict__ mp, int nr, int face_mean, int total, const StepCtl *ctl) {
-    const MGFast &m = *mp;
-    const int g = blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= total || (ctl && ctl->halt)) return;
-    int l = 0, k = g;
-    while (k >= m.nz[l] * nr) {
-        k -= m.nz[l] * nr;
-        ++l;
+    if (nlev == 1) return;
+    __syncthreads();
+    for (int c = warp; c < cols; c += blockDim.x >> 5) {
+        const double *src = s + (size_t)c * st;
+        double *dst = s + (size_t)c * st + nz0;
+        for (int l = 1; l < nlev; ++l) {
+            const int nzc = m.nz[l];
+            for (int I = lane; I < nzc; I += 32)
+                dst[I] = (I == 0 || I == nzc - 1)
+                             ? src[2 * I]
+                             : 0.25 * src[2 * I - 1] + 0.5 * src[2 * I] + 0.25 * src[2 * I + 1];
+            __syncwarp();
+            src = dst;
+            dst += nzc;
+        }
     }
-    const int nz = m.nz[l], i = k / nr, j = k % nr;
-    const double *chi = m.chi[l];
-    const double c = chi[k];
-    double vz = 0.0, vr = 0.0;
-    if (i + 1 < nz) {
-        const double cn = chi[k + nr];
-        const double f = face_mean ? 0.5 * (c + cn) : fmax(c, cn);
-        vz = (1.0 + f) * m.gz[l][j];
-    }
-    if (j + 1 < nr) {
-        const double cn = chi[k + 1];
-        const double f = face_mean ? 0.5 * (c + cn) : fmax(c, cn);
-        vr = (1.0 + f) * m.gr[l][j];
-    }
-    m.cz[l][k] = vz;
-    m.cr[l][k] = vr;
-    if (m.cz32[l]) {
-        m.cz32[l][k] = (float)vz;
-        m.cr32[l][k] = (float)vr;
+    __syncthreads();
+    int at = nz0;
+    for (int l = 1; l < nlev; ++l) {
+        const int nzc = m.nz[l];
+        double *chi = m.chi[l];
+        for (int e = threadIdx.x; e < nzc << lc; e += blockDim.x) {
+            const int c = e & (cols - 1), I = e >> lc, j = j0 + c;
+            if (j < nr) chi[(size_t)I * nr + j] = s[(size_t)c * st + at + I];
+        }
+        at += nzc;
     }
 }
 
@@ -138,29 +135,103 @@ inline int line_chunk(int n) {
     return M;
 }
 
-// One warp per line over all lines of levels [l0, l1).  Computed in Ts.
-template <typename Ts>
-__global__ void k_factor_lines(const MGFast *__restrict__ mp, int l0, int l1, int nr, int M, int nlines,
-                               const StepCtl *ctl) {
+// what a node of the fine level starts from: the right-hand side
+// rho A_j dz / eps0, the operator's diagonal and the Dirichlet data of phi;
+// with phi_prev (a warm solve) the interior starts from 2 phi - phi_prev, the
+// linear extrapolation in time of the last two steps' potentials, and
+// phi_prev takes the last step's
+struct RhsArgs {
+    const double *rho;
+    double *phi;
+    const double *phi_zL;
+    double V;
+    int cold, v_from_ctl;
+    double *phi_prev;
+};
+__device__ __forceinline__ void rhs_node(const MGFast &m, const RhsArgs &a, double V, int nz, int nr, int i, int j,
+                                         double diag) {
+    const size_t k = (size_t)i * nr + j;
+    const bool inner = i > 0 && i < nz - 1 && j < nr - 1;
+    m.f0[k] = inner ? a.rho[k] * m.ga[j] : 0.0;
+    m.dg0[k] = inner ? diag : 0.0;
+    double p;
+    if (i == 0)
+        p = (j == nr - 1) ? 0.0 : V;
+    else if (i == nz - 1)
+        p = a.phi_zL ? a.phi_zL[j] : 0.0;
+    else if (j == nr - 1)
+        p = 0.0;
+    else if (a.cold)
+        p = 0.0;
+    else if (a.phi_prev) {
+        const double t = a.phi[k];
+        p = 2.0 * t - a.phi_prev[k];
+        a.phi_prev[k] = t;
+    } else
+        p = a.phi[k];
+    a.phi[k] = p;
+}
+
+// Set-up, second launch: per row of every level (a block each) the face
+// coefficients, stored for the solve and kept in shared memory for the row's
+// line factors (its first warp); on the fine level also what its nodes start
+// from.  One launch for what were three (coefficients, factors, right-hand
+// side), where the factors made a trip to L2 between each and the next (11 us
+// on c2, 32 us on c3 and in FP64).  Bound by the FP64 pipe: ~14 operations a
+// node, so a row's nodes are spread over the four SM partitions; a warp per
+// row was slower than the three launches.
+constexpr int kSetupThreads = 128;
+template <typename Ts, int M>
+__global__ void __launch_bounds__(kSetupThreads)
+    k_setup_lines(const MGFast *__restrict__ mp, const double *__restrict__ chi0, int nr, int face_mean, RhsArgs a,
+                  const StepCtl *ctl) {
+    constexpr int kPad = 33;
+    __shared__ Ts sd[M * kPad], se[M * kPad];  // cz below + above the row, cr
     const MGFast &m = *mp;
     if (ctl && ctl->halt) return;
-    const int n = nr - 1;
-    const int p = threadIdx.x & 31;
-    int g = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (g >= nlines) return;
-    int l = l0;
-    while (l < l1 && g >= m.nz[l] - 2) {
-        g -= m.nz[l] - 2;
-        ++l;
+    const int n = nr - 1, p = threadIdx.x & 31;
+    // the solve's control block starts cleared
+    if (blockIdx.x == 0)
+        for (int w = threadIdx.x; w < (int)(sizeof(MGCtl) / sizeof(unsigned)); w += blockDim.x)
+            reinterpret_cast<unsigned *>(m.ctl)[w] = 0u;
+    int i = blockIdx.x, l = 0;
+    while (i >= m.nz[l]) i -= m.nz[l++];
+    const int nz = m.nz[l];
+    const double *chi = (l == 0 ? chi0 : m.chi[l]) + (size_t)i * nr;
+    const bool inner = i > 0 && i < nz - 1, mixed = m.cz32[l] != nullptr;
+    const double V = (ctl && a.v_from_ctl) ? ctl->V : a.V;  // in a timestep the source voltage comes with the step
+    auto at = [](int j) { return (j % M) * kPad + j / M; };
+    auto face = [&](double x, double y) { return face_mean ? 0.5 * (x + y) : fmax(x, y); };
+    for (int j = threadIdx.x; j < nr; j += kSetupThreads) {
+        double lo = 0.0, hi = 0.0, right = 0.0;  // cz below and above the row, cr
+        const double c = chi[j], gz = m.gz[l][j];
+        if (i > 0) lo = (1.0 + face(chi[j - nr], c)) * gz;
+        if (i + 1 < nz) hi = (1.0 + face(c, chi[j + nr])) * gz;
+        if (j + 1 < nr) right = (1.0 + face(c, chi[j + 1])) * m.gr[l][j];
+        const size_t k = (size_t)i * nr + j;
+        if (mixed) {
+            m.cz32[l][k] = (float)hi;
+            m.cr32[l][k] = (float)right;
+        }
+        if (!mixed || l == 0) {  // (the mixed path's coarse levels are FP32)
+            m.cz[l][k] = hi;
+            m.cr[l][k] = right;
+        }
+        if (l == 0) {
+            const double left = j > 0 ? (1.0 + face(chi[j - 1], c)) * m.gr[0][j - 1] : 0.0;
+            rhs_node(m, a, V, nz, nr, i, j, lo + hi + left + right);
+        }
+        if (inner && j < n) {
+            sd[at(j)] = (Ts)lo + (Ts)hi;
+            se[at(j)] = (Ts)right;
+        }
     }
-    if (l >= l1) return;
+    __syncthreads();
+    if (!inner || threadIdx.x >= kLine) return;
     const bool f64 = sizeof(Ts) == 8;
-    const Ts *cz = f64 ? (const Ts *)m.cz[l] : (const Ts *)m.cz32[l];
-    const Ts *cr = f64 ? (const Ts *)m.cr[l] : (const Ts *)m.cr32[l];
     Ts *fac = (l == m.nlev - 1) ? (f64 ? (Ts *)m.facc : (Ts *)m.facc32)
                                 : (f64 ? (Ts *)m.fac64[l] : (Ts *)m.fac32[l]);
-    Ts *F = fac + (size_t)g * line_factor_elems(M);
-    const size_t rowk = (size_t)(1 + g) * nr;
+    Ts *F = fac + (size_t)(i - 1) * line_factor_elems(M);
     auto coef = [&](int k, Ts &lo, Ts &dg, Ts &up) {
         const int j = p * M + k;
         if (j >= n) {
@@ -169,60 +240,60 @@ __global__ void k_factor_lines(const MGFast *__restrict__ mp, int l0, int l1, in
             up = 0;
             return;
         }
-        const size_t q = rowk + j;
-        const Ts a = cz[q - nr], c = cz[q], e = cr[q];
-        const Ts d = j > 0 ? cr[q - 1] : (Ts)0;
-        lo = -d;
-        dg = a + c + d + e;
-        up = j < n - 1 ? -e : (Ts)0;
+        lo = j > 0 ? -se[at(j - 1)] : (Ts)0;
+        dg = sd[at(j)] - lo + se[at(j)];
+        up = j < n - 1 ? -se[at(j)] : (Ts)0;
     };
-    auto at = [&](int arr, int k) -> Ts & { return F[((size_t)arr * M + k) * kLine + p]; };
-    const int MI = M - 1;
+    constexpr int MI = M - 1;
     Ts A, B, C;  // reduced (interface) equation of this lane
     Ts loI, dgI, upI;
     coef(M - 1, loI, dgI, upI);
-    if (MI > 0) {
+    if constexpr (MI > 0) {
         // interior Thomas factors
-        Ts lo, dg, up, upm = 0, invd = 0;
+        Ts ell[MI], invd[MI], cp[MI], v[MI], w[MI];
+        Ts upm = 0, iv = 0, lo0 = 0, upL = 0;
+#pragma unroll
         for (int k = 0; k < MI; ++k) {
+            Ts lo, dg, up;
             coef(k, lo, dg, up);
-            Ts ell = 0, d = dg;
+            Ts el = 0, d = dg;
             if (k > 0) {
-                ell = lo * invd;
-                d = dg - ell * upm;
+                el = lo * iv;
+                d = dg - el * upm;
+            } else {
+                lo0 = lo;
             }
-            invd = recip(d);
-            at(0, k) = ell;
-            at(1, k) = invd;
-            at(2, k) = up * invd;
+            iv = recip(d);
+            ell[k] = el;
+            invd[k] = iv;
+            cp[k] = up * iv;
             upm = up;
+            upL = up;
         }
         // spikes: v answers -lo_0 at the first interior unknown, w answers
         // -up_{MI-1} at the last (forward sweep, then backward)
-        Ts lo0, dg0, up0;
-        coef(0, lo0, dg0, up0);
-        Ts vp = -lo0;
-        at(3, 0) = vp;
-        for (int k = 1; k < MI; ++k) {
-            vp = -at(0, k) * vp;
-            at(3, k) = vp;
-        }
-        Ts loL, dgL, upL;
-        coef(MI - 1, loL, dgL, upL);
-        Ts vn = at(3, MI - 1) * at(1, MI - 1), wn = -upL * at(1, MI - 1);
-        at(3, MI - 1) = vn;
-        at(4, MI - 1) = wn;
+        v[0] = -lo0;
+#pragma unroll
+        for (int k = 1; k < MI; ++k) v[k] = -ell[k] * v[k - 1];
+        v[MI - 1] = v[MI - 1] * invd[MI - 1];
+        w[MI - 1] = -upL * invd[MI - 1];
+#pragma unroll
         for (int k = MI - 2; k >= 0; --k) {
-            vn = at(3, k) * at(1, k) - at(2, k) * vn;
-            wn = -at(2, k) * wn;
-            at(3, k) = vn;
-            at(4, k) = wn;
+            v[k] = v[k] * invd[k] - cp[k] * v[k + 1];
+            w[k] = -cp[k] * w[k + 1];
         }
-        const Ts v0n = __shfl_down_sync(0xffffffffu, at(3, 0), 1);
-        const Ts w0n = __shfl_down_sync(0xffffffffu, at(4, 0), 1);
-        const Ts vL = at(3, MI - 1), wL = at(4, MI - 1);
-        A = loI * vL;
-        B = dgI + loI * wL + (p < kLine - 1 ? upI * v0n : (Ts)0);
+#pragma unroll
+        for (int k = 0; k < MI; ++k) {
+            F[(size_t)k * kLine + p] = ell[k];
+            F[(size_t)(M + k) * kLine + p] = invd[k];
+            F[(size_t)(2 * M + k) * kLine + p] = cp[k];
+            F[(size_t)(3 * M + k) * kLine + p] = v[k];
+            F[(size_t)(4 * M + k) * kLine + p] = w[k];
+        }
+        const Ts v0n = __shfl_down_sync(0xffffffffu, v[0], 1);
+        const Ts w0n = __shfl_down_sync(0xffffffffu, w[0], 1);
+        A = loI * v[MI - 1];
+        B = dgI + loI * w[MI - 1] + (p < kLine - 1 ? upI * v0n : (Ts)0);
         C = p < kLine - 1 ? upI * w0n : (Ts)0;
     } else {
         A = loI;
@@ -233,6 +304,7 @@ __global__ void k_factor_lines(const MGFast *__restrict__ mp, int l0, int l1, in
     Gf[p] = loI;
     Gf[kLine + p] = upI;
     // parallel cyclic reduction of the interface system over the lanes
+#pragma unroll
     for (int st = 0; st < 5; ++st) {
         const int s = 1 << st;
         const Ts Bm = __shfl_up_sync(0xffffffffu, B, s), Bp = __shfl_down_sync(0xffffffffu, B, s);
@@ -342,43 +414,13 @@ __device__ __forceinline__ void warp_line_solve(const Ts *F, Ts *Bs, int p) {
     warp_line_solve<Ts, M, false>(q, Bs, p);
 }
 
-// right-hand side rho A_j dz / eps0 and the Dirichlet data of phi; with
-// phi_prev (a warm solve) the interior starts from 2 phi - phi_prev, the
-// linear extrapolation in time of the last two steps' potentials, and
-// phi_prev takes the last step's
-__global__ void k_rhs_bc(const MGFast *__restrict__ mp, const double *rho, double *phi, const double *phi_zL,
-                         double V_arg, int nz, int nr, int cold, const StepCtl *ctl, int v_from_ctl,
-                         double *phi_prev) {
+// a further solve with the operator of the one before: its right-hand side and
+// boundary data alone
+__global__ void k_rhs_bc(const MGFast *__restrict__ mp, RhsArgs a, int nz, int nr, const StepCtl *ctl) {
     const MGFast &m = *mp;
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= nz * nr || (ctl && ctl->halt)) return;
-    const double V = (ctl && v_from_ctl) ? ctl->V : V_arg;  // in a timestep the source voltage comes with the step
-    const int i = k / nr, j = k % nr;
-    double v = 0.0, dg = 0.0;
-    if (i > 0 && i < nz - 1 && j < nr - 1) {
-        v = rho[k] * m.ga[j];
-        const double *cz = m.cz[0], *cr = m.cr[0];
-        dg = cz[k - nr] + cz[k] + (j > 0 ? cr[k - 1] : 0.0) + cr[k];
-    }
-    m.f0[k] = v;
-    m.dg0[k] = dg;
-    double p;
-    if (i == 0)
-        p = (j == nr - 1) ? 0.0 : V;
-    else if (i == nz - 1)
-        p = phi_zL ? phi_zL[j] : 0.0;
-    else if (j == nr - 1)
-        p = 0.0;
-    else if (cold)
-        p = 0.0;
-    else if (phi_prev) {
-        const double t = phi[k];
-        p = 2.0 * t - phi_prev[k];
-        phi_prev[k] = t;
-    } else
-        p = phi[k];
-    phi[k] = p;
-    // the solve's control block starts cleared
+    rhs_node(m, a, (ctl && a.v_from_ctl) ? ctl->V : a.V, nz, nr, k / nr, k % nr, m.dg0[k]);
     for (int w = k; w < (int)(sizeof(MGCtl) / sizeof(unsigned)); w += nz * nr)
         reinterpret_cast<unsigned *>(m.ctl)[w] = 0u;
 }
@@ -1171,7 +1213,7 @@ void raise_smem_limits() {
     static bool done = false;
     if (done) return;
     const int lim = (int)kSolveSmemLimit;
-    cudaFuncSetAttribute(k_chi_levels, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+    cudaFuncSetAttribute(k_setup_levels, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     for (int M = 1; M <= 32; M <<= 1) {
         for (int minb = 1; minb <= 2; ++minb) {
             cudaFuncSetAttribute(solve_kernel<float>(M, minb), cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
@@ -1295,51 +1337,57 @@ bool solve_job(const FieldDims &fd, MGFast &m, double *phi, bool mixed, double t
     return true;
 }
 
-int mg_fast_solve(const FieldDims &fd, MGFast &m, const double *rho, const double *chi, double V,
+template <typename Ts>
+static void launch_setup_lines(int M, int grid, cudaStream_t st, const MGFast *mp, const double *chi, int nr, int mean,
+                               const RhsArgs &a, const StepCtl *ctl) {
+    constexpr int nt = kSetupThreads;
+    switch (M) {
+        case 1: k_setup_lines<Ts, 1><<<grid, nt, 0, st>>>(mp, chi, nr, mean, a, ctl); break;
+        case 2: k_setup_lines<Ts, 2><<<grid, nt, 0, st>>>(mp, chi, nr, mean, a, ctl); break;
+        case 4: k_setup_lines<Ts, 4><<<grid, nt, 0, st>>>(mp, chi, nr, mean, a, ctl); break;
+        case 8: k_setup_lines<Ts, 8><<<grid, nt, 0, st>>>(mp, chi, nr, mean, a, ctl); break;
+        case 16: k_setup_lines<Ts, 16><<<grid, nt, 0, st>>>(mp, chi, nr, mean, a, ctl); break;
+        default: k_setup_lines<Ts, 32><<<grid, nt, 0, st>>>(mp, chi, nr, mean, a, ctl); break;
+    }
+}
+
+int mg_fast_solve(const FieldDims &fd, MGFast &m, const FieldSource &src, double V,
                   const double *phi_zL, double *phi, bool warm, bool mixed, double tol,
                   int max_cycles, double *rel_res, int *launches, StepCtl *sctl, cudaStream_t st,
                   bool v_from_ctl, bool setup, cudaEvent_t at_solve, bool wide, SolveJob *defer,
-                  double *phi_prev, bool report) {
+                  double *phi_prev, bool report, cudaEvent_t after, MGCtl *pinned) {
     const int nz = fd.nz, nr = fd.nr, n = nr - 1, ng = nz * nr;
     const int M = line_chunk(n);
     const int nlev = m.nlev;
     int L = 0;
     raise_smem_limits();
     MGFast *mp = m.self;  // uploaded once (mg_fast_upload)
-    // set-up: levels' chi, coefficients, line factors (skipped when the
-    // operator is the one of the previous solve), right-hand side and
-    // boundary data
+    const RhsArgs ra{src.rho, phi, phi_zL, V, warm ? 0 : 1, v_from_ctl ? 1 : 0, warm ? phi_prev : nullptr};
     if (setup) {
-    cudaMemcpyAsync(m.chi[0], chi, sizeof(double) * ng, cudaMemcpyDeviceToDevice, st);
-    if (nlev > 1) {
-        k_chi_levels<<<(nr + 7) / 8, 256, (size_t)8 * 2 * nz * sizeof(double), st>>>(mp, nr, sctl);
-        ++L;
-    }
-    int total = 0;
-    for (int l = 0; l < nlev; ++l) total += m.nz[l] * nr;
-    k_coefs_levels<<<(total + 255) / 256, 256, 0, st>>>(mp, nr, fd.chi_face == PIC_CHI_MEAN, total, sctl);
-    ++L;
-    {
-        // line factors in the V-cycle's type; one warp per line
-        int lines_all = 0;
-        for (int l = 0; l < nlev; ++l) lines_all += m.nz[l] - 2;
-        if (!mixed) {
-            k_factor_lines<double><<<(lines_all + 7) / 8, 256, 0, st>>>(mp, 0, nlev, nr, M, lines_all, sctl);
-            ++L;
-        } else if (nlev > 1) {
-            k_factor_lines<float><<<(lines_all + 7) / 8, 256, 0, st>>>(mp, 0, nlev, nr, M, lines_all, sctl);
-            ++L;
-        } else {
-            // nz = 3: the single row is phi's own, solved in FP64
-            k_factor_lines<double><<<1, 32, 0, st>>>(mp, 0, 1, nr, M, 1, sctl);
+        int lc = 2;  // four columns (a 32-byte sector a row): c2's FP64 divisions on most SMs
+        size_t smem = 0;
+        while ((smem = (((size_t)2 * nz + kMaxLevels) * sizeof(double)) << lc) > kSolveSmemLimit && lc > 0) --lc;
+        if (src.Ne || nlev > 1) {
+            k_setup_levels<<<(nr + (1 << lc) - 1) >> lc, 256, smem, st>>>(mp, nr, lc, src, sctl);
             ++L;
         }
+        if (after) cudaStreamWaitEvent(st, after, 0);
+        // line factors in the V-cycle's type (nz = 3: the single row is phi's
+        // own, solved in FP64)
+        int rows = 0;
+        for (int l = 0; l < nlev; ++l) rows += m.nz[l];
+        const int mean = fd.chi_face == PIC_CHI_MEAN;
+        if (mixed && nlev > 1)
+            launch_setup_lines<float>(M, rows, st, mp, src.chi, nr, mean, ra, sctl);
+        else
+            launch_setup_lines<double>(M, rows, st, mp, src.chi, nr, mean, ra, sctl);
+        ++L;
+    } else {
+        // the operator is the one of the previous solve
+        if (after) cudaStreamWaitEvent(st, after, 0);
+        k_rhs_bc<<<(ng + 255) / 256, 256, 0, st>>>(mp, ra, nz, nr, sctl);
+        ++L;
     }
-    }
-    k_rhs_bc<<<(ng + 255) / 256, 256, 0, st>>>(mp, rho, phi, phi_zL, V, nz, nr, warm ? 0 : 1, sctl,
-                                               v_from_ctl ? 1 : 0, warm ? phi_prev : nullptr);
-    ++L;
-    // (k_rhs_bc also clears the solve's control block)
     // all cycles in one cooperative launch
     SolveJob job;
     if (!solve_job(fd, m, phi, mixed, tol, max_cycles, sctl, wide, job)) {
@@ -1398,9 +1446,11 @@ int mg_fast_solve(const FieldDims &fd, MGFast &m, const double *rho, const doubl
         return 0;
     }
     if (launches) *launches += L;
-    MGCtl ch;
-    cudaMemcpyAsync(&ch, m.ctl, sizeof(MGCtl), cudaMemcpyDeviceToHost, st);
+    MGCtl local;
+    MGCtl *cp = pinned ? pinned : &local;
+    cudaMemcpyAsync(cp, m.ctl, sizeof(MGCtl), cudaMemcpyDeviceToHost, st);
     cudaStreamSynchronize(st);
+    const MGCtl ch = *cp;
     if (ch.timeout) {
         if (rel_res) *rel_res = 0.0;
         return kSolveTimeout;

@@ -81,6 +81,15 @@ struct MGFast {
     MGFast *self;  // device copy of this struct (kernels read it through a pointer)
 };
 
+// Where a solve's charge and susceptibility come from: computed by the set-up
+// from the species' deposits (Ne, Ni over the node volumes V; rho and chi are
+// then written), or given (Ne null).
+struct FieldSource {
+    const double *Ne, *Ni, *V;
+    double q0, q1, c0, c1;
+    double *rho, *chi;
+};
+
 // Shared-memory layout of the one-launch solve (byte offsets), set on the host.
 struct SolveLayout {
     // from 0 in the line phases: three line buffers, M * 33 values each
@@ -138,15 +147,18 @@ void mg_fast_geometry(const MGFast &m, int nr, double dr, std::vector<double> &o
 // is described in *defer and left to mg_multi_launch; the report to sctl is
 // then the caller's.
 // report false: the report to sctl is left to the caller (launch_efield).
+// after (optional): what the voltage waits for (the set-up's first launch does not).
+// pinned (optional): host memory for the read-back of a solve alone.
 // phi_prev (warm solves only, optional): the potential of the step before
 // phi's; the V-cycles then start from 2 phi - phi_prev on the interior, and
 // phi_prev takes phi's values (the starting value w_0 of Algorithm 1,
 // extrapolated linearly in time).
-int mg_fast_solve(const FieldDims &fd, MGFast &m, const double *rho, const double *chi, double V,
+int mg_fast_solve(const FieldDims &fd, MGFast &m, const FieldSource &src, double V,
                   const double *phi_zL, double *phi, bool warm, bool mixed, double tol,
                   int max_cycles, double *rel_res, int *launches, StepCtl *sctl, cudaStream_t st,
                   bool v_from_ctl = true, bool setup = true, cudaEvent_t at_solve = nullptr,
-                  bool wide = true, SolveJob *defer = nullptr, double *phi_prev = nullptr, bool report = true);
+                  bool wide = true, SolveJob *defer = nullptr, double *phi_prev = nullptr, bool report = true,
+                  cudaEvent_t after = nullptr, MGCtl *pinned = nullptr);
 
 // the launch shape of one reactor's solve (host only); false: not launchable
 bool solve_job(const FieldDims &fd, MGFast &m, double *phi, bool mixed, double tol, int max_cycles,

@@ -104,6 +104,7 @@ struct pic_handle {
     struct HostCtl : CallReport {
         unsigned long long cnt[PIC_NCOUNT];  // pic_moments' counters and absorbed charge
         double qabs[3];
+        MGCtl mg;  // a stand-alone solve's control block
     } *host_ctl = nullptr;
     MGFast mgf;
     RadixTmp rtmp;
@@ -623,7 +624,8 @@ void setup_device(pic_handle *h) {
         m.nz[l] = z;
         m.dz[l] = h->cfg.mesh.L / (z - 1);
         const size_t g = (size_t)z * h->nr;
-        m.chi[l] = (double *)dalloc(h, g * sizeof(double));
+        // (level 0: the caller's chi)
+        if (l > 0) m.chi[l] = (double *)dalloc(h, g * sizeof(double));
         m.cz[l] = (double *)dalloc(h, g * sizeof(double));
         m.cr[l] = (double *)dalloc(h, g * sizeof(double));
         if (h->mixed) {
@@ -888,7 +890,16 @@ void one_step(pic_handle *h, cudaStream_t sb, bool mv, int part = 0, SolveJob *j
                          h->dr, h->sctl, h->mgf.ctl, st);
         h->launches += 2;  // the shared solve's share, E
     } else {
-    k_step_begin<<<1, 1, 0, st>>>(h->sctl, h->rf_d, h->cfg.rf.n, h->cfg.dt, h->cfg.split_every);
+    // the step's voltage and split flag, beside the first launch of the
+    // solve's set-up
+    cudaEvent_t begun = nullptr;
+    if (sb) {
+        cudaEventRecord(h->ev_fork2, st);
+        cudaStreamWaitEvent(sb, h->ev_fork2, 0);
+        begun = h->ev_join2;
+    }
+    k_step_begin<<<1, 1, 0, sb ? sb : st>>>(h->sctl, h->rf_d, h->cfg.rf.n, h->cfg.dt, h->cfg.split_every);
+    if (sb) cudaEventRecord(begun, sb);
     h->launches += 1;
     if (!sb) {
         PhaseTimer t(h, 3);
@@ -900,17 +911,18 @@ void one_step(pic_handle *h, cudaStream_t sb, bool mv, int part = 0, SolveJob *j
     cudaEvent_t fork = sb ? h->ev_fork : nullptr;
     {
         PhaseTimer t(h, 0);
-        launch_finalize(h->N[0], h->N[1], h->V, h->cfg.sp[0].q, h->cfg.sp[1].q, chi_coef(h, 0, true),
-                        chi_coef(h, 1, mv), h->rho, h->chi, h->ng, h->sctl, st);
+        const FieldSource field{h->N[0], h->N[1], h->V, h->cfg.sp[0].q, h->cfg.sp[1].q, chi_coef(h, 0, true),
+                              chi_coef(h, 1, mv), h->rho, h->chi};
         FieldDims fd{h->nz, h->nr, h->dz, h->dr, h->cfg.mesh.L, h->cfg.chi_face};
         int L = 0;
         if (h->cfg.circuit_C > 0.0) {
             // phi_P: the plasma's charge, electrode at 0; phi_L: no charge,
             // electrode at 1, every other boundary at 0; same operator
-            mg_fast_solve(fd, h->mgf, h->rho, h->chi, 0.0, h->has_phiL ? h->phiL_d : nullptr, h->phi_P,
+            mg_fast_solve(fd, h->mgf, field, 0.0, h->has_phiL ? h->phiL_d : nullptr, h->phi_P,
                           true, h->mixed, h->cfg.mg_tol, h->cfg.mg_max_cycles, nullptr, &L, h->sctl, st,
-                          false, true, fork, !h->in_batch);
-            mg_fast_solve(fd, h->mgf, h->zero_grid, h->chi, 1.0, nullptr, h->phi_L, true, h->mixed,
+                          false, true, fork, !h->in_batch, nullptr, nullptr, true, begun);
+            const FieldSource none{nullptr, nullptr, nullptr, 0, 0, 0, 0, h->zero_grid, h->chi};
+            mg_fast_solve(fd, h->mgf, none, 1.0, nullptr, h->phi_L, true, h->mixed,
                           h->cfg.mg_tol, h->cfg.mg_max_cycles, nullptr, &L, h->sctl, st, false, false, nullptr,
                           !h->in_batch);
             k_circuit<<<1, 256, 0, st>>>(h->sctl, h->ds, h->mgf.cz[0], h->phi_P, h->phi_L, h->rho, h->V,
@@ -918,10 +930,10 @@ void one_step(pic_handle *h, cudaStream_t sb, bool mv, int part = 0, SolveJob *j
             k_superpose<<<(h->ng + 255) / 256, 256, 0, st>>>(h->sctl, h->phi_P, h->phi_L, h->phi, h->ng);
             L += 2;
         } else {
-            mg_fast_solve(fd, h->mgf, h->rho, h->chi, 0.0, h->has_phiL ? h->phiL_d : nullptr, h->phi,
+            mg_fast_solve(fd, h->mgf, field, 0.0, h->has_phiL ? h->phiL_d : nullptr, h->phi,
                           true, h->mixed, h->cfg.mg_tol, h->cfg.mg_max_cycles, nullptr, &L, h->sctl, st, true,
                           true, fork, !h->in_batch, part == 1 ? job : nullptr,
-                          h->cfg.mg_guess == PIC_GUESS_LINEAR ? h->phi_prev : nullptr, false);
+                          h->cfg.mg_guess == PIC_GUESS_LINEAR ? h->phi_prev : nullptr, false, begun);
             if (part == 1) {
                 h->launches += L;
                 return;
@@ -934,7 +946,7 @@ void one_step(pic_handle *h, cudaStream_t sb, bool mv, int part = 0, SolveJob *j
         }
         launch_efield<T>(h->phi, h->Ez, h->Er, (typename V2<T>::type *)h->E2, h->nz, h->nr, h->dz,
                          h->dr, h->sctl, h->cfg.circuit_C > 0.0 ? nullptr : h->mgf.ctl, st);
-        h->launches += L + 2;
+        h->launches += L + 1;
     }
     if (sb) cudaStreamWaitEvent(st, h->ev_join, 0);
     }
@@ -1824,15 +1836,27 @@ pic_status pic_field_solve(pic_handle *h, const double *rho, const double *chi, 
                            double *phi, int32_t on_device, pic_solve_info *info) {
     if (!h || !rho || !chi || !phi) return fail(h, PIC_ERR_ARG, "null argument");
     const size_t gb = (size_t)h->ng * sizeof(double);
-    const cudaMemcpyKind kin = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
-    cudaMemcpyAsync(h->tmp_grid[0], rho, gb, kin, h->st);
-    cudaMemcpyAsync(h->tmp_grid[1], chi, gb, kin, h->st);
+    // device arrays are read in place (by the set-up alone) when they can be
+    const bool in_place = on_device && (((uintptr_t)rho | (uintptr_t)chi) & 7) == 0;
+    if (!in_place) {
+        const cudaMemcpyKind kin = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
+        cudaMemcpyAsync(h->tmp_grid[0], rho, gb, kin, h->st);
+        cudaMemcpyAsync(h->tmp_grid[1], chi, gb, kin, h->st);
+    }
+    if (!h->host_ctl && cudaMallocHost((void **)&h->host_ctl, sizeof(*h->host_ctl)) != cudaSuccess) {
+        h->host_ctl = nullptr;
+        cudaGetLastError();
+    }
     FieldDims fd{h->nz, h->nr, h->dz, h->dr, h->cfg.mesh.L, h->cfg.chi_face};
     int L = 0;
     double res = 0.0;
-    const int r = mg_fast_solve(fd, h->mgf, h->tmp_grid[0], h->tmp_grid[1], V,
-                                h->has_phiL ? h->phiL_d : nullptr, h->tmp_grid[2], false,
-                                h->mixed, h->cfg.mg_tol, h->cfg.mg_max_cycles, &res, &L, nullptr, h->st);
+    // (rho and chi are only read: no deposit is given)
+    const FieldSource src{nullptr, nullptr, nullptr, 0, 0, 0, 0, in_place ? const_cast<double *>(rho) : h->tmp_grid[0],
+                          in_place ? const_cast<double *>(chi) : h->tmp_grid[1]};
+    const int r = mg_fast_solve(fd, h->mgf, src, V, h->has_phiL ? h->phiL_d : nullptr, h->tmp_grid[2], false,
+                                h->mixed, h->cfg.mg_tol, h->cfg.mg_max_cycles, &res, &L, nullptr, h->st, true, true,
+                                nullptr, true, nullptr, nullptr, true, nullptr,
+                                h->host_ctl ? &h->host_ctl->mg : nullptr);
     h->launches += L;
     if (r == kSolveTimeout) return fail(h, PIC_ERR_TIMEOUT, "multigrid grid barrier timed out");
     if (r == kSolveNoLaunch) return fail(h, PIC_ERR_CUDA, "multigrid solve could not be launched");

@@ -519,12 +519,13 @@ int window_run(const WindowIn<T> &in, int K, int ckpt, const double *w_host, dou
         // one forward step; `again`: the step's potential is the stored one
         auto fwd = [&](int n, const WinState<T> *Sin, const WinState<T> *Sout, double **Nin, double **Nout,
                        bool again) {
-            launch_finalize(Nin[0], Nin[1], in.V, in.q[0], in.q[1], c_chi[0], c_chi[1], rho, chi, ng, nullptr, st);
             if (again) {
+                launch_finalize(Nin[0], Nin[1], in.V, in.q[0], in.q[1], c_chi[0], c_chi[1], rho, chi, ng, nullptr, st);
                 cudaMemcpyAsync(phi, phi_all[n], (size_t)ng * sizeof(double), cudaMemcpyDeviceToDevice, st);
             } else {
                 const double t = (double)(in.step0 + n) * in.dt;
-                if (mg_fast_solve(fd, *in.mgf, rho, chi, voltage(t), pzl, phi, true, in.mixed, in.tol,
+                const FieldSource src{Nin[0], Nin[1], in.V, in.q[0], in.q[1], c_chi[0], c_chi[1], rho, chi};
+                if (mg_fast_solve(fd, *in.mgf, src, voltage(t), pzl, phi, true, in.mixed, in.tol,
                                   in.max_cycles, nullptr, &L, wctl, st, false, true) == kSolveNoLaunch)
                     throw 1;
                 if (grad) cudaMemcpyAsync(phi_all[n], phi, (size_t)ng * sizeof(double), cudaMemcpyDeviceToDevice, st);
@@ -613,7 +614,8 @@ int window_run(const WindowIn<T> &in, int K, int ckpt, const double *w_host, dou
                     k_adj_rhs<<<blocks(ng), kWT, 0, st>>>(phib, rhof, nz, nr, in.dz, in.dr);
                     // warm start from the previous step's lambda (zero at first):
                     // consecutive adjoint fields are close
-                    if (mg_fast_solve(fd, *in.mgf, rhof, chis[q - 1], 0.0, nullptr, lam, true, in.mixed, in.tol,
+                    const FieldSource src{nullptr, nullptr, nullptr, 0, 0, 0, 0, rhof, chis[q - 1]};
+                    if (mg_fast_solve(fd, *in.mgf, src, 0.0, nullptr, lam, true, in.mixed, in.tol,
                                       in.max_cycles, nullptr, &L, wctl, st, false, true) == kSolveNoLaunch)
                         throw 1;
                     cudaMemsetAsync(chib, 0, (size_t)ng * sizeof(double), st);
