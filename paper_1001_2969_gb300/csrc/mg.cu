@@ -57,10 +57,9 @@ __global__ void __launch_bounds__(256) k_setup_levels(const MGFast *__restrict__
         const size_t k = (size_t)i * nr + j;
         double x;
         if (f.Ne) {
-            const double ne = f.Ne[k] / f.V[k], ni = f.Ni[k] / f.V[k];
-            f.rho[k] = f.q0 * ne + f.q1 * ni;
-            // chi = dt^2/(2 eps0) sum_s q_s^2 n_s / m_s ; c_s = q_s^2 dt^2 / (2 eps0 m_s)
-            x = f.c0 * ne + f.c1 * ni;
+            double rho;
+            node_field(f.Ne[k], f.Ni[k], f.iV[k], f.q0, f.q1, f.c0, f.c1, rho, x);
+            f.rho[k] = rho;
             f.chi[k] = x;
         } else {
             x = f.chi[k];
@@ -177,7 +176,7 @@ __device__ __forceinline__ void rhs_node(const MGFast &m, const RhsArgs &a, doub
 // line factors (its first warp); on the fine level also what its nodes start
 // from.  One launch for what were three (coefficients, factors, right-hand
 // side), where the factors made a trip to L2 between each and the next (11 us
-// on c2, 32 us on c3 and in FP64).  Bound by the FP64 pipe: ~14 operations a
+// on c2, 32 us on c3 and in FP64).  Bound by the FP64 pipe: ~8 operations a
 // node, so a row's nodes are spread over the four SM partitions; a warp per
 // row was slower than the three launches.
 constexpr int kSetupThreads = 128;
@@ -201,13 +200,25 @@ __global__ void __launch_bounds__(kSetupThreads)
     const bool inner = i > 0 && i < nz - 1, mixed = m.cz32[l] != nullptr;
     const double V = (ctl && a.v_from_ctl) ? ctl->V : a.V;  // in a timestep the source voltage comes with the step
     auto at = [](int j) { return (j % M) * kPad + j / M; };
-    auto face = [&](double x, double y) { return face_mean ? 0.5 * (x + y) : fmax(x, y); };
+    // (1 + chi of the face) g; the maximum of two values that are not negative
+    // (nor NaN) by their bit patterns, off the FP64 pipe
+    auto face = [&](double x, double y, double g) {
+        double f;
+        if (face_mean) {
+            f = 0.5 * (x + y);
+        } else {
+            const unsigned long long bx = (unsigned long long)__double_as_longlong(x),
+                                     by = (unsigned long long)__double_as_longlong(y);
+            f = (bx | by) < 0x7ff0000000000000ull ? __longlong_as_double((long long)max(bx, by)) : fmax(x, y);
+        }
+        return fma(f, g, g);
+    };
     for (int j = threadIdx.x; j < nr; j += kSetupThreads) {
         double lo = 0.0, hi = 0.0, right = 0.0;  // cz below and above the row, cr
         const double c = chi[j], gz = m.gz[l][j];
-        if (i > 0) lo = (1.0 + face(chi[j - nr], c)) * gz;
-        if (i + 1 < nz) hi = (1.0 + face(c, chi[j + nr])) * gz;
-        if (j + 1 < nr) right = (1.0 + face(c, chi[j + 1])) * m.gr[l][j];
+        if (i > 0) lo = face(chi[j - nr], c, gz);
+        if (i + 1 < nz) hi = face(c, chi[j + nr], gz);
+        if (j + 1 < nr) right = face(c, chi[j + 1], m.gr[l][j]);
         const size_t k = (size_t)i * nr + j;
         if (mixed) {
             m.cz32[l][k] = (float)hi;
@@ -218,7 +229,7 @@ __global__ void __launch_bounds__(kSetupThreads)
             m.cr[l][k] = right;
         }
         if (l == 0) {
-            const double left = j > 0 ? (1.0 + face(chi[j - 1], c)) * m.gr[0][j - 1] : 0.0;
+            const double left = j > 0 ? face(chi[j - 1], c, m.gr[0][j - 1]) : 0.0;
             rhs_node(m, a, V, nz, nr, i, j, lo + hi + left + right);
         }
         if (inner && j < n) {
@@ -1166,7 +1177,9 @@ __global__ void __launch_bounds__(kSolveThreads, MINB) k_solve_multi(const Solve
 size_t mg_line_factor_elems(int nr) { return (size_t)line_factor_elems(line_chunk(nr - 1)); }
 
 // tiles of one to eight columns, the last one whole, with two neighbour columns each
-size_t mg_tile_elems(int nz, int nr) { return (size_t)nz * (nr + 8) * 3; }
+size_t mg_tile_elems(int nz, int nr, bool with_neighbours) {
+    return (size_t)nz * (nr + 8) * (with_neighbours ? 3 : 1);
+}
 
 int mg_line_chunk(int nr) { return line_chunk(nr - 1); }
 

@@ -82,10 +82,10 @@ struct MGFast {
 };
 
 // Where a solve's charge and susceptibility come from: computed by the set-up
-// from the species' deposits (Ne, Ni over the node volumes V; rho and chi are
+// from the species' deposits (Ne, Ni times the inverse node volumes iV; rho and chi are
 // then written), or given (Ne null).
 struct FieldSource {
-    const double *Ne, *Ni, *V;
+    const double *Ne, *Ni, *iV;
     double q0, q1, c0, c1;
     double *rho, *chi;
 };
@@ -122,9 +122,9 @@ struct SolveJob {
 // line-factor elements of one r-line of a mesh with nr nodes per row
 // (the same count in FP32 and FP64)
 size_t mg_line_factor_elems(int nr);
-// doubles of each tile-wise array (kr, kw, kzp, kwp, ps), and the most blocks
+// doubles of each tile-wise array (kr, kw, kzp, kwp; ps has the neighbour columns), and the most blocks
 // a solve takes (entries of xr and xd)
-size_t mg_tile_elems(int nz, int nr);
+size_t mg_tile_elems(int nz, int nr, bool with_neighbours);
 constexpr int kMaxSolveBlocks = 512;
 // copies of them, so that not every block reads the same few lines of L2
 constexpr int kCopies = 8;

@@ -88,7 +88,7 @@ struct pic_handle {
     int cur_i = 0;  // buffer set holding the ions (flips only in passes that move them)
     int K = 1;      // ion subcycling: the ions move every K-th pass
     double *N[2] = {nullptr, nullptr};
-    double *rho = nullptr, *chi = nullptr, *phi = nullptr, *Ez = nullptr, *Er = nullptr, *V = nullptr;
+    double *rho = nullptr, *chi = nullptr, *phi = nullptr, *Ez = nullptr, *Er = nullptr, *V = nullptr, *iV = nullptr;
     void *E2 = nullptr;
     double *phiL_d = nullptr;
     bool has_phiL = false;
@@ -324,6 +324,11 @@ void node_volumes(const pic_handle *h, std::vector<double> &V) {
             V[(size_t)i * h->nr + j] = v * hz;
         }
     }
+}
+
+__global__ void k_inverse(const double *x, double *y, int n) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k < n) y[k] = 1.0 / x[k];
 }
 
 __global__ void k_iota(int32_t *p, int n) {
@@ -585,6 +590,7 @@ void setup_device(pic_handle *h) {
     h->Ez = (double *)dalloc(h, gb);
     h->Er = (double *)dalloc(h, gb);
     h->V = (double *)dalloc(h, gb);
+    h->iV = (double *)dalloc(h, gb);
     for (int k = 0; k < 3; ++k) h->tmp_grid[k] = (double *)dalloc(h, gb);
     for (int k = 0; k < 5; ++k) h->m_acc[k] = (double *)dalloc(h, gb);
     h->E2 = dalloc(h, (size_t)h->ng * 2 * ts);
@@ -613,6 +619,7 @@ void setup_device(pic_handle *h) {
     std::vector<double> V;
     node_volumes(h, V);
     cudaMemcpyAsync(h->V, V.data(), gb, cudaMemcpyHostToDevice, h->st);
+    k_inverse<<<(h->ng + 255) / 256, 256, 0, h->st>>>(h->V, h->iV, h->ng);
     // multigrid hierarchy: per level nodal chi and face coefficients, the
     // V-cycle's correction and right-hand side, and the r-line factors
     MGFast &m = h->mgf;
@@ -631,11 +638,6 @@ void setup_device(pic_handle *h) {
         if (h->mixed) {
             m.cz32[l] = (float *)dalloc(h, g * sizeof(float));
             m.cr32[l] = (float *)dalloc(h, g * sizeof(float));
-        }
-        const size_t fw = g * (h->mixed ? sizeof(Flag<float>::W) : sizeof(Flag<double>::W));
-        for (void **w : {&m.lu[l], &m.lf[l]}) {
-            *w = dalloc(h, fw);
-            cudaMemsetAsync(*w, 0, fw, h->st);
         }
         const size_t fe = (size_t)(z - 2) * line_fe;
         if (z == 3) {
@@ -662,22 +664,31 @@ void setup_device(pic_handle *h) {
     }
     m.f0 = (double *)dalloc(h, gb);
     m.dg0 = (double *)dalloc(h, gb);
-    const size_t tb = mg_tile_elems(h->nz, h->nr) * sizeof(double);
+    const size_t tb = mg_tile_elems(h->nz, h->nr, !h->mixed) * sizeof(double);
     if (h->mixed) {
-        for (double **z : {&m.kr, &m.kw, &m.kzp, &m.kwp}) {
-            *z = (double *)dalloc(h, tb);
-            cudaMemsetAsync(*z, 0, tb, h->st);
-        }
+        for (double **z : {&m.kr, &m.kw, &m.kzp, &m.kwp}) *z = (double *)dalloc(h, tb);
+        // (read, times zero, by a solve's first GCR step)
+        cudaMemsetAsync(m.kwp, 0, tb, h->st);
     } else {
         m.ps = (double *)dalloc(h, tb);
     }
-    // flagged words and their epoch start at zero: tag 0 is never waited for
-    const size_t xb = (size_t)kMaxSolveBlocks * 8 * kCopies * sizeof(ulonglong2);
-    m.xr = (ulonglong2 *)dalloc(h, xb);
+    // flagged words and their epoch, in one piece; they start at zero: tag 0
+    // is never waited for
+    const size_t fw = h->mixed ? sizeof(Flag<float>::W) : sizeof(Flag<double>::W);
+    size_t fb = (size_t)kMaxSolveBlocks * 8 * kCopies * sizeof(ulonglong2) + 256;
+    for (int l = 0; l < nl; ++l) fb += 2 * (((size_t)m.nz[l] * h->nr * fw + 255) & ~(size_t)255);
+    char *fp = (char *)dalloc(h, fb);
+    cudaMemsetAsync(fp, 0, fb, h->st);
+    m.epoch = (unsigned *)fp;
+    fp += 256;
+    m.xr = (ulonglong2 *)fp;
     m.xd = m.xr + 4 * kCopies * kMaxSolveBlocks;
-    m.epoch = (unsigned *)dalloc(h, sizeof(unsigned));
-    cudaMemsetAsync(m.xr, 0, xb, h->st);
-    cudaMemsetAsync(m.epoch, 0, sizeof(unsigned), h->st);
+    fp += (size_t)kMaxSolveBlocks * 8 * kCopies * sizeof(ulonglong2);
+    for (int l = 0; l < nl; ++l)
+        for (void **w : {&m.lu[l], &m.lf[l]}) {
+            *w = fp;
+            fp += ((size_t)m.nz[l] * h->nr * fw + 255) & ~(size_t)255;
+        }
     m.ctl = (MGCtl *)dalloc(h, sizeof(MGCtl));
     m.self = (MGFast *)dalloc(h, sizeof(MGFast));
     mg_fast_upload(m, h->st);
@@ -911,7 +922,7 @@ void one_step(pic_handle *h, cudaStream_t sb, bool mv, int part = 0, SolveJob *j
     cudaEvent_t fork = sb ? h->ev_fork : nullptr;
     {
         PhaseTimer t(h, 0);
-        const FieldSource field{h->N[0], h->N[1], h->V, h->cfg.sp[0].q, h->cfg.sp[1].q, chi_coef(h, 0, true),
+        const FieldSource field{h->N[0], h->N[1], h->iV, h->cfg.sp[0].q, h->cfg.sp[1].q, chi_coef(h, 0, true),
                               chi_coef(h, 1, mv), h->rho, h->chi};
         FieldDims fd{h->nz, h->nr, h->dz, h->dr, h->cfg.mesh.L, h->cfg.chi_face};
         int L = 0;
@@ -1010,7 +1021,7 @@ void one_step(pic_handle *h, cudaStream_t sb, bool mv, int part = 0, SolveJob *j
         PhaseTimer t(h, 4);
         const StepEnd e{h->ds, h->sp[0].d_nmain[dst], mv ? h->sp[1].d_nmain[idst] : nullptr, h->sp[0].d_nalive,
                         mv ? h->sp[1].d_nalive : nullptr};
-        launch_moments(h->N[0], h->N[1], h->V, h->phi, h->Ez, h->Er, h->m_acc[0], h->m_acc[1],
+        launch_moments(h->N[0], h->N[1], h->iV, h->phi, h->Ez, h->Er, h->m_acc[0], h->m_acc[1],
                        h->m_acc[2], h->m_acc[3], h->m_acc[4], h->ng, h->sctl, e, st);
         h->launches += 1;
     }
@@ -1385,7 +1396,7 @@ pic_status window_t(pic_handle *h, int32_t nsteps, int32_t ckpt, const double *w
         in.perm[s] = d.perm;
         fill_step_args<T>(h, in.args[s], s, cur, 1 - cur, 1 - cur);
     }
-    in.V = h->V;
+    in.iV = h->iV;
     in.phi0 = h->phi;
     in.mgf = &h->mgf;
     in.tol = h->cfg.mg_tol;
@@ -2027,7 +2038,7 @@ pic_status pic_get_fields(pic_handle *h, double *rho, double *chi, double *phi, 
                           double *Er, int32_t on_device) {
     if (!h) return PIC_ERR_ARG;
     // rho and chi as the next step's solve takes them
-    launch_finalize(h->N[0], h->N[1], h->V, h->cfg.sp[0].q, h->cfg.sp[1].q, chi_coef(h, 0, true),
+    launch_finalize(h->N[0], h->N[1], h->iV, h->cfg.sp[0].q, h->cfg.sp[1].q, chi_coef(h, 0, true),
                     chi_coef(h, 1, moves_ions(h, h->step)), h->rho, h->chi, h->ng, nullptr, h->st);
     h->launches += 1;
     const size_t gb = (size_t)h->ng * sizeof(double);

@@ -422,8 +422,16 @@ struct FieldDims {
     double dz, dr, L;
     int chi_face;
 };
-// ctl (may be null): skip when the step has halted
-void launch_finalize(const double *Ne, const double *Ni, const double *V, double q0, double q1,
+// rho = sum q_s n_s and chi = dt^2/(2 eps0) sum_s q_s^2 n_s / m_s of a node
+// (n_s = N_s / V, c_s = q_s^2 dt^2 / (2 eps0 m_s))
+__device__ __forceinline__ void node_field(double Ne, double Ni, double iV, double q0, double q1, double c0, double c1,
+                                           double &rho, double &chi) {
+    const double ne = Ne * iV, ni = Ni * iV;
+    rho = q0 * ne + q1 * ni;
+    chi = c0 * ne + c1 * ni;
+}
+// iV: the inverse node volumes; ctl (may be null): skip when the step has halted
+void launch_finalize(const double *Ne, const double *Ni, const double *iV, double q0, double q1,
                      double chi0, double chi1, double *rho, double *chi, int ng, const StepCtl *ctl,
                      cudaStream_t st);
 // multigrid solve into phi (device); returns cycles, residual and the launch count
@@ -444,7 +452,7 @@ struct StepEnd {
     int32_t *nmain0, *nmain1;
     const int32_t *nalive0, *nalive1;
 };
-void launch_moments(const double *Ne, const double *Ni, const double *V, const double *phi,
+void launch_moments(const double *Ne, const double *Ni, const double *iV, const double *phi,
                     const double *Ez, const double *Er, double *m_ne, double *m_ni,
                     double *m_phi, double *m_ez, double *m_er, int ng, StepCtl *ctl, const StepEnd &e,
                     cudaStream_t st);
