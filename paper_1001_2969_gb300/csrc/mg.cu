@@ -123,9 +123,35 @@ __device__ __forceinline__ double recip(double x) {
 //   ell (forward multipliers), invd (1/pivot), cp (up * invd), v, w
 //   (5 arrays of M), then loI, upI (interface couplings), the five PCR
 //   steps' alpha and gamma, and 1/diagonal of the reduced system.
+//
+// FP64 lines of up to 512 unknowns take 128 lanes (four warps) instead: a warp's
+// FP64 instruction occupies its SM partition's pipe for ~60 cycles, so one warp
+// per line left three of the four pipes idle (7700 cycles a line at M = 16).
+// The chunks are a quarter as long, the interface system has seven reduction
+// steps, and lanes exchange through shared memory.  Longer lines' factors
+// would not fit shared memory that way.
 constexpr int kLine = 32;  // lanes per line
 
-__host__ __device__ constexpr int line_factor_elems(int M) { return 5 * M * kLine + 2 * kLine + 10 * kLine + kLine; }
+// how a line of up to 32 M unknowns is laid out
+template <typename Ts, int M>
+struct Shape {
+    static constexpr bool group = sizeof(Ts) == 8 && M <= 16;
+    static constexpr int lanes = group ? 128 : kLine;
+    static constexpr int chunk = group ? (M > 4 ? M / 4 : 1) : M;
+    static constexpr int steps = group ? 7 : 5;
+    static constexpr int row = lanes + 1;          // a line buffer's row of one unknown of every chunk, padded
+    static constexpr int unknowns = lanes * chunk;  // with padding
+    static constexpr int elems = 5 * chunk * lanes + (3 + 2 * steps) * lanes;
+    // position of unknown j in a line buffer
+    static __device__ __forceinline__ int at(int j) { return (j % chunk) * row + j / chunk; }
+};
+int line_elems(int M, bool f64) {
+    if (!f64 || M > 16) return 5 * M * kLine + 13 * kLine;
+    return 5 * (M > 4 ? M / 4 : 1) * 128 + 17 * 128;
+}
+int line_buffer(int M, bool f64) {
+    return f64 && M <= 16 ? (M > 4 ? M / 4 : 1) * 129 : M * 33;
+}
 
 // chunk per lane: the least power of two M with 32 M >= n
 inline int line_chunk(int n) {
@@ -184,11 +210,13 @@ template <typename Ts, int M>
 __global__ void __launch_bounds__(kSetupThreads)
     k_setup_lines(const MGFast *__restrict__ mp, const double *__restrict__ chi0, int nr, int face_mean, RhsArgs a,
                   const StepCtl *ctl) {
-    constexpr int kPad = 33;
-    __shared__ Ts sd[M * kPad], se[M * kPad];  // cz below + above the row, cr
+    using Sh = Shape<Ts, M>;
+    constexpr int MC = Sh::chunk, NL = Sh::lanes;
+    __shared__ Ts sd[MC * Sh::row], se[MC * Sh::row];  // cz below + above the row, cr
+    __shared__ Ts sx[2][6][Sh::group ? NL : 1];         // exchange between the lanes' warps
     const MGFast &m = *mp;
     if (ctl && ctl->halt) return;
-    const int n = nr - 1, p = threadIdx.x & 31;
+    const int n = nr - 1, p = threadIdx.x & (NL - 1);
     // the solve's control block starts cleared
     if (blockIdx.x == 0)
         for (int w = threadIdx.x; w < (int)(sizeof(MGCtl) / sizeof(unsigned)); w += blockDim.x)
@@ -199,7 +227,6 @@ __global__ void __launch_bounds__(kSetupThreads)
     const double *chi = (l == 0 ? chi0 : m.chi[l]) + (size_t)i * nr;
     const bool inner = i > 0 && i < nz - 1, mixed = m.cz32[l] != nullptr;
     const double V = (ctl && a.v_from_ctl) ? ctl->V : a.V;  // in a timestep the source voltage comes with the step
-    auto at = [](int j) { return (j % M) * kPad + j / M; };
     // (1 + chi of the face) g; the maximum of two values that are not negative
     // (nor NaN) by their bit patterns, off the FP64 pipe
     auto face = [&](double x, double y, double g) {
@@ -233,32 +260,53 @@ __global__ void __launch_bounds__(kSetupThreads)
             rhs_node(m, a, V, nz, nr, i, j, lo + hi + left + right);
         }
         if (inner && j < n) {
-            sd[at(j)] = (Ts)lo + (Ts)hi;
-            se[at(j)] = (Ts)right;
+            sd[Sh::at(j)] = (Ts)lo + (Ts)hi;
+            se[Sh::at(j)] = (Ts)right;
         }
     }
     __syncthreads();
-    if (!inner || threadIdx.x >= kLine) return;
+    if (!inner || threadIdx.x >= NL) return;
     const bool f64 = sizeof(Ts) == 8;
     Ts *fac = (l == m.nlev - 1) ? (f64 ? (Ts *)m.facc : (Ts *)m.facc32)
                                 : (f64 ? (Ts *)m.fac64[l] : (Ts *)m.fac32[l]);
-    Ts *F = fac + (size_t)(i - 1) * line_factor_elems(M);
+    Ts *F = fac + (size_t)(i - 1) * Sh::elems;
     auto coef = [&](int k, Ts &lo, Ts &dg, Ts &up) {
-        const int j = p * M + k;
+        const int j = p * MC + k;
         if (j >= n) {
             lo = 0;
             dg = 1;
             up = 0;
             return;
         }
-        lo = j > 0 ? -se[at(j - 1)] : (Ts)0;
-        dg = sd[at(j)] - lo + se[at(j)];
-        up = j < n - 1 ? -se[at(j)] : (Ts)0;
+        lo = j > 0 ? -se[Sh::at(j - 1)] : (Ts)0;
+        dg = sd[Sh::at(j)] - lo + se[Sh::at(j)];
+        up = j < n - 1 ? -se[Sh::at(j)] : (Ts)0;
     };
-    constexpr int MI = M - 1;
+    constexpr int MI = MC - 1;
+    // values of the lanes s to the left and right (undefined past the ends)
+    int turn = 0;
+    auto swap = [&](auto &...x) {
+        if constexpr (Sh::group) {
+            int w = 0;
+            ((sx[turn][w++][p] = x), ...);
+            __syncthreads();
+        }
+    };
+    auto left = [&](Ts x, int w, int s) -> Ts {
+        if constexpr (Sh::group)
+            return sx[turn][w][(p - s) & (NL - 1)];
+        else
+            return __shfl_up_sync(0xffffffffu, x, s);
+    };
+    auto right = [&](Ts x, int w, int s) -> Ts {
+        if constexpr (Sh::group)
+            return sx[turn][w][(p + s) & (NL - 1)];
+        else
+            return __shfl_down_sync(0xffffffffu, x, s);
+    };
     Ts A, B, C;  // reduced (interface) equation of this lane
     Ts loI, dgI, upI;
-    coef(M - 1, loI, dgI, upI);
+    coef(MC - 1, loI, dgI, upI);
     if constexpr (MI > 0) {
         // interior Thomas factors
         Ts ell[MI], invd[MI], cp[MI], v[MI], w[MI];
@@ -295,43 +343,45 @@ __global__ void __launch_bounds__(kSetupThreads)
         }
 #pragma unroll
         for (int k = 0; k < MI; ++k) {
-            F[(size_t)k * kLine + p] = ell[k];
-            F[(size_t)(M + k) * kLine + p] = invd[k];
-            F[(size_t)(2 * M + k) * kLine + p] = cp[k];
-            F[(size_t)(3 * M + k) * kLine + p] = v[k];
-            F[(size_t)(4 * M + k) * kLine + p] = w[k];
+            F[(size_t)k * NL + p] = ell[k];
+            F[(size_t)(MC + k) * NL + p] = invd[k];
+            F[(size_t)(2 * MC + k) * NL + p] = cp[k];
+            F[(size_t)(3 * MC + k) * NL + p] = v[k];
+            F[(size_t)(4 * MC + k) * NL + p] = w[k];
         }
-        const Ts v0n = __shfl_down_sync(0xffffffffu, v[0], 1);
-        const Ts w0n = __shfl_down_sync(0xffffffffu, w[0], 1);
+        swap(v[0], w[0]);
+        const Ts v0n = right(v[0], 0, 1), w0n = right(w[0], 1, 1);
+        turn ^= 1;
         A = loI * v[MI - 1];
-        B = dgI + loI * w[MI - 1] + (p < kLine - 1 ? upI * v0n : (Ts)0);
-        C = p < kLine - 1 ? upI * w0n : (Ts)0;
+        B = dgI + loI * w[MI - 1] + (p < NL - 1 ? upI * v0n : (Ts)0);
+        C = p < NL - 1 ? upI * w0n : (Ts)0;
     } else {
         A = loI;
         B = dgI;
         C = upI;
     }
-    Ts *Gf = F + (size_t)5 * M * kLine;
+    Ts *Gf = F + (size_t)5 * MC * NL;
     Gf[p] = loI;
-    Gf[kLine + p] = upI;
+    Gf[NL + p] = upI;
     // parallel cyclic reduction of the interface system over the lanes
 #pragma unroll
-    for (int st = 0; st < 5; ++st) {
+    for (int st = 0; st < Sh::steps; ++st) {
         const int s = 1 << st;
-        const Ts Bm = __shfl_up_sync(0xffffffffu, B, s), Bp = __shfl_down_sync(0xffffffffu, B, s);
-        const Ts Am = __shfl_up_sync(0xffffffffu, A, s), Ap = __shfl_down_sync(0xffffffffu, A, s);
-        const Ts Cm = __shfl_up_sync(0xffffffffu, C, s), Cp = __shfl_down_sync(0xffffffffu, C, s);
+        swap(A, B, C);
+        const Ts Am = left(A, 0, s), Bm = left(B, 1, s), Cm = left(C, 2, s);
+        const Ts Ap = right(A, 0, s), Bp = right(B, 1, s), Cp = right(C, 2, s);
+        turn ^= 1;
         Ts al = 0, ga = 0;
         if (p >= s) al = -A * recip(Bm);
-        if (p + s < kLine) ga = -C * recip(Bp);
-        Gf[2 * kLine + st * kLine + p] = al;
-        Gf[7 * kLine + st * kLine + p] = ga;
-        const Ts nB = B + (p >= s ? al * Cm : (Ts)0) + (p + s < kLine ? ga * Ap : (Ts)0);
+        if (p + s < NL) ga = -C * recip(Bp);
+        Gf[(2 + st) * NL + p] = al;
+        Gf[(2 + Sh::steps + st) * NL + p] = ga;
+        const Ts nB = B + (p >= s ? al * Cm : (Ts)0) + (p + s < NL ? ga * Ap : (Ts)0);
         A = p >= s ? al * Am : (Ts)0;
-        C = p + s < kLine ? ga * Cp : (Ts)0;
+        C = p + s < NL ? ga * Cp : (Ts)0;
         B = nB;
     }
-    Gf[12 * kLine + p] = recip(B);
+    Gf[(2 + 2 * Sh::steps) * NL + p] = recip(B);
 }
 
 // Warp solve of one line: right-hand side in Bs and solution out to the same
@@ -416,6 +466,52 @@ __device__ __forceinline__ void warp_line_solve(const LineFactors<Ts, M, REG> &q
             Bs[k * kRow + p] = fma_(q.template at<4>(k), I, fma_(q.template at<3>(k), Ip, z[k]));
     }
     Bs[(M - 1) * kRow + p] = I;
+}
+
+// The same by 128 threads (p: the thread's lane; X: 2 x 128 values of shared
+// memory of their own; bar: a named barrier of their own)
+template <typename Ts, int M>
+__device__ __forceinline__ void group_line_solve(const Ts *__restrict__ F, Ts *Bs, Ts *X, int p, int bar) {
+    using Sh = Shape<Ts, M>;
+    constexpr int MC = Sh::chunk, MI = MC - 1, NL = Sh::lanes;
+    const Ts *G = F + 5 * MC * NL;
+    Ts z[MC];
+#pragma unroll
+    for (int k = 0; k < MC; ++k) z[k] = Bs[k * Sh::row + p];
+    int turn = 0;
+    auto share = [&](Ts x) {
+        turn ^= NL;
+        X[turn + p] = x;
+        asm volatile("bar.sync %0, 128;" ::"r"(bar) : "memory");
+    };
+    Ts r = z[MC - 1];
+    if constexpr (MI > 0) {
+#pragma unroll
+        for (int k = 1; k < MI; ++k) z[k] = fma_(-F[k * NL + p], z[k - 1], z[k]);
+#pragma unroll
+        for (int k = 0; k < MI; ++k) z[k] *= F[(MC + k) * NL + p];
+#pragma unroll
+        for (int k = MI - 2; k >= 0; --k) z[k] = fma_(-F[(2 * MC + k) * NL + p], z[k + 1], z[k]);
+        share(z[0]);
+        r = fma_(-G[p], z[MI - 1], r);
+        if (p < NL - 1) r = fma_(-G[NL + p], X[turn + p + 1], r);
+    }
+#pragma unroll
+    for (int st = 0; st < Sh::steps; ++st) {
+        const int s = 1 << st;
+        share(r);
+        const Ts rm = X[turn + ((p - s) & (NL - 1))], rp = X[turn + ((p + s) & (NL - 1))];
+        r = fma_(G[(2 + Sh::steps + st) * NL + p], rp, fma_(G[(2 + st) * NL + p], rm, r));
+    }
+    const Ts I = r * G[(2 + 2 * Sh::steps) * NL + p];
+    if constexpr (MI > 0) {
+        share(I);
+        const Ts Ip = X[turn + ((p - 1) & (NL - 1))];  // lane 0: v is zero there
+#pragma unroll
+        for (int k = 0; k < MI; ++k)
+            Bs[k * Sh::row + p] = fma_(F[(4 * MC + k) * NL + p], I, fma_(F[(3 * MC + k) * NL + p], Ip, z[k]));
+    }
+    Bs[(MC - 1) * Sh::row + p] = I;
 }
 
 template <typename Ts, int M>
@@ -549,11 +645,12 @@ __device__ __forceinline__ void block_max2(unsigned long long &a, unsigned long 
 template <int M>
 __device__ __noinline__ void solve_row(const MGFast &m, double *phi, int nr, double tol, int max_cycles,
                                           double *B, double *F) {
+    using Sh = Shape<double, M>;
     __shared__ unsigned long long s_max[2][kSolveThreads / 32];
+    __shared__ double s_x[256];
     const int tid = threadIdx.x, n = nr - 1;
     const double *cz = m.cz[0], *cr = m.cr[0];
-    auto at = [](int j) { return (j % M) * kRow + j / M; };
-    for (int k = tid; k < line_factor_elems(M); k += kSolveThreads) F[k] = m.facc[k];
+    for (int k = tid; k < Sh::elems; k += kSolveThreads) F[k] = m.facc[k];
     double bn = 0.0;
     for (int cyc = 0;; ++cyc) {
         unsigned long long rmax = 0ull, bmax = 0ull;
@@ -584,19 +681,23 @@ __device__ __noinline__ void solve_row(const MGFast &m, double *phi, int nr, dou
         if (d == 3)
             for (int j = tid; j < n; j += kSolveThreads) phi[nr + j] = 0.0;
         if (d) return;
-        for (int j = tid; j < kLine * M; j += kSolveThreads) {
+        for (int j = tid; j < Sh::unknowns; j += kSolveThreads) {
             double rhs = 0.0;
             if (j < n) {
                 const size_t k = (size_t)nr + j;
                 rhs = m.f0[k] + cz[k - nr] * phi[k - nr] + cz[k] * phi[k + nr];
                 if (j == n - 1) rhs += cr[k] * phi[k + 1];
             }
-            B[at(j)] = rhs;
+            B[Sh::at(j)] = rhs;
         }
         __syncthreads();
-        if (tid < 32) warp_line_solve<double, M>(F, B, tid);
+        if constexpr (Sh::group) {
+            if (tid < 128) group_line_solve<double, M>(F, B, s_x, tid, 1);
+        } else {
+            if (tid < 32) warp_line_solve<double, M>(F, B, tid);
+        }
         __syncthreads();
-        for (int j = tid; j < n; j += kSolveThreads) phi[nr + j] = B[at(j)];
+        for (int j = tid; j < n; j += kSolveThreads) phi[nr + j] = B[Sh::at(j)];
         __syncthreads();
     }
 }
@@ -624,8 +725,8 @@ __device__ __forceinline__ void solve_body(const MGFast *__restrict__ mp, double
     const MGFast &m = s_m;
     MGCtl *ctl = m.ctl;
     const int n = nr - 1, nz0 = m.nz[0], L = m.nlev - 1;
-    constexpr int NW = kLine * M;  // unknowns of a line with its padding
-    constexpr int LFE = line_factor_elems(M);
+    using Sh = Shape<Tv, M>;
+    constexpr int NW = Sh::unknowns, LFE = Sh::elems;
     if (L == 0) {
         if (bid == 0)
             solve_row<M>(m, phi, nr, tol, max_cycles, reinterpret_cast<double *>(smem_raw),
@@ -681,7 +782,8 @@ __device__ __forceinline__ void solve_body(const MGFast *__restrict__ mp, double
     }
     // line buffers: the two reds, the black line
     Tv *const Bf = reinterpret_cast<Tv *>(smem_raw);
-    constexpr int BL = M * kRow;
+    constexpr int BL = Sh::chunk * Sh::row;
+    __shared__ Tv s_x[Sh::group ? 512 : 1];  // a group's exchange: 2 x 128 values each
     double *St = reinterpret_cast<double *>(smem_raw);
     const int tw = lay.tw, ltw = __ffs(tw) - 1, sw = tw + 2, ntile = (n + tw - 1) >> ltw, tn = tw * (nz0 - 2);
     // e / sw for e < sw * nz0 (< 2^17): e * ceil(2^32 / sw) >> 32
@@ -689,8 +791,6 @@ __device__ __forceinline__ void solve_body(const MGFast *__restrict__ mp, double
     auto div_sw = [&](int e) { return (int)__umulhi((unsigned)e, sw_inv); };
     Tv *T0 = reinterpret_cast<Tv *>(smem_raw + lay.offT), *T1 = T0 + (size_t)tw * nz0;
     Wv *lu0 = (Wv *)m.lu[0], *lf0 = (Wv *)m.lf[0];
-    // position of unknown j in a line buffer
-    auto at = [](int j) { return (j % M) * kRow + j / M; };
     bool fail = false;
     int g = 0;  // units done
     int cyc = 0;
@@ -1042,8 +1142,9 @@ __device__ __forceinline__ void solve_body(const MGFast *__restrict__ mp, double
             // come into registers while the coarse rows are on their way
             if (!ld_wait(ld, slot) || (deep && !ld_wait(ld, kMaxSlots))) fail = true;
             constexpr bool kReg = WIDE && sizeof(Tv) == 4 && M <= 16;
+            const Tv *F = slots + (size_t)slot * 3 * LFE;
             LineFactors<Tv, M, kReg> lf;
-            if (warp < 3) lf.load(slots + (size_t)(slot * 3 + (warp == 0 ? 0 : 3 - warp)) * LFE, lane);
+            if (!Sh::group && warp < 3) lf.load(F + (size_t)(warp == 0 ? 0 : 3 - warp) * LFE, lane);
             Tv um0[kE];  // deep: the coarsest row
             if (deep) {
                 const Wv *p[kE];
@@ -1053,15 +1154,19 @@ __device__ __forceinline__ void solve_body(const MGFast *__restrict__ mp, double
                 flag_wait<Tv, kE>(p, x, tag, &ctl->timeout, fail);
 #pragma unroll
                 for (int s = 0; s < kE; ++s)
-                    if (tid + s * nt < NW) Bf[at(tid + s * nt)] = x[s];
+                    if (tid + s * nt < NW) Bf[Sh::at(tid + s * nt)] = x[s];
                 if (__syncthreads_or(fail)) {
                     fail = true;
                     break;
                 }
-                if (warp == 0) warp_line_solve<Tv, M>(FC, Bf, lane);
+                if constexpr (Sh::group) {
+                    if (tid < 128) group_line_solve<Tv, M>(FC, Bf, s_x, tid, 1);
+                } else {
+                    if (warp == 0) warp_line_solve<Tv, M>(FC, Bf, lane);
+                }
                 __syncthreads();
 #pragma unroll
-                for (int s = 0; s < kE; ++s) um0[s] = tid + s * nt < NW ? Bf[at(tid + s * nt)] : (Tv)0;
+                for (int s = 0; s < kE; ++s) um0[s] = tid + s * nt < NW ? Bf[Sh::at(tid + s * nt)] : (Tv)0;
             }
             Tv z[4][kE], fx[3 * kE], ux[3 * kE];  // z: cz below ra, ra + 1, ra + 2 and above it
             {
@@ -1102,7 +1207,7 @@ __device__ __forceinline__ void solve_body(const MGFast *__restrict__ mp, double
             for (int s = 0; s < kE; ++s) {
                 const int j = tid + s * nt;
                 if (j >= NW) break;
-                Tv *B = Bf + at(j);
+                Tv *B = Bf + Sh::at(j);
                 B[0] = fx[3 * s] + z[0][s] * ux[3 * s] + z[1][s] * ux[3 * s + 1];
                 B[BL] = fx[3 * s + 2] + z[2][s] * ux[3 * s + 1] + z[3][s] * ux[3 * s + 2];
             }
@@ -1110,13 +1215,18 @@ __device__ __forceinline__ void solve_body(const MGFast *__restrict__ mp, double
                 fail = true;
                 break;
             }
-            if (warp < 2) warp_line_solve<Tv, M, kReg>(lf, Bf + warp * BL, lane);
+            if constexpr (Sh::group) {  // a red line each half of the block
+                const int w = tid >> 7;
+                group_line_solve<Tv, M>(F + (size_t)2 * w * LFE, Bf + w * BL, s_x + 256 * w, tid & 127, 1 + w);
+            } else {
+                if (warp < 2) warp_line_solve<Tv, M, kReg>(lf, Bf + warp * BL, lane);
+            }
             __syncthreads();
 #pragma unroll
             for (int s = 0; s < kE; ++s) {
                 const int j = tid + s * nt;
                 if (j >= NW) break;
-                Tv *B = Bf + at(j);
+                Tv *B = Bf + Sh::at(j);
                 const Tv x0 = B[0], x1 = B[BL];
                 B[2 * BL] = fx[3 * s + 1] + z[1][s] * x0 + z[2][s] * x1;
                 if (j < n) {
@@ -1126,13 +1236,17 @@ __device__ __forceinline__ void solve_body(const MGFast *__restrict__ mp, double
                 }
             }
             __syncthreads();
-            if (warp == 2) warp_line_solve<Tv, M, kReg>(lf, Bf + 2 * BL, lane);
+            if constexpr (Sh::group) {
+                if (tid < 128) group_line_solve<Tv, M>(F + LFE, Bf + 2 * BL, s_x, tid, 1);
+            } else {
+                if (warp == 2) warp_line_solve<Tv, M, kReg>(lf, Bf + 2 * BL, lane);
+            }
             __syncthreads();
             if (nun > S) request(g + S, slot);
 #pragma unroll
             for (int s = 0; s < kE; ++s) {
                 const int j = tid + s * nt;
-                if (j < n) Fv::store(u + nr + j, Bf[2 * BL + at(j)], tag);
+                if (j < n) Fv::store(u + nr + j, Bf[2 * BL + Sh::at(j)], tag);
             }
         }
         if (fail) break;
@@ -1156,8 +1270,8 @@ __global__ void __launch_bounds__(kSolveThreads, MINB)
 // The solves of several reactors (one line chunk M, one precision) in one
 // cooperative launch: job k takes blocks [block0, block0 + nblocks) and hands
 // its words to its own blocks only, so the reactors proceed side by side.
-template <typename Tv, int M, int MINB>
-__global__ void __launch_bounds__(kSolveThreads, MINB) k_solve_multi(const SolveJob *__restrict__ jobs, int njobs) {
+template <typename Tv, int M>
+__global__ void __launch_bounds__(kSolveThreads, 2) k_solve_multi(const SolveJob *__restrict__ jobs, int njobs) {
     int lo = 0, hi = njobs - 1;  // the job whose block range holds this block
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
@@ -1169,12 +1283,12 @@ __global__ void __launch_bounds__(kSolveThreads, MINB) k_solve_multi(const Solve
     const SolveJob &j = jobs[lo];
     const int bid = (int)blockIdx.x - j.block0;
     if (bid >= j.nblocks) return;
-    solve_body<Tv, M, MINB == 1>(j.mp, j.phi, j.nr, j.lay, j.tol, j.max_cycles, j.sctl, bid, j.nblocks);
+    solve_body<Tv, M, false>(j.mp, j.phi, j.nr, j.lay, j.tol, j.max_cycles, j.sctl, bid, j.nblocks);
 }
 
 }  // namespace
 
-size_t mg_line_factor_elems(int nr) { return (size_t)line_factor_elems(line_chunk(nr - 1)); }
+size_t mg_line_factor_elems(int nr, bool f64) { return (size_t)line_elems(line_chunk(nr - 1), f64); }
 
 // tiles of one to eight columns, the last one whole, with two neighbour columns each
 size_t mg_tile_elems(int nz, int nr, bool with_neighbours) {
@@ -1190,20 +1304,15 @@ void *solve_fn(int minb) {
     return minb == 2 ? (void *)k_solve_persistent<Tv, M, 2> : (void *)k_solve_persistent<Tv, M, 1>;
 }
 
-template <typename Tv, int M>
-void *multi_fn(int minb) {
-    return minb == 2 ? (void *)k_solve_multi<Tv, M, 2> : (void *)k_solve_multi<Tv, M, 1>;
-}
-
 template <typename Tv>
-void *multi_kernel(int M, int minb) {
+void *multi_kernel(int M) {
     switch (M) {
-        case 1: return multi_fn<Tv, 1>(minb);
-        case 2: return multi_fn<Tv, 2>(minb);
-        case 4: return multi_fn<Tv, 4>(minb);
-        case 8: return multi_fn<Tv, 8>(minb);
-        case 16: return multi_fn<Tv, 16>(minb);
-        default: return multi_fn<Tv, 32>(minb);
+        case 1: return (void *)k_solve_multi<Tv, 1>;
+        case 2: return (void *)k_solve_multi<Tv, 2>;
+        case 4: return (void *)k_solve_multi<Tv, 4>;
+        case 8: return (void *)k_solve_multi<Tv, 8>;
+        case 16: return (void *)k_solve_multi<Tv, 16>;
+        default: return (void *)k_solve_multi<Tv, 32>;
     }
 }
 
@@ -1225,15 +1334,21 @@ constexpr size_t kSolveSmemLimit = 220 * 1024;
 void raise_smem_limits() {
     static bool done = false;
     if (done) return;
-    const int lim = (int)kSolveSmemLimit;
-    cudaFuncSetAttribute(k_setup_levels, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+    // (what the kernel's static shared memory leaves of a block's 227 KB)
+    auto raise = [](void *fn) {
+        cudaFuncAttributes a;
+        if (cudaFuncGetAttributes(&a, fn) == cudaSuccess)
+            cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)std::min(kSolveSmemLimit, 227 * 1024 - a.sharedSizeBytes));
+    };
+    raise((void *)k_setup_levels);
     for (int M = 1; M <= 32; M <<= 1) {
         for (int minb = 1; minb <= 2; ++minb) {
-            cudaFuncSetAttribute(solve_kernel<float>(M, minb), cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-            cudaFuncSetAttribute(solve_kernel<double>(M, minb), cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-            cudaFuncSetAttribute(multi_kernel<float>(M, minb), cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-            cudaFuncSetAttribute(multi_kernel<double>(M, minb), cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+            raise(solve_kernel<float>(M, minb));
+            raise(solve_kernel<double>(M, minb));
         }
+        raise(multi_kernel<float>(M));
+        raise(multi_kernel<double>(M));
     }
     done = true;
 }
@@ -1283,7 +1398,7 @@ bool solve_job(const FieldDims &fd, MGFast &m, double *phi, bool mixed, double t
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     const size_t es = mixed ? sizeof(float) : sizeof(double);
-    const size_t LFE = (size_t)line_factor_elems(M);
+    const size_t LFE = (size_t)line_elems(M, !mixed || m.nlev == 1);
     SolveLayout lay{};
     const int L = m.nlev - 1;
     size_t off = 0;
@@ -1295,7 +1410,7 @@ bool solve_job(const FieldDims &fd, MGFast &m, double *phi, bool mixed, double t
     int grid = 1;
     const int minb = wide ? 1 : 2;
     if (L == 0) {
-        take((size_t)M * kRow * sizeof(double));
+        take((size_t)line_buffer(M, true) * sizeof(double));
         lay.offC = take(LFE * sizeof(double));
         lay.tw = 4;
     } else {
@@ -1305,13 +1420,14 @@ bool solve_job(const FieldDims &fd, MGFast &m, double *phi, bool mixed, double t
         lay.tw = mixed && (!wide || n > 4 * nsm) ? 8 : 4;
         // the line buffers of the line phases share their space with the residual phase's tile (with its two neighbour columns) and
         // restriction buffers (very tall meshes: narrower tiles)
-        const size_t line = (size_t)3 * M * kRow * es;
+        const size_t line = (size_t)3 * line_buffer(M, !mixed) * es;
         const size_t fac = LFE * es + (size_t)3 * LFE * es + 512;
         size_t tile = 0, both = 0;
         for (;; lay.tw /= 2) {
             tile = ((size_t)(lay.tw + 2) * nz * sizeof(double) + 127) & ~(size_t)127;
             both = std::max(line, tile + (size_t)lay.tw * (2 * nz + kMaxLevels) * es);
-            if (lay.tw == 1 || both + fac <= kSolveSmemLimit) break;
+            // (FP64: room for the static exchange buffers too)
+            if (lay.tw == 1 || both + fac + (mixed ? 0 : 8192) <= kSolveSmemLimit) break;
         }
         lay.offT = (int)tile;
         take(both);
@@ -1504,7 +1620,7 @@ std::vector<std::pair<int, int>> mg_multi_plan(std::vector<SolveJob> &jobs, bool
             want += jobs[b].nblocks;
             ++b;
         }
-        void *fn = jobs[a].mixed ? multi_kernel<float>(jobs[a].M, 2) : multi_kernel<double>(jobs[a].M, 2);
+        void *fn = jobs[a].mixed ? multi_kernel<float>(jobs[a].M) : multi_kernel<double>(jobs[a].M);
         kinds.push_back({a, b, fn, smem, want});
         want_all += want;
         a = b;

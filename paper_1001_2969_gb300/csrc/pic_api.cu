@@ -624,7 +624,7 @@ void setup_device(pic_handle *h) {
     // V-cycle's correction and right-hand side, and the r-line factors
     MGFast &m = h->mgf;
     memset(&m, 0, sizeof(m));
-    const size_t line_fe = mg_line_factor_elems(h->nr);
+    const size_t line_fe = mg_line_factor_elems(h->nr, !h->mixed);
     int nl = 0;
     for (int z = h->nz;; z = (z + 1) / 2) {
         const int l = nl++;
@@ -641,7 +641,7 @@ void setup_device(pic_handle *h) {
         }
         const size_t fe = (size_t)(z - 2) * line_fe;
         if (z == 3) {
-            m.facc = (double *)dalloc(h, fe * sizeof(double));
+            m.facc = (double *)dalloc(h, mg_line_factor_elems(h->nr, true) * sizeof(double));
             if (h->mixed) m.facc32 = (float *)dalloc(h, fe * sizeof(float));
         } else if (!h->mixed)
             m.fac64[l] = (double *)dalloc(h, fe * sizeof(double));
