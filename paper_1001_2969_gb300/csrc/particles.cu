@@ -187,15 +187,15 @@ struct Rel {
 };
 
 // electrons: the gas at rest; ions: an atom drawn from the gas Maxwellian
-template <typename T>
+template <typename T, int S>
 __device__ __forceinline__ Rel<T> relative(const StepArgs<T> &a, uint64_t id, uint32_t step, const PS<T> &p) {
     Rel<T> r;
     r.gx = p.vr;
     r.gy = p.vt;
     r.gz = p.vz;
     r.vnx = r.vny = r.vnz = 0;
-    if (a.s == 1) {
-        const uint4 y = draw(a.key0, a.key1, id, step, 1, a.s);
+    if constexpr (S == 1) {
+        const uint4 y = draw(a.key0, a.key1, id, step, 1, S);
         T n0, n1, n2, n3;
         normals(y.x, y.y, n0, n1);
         normals(y.z, y.w, n2, n3);
@@ -214,7 +214,7 @@ __device__ __forceinline__ Rel<T> relative(const StepArgs<T> &a, uint64_t id, ui
 // channel of a candidate whose stream-0 draw is x: -1 for a null collision
 // (also an inelastic channel picked below its threshold); counts nu_max
 // overruns and real collisions
-template <typename T>
+template <typename T, int S>
 __device__ __forceinline__ int choose(const StepArgs<T> &a, BlockTally *bt, const uint4 x, const Rel<T> &r) {
     T nu[kMaxCh];
     sigma_all(a.xs, r.E, nu);
@@ -225,7 +225,7 @@ __device__ __forceinline__ int choose(const StepArgs<T> &a, BlockTally *bt, cons
         nu[ch] = ch < a.xs.n_ch ? ngg * nu[ch] : (T)0;
         tot += nu[ch];
     }
-    if (tot > a.nu_max) atomicAdd(&bt->cnt[PIC_C_NUOVER + a.s], 1ull);
+    if (tot > a.nu_max) atomicAdd(&bt->cnt[PIC_C_NUOVER + S], 1ull);
     const T sel = unif<T>(x.y) * a.nu_max;
     T cum = 0;
     int ch = -1;
@@ -237,26 +237,28 @@ __device__ __forceinline__ int choose(const StepArgs<T> &a, BlockTally *bt, cons
         }
     }
     if (ch < 0) return -1;
-    const int kind = a.xs.kind[ch];
-    if ((kind == PIC_XS_EXCITE || kind == PIC_XS_IONIZE) && r.E <= a.xs.thr[ch]) return -1;
-    atomicAdd(&bt->cnt[PIC_C_COLL + a.s * 4 + ch], 1ull);
+    if constexpr (S == 0) {  // (ions exchange charge only)
+        const int kind = a.xs.kind[ch];
+        if ((kind == PIC_XS_EXCITE || kind == PIC_XS_IONIZE) && r.E <= a.xs.thr[ch]) return -1;
+    }
+    atomicAdd(&bt->cnt[PIC_C_COLL + S * 4 + ch], 1ull);
     return ch;
 }
 
 // the collision on channel ch (Vahedi-Surendra scattering, ionisation
 // births, charge exchange)
-template <typename T>
+template <typename T, int S>
 __device__ __forceinline__ void scatter(const StepArgs<T> &a, BlockTally *bt, uint64_t id, uint32_t step,
                                         const uint4 x, int ch, const Rel<T> &r, PS<T> &p) {
-    const int kind = a.xs.kind[ch];
-    const T thr = a.xs.thr[ch];
-    const T g = r.g, E = r.E;
-    if (kind == PIC_XS_CX) {
+    if constexpr (S == 1) {  // charge exchange, the ions' one kind
         p.vr = r.vnx;
         p.vt = r.vny;
         p.vz = r.vnz;
         return;
     }
+    const int kind = a.xs.kind[ch];
+    const T thr = a.xs.thr[ch];
+    const T g = r.g, E = r.E;
     const T ux = r.gx / g, uy = r.gy / g, uz = r.gz / g;
     T dx, dy, dz;
     if (kind == PIC_XS_ELASTIC) {
@@ -275,8 +277,8 @@ __device__ __forceinline__ void scatter(const StepArgs<T> &a, BlockTally *bt, ui
         p.vt = gn * dy;
         p.vz = gn * dz;
     } else {  // ionisation
-        const uint4 y = draw(a.key0, a.key1, id, step, 1, a.s);
-        const uint4 zz = draw(a.key0, a.key1, id, step, 2, a.s);
+        const uint4 y = draw(a.key0, a.key1, id, step, 1, S);
+        const uint4 zz = draw(a.key0, a.key1, id, step, 2, S);
         const T Eej = a.xs.B * m_tan(unif<T>(y.x) * m_atan((E - thr) / ((T)2 * a.xs.B)));
         T Esc = E - thr - Eej;
         if (Esc < (T)0) Esc = (T)0;
@@ -303,21 +305,21 @@ __device__ __forceinline__ void scatter(const StepArgs<T> &a, BlockTally *bt, ui
         ion.ar = p.ar * a.ion_acc;
         ion.az = p.az * a.ion_acc;
         ion.at = a.xyz ? p.at * a.ion_acc : (T)0;
-        emit_birth(a, bt, 0, a.s, id, 0, e2);
-        emit_birth(a, bt, 1, a.s, id, 1, ion);
+        emit_birth(a, bt, 0, S, id, 0, e2);
+        emit_birth(a, bt, 1, S, id, 1, ion);
     }
 }
 
 // the whole Monte Carlo step of one particle
-template <typename T>
+template <typename T, int S>
 __device__ __forceinline__ void collide(const StepArgs<T> &a, BlockTally *bt, uint64_t id, uint32_t step,
                                         PS<T> &p) {
-    const uint4 x = draw(a.key0, a.key1, id, step, 0, a.s);
+    const uint4 x = draw(a.key0, a.key1, id, step, 0, S);
     if ((unsigned long long)x.x >= a.t_null) return;
-    atomicAdd(&bt->cnt[PIC_C_CAND + a.s], 1ull);
-    const Rel<T> r = relative(a, id, step, p);
-    const int ch = choose(a, bt, x, r);
-    if (ch >= 0) scatter(a, bt, id, step, x, ch, r, p);
+    atomicAdd(&bt->cnt[PIC_C_CAND + S], 1ull);
+    const Rel<T> r = relative<T, S>(a, id, step, p);
+    const int ch = choose<T, S>(a, bt, x, r);
+    if (ch >= 0) scatter<T, S>(a, bt, id, step, x, ch, r, p);
 }
 
 // cp.async of 4, 8 or 16 bytes (global -> shared; both ends aligned to the size)
@@ -354,7 +356,9 @@ constexpr int kEedfCopies = 8;
 // a time, ahead of their use (for latency-bound passes)
 // PPT: particles per thread in a unit (32 * PPT particles per warp)
 // XYZ: the global X-Y-Z pusher (a_theta carried; a.xyz set)
-template <typename T, bool PF, int kPPT, bool XYZ>
+// S: the species, 0 electrons (Vahedi-Surendra scattering and births, EEDF), 1
+// ions (charge exchange)
+template <typename T, bool PF, int kPPT, bool XYZ, int S>
 __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 4 : 2) k_step(StepArgs<T> a) {
     constexpr int kChunk = kThreads * kPPT;  // the block's staging slots
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -375,7 +379,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 4 : 2) k_step(StepA
     const bool do_split = a.ctl->do_split != 0;
     for (int k = tid; k < PIC_NCOUNT; k += blockDim.x) bt.cnt[k] = 0;
     if (tid < 3) bt.q[tid] = 0.0;
-    if (a.eedf)
+    if (S == 0 && a.eedf)
         for (int k = tid; k < a.eedf_bins * kEedfCopies; k += blockDim.x) s_eedf[k] = (T)0;
     __syncthreads();  // tallies and EEDF cleared before any thread adds to them
     const int n = *a.n_alive;
@@ -480,13 +484,13 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 4 : 2) k_step(StepA
             }
             int wall = alive ? wall_of(p.i, p.oz, p.j, a.nz, a.nr) : -1;
             if (wall >= 0) {
-                atomicAdd(&bt.cnt[PIC_C_ABS + a.s * 3 + wall], 1ull);
-                atomicAdd(&bt.q[wall], (double)p.w * a.qch[a.s]);
+                atomicAdd(&bt.cnt[PIC_C_ABS + S * 3 + wall], 1ull);
+                atomicAdd(&bt.q[wall], (double)p.w * a.qch[S]);
                 alive = false;
             }
             if (alive) {
-                collide(a, &bt, id, step, p);
-                if (a.eedf) {
+                collide<T, S>(a, &bt, id, step, p);
+                if (S == 0 && a.eedf) {
                     const T Ek = a.half_m_e * (p.vr * p.vr + p.vt * p.vt + p.vz * p.vz);
                     const T x = Ek * a.eedf_scale;
                     if (x >= (T)0 && x < (T)a.eedf_bins)
@@ -504,11 +508,11 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 4 : 2) k_step(StepA
                             rem = p.w - (T)Nc * wr_;
                         }
                         if (Nc > 0) {
-                            atomicAdd(&bt.cnt[PIC_C_SPLITS + a.s], 1ull);
+                            atomicAdd(&bt.cnt[PIC_C_SPLITS + S], 1ull);
                             PS<T> cp = p;
                             cp.w = wr_;
                             p.w = rem;
-                            for (int c = 0; c < Nc; ++c) emit_birth(a, &bt, a.s, a.s, id, 2 + c, cp);
+                            for (int c = 0; c < Nc; ++c) emit_birth(a, &bt, S, S, id, 2 + c, cp);
                         }
                     }
                 }
@@ -518,8 +522,8 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 4 : 2) k_step(StepA
                     first_push(a, p);
                 wall = wall_of(p.i, p.oz, p.j, a.nz, a.nr);
                 if (wall >= 0) {
-                    atomicAdd(&bt.cnt[PIC_C_ABS + a.s * 3 + wall], 1ull);
-                    atomicAdd(&bt.q[wall], (double)p.w * a.qch[a.s]);
+                    atomicAdd(&bt.cnt[PIC_C_ABS + S * 3 + wall], 1ull);
+                    atomicAdd(&bt.q[wall], (double)p.w * a.qch[S]);
                     alive = false;
                 }
             }
@@ -558,10 +562,10 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 4 : 2) k_step(StepA
             }
         }
         if (head && out_cell >= 0) {
-            atomicAdd(a.counts[a.s] + out_cell, rend - lane);
+            atomicAdd(a.counts[S] + out_cell, rend - lane);
             int ci, cj;
             decode_cell(out_cell, a.ncz, a.inv_ncz, ci, cj);
-            double *g = a.N[a.s] + (size_t)ci * a.nr + cj;
+            double *g = a.N[S] + (size_t)ci * a.nr + cj;
             atomicAdd(g, (double)c00);
             atomicAdd(g + 1, (double)c01);
             atomicAdd(g + a.nr, (double)c10);
@@ -681,7 +685,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 4 : 2) k_step(StepA
         atomicAdd(&a.ds->qabs[tid], bt.q[tid]);
         atomicAdd(&a.ds->qstep[tid], bt.q[tid]);
     }
-    if (a.eedf)
+    if (S == 0 && a.eedf)
         for (int k = tid; k < a.eedf_bins; k += blockDim.x) {
             double v = 0.0;
             for (int c = 0; c < kEedfCopies; ++c) v += (double)s_eedf[k * kEedfCopies + c];
@@ -689,7 +693,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 4 : 2) k_step(StepA
         }
 }
 
-template <typename T, bool PF, int PPT, bool XYZ>
+template <typename T, bool PF, int PPT, bool XYZ, int S>
 void launch_shape(const StepArgs<T> &a, int grid, cudaStream_t st) {
     const size_t stage =
         PF ? (size_t)kThreads * PPT *
@@ -700,22 +704,29 @@ void launch_shape(const StepArgs<T> &a, int grid, cudaStream_t st) {
     // dynamic plus static shared memory above 48 KB needs the opt-in: set
     // it for every size (the static tallies come on top of `smem`)
     if (smem > 0)
-        cudaFuncSetAttribute(k_step<T, PF, PPT, XYZ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaFuncSetAttribute(k_step<T, PF, PPT, XYZ, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     // blocks claim chunks until none is left: as many as are resident at once
     int per_sm = 0, dev = 0, nsm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_step<T, PF, PPT, XYZ>, kThreads, smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_step<T, PF, PPT, XYZ, S>, kThreads, smem);
     if (per_sm > 0 && nsm > 0) grid = std::min(grid, per_sm * nsm);
-    k_step<T, PF, PPT, XYZ><<<grid, kThreads, smem, st>>>(a);
+    k_step<T, PF, PPT, XYZ, S><<<grid, kThreads, smem, st>>>(a);
 }
 
 template <typename T, bool PF, int PPT>
 void launch_variant(const StepArgs<T> &a, int grid, cudaStream_t st) {
-    if (a.xyz)
-        launch_shape<T, PF, PPT, true>(a, grid, st);
-    else
-        launch_shape<T, PF, PPT, false>(a, grid, st);
+    if (a.s == 0) {
+        if (a.xyz)
+            launch_shape<T, PF, PPT, true, 0>(a, grid, st);
+        else
+            launch_shape<T, PF, PPT, false, 0>(a, grid, st);
+    } else {
+        if (a.xyz)
+            launch_shape<T, PF, PPT, true, 1>(a, grid, st);
+        else
+            launch_shape<T, PF, PPT, false, 1>(a, grid, st);
+    }
 }
 
 // variant: bit 0 = prefetch the chunk into shared memory, bit 1 = 8
