@@ -113,10 +113,10 @@ __device__ __forceinline__ void scatter_dir(T ux, T uy, T uz, T cc, T uphi, T &o
         oz = cc * uz;
         return;
     }
-    const T s = m_sqrt(s2);
-    ox = cc * ux + sc * (cp * uy + sp * ux * uz) / s;
-    oy = cc * uy + sc * (-cp * ux + sp * uy * uz) / s;
-    oz = cc * uz + sc * (-sp * s2) / s;
+    const T s = m_sqrt(s2), inv = m_inv(s);
+    ox = cc * ux + m_quot(sc * (cp * uy + sp * ux * uz), s, inv);
+    oy = cc * uy + m_quot(sc * (-cp * ux + sp * uy * uz), s, inv);
+    oz = cc * uz + m_quot(sc * (-sp * s2), s, inv);
 }
 
 template <typename T>
@@ -259,7 +259,8 @@ __device__ __forceinline__ void scatter(const StepArgs<T> &a, BlockTally *bt, ui
     const int kind = a.xs.kind[ch];
     const T thr = a.xs.thr[ch];
     const T g = r.g, E = r.E;
-    const T ux = r.gx / g, uy = r.gy / g, uz = r.gz / g;
+    const T ig = m_inv(g);
+    const T ux = m_quot(r.gx, g, ig), uy = m_quot(r.gy, g, ig), uz = m_quot(r.gz, g, ig);
     T dx, dy, dz;
     if (kind == PIC_XS_ELASTIC) {
         const T cc = cos_chi(a.scatter, E, unif<T>(x.z));
@@ -436,7 +437,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 4 : 2) k_step(StepA
             if (!in_mesh) p.i = p.j = 0;
             // gather E at x~ with the deposit's shape factors (Sec. 2.4)
             T s0, s1;
-            shape_r(a.weighting, p.j, p.orr, s0, s1);
+            shape_r(a.weighting, p.j, p.orr, s0, s1, a.inv_t);
             const T z0 = (T)1 - p.oz, z1 = p.oz;
             const auto *Ep = a.E + (size_t)p.i * a.nr + p.j;
             const auto e00 = Ep[0], e01 = Ep[1], e10 = Ep[a.nr], e11 = Ep[a.nr + 1];
@@ -476,9 +477,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 4 : 2) k_step(StepA
                 }
             }
             bool alive = true;
-            // one test for all: a NaN or infinity anywhere makes the sum
-            // non-finite (the values are far below overflow)
-            if (!in_mesh || !m_finite(p.oz + p.orr + p.vr + p.vt + p.vz + p.w)) {
+            if (!in_mesh || !all_finite(p.oz, p.orr, p.vr, p.vt, p.vz, p.w)) {
                 atomicOr(&a.ds->status, ST_NAN);
                 alive = false;
             }
@@ -531,7 +530,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 4 : 2) k_step(StepA
                 out_cell = p.j * a.ncz + p.i;
                 // deposit weights at the new x~ (Sec. 2.4)
                 T r0, r1;
-                shape_r(a.weighting, p.j, p.orr, r0, r1);
+                shape_r(a.weighting, p.j, p.orr, r0, r1, a.inv_t);
                 const T y0 = (T)1 - p.oz, y1 = p.oz;
                 c00 = p.w * y0 * r0;
                 c01 = p.w * y0 * r1;
@@ -550,6 +549,9 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 4 : 2) k_step(StepA
         const int rend = above ? __ffs(above) - 1 : 32;
 #pragma unroll
         for (int d = 1; d < 32; d <<= 1) {
+            // (FP64: no additions past the longest run; FP32, whose additions
+            // are cheap, gains nothing by looking)
+            if (sizeof(T) == 8 && !__any_sync(0xffffffffu, lane + d < rend)) break;
             const T t00 = __shfl_down_sync(0xffffffffu, c00, d);
             const T t01 = __shfl_down_sync(0xffffffffu, c01, d);
             const T t10 = __shfl_down_sync(0xffffffffu, c10, d);

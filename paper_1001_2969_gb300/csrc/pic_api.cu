@@ -90,6 +90,7 @@ struct pic_handle {
     double *N[2] = {nullptr, nullptr};
     double *rho = nullptr, *chi = nullptr, *phi = nullptr, *Ez = nullptr, *Er = nullptr, *V = nullptr, *iV = nullptr;
     void *E2 = nullptr;
+    double *inv_t = nullptr;  // 1 / (2j + 1) per radial cell (FP64 path)
     double *phiL_d = nullptr;
     bool has_phiL = false;
     // external circuit: the two superposition parts of phi and an empty charge grid
@@ -329,6 +330,11 @@ void node_volumes(const pic_handle *h, std::vector<double> &V) {
 __global__ void k_inverse(const double *x, double *y, int n) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k < n) y[k] = 1.0 / x[k];
+}
+
+__global__ void k_inverse_odd(double *y, int n) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k < n) y[k] = 1.0 / (2.0 * k + 1.0);
 }
 
 __global__ void k_iota(int32_t *p, int n) {
@@ -620,6 +626,10 @@ void setup_device(pic_handle *h) {
     node_volumes(h, V);
     cudaMemcpyAsync(h->V, V.data(), gb, cudaMemcpyHostToDevice, h->st);
     k_inverse<<<(h->ng + 255) / 256, 256, 0, h->st>>>(h->V, h->iV, h->ng);
+    if (!h->mixed) {
+        h->inv_t = (double *)dalloc(h, (size_t)h->ncr * sizeof(double));
+        k_inverse_odd<<<(h->ncr + 255) / 256, 256, 0, h->st>>>(h->inv_t, h->ncr);
+    }
     // multigrid hierarchy: per level nodal chi and face coefficients, the
     // V-cycle's correction and right-hand side, and the r-line factors
     MGFast &m = h->mgf;
@@ -797,6 +807,7 @@ void fill_step_args(pic_handle *h, StepArgs<T> &a, int s, int src_set, int dst_s
     a.key1 = (uint32_t)(h->cfg.seed >> 32);
     a.ctl = h->sctl;
     a.w_ref = (const T *)h->sp[s].w_ref;
+    a.inv_t = (const T *)h->inv_t;
     a.E = (const typename V2<T>::type *)h->E2;
     SpecDev &d = h->sp[s];
     a.src_main = view<T>(d.main[src_set]);

@@ -294,6 +294,7 @@ struct StepArgs {
     const StepCtl *ctl;  // step number (Philox counter), split flag, halt
     // splitting
     const T *w_ref;  // [ncr]
+    const T *inv_t;  // [ncr] 1 / (2j + 1), FP64 (null on the mixed path)
     // fields at the nodes {E_z, E_r}
     const typename V2<T>::type *E;
     // input set, read through perm

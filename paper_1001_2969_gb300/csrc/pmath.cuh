@@ -36,6 +36,27 @@ __device__ __forceinline__ bool m_finite(double x) { return isfinite(x); }
 // where the result feeds positions/weights (never a threshold test on its own)
 __device__ __forceinline__ float m_div(float a, float b) { return __fdividef(a, b); }
 __device__ __forceinline__ double m_div(double a, double b) { return a / b; }
+// quotients of one divisor.  An FP64 division is some twelve operations on
+// GB300's narrow FP64 pipe, which bounds the FP64 pass: the divisor's inverse is
+// taken once (m_inv) and each quotient corrected by its residual, which leaves
+// it rounded as the division would be but for the last half unit.  FP32
+// divides.
+__device__ __forceinline__ float m_inv(float) { return 0.0f; }
+__device__ __forceinline__ double m_inv(double x) { return 1.0 / x; }
+__device__ __forceinline__ float m_quot(float a, float b, float) { return a / b; }
+__device__ __forceinline__ double m_quot(double a, double b, double inv) {
+    const double q = a * inv;
+    return fma(fma(-q, b, a), inv, q);
+}
+// no value is a NaN or infinite: in FP32 their sum is finite (the values are
+// far below overflow), in FP64 their exponents tell, off the FP64 pipe
+__device__ __forceinline__ bool all_finite(float a, float b, float c, float d, float e, float f) {
+    return isfinite(a + b + c + d + e + f);
+}
+__device__ __forceinline__ bool all_finite(double a, double b, double c, double d, double e, double f) {
+    auto bad = [](double x) { return (__double2hiint(x) & 0x7ff00000) == 0x7ff00000; };
+    return !(bad(a) | bad(b) | bad(c) | bad(d) | bad(e) | bad(f));
+}
 __device__ __forceinline__ float m_rsqrt(float x) { return rsqrtf(x); }
 __device__ __forceinline__ double m_rsqrt(double x) { return 1.0 / sqrt(x); }
 
@@ -127,8 +148,9 @@ __device__ __forceinline__ void store_p(const PBuf<T> &b, int idx, const PS<T> &
 
 // radial shape factors of Eq. (9) (z-r^2) or Eq. (8) (z-r) in offset form:
 // z-r^2: S_{j+1} = (r^2 - r_j^2)/(r_{j+1}^2 - r_j^2) = o (2j + o)/(2j + 1)
+// inv_t (FP64, nullable): 1 / (2j + 1) per radial cell
 template <typename T>
-__device__ __forceinline__ void shape_r(int weighting, int j, T o, T &s0, T &s1) {
+__device__ __forceinline__ void shape_r(int weighting, int j, T o, T &s0, T &s1, const T *inv_t = nullptr) {
     if (weighting == PIC_WEIGHT_ZR) {
         s1 = o;
         s0 = (T)1 - o;
@@ -139,8 +161,9 @@ __device__ __forceinline__ void shape_r(int weighting, int j, T o, T &s0, T &s1)
         s0 = ((T)1 - o) * (t + o) * it;
     } else {
         const T t = (T)(2 * j + 1);
-        s1 = m_div(o * ((T)(2 * j) + o), t);
-        s0 = m_div(((T)1 - o) * (t + o), t);
+        const T it = inv_t ? inv_t[j] : m_inv(t);
+        s1 = m_quot(o * (t - (T)1 + o), t, it);
+        s0 = m_quot(((T)1 - o) * (t + o), t, it);
     }
 }
 
@@ -184,8 +207,9 @@ __device__ __forceinline__ void first_push(const StepArgs<T> &a, PS<T> &p, const
             sn = dy * inv;
         } else {
             rn = m_sqrt(q2);
-            c = xr / rn;
-            sn = dy / rn;
+            const T inv = m_inv(rn);
+            c = m_quot(xr, rn, inv);
+            sn = m_quot(dy, rn, inv);
         }
     }
     const T den = rn + r;
@@ -234,8 +258,9 @@ __device__ __forceinline__ void first_push_xyz(const StepArgs<T> &a, PS<T> &p, c
             sn = dy * inv;
         } else {
             rn = m_sqrt(q2);
-            c = xr / rn;
-            sn = dy / rn;
+            const T inv = m_inv(rn);
+            c = m_quot(xr, rn, inv);
+            sn = m_quot(dy, rn, inv);
         }
     }
     const T den = rn + r;
