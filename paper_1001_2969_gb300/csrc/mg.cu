@@ -557,9 +557,10 @@ __global__ void k_rhs_bc(const MGFast *__restrict__ mp, RhsArgs a, int nz, int n
 // that owns them, and nothing drops them from L1.
 // Words are reused every cycle under a new tag.  That is safe: a tile phase
 // starts with every row of the cycle's level-0 correction, each of which comes
-// after all its unit's reads and after those of all units above it; and rows
-// of the next correction are written after the exchange of norms that ends
-// the tile phase, to which every block comes with its own reads done.
+// after all its unit's reads and after those of all units above it; rows of
+// the next correction start with the coarsest, for which all tile phases of
+// that cycle must be through; and no block is more than a cycle ahead of
+// another's look at the norms, which are kept in two sets.
 // Measured, a whole stand-alone solve (with its set-up launches) against the
 // same phases between grid barriers, which took ~1 us each and cost every
 // phase its L1: 33 x 65 mixed 216 -> 157 us, 65 x 300 mixed 326 -> 228,
@@ -1095,42 +1096,48 @@ __device__ __forceinline__ void solve_body(const MGFast *__restrict__ mp, double
             if (cyc == 0) Flag<double>::store(to + 1, __longlong_as_double((long long)bmax), tag);
         }
         xr += (size_t)(bid % kCopies) * 2 * kMaxSolveBlocks;
-        rmax = bmax = 0ull;
-        for (int e = tid; e < P; e += nt) {
-            const ulonglong2 *p[2] = {xr + 2 * e, cyc == 0 ? xr + 2 * e + 1 : nullptr};
-            double x[2];
-            flag_wait<double, 2>(p, x, tag, &ctl->timeout, fail);
-            rmax = max(rmax, (unsigned long long)__double_as_longlong(x[0]));
-            bmax = max(bmax, (unsigned long long)__double_as_longlong(x[1]));
-        }
-        block_max2(rmax, bmax, s_max[1]);
-        if (__syncthreads_or(fail)) break;
-        const double rn = __longlong_as_double((long long)rmax);
-        if (cyc == 0) bn = __longlong_as_double((long long)bmax);
-        int decide = 0;  // 0 continue, 1 converged, 2 out of cycles, 3 zero right-hand side
-        if (bn == 0.0)
-            decide = 3;
-        else if (tol > 0.0 && rn <= tol * bn)
-            decide = 1;
-        else if (cyc >= max_cycles)
-            decide = tol > 0.0 ? 2 : 1;
-        if (bid == 0 && tid == 0) {
-            ctl->last_res = rn;
-            ctl->bnorm = bn;
-            ctl->cycles = cyc;
-            if (decide == 1) ctl->converged = 1;
-            if (decide == 3) ctl->zero_rhs = 1;
-        }
-        if (decide == 3)
-            for (int t = bid; t < ntile; t += P)
-                for (int e = tid; e < tn; e += nt) {
-                    const int j = t * tw + (e & (tw - 1));
-                    if (j < n) phi[(size_t)(1 + (e >> ltw)) * nr + j] = 0.0;
-                }
-        if (decide != 0) break;  // phi holds the iterate of this residual
+        // ---- decision: every block reads every block's maxima, and comes to
+        // the same: 0 continue, 1 converged, 2 out of cycles, 3 zero right-hand
+        // side, 4 a wait gave up.  phi holds the iterate of this residual.  The
+        // line phases start without it (they do not change phi): a block looks
+        // while it waits for its coarse rows, the one with the coarsest row,
+        // which all others wait for, when it has handed that on.
+        auto check = [&]() -> int {
+            unsigned long long rm = 0ull, bm = 0ull;
+            for (int e = tid; e < P; e += nt) {
+                const ulonglong2 *p[2] = {xr + 2 * e, cyc == 0 ? xr + 2 * e + 1 : nullptr};
+                double x[2];
+                flag_wait<double, 2>(p, x, tag, &ctl->timeout, fail);
+                rm = max(rm, (unsigned long long)__double_as_longlong(x[0]));
+                bm = max(bm, (unsigned long long)__double_as_longlong(x[1]));
+            }
+            block_max2(rm, bm, s_max[1]);
+            if (__syncthreads_or(fail)) {
+                fail = true;
+                return 4;
+            }
+            const double rn = __longlong_as_double((long long)rm);
+            if (cyc == 0) bn = __longlong_as_double((long long)bm);
+            int d = 0;
+            if (bn == 0.0)
+                d = 3;
+            else if (tol > 0.0 && rn <= tol * bn)
+                d = 1;
+            else if (cyc >= max_cycles)
+                d = tol > 0.0 ? 2 : 1;
+            if (bid == 0 && tid == 0) {
+                ctl->last_res = rn;
+                ctl->bnorm = bn;
+                ctl->cycles = cyc;
+                if (d == 1) ctl->converged = 1;
+                if (d == 3) ctl->zero_rhs = 1;
+            }
+            return d;
+        };
+        int decide = -1;  // not looked yet
         // ---- up: per unit, a black line with the two red lines beside it ----
         constexpr int kE = (NW + nt - 1) / nt;  // unknowns of a line per thread
-        for (int k = 0; k < nun && !fail; ++k, ++g) {
+        for (int k = 0; k < nun; ++k, ++g) {
             int l, q;
             unit_at(bid + k * P, l, q);
             const int nzc = m.nz[l + 1], slot = nun <= S ? k : g % S;
@@ -1181,6 +1188,7 @@ __device__ __forceinline__ void solve_body(const MGFast *__restrict__ mp, double
                     for (int w = 0; w < 3; ++w) p[3 * s + w] = j < n ? f + (size_t)w * nr + j : nullptr;
                 }
                 flag_wait<Tv, 3 * kE>(p, fx, tag, &ctl->timeout, fail);
+                if (!deep && decide < 0 && (decide = check()) != 0) break;
                 if (!deep) {
                     // coarse rows below ra, between (row ra + 1) and above
                     // ra + 2: q, q + 1, q + 2, zero at the level's ends
@@ -1249,7 +1257,14 @@ __device__ __forceinline__ void solve_body(const MGFast *__restrict__ mp, double
                 if (j < n) Fv::store(u + nr + j, Bf[2 * BL + Sh::at(j)], tag);
             }
         }
-        if (fail) break;
+        if (!fail && decide < 0) decide = check();
+        if (decide == 3)
+            for (int t = bid; t < ntile; t += P)
+                for (int e = tid; e < tn; e += nt) {
+                    const int j = t * tw + (e & (tw - 1));
+                    if (j < n) phi[(size_t)(1 + (e >> ltw)) * nr + j] = 0.0;
+                }
+        if (fail || decide != 0) break;
     }
     // leave with no copy in flight (bounded waits), the tags used up
     if (fail && tid == 0) atomicExch(&ctl->timeout, 1);
