@@ -176,6 +176,12 @@ __device__ void emit_birth(const StepArgs<T> &a, BlockTally *bt, int ts, int ps,
     a.bkey[ts][slot] = ((uint64_t)ps << 63) | (pid << 16) | (uint64_t)k;
 }
 
+// the pass's species: fixed in the ions' instantiation
+template <int S, typename T>
+__device__ __forceinline__ int species(const StepArgs<T> &a) {
+    return S == 1 ? 1 : a.s;
+}
+
 // Null-collision Monte Carlo (Sec. 2.6) on the post-final-push state, in
 // three parts: the relative velocity against the target, the channel of a
 // candidate, and the collision itself.
@@ -194,8 +200,8 @@ __device__ __forceinline__ Rel<T> relative(const StepArgs<T> &a, uint64_t id, ui
     r.gy = p.vt;
     r.gz = p.vz;
     r.vnx = r.vny = r.vnz = 0;
-    if constexpr (S == 1) {
-        const uint4 y = draw(a.key0, a.key1, id, step, 1, S);
+    if (species<S>(a) == 1) {
+        const uint4 y = draw(a.key0, a.key1, id, step, 1, species<S>(a));
         T n0, n1, n2, n3;
         normals(y.x, y.y, n0, n1);
         normals(y.z, y.w, n2, n3);
@@ -225,7 +231,7 @@ __device__ __forceinline__ int choose(const StepArgs<T> &a, BlockTally *bt, cons
         nu[ch] = ch < a.xs.n_ch ? ngg * nu[ch] : (T)0;
         tot += nu[ch];
     }
-    if (tot > a.nu_max) atomicAdd(&bt->cnt[PIC_C_NUOVER + S], 1ull);
+    if (tot > a.nu_max) atomicAdd(&bt->cnt[PIC_C_NUOVER + species<S>(a)], 1ull);
     const T sel = unif<T>(x.y) * a.nu_max;
     T cum = 0;
     int ch = -1;
@@ -237,11 +243,11 @@ __device__ __forceinline__ int choose(const StepArgs<T> &a, BlockTally *bt, cons
         }
     }
     if (ch < 0) return -1;
-    if constexpr (S == 0) {  // (ions exchange charge only)
+    if constexpr (S != 1) {  // (ions exchange charge only)
         const int kind = a.xs.kind[ch];
         if ((kind == PIC_XS_EXCITE || kind == PIC_XS_IONIZE) && r.E <= a.xs.thr[ch]) return -1;
     }
-    atomicAdd(&bt->cnt[PIC_C_COLL + S * 4 + ch], 1ull);
+    atomicAdd(&bt->cnt[PIC_C_COLL + species<S>(a) * 4 + ch], 1ull);
     return ch;
 }
 
@@ -259,6 +265,12 @@ __device__ __forceinline__ void scatter(const StepArgs<T> &a, BlockTally *bt, ui
     const int kind = a.xs.kind[ch];
     const T thr = a.xs.thr[ch];
     const T g = r.g, E = r.E;
+    if (kind == PIC_XS_CX) {
+        p.vr = r.vnx;
+        p.vt = r.vny;
+        p.vz = r.vnz;
+        return;
+    }
     const T ig = m_inv(g);
     const T ux = m_quot(r.gx, g, ig), uy = m_quot(r.gy, g, ig), uz = m_quot(r.gz, g, ig);
     T dx, dy, dz;
@@ -278,8 +290,8 @@ __device__ __forceinline__ void scatter(const StepArgs<T> &a, BlockTally *bt, ui
         p.vt = gn * dy;
         p.vz = gn * dz;
     } else {  // ionisation
-        const uint4 y = draw(a.key0, a.key1, id, step, 1, S);
-        const uint4 zz = draw(a.key0, a.key1, id, step, 2, S);
+        const uint4 y = draw(a.key0, a.key1, id, step, 1, species<S>(a));
+        const uint4 zz = draw(a.key0, a.key1, id, step, 2, species<S>(a));
         const T Eej = a.xs.B * m_tan(unif<T>(y.x) * m_atan((E - thr) / ((T)2 * a.xs.B)));
         T Esc = E - thr - Eej;
         if (Esc < (T)0) Esc = (T)0;
@@ -306,8 +318,8 @@ __device__ __forceinline__ void scatter(const StepArgs<T> &a, BlockTally *bt, ui
         ion.ar = p.ar * a.ion_acc;
         ion.az = p.az * a.ion_acc;
         ion.at = a.xyz ? p.at * a.ion_acc : (T)0;
-        emit_birth(a, bt, 0, S, id, 0, e2);
-        emit_birth(a, bt, 1, S, id, 1, ion);
+        emit_birth(a, bt, 0, species<S>(a), id, 0, e2);
+        emit_birth(a, bt, 1, species<S>(a), id, 1, ion);
     }
 }
 
@@ -315,9 +327,9 @@ __device__ __forceinline__ void scatter(const StepArgs<T> &a, BlockTally *bt, ui
 template <typename T, int S>
 __device__ __forceinline__ void collide(const StepArgs<T> &a, BlockTally *bt, uint64_t id, uint32_t step,
                                         PS<T> &p) {
-    const uint4 x = draw(a.key0, a.key1, id, step, 0, S);
+    const uint4 x = draw(a.key0, a.key1, id, step, 0, species<S>(a));
     if ((unsigned long long)x.x >= a.t_null) return;
-    atomicAdd(&bt->cnt[PIC_C_CAND + S], 1ull);
+    atomicAdd(&bt->cnt[PIC_C_CAND + species<S>(a)], 1ull);
     const Rel<T> r = relative<T, S>(a, id, step, p);
     const int ch = choose<T, S>(a, bt, x, r);
     if (ch >= 0) scatter<T, S>(a, bt, id, step, x, ch, r, p);
@@ -357,8 +369,10 @@ constexpr int kEedfCopies = 8;
 // a time, ahead of their use (for latency-bound passes)
 // PPT: particles per thread in a unit (32 * PPT particles per warp)
 // XYZ: the global X-Y-Z pusher (a_theta carried; a.xyz set)
-// S: the species, 0 electrons (Vahedi-Surendra scattering and births, EEDF), 1
-// ions (charge exchange)
+// S: 1 the ions (charge exchange alone: fewer registers, no spills, c2 230 -> 221
+// us), 0 the electrons.  Fixing the species at compile time for the electrons
+// too gave 2 %, but the compiler then contracts the scattering differently and
+// one electron in a thousand moves by an FP32 rounding: not done.
 template <typename T, bool PF, int kPPT, bool XYZ, int S>
 __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 4 : 2) k_step(StepArgs<T> a) {
     constexpr int kChunk = kThreads * kPPT;  // the block's staging slots
@@ -380,7 +394,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 4 : 2) k_step(StepA
     const bool do_split = a.ctl->do_split != 0;
     for (int k = tid; k < PIC_NCOUNT; k += blockDim.x) bt.cnt[k] = 0;
     if (tid < 3) bt.q[tid] = 0.0;
-    if (S == 0 && a.eedf)
+    if (S != 1 && a.eedf)
         for (int k = tid; k < a.eedf_bins * kEedfCopies; k += blockDim.x) s_eedf[k] = (T)0;
     __syncthreads();  // tallies and EEDF cleared before any thread adds to them
     const int n = *a.n_alive;
@@ -483,13 +497,13 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 4 : 2) k_step(StepA
             }
             int wall = alive ? wall_of(p.i, p.oz, p.j, a.nz, a.nr) : -1;
             if (wall >= 0) {
-                atomicAdd(&bt.cnt[PIC_C_ABS + S * 3 + wall], 1ull);
-                atomicAdd(&bt.q[wall], (double)p.w * a.qch[S]);
+                atomicAdd(&bt.cnt[PIC_C_ABS + species<S>(a) * 3 + wall], 1ull);
+                atomicAdd(&bt.q[wall], (double)p.w * a.qch[species<S>(a)]);
                 alive = false;
             }
             if (alive) {
                 collide<T, S>(a, &bt, id, step, p);
-                if (S == 0 && a.eedf) {
+                if (S != 1 && a.eedf) {
                     const T Ek = a.half_m_e * (p.vr * p.vr + p.vt * p.vt + p.vz * p.vz);
                     const T x = Ek * a.eedf_scale;
                     if (x >= (T)0 && x < (T)a.eedf_bins)
@@ -507,11 +521,11 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 4 : 2) k_step(StepA
                             rem = p.w - (T)Nc * wr_;
                         }
                         if (Nc > 0) {
-                            atomicAdd(&bt.cnt[PIC_C_SPLITS + S], 1ull);
+                            atomicAdd(&bt.cnt[PIC_C_SPLITS + species<S>(a)], 1ull);
                             PS<T> cp = p;
                             cp.w = wr_;
                             p.w = rem;
-                            for (int c = 0; c < Nc; ++c) emit_birth(a, &bt, S, S, id, 2 + c, cp);
+                            for (int c = 0; c < Nc; ++c) emit_birth(a, &bt, species<S>(a), species<S>(a), id, 2 + c, cp);
                         }
                     }
                 }
@@ -521,8 +535,8 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 4 : 2) k_step(StepA
                     first_push(a, p);
                 wall = wall_of(p.i, p.oz, p.j, a.nz, a.nr);
                 if (wall >= 0) {
-                    atomicAdd(&bt.cnt[PIC_C_ABS + S * 3 + wall], 1ull);
-                    atomicAdd(&bt.q[wall], (double)p.w * a.qch[S]);
+                    atomicAdd(&bt.cnt[PIC_C_ABS + species<S>(a) * 3 + wall], 1ull);
+                    atomicAdd(&bt.q[wall], (double)p.w * a.qch[species<S>(a)]);
                     alive = false;
                 }
             }
@@ -564,10 +578,10 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 4 : 2) k_step(StepA
             }
         }
         if (head && out_cell >= 0) {
-            atomicAdd(a.counts[S] + out_cell, rend - lane);
+            atomicAdd(a.counts[species<S>(a)] + out_cell, rend - lane);
             int ci, cj;
             decode_cell(out_cell, a.ncz, a.inv_ncz, ci, cj);
-            double *g = a.N[S] + (size_t)ci * a.nr + cj;
+            double *g = a.N[species<S>(a)] + (size_t)ci * a.nr + cj;
             atomicAdd(g, (double)c00);
             atomicAdd(g + 1, (double)c01);
             atomicAdd(g + a.nr, (double)c10);
@@ -687,7 +701,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 4 : 2) k_step(StepA
         atomicAdd(&a.ds->qabs[tid], bt.q[tid]);
         atomicAdd(&a.ds->qstep[tid], bt.q[tid]);
     }
-    if (S == 0 && a.eedf)
+    if (S != 1 && a.eedf)
         for (int k = tid; k < a.eedf_bins; k += blockDim.x) {
             double v = 0.0;
             for (int c = 0; c < kEedfCopies; ++c) v += (double)s_eedf[k * kEedfCopies + c];

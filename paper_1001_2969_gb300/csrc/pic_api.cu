@@ -961,13 +961,19 @@ void one_step(pic_handle *h, cudaStream_t sb, bool mv, int part = 0, SolveJob *j
                 return;
             }
         }
+        cudaStream_t es = st;
         if (sb) {
             cudaStreamWaitEvent(sb, h->ev_fork, 0);
             sort_branch<T>(h, src, isrc, mv, sb);
             cudaEventRecord(h->ev_join, sb);
+            // E on the second branch, beside the end of the sort
+            cudaEventRecord(h->ev_fork2, st);
+            cudaStreamWaitEvent(sb, h->ev_fork2, 0);
+            es = sb;
         }
         launch_efield<T>(h->phi, h->Ez, h->Er, (typename V2<T>::type *)h->E2, h->nz, h->nr, h->dz,
-                         h->dr, h->sctl, h->cfg.circuit_C > 0.0 ? nullptr : h->mgf.ctl, st);
+                         h->dr, h->sctl, h->cfg.circuit_C > 0.0 ? nullptr : h->mgf.ctl, es);
+        if (sb) cudaEventRecord(h->ev_join2, sb);
         h->launches += L + 1;
     }
     if (sb) cudaStreamWaitEvent(st, h->ev_join, 0);
@@ -989,6 +995,7 @@ void one_step(pic_handle *h, cudaStream_t sb, bool mv, int part = 0, SolveJob *j
             PhaseTimer t(h, 3);
             sort_finish(h, src, isrc, st, h->in_batch ? nullptr : &r);
         }
+        if (sb) cudaStreamWaitEvent(st, h->ev_join2, 0);  // E
         if (h->in_batch) {  // its births numbering has one block: too few to clear with
             k_pass_reset<<<std::max(1, std::min(152 * 4, (std::max(h->ng, h->ncell) + 255) / 256)), 256, 0, st>>>(r);
             h->launches += 1;
