@@ -945,9 +945,12 @@ __device__ __forceinline__ void solve_body(const MGFast *__restrict__ mp, double
                 // narrow, and every thread dividing cost microseconds
                 if (warp == 0) {
                     const double t = over_warps(1);
-                    const double rw = __shfl_sync(0xffffffffu, t, 0), ww = __shfl_sync(0xffffffffu, t, 1),
-                                 wwp = __shfl_sync(0xffffffffu, t, 2), rwp = __shfl_sync(0xffffffffu, t, 3);
+                    const double rw = __shfl_sync(0xffffffffu, t, 0), ww = __shfl_sync(0xffffffffu, t, 1);
+                    double wwp = __shfl_sync(0xffffffffu, t, 2), rwp = __shfl_sync(0xffffffffu, t, 3);
                     if (lane == 0) {
+                        // no previous direction (a solve's first step): what lies
+                        // there is an earlier solve's, perhaps not finite
+                        if (!(s_ab[3] > 0.0)) wwp = rwp = 0.0;
                         const double beta = wwp * s_ab[3];
                         const double den = ww - beta * wwp;
                         s_ab[0] = beta;
@@ -958,8 +961,9 @@ __device__ __forceinline__ void solve_body(const MGFast *__restrict__ mp, double
                 __syncthreads();
             }
             const double beta = s_ab[0], alpha = s_ab[1];
-            // 1 / |q|^2 for the next step's beta, off this one's path
-            if (tid == nt - 1) s_ab[3] = s_ab[2] > 0.0 ? 1.0 / s_ab[2] : 0.0;
+            // 1 / |q|^2 for the next step's beta, off this one's path (none where
+            // the inverse would not be finite: the next step starts anew)
+            if (tid == nt - 1) s_ab[3] = s_ab[2] >= 2.2250738585072014e-308 ? 1.0 / s_ab[2] : 0.0;
             const bool one = bid + P >= ntile;  // the block's only tile: z is still in St
             for (int t = bid; t < ntile; t += P) {
                 const int j0 = t * tw;

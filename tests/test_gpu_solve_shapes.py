@@ -42,3 +42,23 @@ def test_solve_shapes(mesh, prec):
     ref = o.grid("phi")
     assert np.abs(phi - ref).max() <= (1e-11 if fixed else 1e-8) * np.abs(ref).max()
     assert np.array_equal(phi, again)
+
+
+@pytest.mark.parametrize("prec", ["fp64", "mixed"])
+def test_solve_after_a_solve_that_was_not_finite(prec):
+    """What a solve of non-finite charge leaves in the handle's workspace does not reach the next."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1001_2969_gb300 import pic
+
+    cfg = W.scaled(W.config("c1", precision=prec, mg_max_cycles=30), 0)
+    chi = W.random_grid(cfg, seed=1, scale=2.0)
+    rho = 1e-5 * (W.random_grid(cfg, seed=2, smooth=False) - 0.5)
+    bad = rho.copy()
+    bad[7, 11] = np.nan
+    fresh = pic.pic_field_solve(pic.pic_init(cfg, load=False), rho, chi, 60.0)
+    h = pic.pic_init(cfg, load=False)
+    assert pic.pic_field_solve(h, bad, chi, 60.0)[3] == pic.PIC_ERR_NOT_CONVERGED
+    phi, cyc, _, st = pic.pic_field_solve(h, rho, chi, 60.0)
+    assert st == fresh[3] == 0 and cyc == fresh[1] and np.array_equal(phi, fresh[0])
