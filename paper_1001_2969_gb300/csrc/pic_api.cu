@@ -1501,6 +1501,8 @@ pic_status finish_call(pic_handle *h, int64_t step0, int cur0, int cur_i0, int32
         const int32_t z[3] = {0, 0, 0};
         cudaMemcpyAsync(&h->sctl->halt, z, 2 * sizeof(int32_t), cudaMemcpyHostToDevice, h->st);
         cudaMemcpyAsync(&h->sctl->sort_pending, z, 3 * sizeof(int32_t), cudaMemcpyHostToDevice, h->st);
+        // (a pass whose sort failed had moved the device's step number on)
+        cudaMemcpyAsync(&h->sctl->step, &h->step, sizeof(int64_t), cudaMemcpyHostToDevice, h->st);
         cudaMemsetAsync(&h->ds->status, 0, 4, h->st);
         const int why = c.sort_fail ? c.sort_fail_status : c.halt_status;
         if (h->K > 1) {
