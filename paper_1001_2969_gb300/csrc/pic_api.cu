@@ -387,11 +387,10 @@ __global__ void k_step_begin(StepCtl *c, const double *rf, int nrf, double dt, i
     c->do_split = split_every > 0 && (c->step % split_every) == split_every - 1;
 }
 
-// a pass that holds the ions: the births its newborn ions join start at
-// the buffer's present count (skipped once the step has failed, so that a
-// dropped pass's newborns can be cut off again)
-// zero what the particle passes accumulate into (a batch's reactors; else k_birth_finish does)
-__global__ void k_pass_reset(PassReset r) {
+// zero what the particle passes accumulate into (a batch's reactors; else
+// k_birth_finish does); a failed step keeps its births
+__global__ void k_pass_reset(PassReset r, const StepCtl *c) {
+    if (c->halt) return;
     const int t = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
     for (int s = 0; s < 2; ++s) {
         if (r.N[s])
@@ -406,6 +405,9 @@ __global__ void k_pass_reset(PassReset r) {
     }
 }
 
+// a pass that holds the ions: the births its newborn ions join start at
+// the buffer's present count (skipped once the step has failed, so that a
+// dropped pass's newborns can be cut off again)
 __global__ void k_hold_ions(const StepCtl *c, int32_t *nb0, const int32_t *nb) {
     if (c->halt) return;
     *nb0 = *nb;
@@ -997,7 +999,8 @@ void one_step(pic_handle *h, cudaStream_t sb, bool mv, int part = 0, SolveJob *j
         }
         if (sb) cudaStreamWaitEvent(st, h->ev_join2, 0);  // E
         if (h->in_batch) {  // its births numbering has one block: too few to clear with
-            k_pass_reset<<<std::max(1, std::min(152 * 4, (std::max(h->ng, h->ncell) + 255) / 256)), 256, 0, st>>>(r);
+            k_pass_reset<<<std::max(1, std::min(152 * 4, (std::max(h->ng, h->ncell) + 255) / 256)), 256, 0, st>>>(
+                r, h->sctl);
             h->launches += 1;
         }
         // (else always 0)
@@ -1511,23 +1514,16 @@ pic_status finish_call(pic_handle *h, int64_t step0, int cur0, int cur_i0, int32
                 resync_ions<float>(h, cut);
             else
                 resync_ions<double>(h, cut);
-            if (!(why & (ST_CAPACITY | ST_BIRTH_OVERFLOW))) {
-                if (h->mixed)
-                    deposit_current<float>(h);
-                else
-                    deposit_current<double>(h);
-            }
         }
-        if (why & (ST_CAPACITY | ST_BIRTH_OVERFLOW)) {
-            if (h->mixed)
-                deposit_current<float>(h);
-            else
-                deposit_current<double>(h);
-            cudaStreamSynchronize(h->st);
+        // (the dropped pass's deposit took the place of the state's)
+        if (h->mixed)
+            deposit_current<float>(h);
+        else
+            deposit_current<double>(h);
+        cudaStreamSynchronize(h->st);
+        if (why & (ST_CAPACITY | ST_BIRTH_OVERFLOW))
             return fail(h, PIC_ERR_CAPACITY, (why & ST_CAPACITY) ? "particle capacity exceeded"
                                                                  : "births capacity exceeded");
-        }
-        cudaStreamSynchronize(h->st);
         return fail(h, PIC_ERR_TIMEOUT, c.sort_fail ? "births numbering: grid barrier timed out"
                                                     : "multigrid grid barrier timed out");
     }

@@ -561,21 +561,28 @@ __device__ bool radix_births(const uint64_t *key, uint64_t *id, int nb, StepCtl 
 // Cooperative when it has more than one block (the radix sort's barriers).
 __global__ void __launch_bounds__(kRadixThreads) k_birth_finish(BirthJob b, PassReset r, int reset) {
     const int tid = threadIdx.x, t = blockIdx.x * blockDim.x + tid, all = gridDim.x * blockDim.x;
-    if (reset) {
+    StepCtl *ctl = b.ctl;
+    if (reset && !ctl->halt) {
         for (int s = 0; s < 2; ++s) {
             if (r.N[s])
                 for (int k = t; k < r.ng; k += all) r.N[s][k] = 0.0;
             if (r.counts[s])
                 for (int k = t; k < r.ncell; k += all) r.counts[s][k] = 0;
         }
-        if (t == 0) {
+        if (t == 0) r.chunk_next[0] = r.chunk_next[1] = 0;
+    }
+    // the coming pass writes its births over those of the pass before the one
+    // sorted here: they are the state's until this sort is done, and stay
+    // where it failed
+    auto drop_births = [&]() {
+        if (reset && t == 0 && !*(const volatile int32_t *)&ctl->halt)
             for (int s = 0; s < 2; ++s)
                 if (r.nbirths[s]) *r.nbirths[s] = 0;
-            r.chunk_next[0] = r.chunk_next[1] = 0;
-        }
+    };
+    if (sort_skip(ctl)) {
+        drop_births();
+        return;
     }
-    StepCtl *ctl = b.ctl;
-    if (sort_skip(ctl)) return;
     // every block reads the counts and the bases before the first barrier;
     // block 0 moves the bases on at the end
     int nb[2], first[2];
@@ -598,6 +605,7 @@ __global__ void __launch_bounds__(kRadixThreads) k_birth_finish(BirthJob b, Pass
             *b.nalive[s] = *b.ntotal[s];
         }
         ctl->sort_pending = 0;
+        drop_births();
     }
 }
 

@@ -75,3 +75,27 @@ def test_a_failed_step_fails_again_and_leaves_the_step_number(short):
             pic.pic_step(h, n)
         assert err.value.status == pic.PIC_ERR_CAPACITY
         same(pic, h, ref)
+
+
+@pytest.mark.parametrize("batched", [False, True])
+@pytest.mark.parametrize("short", ["capacity", "births"])
+def test_a_failed_call_of_several_steps_keeps_births_and_deposit(short, batched):
+    """The pass that overflows is followed by further steps of its call, whose kernels find out."""
+    pic, h, ref = pair(short)
+    assert pic.pic_step(ref, 2) == 0
+    b = pic.pic_batch_init([h]) if batched else None
+    for _ in range(2):
+        if batched:
+            with pytest.raises(pic.PicError):
+                b.step(5)
+        else:
+            with pytest.raises(pic.PicError) as err:
+                pic.pic_step(h, 5)
+            assert err.value.status == pic.PIC_ERR_CAPACITY
+        same(pic, h, ref)
+    for x in (h, ref):  # on from there, from a step that does not split
+        pic.pic_set_step(x, 0)
+        assert pic.pic_step(x, 2) == 0
+    same(pic, h, ref, grids=("rho", "chi", "phi"))
+    if batched:
+        b.close()
