@@ -1440,15 +1440,16 @@ pic_status window_t(pic_handle *h, int32_t nsteps, int32_t ckpt, const double *w
     return cuda_check(h, "window");
 }
 
-// After a failed call with ion subcycling: the ions as the last completed
-// step left them.  A dropped pass that held them had appended its newborn
-// ions to their births (cut off again); a dropped pass that moved them had
-// recounted their cells.  So the counts, the permutation and the count of
-// ions are rebuilt from the state, and the deposit with them.
+// After a failed call: the counts, the permutation and the count of species s
+// rebuilt from its stored state.  With ion subcycling the ions need it: a
+// dropped pass that held them had appended its newborn ions to their births
+// (cut off again), one that moved them had recounted their cells.  A sort
+// that failed in the births numbering had ranked the dropped pass's particles
+// already: both species need it.
 template <typename T>
-void resync_ions(pic_handle *h, bool cut_births) {
-    SpecDev &d = h->sp[1];
-    const int c = h->cur_i;
+void resync(pic_handle *h, int s, bool cut_births) {
+    SpecDev &d = h->sp[s];
+    const int c = par_of(h, s);
     if (cut_births) cudaMemcpyAsync(d.d_nbirths[c], d.d_nb0, sizeof(int32_t), cudaMemcpyDeviceToDevice, h->st);
     cudaMemsetAsync(d.d_nb0, 0, sizeof(int32_t), h->st);
     cudaMemsetAsync(d.counts, 0, (size_t)h->ncell * sizeof(int32_t), h->st);
@@ -1508,12 +1509,14 @@ pic_status finish_call(pic_handle *h, int64_t step0, int cur0, int cur_i0, int32
         cudaMemcpyAsync(&h->sctl->step, &h->step, sizeof(int64_t), cudaMemcpyHostToDevice, h->st);
         cudaMemsetAsync(&h->ds->status, 0, 4, h->st);
         const int why = c.sort_fail ? c.sort_fail_status : c.halt_status;
-        if (h->K > 1) {
-            const bool cut = c.sort_fail && !moves_ions(h, c.sort_fail_step);
+        const bool ranked = c.sort_fail && !(why & (ST_CAPACITY | ST_BIRTH_OVERFLOW));
+        for (int s = 0; s < 2; ++s) {
+            if (!ranked && !(s == 1 && h->K > 1)) continue;
+            const bool cut = s == 1 && h->K > 1 && c.sort_fail && !moves_ions(h, c.sort_fail_step);
             if (h->mixed)
-                resync_ions<float>(h, cut);
+                resync<float>(h, s, cut);
             else
-                resync_ions<double>(h, cut);
+                resync<double>(h, s, cut);
         }
         // (the dropped pass's deposit took the place of the state's)
         if (h->mixed)
