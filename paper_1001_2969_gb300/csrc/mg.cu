@@ -160,6 +160,17 @@ inline int line_chunk(int n) {
     return M;
 }
 
+// The solve's control block starts cleared, with the one decision all of the
+// solve's blocks take whether it runs (one thread of the set-up calls it).
+// They do not look at `halt` themselves: the cell sort beside the solve may
+// set it, and blocks that went on without the others would leave words behind
+// under tags that the next solve uses again.
+__device__ __forceinline__ void begin_solve(const MGFast &m, const StepCtl *ctl) {
+    MGCtl c{};
+    c.skip = ctl && *(const volatile int32_t *)&ctl->halt;
+    *m.ctl = c;
+}
+
 // what a node of the fine level starts from: the right-hand side
 // rho A_j dz / eps0, the operator's diagonal and the Dirichlet data of phi;
 // with phi_prev (a warm solve) the interior starts from 2 phi - phi_prev, the
@@ -215,12 +226,9 @@ __global__ void __launch_bounds__(kSetupThreads)
     __shared__ Ts sd[MC * Sh::row], se[MC * Sh::row];  // cz below + above the row, cr
     __shared__ Ts sx[2][6][Sh::group ? NL : 1];         // exchange between the lanes' warps
     const MGFast &m = *mp;
+    if (blockIdx.x == 0 && threadIdx.x == 0) begin_solve(m, ctl);
     if (ctl && ctl->halt) return;
     const int n = nr - 1, p = threadIdx.x & (NL - 1);
-    // the solve's control block starts cleared
-    if (blockIdx.x == 0)
-        for (int w = threadIdx.x; w < (int)(sizeof(MGCtl) / sizeof(unsigned)); w += blockDim.x)
-            reinterpret_cast<unsigned *>(m.ctl)[w] = 0u;
     int i = blockIdx.x, l = 0;
     while (i >= m.nz[l]) i -= m.nz[l++];
     const int nz = m.nz[l];
@@ -526,10 +534,9 @@ __device__ __forceinline__ void warp_line_solve(const Ts *F, Ts *Bs, int p) {
 __global__ void k_rhs_bc(const MGFast *__restrict__ mp, RhsArgs a, int nz, int nr, const StepCtl *ctl) {
     const MGFast &m = *mp;
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= nz * nr || (ctl && ctl->halt)) return;
+    if (k >= nz * nr) return;
+    if (k == 0) begin_solve(m, ctl);
     rhs_node(m, a, (ctl && a.v_from_ctl) ? ctl->V : a.V, nz, nr, k / nr, k % nr, m.dg0[k]);
-    for (int w = k; w < (int)(sizeof(MGCtl) / sizeof(unsigned)); w += nz * nr)
-        reinterpret_cast<unsigned *>(m.ctl)[w] = 0u;
 }
 
 // ---------------------------------------------------------------------------
@@ -560,7 +567,9 @@ __global__ void k_rhs_bc(const MGFast *__restrict__ mp, RhsArgs a, int nz, int n
 // after all its unit's reads and after those of all units above it; rows of
 // the next correction start with the coarsest, for which all tile phases of
 // that cycle must be through; and no block is more than a cycle ahead of
-// another's look at the norms, which are kept in two sets.
+// another's look at the norms, which are kept in two sets.  A solve's tags
+// start where the one before ended (block 0 moves `epoch` on), so either all
+// of its blocks run or none does (MGCtl::skip).
 // Measured, a whole stand-alone solve (with its set-up launches) against the
 // same phases between grid barriers, which took ~1 us each and cost every
 // phase its L1: 33 x 65 mixed 216 -> 157 us, 65 x 300 mixed 326 -> 228,
@@ -708,9 +717,8 @@ __device__ __noinline__ void solve_row(const MGFast &m, double *phi, int nr, dou
 template <typename Tv, int M, bool WIDE>
 __device__ __forceinline__ void solve_body(const MGFast *__restrict__ mp, double *phi, int nr,
                                            const SolveLayout &lay, double tol, int max_cycles,
-                                           const StepCtl *sctl, const int bid, const int P) {
+                                           const int bid, const int P) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    if (sctl && sctl->halt) return;  // an earlier failure of this step
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     constexpr int nt = kSolveThreads;
     constexpr int kU = WIDE ? 4 : 2;  // elements per thread and batch in the residual phase
@@ -725,6 +733,7 @@ __device__ __forceinline__ void solve_body(const MGFast *__restrict__ mp, double
     }
     const MGFast &m = s_m;
     MGCtl *ctl = m.ctl;
+    if (ctl->skip) return;  // an earlier failure of this step
     const int n = nr - 1, nz0 = m.nz[0], L = m.nlev - 1;
     using Sh = Shape<Tv, M>;
     constexpr int NW = Sh::unknowns, LFE = Sh::elems;
@@ -1282,8 +1291,8 @@ __device__ __forceinline__ void solve_body(const MGFast *__restrict__ mp, double
 template <typename Tv, int M, int MINB>
 __global__ void __launch_bounds__(kSolveThreads, MINB)
     k_solve_persistent(const MGFast *__restrict__ mp, double *phi, int nr, SolveLayout lay, double tol,
-                       int max_cycles, const StepCtl *sctl) {
-    solve_body<Tv, M, MINB == 1>(mp, phi, nr, lay, tol, max_cycles, sctl, blockIdx.x, gridDim.x);
+                       int max_cycles) {
+    solve_body<Tv, M, MINB == 1>(mp, phi, nr, lay, tol, max_cycles, blockIdx.x, gridDim.x);
 }
 
 // The solves of several reactors (one line chunk M, one precision) in one
@@ -1302,7 +1311,7 @@ __global__ void __launch_bounds__(kSolveThreads, 2) k_solve_multi(const SolveJob
     const SolveJob &j = jobs[lo];
     const int bid = (int)blockIdx.x - j.block0;
     if (bid >= j.nblocks) return;
-    solve_body<Tv, M, false>(j.mp, j.phi, j.nr, j.lay, j.tol, j.max_cycles, j.sctl, bid, j.nblocks);
+    solve_body<Tv, M, false>(j.mp, j.phi, j.nr, j.lay, j.tol, j.max_cycles, bid, j.nblocks);
 }
 
 }  // namespace
@@ -1408,8 +1417,8 @@ void mg_fast_upload(MGFast &m, cudaStream_t st) {
 
 // The launch shape of one reactor's one-launch solve (shared-memory layout,
 // blocks, kernel); false when it cannot be launched.
-bool solve_job(const FieldDims &fd, MGFast &m, double *phi, bool mixed, double tol, int max_cycles,
-               const StepCtl *sctl, bool wide, SolveJob &job) {
+bool solve_job(const FieldDims &fd, MGFast &m, double *phi, bool mixed, double tol, int max_cycles, bool wide,
+               SolveJob &job) {
     const int nz = fd.nz, nr = fd.nr, n = nr - 1;
     const int M = line_chunk(n);
     raise_smem_limits();
@@ -1474,7 +1483,6 @@ bool solve_job(const FieldDims &fd, MGFast &m, double *phi, bool mixed, double t
     job.lay = lay;
     job.tol = tol;
     job.max_cycles = max_cycles;
-    job.sctl = sctl;
     job.block0 = 0;
     job.nblocks = grid;
     job.M = M;
@@ -1538,7 +1546,7 @@ int mg_fast_solve(const FieldDims &fd, MGFast &m, const FieldSource &src, double
     }
     // all cycles in one cooperative launch
     SolveJob job;
-    if (!solve_job(fd, m, phi, mixed, tol, max_cycles, sctl, wide, job)) {
+    if (!solve_job(fd, m, phi, mixed, tol, max_cycles, wide, job)) {
         if (at_solve) cudaEventRecord(at_solve, st);
         if (launches) *launches += L;
         return kSolveNoLaunch;
@@ -1555,8 +1563,7 @@ int mg_fast_solve(const FieldDims &fd, MGFast &m, const FieldSource &src, double
     const int grid = job.nblocks;
     int nrv = nr, mc = max_cycles;
     double tv = tol;
-    const StepCtl *sc = sctl;
-    void *args[] = {(void *)&mp, (void *)&phi, (void *)&nrv, (void *)&lay, (void *)&tv, (void *)&mc, (void *)&sc};
+    void *args[] = {(void *)&mp, (void *)&phi, (void *)&nrv, (void *)&lay, (void *)&tv, (void *)&mc};
     // the highest stream priority: when a step sorts beside the solve, the
     // solve's blocks take SMs as soon as the sort's short blocks retire
     static int prio = 1;

@@ -10,6 +10,7 @@ namespace pic {
 // device-side control of one solve (the one-launch V-cycles)
 struct MGCtl {
     int converged, zero_rhs, cycles, timeout;
+    int skip, pad;  // the step had halted when the solve was set up: its blocks do nothing
     double last_res, bnorm;
 };
 
@@ -111,7 +112,6 @@ struct SolveJob {
     SolveLayout lay;
     double tol;
     int max_cycles;
-    const StepCtl *sctl;
     int block0, nblocks;  // this job's blocks in the launch
     // host side
     int M, mixed, minb;
@@ -161,8 +161,8 @@ int mg_fast_solve(const FieldDims &fd, MGFast &m, const FieldSource &src, double
                   cudaEvent_t after = nullptr, MGCtl *pinned = nullptr);
 
 // the launch shape of one reactor's solve (host only); false: not launchable
-bool solve_job(const FieldDims &fd, MGFast &m, double *phi, bool mixed, double tol, int max_cycles,
-               const StepCtl *sctl, bool wide, SolveJob &job);
+bool solve_job(const FieldDims &fd, MGFast &m, double *phi, bool mixed, double tol, int max_cycles, bool wide,
+               SolveJob &job);
 
 // Plan deferred solves for shared cooperative launches: jobs of one (precision,
 // line chunk) kind share a launch; each kind gets SMs in proportion to the

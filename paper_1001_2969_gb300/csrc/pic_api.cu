@@ -1188,7 +1188,7 @@ void capture_batch(pic_batch *b, pic_batch::Graph &g) {
         if (h->cfg.circuit_C > 0.0) continue;
         FieldDims fd{h->nz, h->nr, h->dz, h->dr, h->cfg.mesh.L, h->cfg.chi_face};
         SolveJob j;
-        if (!solve_job(fd, h->mgf, h->phi, h->mixed, h->cfg.mg_tol, h->cfg.mg_max_cycles, h->sctl, false, j))
+        if (!solve_job(fd, h->mgf, h->phi, h->mixed, h->cfg.mg_tol, h->cfg.mg_max_cycles, false, j))
             continue;
         jobs.push_back(j);
         shared[k] = 1;
