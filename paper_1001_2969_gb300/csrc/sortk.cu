@@ -454,6 +454,10 @@ __device__ bool radix_births(const uint64_t *key, uint64_t *id, int nb, StepCtl 
         if (tid == 0) sort_failed(ctl, ST_TIMEOUT);
         return false;
     };
+    // (No barrier lies between the first species' last loop, which may read
+    // v0, and this fill for the second: both give entry e to the same thread,
+    // and must go on doing so.  Keys, digit counts and the flag of the first
+    // are read before its last barrier but one.)
     for (int e = blockIdx.x * blockDim.x + tid; e < nb; e += gridDim.x * blockDim.x) {
         t.k0[e] = key[e];
         t.v0[e] = (uint32_t)e;
@@ -549,6 +553,7 @@ __device__ bool radix_births(const uint64_t *key, uint64_t *id, int nb, StepCtl 
         va = vb;
         vb = tv;
     }
+    // (entry r by the thread that fills v0[r] for the next species)
     for (int r = blockIdx.x * blockDim.x + tid; r < nb; r += gridDim.x * blockDim.x) id[va[r]] = base + stride * (uint64_t)r;
     return true;
 }
