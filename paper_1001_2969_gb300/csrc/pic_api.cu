@@ -1534,6 +1534,18 @@ pic_status finish_call(pic_handle *h, int64_t step0, int cur0, int cur_i0, int32
     return result;
 }
 
+// device memory of the GPU in use, aligned for FP64: a kernel can read it as
+// it stands (another GPU's, which a copy takes, would need peer access)
+bool here_and_aligned(const double *p) {
+    cudaPointerAttributes a;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return a.type == cudaMemoryTypeDevice && a.device == dev && ((uintptr_t)p & 7) == 0;
+}
+
 // Finish the last pass's deferred sort (rank, births numbering, sorted
 // counts) before the particle state is read or replaced.  A failure there
 // (the numbering's grid barrier timing out) drops that pass, as in a call.
@@ -1867,7 +1879,7 @@ pic_status pic_field_solve(pic_handle *h, const double *rho, const double *chi, 
     if (!h || !rho || !chi || !phi) return fail(h, PIC_ERR_ARG, "null argument");
     const size_t gb = (size_t)h->ng * sizeof(double);
     // device arrays are read in place (by the set-up alone) when they can be
-    const bool in_place = on_device && (((uintptr_t)rho | (uintptr_t)chi) & 7) == 0;
+    const bool in_place = on_device && here_and_aligned(rho) && here_and_aligned(chi);
     if (!in_place) {
         const cudaMemcpyKind kin = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
         cudaMemcpyAsync(h->tmp_grid[0], rho, gb, kin, h->st);
