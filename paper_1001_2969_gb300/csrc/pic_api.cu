@@ -344,7 +344,7 @@ __global__ void k_iota(int32_t *p, int n) {
 
 // pic_moments in one launch: the five averages and the EEDF scaled into their
 // buffers (null: skipped), the counters and the absorbed charge to pinned host
-// memory, and (reset) all of them cleared behind it.  blockIdx.y: the array.
+// memory (null: not there), and (reset) all of them cleared behind it.  blockIdx.y: the array.
 struct MomentsOut {
     double *src[6], *dst[6];
     int ng, nb, reset;
@@ -364,10 +364,10 @@ __global__ void k_moments_out(MomentsOut m) {
     if (a == 5 && blockIdx.x == 0) {
         const int t = threadIdx.x;
         if (t < PIC_NCOUNT) {
-            m.cnt[t] = m.ds->cnt[t];
+            if (m.cnt) m.cnt[t] = m.ds->cnt[t];
             if (m.reset) m.ds->cnt[t] = 0ull;
         } else if (t >= 32 && t < 35) {
-            m.qabs[t - 32] = m.ds->qabs[t - 32];
+            if (m.qabs) m.qabs[t - 32] = m.ds->qabs[t - 32];
             if (m.reset) m.ds->qabs[t - 32] = 0.0;
         } else if (t == 64 && m.reset) {
             m.ctl->mg_cycles = 0ull;
@@ -1050,15 +1050,21 @@ void one_step(pic_handle *h, cudaStream_t sb, bool mv, int part = 0, SolveJob *j
     h->cur_i = idst;
 }
 
+// the handle's pinned block, asked for when first needed; false: there is none
+bool pin_report(pic_handle *h) {
+    if (!h->host_ctl && cudaMallocHost((void **)&h->host_ctl, sizeof(*h->host_ctl)) != cudaSuccess) {
+        h->host_ctl = nullptr;
+        cudaGetLastError();
+    }
+    return h->host_ctl != nullptr;
+}
+
 // the end of a call on stream `on`: the capacity check of the last pass's sort
 // and the report to pinned memory.  Rank, births numbering and the sorted
 // counts stay pending; the next step's graph runs them beside its solve, or
 // complete_sort() before the state is read.
 void call_tail(pic_handle *h, cudaStream_t on) {
-    if (!h->host_ctl && cudaMallocHost((void **)&h->host_ctl, sizeof(*h->host_ctl)) != cudaSuccess) {
-        h->host_ctl = nullptr;
-        cudaGetLastError();
-    }
+    pin_report(h);
     const int32_t *counts[2] = {h->sp[0].counts, h->sp[1].counts};
     const int64_t cap[2] = {h->sp[0].cap, h->sp[1].cap};
     launch_call_tail(counts, h->ncell, cap, h->ds, h->sctl, h->host_ctl, on);
@@ -1885,10 +1891,7 @@ pic_status pic_field_solve(pic_handle *h, const double *rho, const double *chi, 
         cudaMemcpyAsync(h->tmp_grid[0], rho, gb, kin, h->st);
         cudaMemcpyAsync(h->tmp_grid[1], chi, gb, kin, h->st);
     }
-    if (!h->host_ctl && cudaMallocHost((void **)&h->host_ctl, sizeof(*h->host_ctl)) != cudaSuccess) {
-        h->host_ctl = nullptr;
-        cudaGetLastError();
-    }
+    pin_report(h);
     FieldDims fd{h->nz, h->nr, h->dz, h->dr, h->cfg.mesh.L, h->cfg.chi_face};
     int L = 0;
     double res = 0.0;
@@ -1941,13 +1944,17 @@ pic_status pic_moments(pic_handle *h, pic_moments_out *out, int32_t reset) {
     mo.reset = reset ? 1 : 0;
     mo.ds = h->ds;
     mo.ctl = h->sctl;
-    if (!h->host_ctl && cudaMallocHost((void **)&h->host_ctl, sizeof(*h->host_ctl)) != cudaSuccess) {
-        h->host_ctl = nullptr;
-        cudaGetLastError();
-        return fail(h, PIC_ERR_CUDA, "moments: pinned memory");
+    // (no pinned memory to be had: the counters are copied ahead of the launch)
+    DevScalars local;
+    const bool pinned = pin_report(h);
+    if (pinned) {
+        mo.cnt = h->host_ctl->cnt;
+        mo.qabs = h->host_ctl->qabs;
+    } else {
+        cudaMemcpyAsync(&local, h->ds, sizeof(local), cudaMemcpyDeviceToHost, h->st);
     }
-    mo.cnt = h->host_ctl->cnt;
-    mo.qabs = h->host_ctl->qabs;
+    const unsigned long long *cnt = pinned ? h->host_ctl->cnt : local.cnt;
+    const double *qabs = pinned ? h->host_ctl->qabs : local.qabs;
     k_moments_out<<<dim3(std::max(1, std::min(64, (h->ng + 255) / 256)), 6), 256, 0, h->st>>>(mo);
     h->launches += 1;
     if (!out->on_device) {
@@ -1961,12 +1968,12 @@ pic_status pic_moments(pic_handle *h, pic_moments_out *out, int32_t reset) {
     const pic_status ce = cuda_check(h, "moments");
     if (ce != PIC_OK) return ce;
     if (out->counters) {
-        for (int k = 0; k < PIC_NCOUNT; ++k) out->counters[k] = (int64_t)h->host_ctl->cnt[k];
+        for (int k = 0; k < PIC_NCOUNT; ++k) out->counters[k] = (int64_t)cnt[k];
         out->counters[PIC_C_MGCYC] = h->mg_cycles_total;
         out->counters[PIC_C_STEPS] = h->steps_total;
     }
     if (out->charge)
-        for (int k = 0; k < 3; ++k) out->charge[k] = h->host_ctl->qabs[k];
+        for (int k = 0; k < 3; ++k) out->charge[k] = qabs[k];
     out->nsamples = h->nsamples;
     if (reset) {
         h->nsamples = 0;
