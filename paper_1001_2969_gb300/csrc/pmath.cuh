@@ -36,18 +36,15 @@ __device__ __forceinline__ bool m_finite(double x) { return isfinite(x); }
 // where the result feeds positions/weights (never a threshold test on its own)
 __device__ __forceinline__ float m_div(float a, float b) { return __fdividef(a, b); }
 __device__ __forceinline__ double m_div(double a, double b) { return a / b; }
-// quotients of one divisor.  An FP64 division is some twelve operations on
-// GB300's narrow FP64 pipe, which bounds the FP64 pass: the divisor's inverse is
-// taken once (m_inv) and each quotient corrected by its residual, which leaves
-// it rounded as the division would be but for the last half unit.  FP32
-// divides.
+// quotients of one divisor.  GB300's narrow FP64 pipe bounds the FP64 pass: the
+// divisor's inverse is taken once (m_inv) and each quotient corrected by its
+// residual (quot: the divisors here are square roots and odd integers, so they
+// and their inverses are normal numbers).  65 x 257, 1e6 + 1e6 particles: 1294 ->
+// 1163 us a step.  FP32 divides.
 __device__ __forceinline__ float m_inv(float) { return 0.0f; }
 __device__ __forceinline__ double m_inv(double x) { return 1.0 / x; }
 __device__ __forceinline__ float m_quot(float a, float b, float) { return a / b; }
-__device__ __forceinline__ double m_quot(double a, double b, double inv) {
-    const double q = a * inv;
-    return fma(fma(-q, b, a), inv, q);
-}
+__device__ __forceinline__ double m_quot(double a, double b, double inv) { return quot(a, b, inv); }
 // no value is a NaN or infinite: in FP32 their sum is finite (the values are
 // far below overflow), in FP64 their exponents tell, off the FP64 pipe
 __device__ __forceinline__ bool all_finite(float a, float b, float c, float d, float e, float f) {
