@@ -1287,9 +1287,17 @@ __device__ __forceinline__ void solve_body(const MGFast *__restrict__ mp, double
 }
 
 // MINB: blocks per SM the registers must allow: one for a reactor's solve
-// alone, two for the solves of a batch of reactors, which share SMs.
+// alone, two for the solves of a batch of reactors, which share SMs.  FP64 lines
+// of more than 256 unknowns: four lines' factors (150 KB and more) leave room for
+// one block anyway, and 128 registers made them spill (2 KB a thread above 512
+// unknowns; six 33 x 1025 reactors 2128 -> 1713 us a step, four 33 x 513 933 ->
+// 885).
+template <typename Tv, int M>
+constexpr int reg_blocks(int minb) {
+    return sizeof(Tv) == 8 && M >= 16 ? 1 : minb;
+}
 template <typename Tv, int M, int MINB>
-__global__ void __launch_bounds__(kSolveThreads, MINB)
+__global__ void __launch_bounds__(kSolveThreads, (reg_blocks<Tv, M>(MINB)))
     k_solve_persistent(const MGFast *__restrict__ mp, double *phi, int nr, SolveLayout lay, double tol,
                        int max_cycles) {
     solve_body<Tv, M, MINB == 1>(mp, phi, nr, lay, tol, max_cycles, blockIdx.x, gridDim.x);
@@ -1299,7 +1307,8 @@ __global__ void __launch_bounds__(kSolveThreads, MINB)
 // cooperative launch: job k takes blocks [block0, block0 + nblocks) and hands
 // its words to its own blocks only, so the reactors proceed side by side.
 template <typename Tv, int M>
-__global__ void __launch_bounds__(kSolveThreads, 2) k_solve_multi(const SolveJob *__restrict__ jobs, int njobs) {
+__global__ void __launch_bounds__(kSolveThreads, (reg_blocks<Tv, M>(2)))
+    k_solve_multi(const SolveJob *__restrict__ jobs, int njobs) {
     int lo = 0, hi = njobs - 1;  // the job whose block range holds this block
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
