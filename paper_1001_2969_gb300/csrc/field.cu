@@ -25,20 +25,18 @@
 
 namespace pic {
 
-// (V: node volumes and their inverses: no FP64 divisions per node on GB300's
-// narrow FP64 pipe)
-__global__ void k_finalize(const double *Ne, const double *Ni, const double2 *V, double q0,
+__global__ void k_finalize(const double *Ne, const double *Ni, const double2 *iV, double q0,
                            double q1, double c0, double c1, double *rho, double *chi, int ng,
                            const StepCtl *ctl) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= ng || (ctl && ctl->halt)) return;
-    node_field(Ne[k], Ni[k], V[k], q0, q1, c0, c1, rho[k], chi[k]);
+    node_field(Ne[k], Ni[k], iV[k], q0, q1, c0, c1, rho[k], chi[k]);
 }
 
-void launch_finalize(const double *Ne, const double *Ni, const double2 *V, double q0, double q1,
+void launch_finalize(const double *Ne, const double *Ni, const double2 *iV, double q0, double q1,
                      double c0, double c1, double *rho, double *chi, int ng, const StepCtl *ctl,
                      cudaStream_t st) {
-    k_finalize<<<(ng + 255) / 256, 256, 0, st>>>(Ne, Ni, V, q0, q1, c0, c1, rho, chi, ng, ctl);
+    k_finalize<<<(ng + 255) / 256, 256, 0, st>>>(Ne, Ni, iV, q0, q1, c0, c1, rho, chi, ng, ctl);
 }
 
 // ---- level set-up ----
@@ -413,30 +411,29 @@ int mg_solve(const FieldDims &fd, MGWork &mg, const double *rho, const double *c
 
 // E = -grad phi: central inside, one-sided first order on the boundary rows
 // and on r = R, E_r = 0 on the axis
-// (iz = 1/dz, ir = 1/dr, each quotient corrected: no FP64 divisions per node)
+// (iz, ir: the inverses of 2 dz and 2 dr)
 // (solved not null: one thread reports the solve before it to ctl; should
 // that halt the step, what the others still write is not read)
 template <typename T>
 __global__ void k_efield(const double *phi, double *Ez, double *Er, typename V2<T>::type *E2,
-                         int nz, int nr, double dz, double dr, double iz, double ir, StepCtl *ctl,
-                         const MGCtl *solved) {
+                         int nz, int nr, double2 iz, double2 ir, StepCtl *ctl, const MGCtl *solved) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (solved && k == 0) solve_report(solved, ctl, 0);
     if (k >= nz * nr || (ctl && ctl->halt)) return;
     const int i = k / nr, j = k % nr;
     double ez, er;
     if (i == 0)
-        ez = quot(phi[k] - phi[k + nr], dz, iz);
+        ez = quot(2.0 * (phi[k] - phi[k + nr]), iz);
     else if (i == nz - 1)
-        ez = quot(phi[k - nr] - phi[k], dz, iz);
+        ez = quot(2.0 * (phi[k - nr] - phi[k]), iz);
     else
-        ez = quot(phi[k - nr] - phi[k + nr], 2.0 * dz, 0.5 * iz);
+        ez = quot(phi[k - nr] - phi[k + nr], iz);
     if (j == 0)
         er = 0.0;
     else if (j == nr - 1)
-        er = quot(phi[k - 1] - phi[k], dr, ir);
+        er = quot(2.0 * (phi[k - 1] - phi[k]), ir);
     else
-        er = quot(phi[k - 1] - phi[k + 1], 2.0 * dr, 0.5 * ir);
+        er = quot(phi[k - 1] - phi[k + 1], ir);
     Ez[k] = ez;
     Er[k] = er;
     typename V2<T>::type e;
@@ -448,14 +445,15 @@ __global__ void k_efield(const double *phi, double *Ez, double *Er, typename V2<
 template <typename T>
 void launch_efield(const double *phi, double *Ez, double *Er, typename V2<T>::type *E2, int nz,
                    int nr, double dz, double dr, StepCtl *ctl, const MGCtl *solved, cudaStream_t st) {
-    k_efield<T><<<nblk(nz * nr), 256, 0, st>>>(phi, Ez, Er, E2, nz, nr, dz, dr, 1.0 / dz, 1.0 / dr, ctl, solved);
+    k_efield<T><<<nblk(nz * nr), 256, 0, st>>>(phi, Ez, Er, E2, nz, nr, inverse_pair(2.0 * dz),
+                                          inverse_pair(2.0 * dr), ctl, solved);
 }
 template void launch_efield<float>(const double *, double *, double *, float2 *, int, int, double,
                                    double, StepCtl *, const MGCtl *, cudaStream_t);
 template void launch_efield<double>(const double *, double *, double *, double2 *, int, int,
                                     double, double, StepCtl *, const MGCtl *, cudaStream_t);
 
-__global__ void k_moments(const double *Ne, const double *Ni, const double2 *V, const double *phi,
+__global__ void k_moments(const double *Ne, const double *Ni, const double2 *iV, const double *phi,
                           const double *Ez, const double *Er, double *m_ne, double *m_ni,
                           double *m_phi, double *m_ez, double *m_er, int ng, StepCtl *c, StepEnd e) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
@@ -477,18 +475,19 @@ __global__ void k_moments(const double *Ne, const double *Ni, const double2 *V, 
         }
     }
     if (k >= ng || c->halt) return;
-    const double2 v = V[k];
-    m_ne[k] += quot(Ne[k], v.x, v.y);
-    m_ni[k] += quot(Ni[k], v.x, v.y);
+    // (one fused operation: the inverse's half unit stands for the quotient's)
+    const double v = iV[k].x;
+    m_ne[k] = fma(Ne[k], v, m_ne[k]);
+    m_ni[k] = fma(Ni[k], v, m_ni[k]);
     m_phi[k] += phi[k];
     m_ez[k] += Ez[k];
     m_er[k] += Er[k];
 }
 
-void launch_moments(const double *Ne, const double *Ni, const double2 *V, const double *phi, const double *Ez,
+void launch_moments(const double *Ne, const double *Ni, const double2 *iV, const double *phi, const double *Ez,
                     const double *Er, double *m_ne, double *m_ni, double *m_phi, double *m_ez,
                     double *m_er, int ng, StepCtl *ctl, const StepEnd &e, cudaStream_t st) {
-    k_moments<<<nblk(ng), 256, 0, st>>>(Ne, Ni, V, phi, Ez, Er, m_ne, m_ni, m_phi, m_ez, m_er, ng, ctl, e);
+    k_moments<<<nblk(ng), 256, 0, st>>>(Ne, Ni, iV, phi, Ez, Er, m_ne, m_ni, m_phi, m_ez, m_er, ng, ctl, e);
 }
 
 }  // namespace pic

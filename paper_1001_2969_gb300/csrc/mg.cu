@@ -58,7 +58,7 @@ __global__ void __launch_bounds__(256) k_setup_levels(const MGFast *__restrict__
         double x;
         if (f.Ne) {
             double rho;
-            node_field(f.Ne[k], f.Ni[k], f.V[k], f.q0, f.q1, f.c0, f.c1, rho, x);
+            node_field(f.Ne[k], f.Ni[k], f.iV[k], f.q0, f.q1, f.c0, f.c1, rho, x);
             f.rho[k] = rho;
             f.chi[k] = x;
         } else {

@@ -83,11 +83,11 @@ struct MGFast {
 };
 
 // Where a solve's charge and susceptibility come from: computed by the set-up
-// from the species' deposits (Ne and Ni over the node volumes V, which come with
-// their inverses; rho and chi are then written), or given (Ne null).
+// from the species' deposits (Ne, Ni) and the node volumes' inverses (rho and chi
+// are then written), or given (Ne null).
 struct FieldSource {
     const double *Ne, *Ni;
-    const double2 *V;
+    const double2 *iV;
     double q0, q1, c0, c1;
     double *rho, *chi;
 };

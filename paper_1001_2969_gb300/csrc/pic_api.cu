@@ -89,7 +89,7 @@ struct pic_handle {
     int K = 1;      // ion subcycling: the ions move every K-th pass
     double *N[2] = {nullptr, nullptr};
     double *rho = nullptr, *chi = nullptr, *phi = nullptr, *Ez = nullptr, *Er = nullptr, *V = nullptr;
-    double2 *V2 = nullptr;  // node volumes and their inverses
+    double2 *iV = nullptr;  // node volumes' inverses
     void *E2 = nullptr;
     double *inv_t = nullptr;  // 1 / (2j + 1) per radial cell (FP64 path)
     double *phiL_d = nullptr;
@@ -328,10 +328,9 @@ void node_volumes(const pic_handle *h, std::vector<double> &V) {
     }
 }
 
-// {x, 1/x}
 __global__ void k_inverse(const double *x, double2 *y, int n) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k < n) y[k] = make_double2(x[k], 1.0 / x[k]);
+    if (k < n) y[k] = inverse_pair(x[k]);
 }
 
 __global__ void k_inverse_odd(double *y, int n) {
@@ -600,7 +599,7 @@ void setup_device(pic_handle *h) {
     h->Ez = (double *)dalloc(h, gb);
     h->Er = (double *)dalloc(h, gb);
     h->V = (double *)dalloc(h, gb);
-    h->V2 = (double2 *)dalloc(h, 2 * gb);
+    h->iV = (double2 *)dalloc(h, 2 * gb);
     for (int k = 0; k < 3; ++k) h->tmp_grid[k] = (double *)dalloc(h, gb);
     for (int k = 0; k < 5; ++k) h->m_acc[k] = (double *)dalloc(h, gb);
     h->E2 = dalloc(h, (size_t)h->ng * 2 * ts);
@@ -629,7 +628,7 @@ void setup_device(pic_handle *h) {
     std::vector<double> V;
     node_volumes(h, V);
     cudaMemcpyAsync(h->V, V.data(), gb, cudaMemcpyHostToDevice, h->st);
-    k_inverse<<<(h->ng + 255) / 256, 256, 0, h->st>>>(h->V, h->V2, h->ng);
+    k_inverse<<<(h->ng + 255) / 256, 256, 0, h->st>>>(h->V, h->iV, h->ng);
     if (!h->mixed) {
         h->inv_t = (double *)dalloc(h, (size_t)h->ncr * sizeof(double));
         k_inverse_odd<<<(h->ncr + 255) / 256, 256, 0, h->st>>>(h->inv_t, h->ncr);
@@ -937,7 +936,7 @@ void one_step(pic_handle *h, cudaStream_t sb, bool mv, int part = 0, SolveJob *j
     cudaEvent_t fork = sb ? h->ev_fork : nullptr;
     {
         PhaseTimer t(h, 0);
-        const FieldSource field{h->N[0], h->N[1], h->V2, h->cfg.sp[0].q, h->cfg.sp[1].q, chi_coef(h, 0, true),
+        const FieldSource field{h->N[0], h->N[1], h->iV, h->cfg.sp[0].q, h->cfg.sp[1].q, chi_coef(h, 0, true),
                               chi_coef(h, 1, mv), h->rho, h->chi};
         FieldDims fd{h->nz, h->nr, h->dz, h->dr, h->cfg.mesh.L, h->cfg.chi_face};
         int L = 0;
@@ -1044,7 +1043,7 @@ void one_step(pic_handle *h, cudaStream_t sb, bool mv, int part = 0, SolveJob *j
         PhaseTimer t(h, 4);
         const StepEnd e{h->ds, h->sp[0].d_nmain[dst], mv ? h->sp[1].d_nmain[idst] : nullptr, h->sp[0].d_nalive,
                         mv ? h->sp[1].d_nalive : nullptr};
-        launch_moments(h->N[0], h->N[1], h->V2, h->phi, h->Ez, h->Er, h->m_acc[0], h->m_acc[1],
+        launch_moments(h->N[0], h->N[1], h->iV, h->phi, h->Ez, h->Er, h->m_acc[0], h->m_acc[1],
                        h->m_acc[2], h->m_acc[3], h->m_acc[4], h->ng, h->sctl, e, st);
         h->launches += 1;
     }
@@ -1425,7 +1424,7 @@ pic_status window_t(pic_handle *h, int32_t nsteps, int32_t ckpt, const double *w
         in.perm[s] = d.perm;
         fill_step_args<T>(h, in.args[s], s, cur, 1 - cur, 1 - cur);
     }
-    in.V = h->V2;
+    in.iV = h->iV;
     in.phi0 = h->phi;
     in.mgf = &h->mgf;
     in.tol = h->cfg.mg_tol;
@@ -2078,7 +2077,7 @@ pic_status pic_get_fields(pic_handle *h, double *rho, double *chi, double *phi, 
                           double *Er, int32_t on_device) {
     if (!h) return PIC_ERR_ARG;
     // rho and chi as the next step's solve takes them
-    launch_finalize(h->N[0], h->N[1], h->V2, h->cfg.sp[0].q, h->cfg.sp[1].q, chi_coef(h, 0, true),
+    launch_finalize(h->N[0], h->N[1], h->iV, h->cfg.sp[0].q, h->cfg.sp[1].q, chi_coef(h, 0, true),
                     chi_coef(h, 1, moves_ions(h, h->step)), h->rho, h->chi, h->ng, nullptr, h->st);
     h->launches += 1;
     const size_t gb = (size_t)h->ng * sizeof(double);

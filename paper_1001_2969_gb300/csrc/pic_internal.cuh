@@ -3,6 +3,7 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stdint.h>
 
 #include "pic.h"
@@ -423,28 +424,27 @@ struct FieldDims {
     double dz, dr, L;
     int chi_face;
 };
-// a / b by the inverse of b (correctly rounded, taken once for many quotients)
-// and one residual correction, after Markstein (IBM J. Res. Dev. 34, 1990): the
-// product a inv is off by at most 1.5 units in the last place, the residual
-// a - q b is a single fused operation, and the corrected quotient is the
-// division's but for cases within ~2^-51 units of a rounding tie.  For b, 1/b,
-// a and a/b in the normal range and |a| > 2^-960 (or zero); an infinite a
-// gives a NaN.
-__device__ __forceinline__ double quot(double a, double b, double inv) {
-    const double q = a * inv;
-    return fma(fma(-q, b, a), inv, q);
+// a / b where b's inverse w is known to twice the precision (inverse_pair): two
+// operations of GB300's narrow FP64 pipe instead of a division.  The tail a w.y
+// is below half a unit of a w.x, so the result is the division's but for cases
+// within ~2^-52 units of a rounding tie (b, 1/b, a and a/b in the normal range;
+// an infinite a gives a NaN).
+__host__ __device__ inline double2 inverse_pair(double b) {
+    const double x = 1.0 / b;
+    return {x, fma(-b, x, 1.0) * x};
 }
+__device__ __forceinline__ double quot(double a, double2 w) { return fma(a, w.x, a * w.y); }
 
 // rho = sum q_s n_s and chi = dt^2/(2 eps0) sum_s q_s^2 n_s / m_s of a node
-// (n_s = N_s / V, v = {V, 1/V}, c_s = q_s^2 dt^2 / (2 eps0 m_s))
-__device__ __forceinline__ void node_field(double Ne, double Ni, double2 v, double q0, double q1, double c0, double c1,
+// (n_s = N_s / V, iV: V's inverse, c_s = q_s^2 dt^2 / (2 eps0 m_s))
+__device__ __forceinline__ void node_field(double Ne, double Ni, double2 iV, double q0, double q1, double c0, double c1,
                                            double &rho, double &chi) {
-    const double ne = quot(Ne, v.x, v.y), ni = quot(Ni, v.x, v.y);
+    const double ne = quot(Ne, iV), ni = quot(Ni, iV);
     rho = q0 * ne + q1 * ni;
     chi = c0 * ne + c1 * ni;
 }
-// V: the node volumes and their inverses; ctl (may be null): skip when the step has halted
-void launch_finalize(const double *Ne, const double *Ni, const double2 *V, double q0, double q1,
+// iV: the node volumes' inverses; ctl (may be null): skip when the step has halted
+void launch_finalize(const double *Ne, const double *Ni, const double2 *iV, double q0, double q1,
                      double chi0, double chi1, double *rho, double *chi, int ng, const StepCtl *ctl,
                      cudaStream_t st);
 // multigrid solve into phi (device); returns cycles, residual and the launch count
@@ -465,7 +465,7 @@ struct StepEnd {
     int32_t *nmain0, *nmain1;
     const int32_t *nalive0, *nalive1;
 };
-void launch_moments(const double *Ne, const double *Ni, const double2 *V, const double *phi,
+void launch_moments(const double *Ne, const double *Ni, const double2 *iV, const double *phi,
                     const double *Ez, const double *Er, double *m_ne, double *m_ni,
                     double *m_phi, double *m_ez, double *m_er, int ng, StepCtl *ctl, const StepEnd &e,
                     cudaStream_t st);

@@ -38,13 +38,19 @@ __device__ __forceinline__ float m_div(float a, float b) { return __fdividef(a, 
 __device__ __forceinline__ double m_div(double a, double b) { return a / b; }
 // quotients of one divisor.  GB300's narrow FP64 pipe bounds the FP64 pass: the
 // divisor's inverse is taken once (m_inv) and each quotient corrected by its
-// residual (quot: the divisors here are square roots and odd integers, so they
-// and their inverses are normal numbers).  65 x 257, 1e6 + 1e6 particles: 1294 ->
-// 1163 us a step.  FP32 divides.
+// residual (after Markstein, IBM J. Res. Dev. 34, 1990): the product is off by at
+// most 1.5 units in the last place, the residual is one fused operation, and the
+// corrected quotient is the division's but for cases within ~2^-51 units of a
+// rounding tie.  For a divisor, an inverse and quotients in the normal range and
+// a numerator that is zero or above 2^-960; the divisors here are square roots and odd integers.
+// 65 x 257, 1e6 + 1e6 particles: 1294 -> 1163 us a step.  FP32 divides.
 __device__ __forceinline__ float m_inv(float) { return 0.0f; }
 __device__ __forceinline__ double m_inv(double x) { return 1.0 / x; }
 __device__ __forceinline__ float m_quot(float a, float b, float) { return a / b; }
-__device__ __forceinline__ double m_quot(double a, double b, double inv) { return quot(a, b, inv); }
+__device__ __forceinline__ double m_quot(double a, double b, double inv) {
+    const double q = a * inv;
+    return fma(fma(-q, b, a), inv, q);
+}
 // no value is a NaN or infinite: in FP32 their sum is finite (the values are
 // far below overflow), in FP64 their exponents tell, off the FP64 pipe
 __device__ __forceinline__ bool all_finite(float a, float b, float c, float d, float e, float f) {

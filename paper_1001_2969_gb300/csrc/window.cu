@@ -329,21 +329,21 @@ __global__ void k_win_back(StepArgs<T> a, WinState<T> prev, WinState<T> cur, int
 }
 
 // adjoint of E = -grad phi (the stencils of k_efield) onto phi_bar
-__global__ void k_efield_adj(const double *Ebz, const double *Ebr, double *phib, int nz, int nr, double dz,
-                             double dr, double iz, double ir) {
+__global__ void k_efield_adj(const double *Ebz, const double *Ebr, double *phib, int nz, int nr, double2 iz,
+                             double2 ir) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= nz * nr) return;
     const int i = k / nr, j = k % nr;
     const double ez = Ebz[k], er = Ebr[k];
     if (ez != 0.0) {
         const bool end = i == 0 || i == nz - 1;
-        const double e = end ? quot(ez, dz, iz) : quot(ez, 2.0 * dz, 0.5 * iz);
+        const double e = quot(end ? 2.0 * ez : ez, iz);
         atomicAdd(phib + (i == nz - 1 ? k : k + nr), -e);
         atomicAdd(phib + (i == 0 ? k : k - nr), e);
     }
     if (er != 0.0 && j > 0) {
         const bool end = j == nr - 1;
-        const double e = end ? quot(er, dr, ir) : quot(er, 2.0 * dr, 0.5 * ir);
+        const double e = quot(end ? 2.0 * er : er, ir);
         atomicAdd(phib + (end ? k : k + 1), -e);
         atomicAdd(phib + k - 1, e);
     }
@@ -390,7 +390,7 @@ __global__ void k_face_adj(const double *lam, const double *phi, const double *c
 // per node: rho_bar, N_bar of both species (plus the functional's own term
 // for the ions), and the Dirichlet rows' adjoints -> parameter gradients
 __global__ void k_node_adj(const double *lam, const double *chi, const double *phib, const double *chib,
-                           const double2 *V, const double *w, double *Nb0, double *Nb1, int nz, int nr,
+                           const double2 *iV, const double *w, double *Nb0, double *Nb1, int nz, int nr,
                            double dz, double dr, int face_mean, double q0, double q1, double c0, double c1,
                            double jscale, double sin_t, double *Ab, double *phizLb) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
@@ -399,9 +399,8 @@ __global__ void k_node_adj(const double *lam, const double *chi, const double *p
     const bool inner = i > 0 && i < nz - 1 && j < nr - 1;
     const double rhob = inner ? lam[k] * area_z(j, dr) * dz / kEps0 : 0.0;
     const double cb = chib[k];
-    const double2 v = V[k];
-    Nb0[k] = quot(q0 * rhob + c0 * cb, v.x, v.y);
-    Nb1[k] = quot(q1 * rhob + c1 * cb, v.x, v.y) + jscale * w[k];
+    Nb0[k] = quot(q0 * rhob + c0 * cb, iV[k]);
+    Nb1[k] = quot(q1 * rhob + c1 * cb, iV[k]) + jscale * w[k];
     auto face = [&](int lo, int hi) {
         return face_mean ? 0.5 * (chi[lo] + chi[hi]) : fmax(chi[lo], chi[hi]);
     };
@@ -512,11 +511,11 @@ int window_run(const WindowIn<T> &in, int K, int ckpt, const double *w_host, dou
         auto fwd = [&](int n, const WinState<T> *Sin, const WinState<T> *Sout, double **Nin, double **Nout,
                        bool again) {
             if (again) {
-                launch_finalize(Nin[0], Nin[1], in.V, in.q[0], in.q[1], c_chi[0], c_chi[1], rho, chi, ng, nullptr, st);
+                launch_finalize(Nin[0], Nin[1], in.iV, in.q[0], in.q[1], c_chi[0], c_chi[1], rho, chi, ng, nullptr, st);
                 cudaMemcpyAsync(phi, phi_all[n], (size_t)ng * sizeof(double), cudaMemcpyDeviceToDevice, st);
             } else {
                 const double t = (double)(in.step0 + n) * in.dt;
-                const FieldSource src{Nin[0], Nin[1], in.V, in.q[0], in.q[1], c_chi[0], c_chi[1], rho, chi};
+                const FieldSource src{Nin[0], Nin[1], in.iV, in.q[0], in.q[1], c_chi[0], c_chi[1], rho, chi};
                 if (mg_fast_solve(fd, *in.mgf, src, voltage(t), pzl, phi, true, in.mixed, in.tol,
                                   in.max_cycles, nullptr, &L, wctl, st, false, true) == kSolveNoLaunch)
                     throw 1;
@@ -602,8 +601,8 @@ int window_run(const WindowIn<T> &in, int K, int ckpt, const double *w_host, dou
                     }
                     pb = 1 - pb;
                     cudaMemsetAsync(phib, 0, (size_t)ng * sizeof(double), st);
-                    k_efield_adj<<<blocks(ng), kWT, 0, st>>>(Ebz, Ebr, phib, nz, nr, in.dz, in.dr, 1.0 / in.dz,
-                                                            1.0 / in.dr);
+                    k_efield_adj<<<blocks(ng), kWT, 0, st>>>(Ebz, Ebr, phib, nz, nr, inverse_pair(2.0 * in.dz),
+                                                            inverse_pair(2.0 * in.dr));
                     k_adj_rhs<<<blocks(ng), kWT, 0, st>>>(phib, rhof, nz, nr, in.dz, in.dr);
                     // warm start from the previous step's lambda (zero at first):
                     // consecutive adjoint fields are close
@@ -616,7 +615,7 @@ int window_run(const WindowIn<T> &in, int K, int ckpt, const double *w_host, dou
                         lam, phi_all[n], chis[q - 1], chib, nz, nr, in.mgf->gz[0], in.mgf->gr[0], in.chi_face == PIC_CHI_MEAN);
                     const double t = (double)(in.step0 + n) * in.dt;
                     const double sin_t = std::sin(2.0 * kPi * in.rf_freq[0] * t + in.rf_phase[0]);
-                    k_node_adj<<<blocks(ng), kWT, 0, st>>>(lam, chis[q - 1], phib, chib, in.V, w_d, Nb[0], Nb[1], nz,
+                    k_node_adj<<<blocks(ng), kWT, 0, st>>>(lam, chis[q - 1], phib, chib, in.iV, w_d, Nb[0], Nb[1], nz,
                                                           nr, in.dz, in.dr, in.chi_face == PIC_CHI_MEAN, in.q[0],
                                                           in.q[1], c_chi[0], c_chi[1], n > 1 ? 1.0 / K : 0.0, sin_t,
                                                           acc + 1, acc + 2);

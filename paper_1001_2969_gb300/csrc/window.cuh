@@ -34,7 +34,7 @@ struct WindowIn {
     const int32_t *perm[2];   // the sorted store's permutation
     int nmain[2];
     StepArgs<T> args[2];      // the production pass's constants per species
-    const double2 *V;         // node volumes and their inverses
+    const double2 *iV;        // node volumes' inverses
     const double *phi0;       // the first solve's start
     MGFast *mgf;
     double tol;
