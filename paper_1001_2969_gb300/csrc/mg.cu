@@ -124,20 +124,25 @@ __device__ __forceinline__ double recip(double x) {
 //   (5 arrays of M), then loI, upI (interface couplings), the five PCR
 //   steps' alpha and gamma, and 1/diagonal of the reduced system.
 //
-// FP64 lines of up to 512 unknowns take 128 lanes (four warps) instead: a warp's
+// FP64 lines of 65 to 512 unknowns take 128 lanes (four warps) instead: a warp's
 // FP64 instruction occupies its SM partition's pipe for ~60 cycles, so one warp
 // per line left three of the four pipes idle (7700 cycles a line at M = 16).
 // The chunks are a quarter as long, the interface system has seven reduction
 // steps, and lanes exchange through shared memory.  Longer lines' factors
-// would not fit shared memory that way.
+// would not fit shared memory that way; shorter ones have under two unknowns a
+// lane, gain nothing, and their factors take four times the space, so that
+// tall meshes reload them every cycle (whole solves, 32 / 128 lanes: 1025 x 65
+// 682 / 818 us, 33 x 65 202 / 224; 65 x 129 310 / 291).
 constexpr int kLine = 32;  // lanes per line
+
+constexpr bool grouped(int M, bool f64) { return f64 && M >= 4 && M <= 16; }
 
 // how a line of up to 32 M unknowns is laid out
 template <typename Ts, int M>
 struct Shape {
-    static constexpr bool group = sizeof(Ts) == 8 && M <= 16;
+    static constexpr bool group = grouped(M, sizeof(Ts) == 8);
     static constexpr int lanes = group ? 128 : kLine;
-    static constexpr int chunk = group ? (M > 4 ? M / 4 : 1) : M;
+    static constexpr int chunk = group ? M / 4 : M;
     static constexpr int steps = group ? 7 : 5;
     static constexpr int row = lanes + 1;          // a line buffer's row of one unknown of every chunk, padded
     static constexpr int unknowns = lanes * chunk;  // with padding
@@ -146,11 +151,11 @@ struct Shape {
     static __device__ __forceinline__ int at(int j) { return (j % chunk) * row + j / chunk; }
 };
 int line_elems(int M, bool f64) {
-    if (!f64 || M > 16) return 5 * M * kLine + 13 * kLine;
-    return 5 * (M > 4 ? M / 4 : 1) * 128 + 17 * 128;
+    if (!grouped(M, f64)) return 5 * M * kLine + 13 * kLine;
+    return 5 * (M / 4) * 128 + 17 * 128;
 }
 int line_buffer(int M, bool f64) {
-    return f64 && M <= 16 ? (M > 4 ? M / 4 : 1) * 129 : M * 33;
+    return grouped(M, f64) ? (M / 4) * 129 : M * 33;
 }
 
 // chunk per lane: the least power of two M with 32 M >= n

@@ -121,7 +121,7 @@ struct SolveJob {
 };
 
 // line-factor elements of one r-line of a mesh with nr nodes per row
-// (in FP64 up to 512 unknowns are solved by more lanes: f64)
+// (in FP64 65 to 512 unknowns are solved by more lanes: f64)
 size_t mg_line_factor_elems(int nr, bool f64);
 // doubles of each tile-wise array (kr, kw, kzp, kwp; ps has the neighbour columns), and the most blocks
 // a solve takes (entries of xr and xd)
