@@ -158,6 +158,16 @@ int line_buffer(int M, bool f64) {
     return grouped(M, f64) ? (M / 4) * 129 : M * 33;
 }
 
+// FP64 lines of more than 128 unknowns: four lines' factors (110 KB and more)
+// leave an SM room for one block, however few registers it takes.  A batch's
+// solves of such lines have an SM per block too, then: all its registers (128
+// made them spill, 2 KB a thread above 512 unknowns), up to as many blocks as a
+// reactor alone, and wider residual tiles the fewer they get (fit_tiles).
+// Steps of batches, against 128 registers, a block per two rows and tiles of 4
+// columns: six 33 x 1025 reactors 2130 -> 1375 us, forty 17 x 700 4340 -> 2360,
+// sixteen 33 x 513 1620 -> 1260, forty 33 x 257 2510 -> 2020.
+constexpr bool one_block(int M, bool f64) { return f64 && M >= 8; }
+
 // chunk per lane: the least power of two M with 32 M >= n
 inline int line_chunk(int n) {
     int M = 1;
@@ -1292,17 +1302,10 @@ __device__ __forceinline__ void solve_body(const MGFast *__restrict__ mp, double
 }
 
 // MINB: blocks per SM the registers must allow: one for a reactor's solve
-// alone, two for the solves of a batch of reactors, which share SMs.  FP64 lines
-// of more than 256 unknowns: four lines' factors (150 KB and more) leave room for
-// one block anyway, and 128 registers made them spill (2 KB a thread above 512
-// unknowns; six 33 x 1025 reactors 2128 -> 1713 us a step, four 33 x 513 933 ->
-// 885).
-template <typename Tv, int M>
-constexpr int reg_blocks(int minb) {
-    return sizeof(Tv) == 8 && M >= 16 ? 1 : minb;
-}
+// alone, two for the solves of a batch of reactors, which share SMs (one where
+// one_block says so).
 template <typename Tv, int M, int MINB>
-__global__ void __launch_bounds__(kSolveThreads, (reg_blocks<Tv, M>(MINB)))
+__global__ void __launch_bounds__(kSolveThreads, one_block(M, sizeof(Tv) == 8) ? 1 : MINB)
     k_solve_persistent(const MGFast *__restrict__ mp, double *phi, int nr, SolveLayout lay, double tol,
                        int max_cycles) {
     solve_body<Tv, M, MINB == 1>(mp, phi, nr, lay, tol, max_cycles, blockIdx.x, gridDim.x);
@@ -1312,7 +1315,7 @@ __global__ void __launch_bounds__(kSolveThreads, (reg_blocks<Tv, M>(MINB)))
 // cooperative launch: job k takes blocks [block0, block0 + nblocks) and hands
 // its words to its own blocks only, so the reactors proceed side by side.
 template <typename Tv, int M>
-__global__ void __launch_bounds__(kSolveThreads, (reg_blocks<Tv, M>(2)))
+__global__ void __launch_bounds__(kSolveThreads, one_block(M, sizeof(Tv) == 8) ? 1 : 2)
     k_solve_multi(const SolveJob *__restrict__ jobs, int njobs) {
     int lo = 0, hi = njobs - 1;  // the job whose block range holds this block
     while (lo < hi) {
@@ -1332,9 +1335,11 @@ __global__ void __launch_bounds__(kSolveThreads, (reg_blocks<Tv, M>(2)))
 
 size_t mg_line_factor_elems(int nr, bool f64) { return (size_t)line_elems(line_chunk(nr - 1), f64); }
 
-// tiles of one to eight columns, the last one whole, with two neighbour columns each
+// tiles of one to eight columns (FP64: to kWideTile), the last one whole, FP64
+// with two neighbour columns each
+constexpr int kWideTile = 32;
 size_t mg_tile_elems(int nz, int nr, bool with_neighbours) {
-    return (size_t)nz * (nr + 8) * (with_neighbours ? 3 : 1);
+    return with_neighbours ? (size_t)nz * (nr + kWideTile) * 3 : (size_t)nz * (nr + 8);
 }
 
 int mg_line_chunk(int nr) { return line_chunk(nr - 1); }
@@ -1429,6 +1434,19 @@ void mg_fast_upload(MGFast &m, cudaStream_t st) {
     cudaStreamSynchronize(st);
 }
 
+size_t tile_bytes(int tw, int nz) { return ((size_t)(tw + 2) * nz * sizeof(double) + 127) & ~(size_t)127; }
+
+// Residual tiles for the job's number of blocks, no wider than the layout has
+// room for: the widest, but for those that would leave a block without one.  A
+// tile of a short mesh fills half a block's threads at 4 columns and costs a
+// fixed chain of trips to L2.
+void fit_tiles(SolveJob &j) {
+    if (!j.lay.tw_max) return;
+    j.lay.tw = j.lay.tw_max;
+    while (j.lay.tw > 4 && (j.nr - 1 + j.lay.tw / 2 - 1) / (j.lay.tw / 2) <= j.nblocks) j.lay.tw /= 2;
+    j.lay.offT = (int)tile_bytes(j.lay.tw, j.nz);
+}
+
 // The launch shape of one reactor's one-launch solve (shared-memory layout,
 // blocks, kernel); false when it cannot be launched.
 bool solve_job(const FieldDims &fd, MGFast &m, double *phi, bool mixed, double tol, int max_cycles, bool wide,
@@ -1449,7 +1467,7 @@ bool solve_job(const FieldDims &fd, MGFast &m, double *phi, bool mixed, double t
         off += (b + 127) & ~(size_t)127;
         return (int)o;
     };
-    int grid = 1;
+    int grid = 1, most = 1;
     const int minb = wide ? 1 : 2;
     if (L == 0) {
         take((size_t)line_buffer(M, true) * sizeof(double));
@@ -1457,26 +1475,29 @@ bool solve_job(const FieldDims &fd, MGFast &m, double *phi, bool mixed, double t
         lay.tw = 4;
     } else {
         // residual tiles of 4 columns (a 32-byte sector of flagged words per
-        // row) while there are as many SMs, and on the FP64 path, whose factor
-        // lines leave no room for more; else 8
-        lay.tw = mixed && (!wide || n > 4 * nsm) ? 8 : 4;
+        // row) while there are as many SMs, and on the FP64 path alone, whose
+        // factor lines leave no room for more; else 8, or what fit_tiles takes
+        const bool one = one_block(M, !mixed), fit = one && !wide;
+        lay.tw = fit ? kWideTile : mixed && (!wide || n > 4 * nsm) ? 8 : 4;
         // the line buffers of the line phases share their space with the residual phase's tile (with its two neighbour columns) and
         // restriction buffers (very tall meshes: narrower tiles)
         const size_t line = (size_t)3 * line_buffer(M, !mixed) * es;
         const size_t fac = LFE * es + (size_t)3 * LFE * es + 512;
         size_t tile = 0, both = 0;
         for (;; lay.tw /= 2) {
-            tile = ((size_t)(lay.tw + 2) * nz * sizeof(double) + 127) & ~(size_t)127;
+            tile = tile_bytes(lay.tw, nz);
             both = std::max(line, tile + (size_t)lay.tw * (2 * nz + kMaxLevels) * es);
             // (FP64: room for the static exchange buffers too)
             if (lay.tw == 1 || both + fac + (mixed ? 0 : 8192) <= kSolveSmemLimit) break;
         }
         lay.offT = (int)tile;
+        if (fit && lay.tw > 4) lay.tw_max = lay.tw;
         take(both);
         lay.offC = take(LFE * es);
         // a block per tile and per unit of the line phases
-        const int units = (2 << L) - 2 - L, ntile = (n + lay.tw - 1) / lay.tw;
-        grid = wide ? std::min(nsm, std::max(units, ntile)) : std::max(1, (nz - 1) / 2);
+        const int units = (2 << L) - 2 - L, tw = std::min(lay.tw, fit ? 4 : 8), ntile = (n + tw - 1) / tw;
+        most = std::min(nsm, std::max(units, ntile));
+        grid = wide ? most : std::max(1, (nz - 1) / 2);
         // factor slots: all of a block's units, as far as they fit (a batch's
         // blocks: two to an SM)
         const size_t room = wide ? kSolveSmemLimit : kSolveSmemLimit / 2;
@@ -1493,17 +1514,20 @@ bool solve_job(const FieldDims &fd, MGFast &m, double *phi, bool mixed, double t
     grid = std::min(std::min(grid, nsm * per_sm), kMaxSolveBlocks);
     job.mp = m.self;
     job.phi = phi;
+    job.nz = nz;
     job.nr = nr;
     job.lay = lay;
     job.tol = tol;
     job.max_cycles = max_cycles;
     job.block0 = 0;
     job.nblocks = grid;
+    job.most = lay.tw_max ? std::max(most, grid) : grid;
     job.M = M;
     job.mixed = mixed ? 1 : 0;
     job.minb = minb;
     job.smem = sp;
     job.fn = fn;
+    fit_tiles(job);
     return true;
 }
 
@@ -1688,10 +1712,10 @@ std::vector<std::pair<int, int>> mg_multi_plan(std::vector<SolveJob> &jobs, bool
             const size_t e = std::min(k.b, a + (size_t)cap);
             int want = 0;
             for (size_t j = a; j < e; ++j) want += jobs[j].nblocks;
-            const double scale = want > cap ? (double)cap / want : 1.0;
+            const double scale = (double)cap / want;
             int used = 0;
             for (size_t j = a; j < e; ++j) {
-                jobs[j].nblocks = std::max(1, (int)(jobs[j].nblocks * scale));
+                jobs[j].nblocks = std::max(1, std::min(jobs[j].most, (int)(jobs[j].nblocks * scale)));
                 used += jobs[j].nblocks;
             }
             while (used > cap) {  // the one-block floors overshot: trim the largest
@@ -1704,6 +1728,7 @@ std::vector<std::pair<int, int>> mg_multi_plan(std::vector<SolveJob> &jobs, bool
             }
             used = 0;
             for (size_t j = a; j < e; ++j) {
+                fit_tiles(jobs[j]);
                 jobs[j].block0 = used;
                 jobs[j].fn = k.fn;
                 jobs[j].smem = k.smem;

@@ -100,6 +100,7 @@ struct SolveLayout {
     int offC;   // factors of the coarsest row
     int slots;  // factor slots
     int tw;     // columns per residual tile
+    int tw_max; // the most there is room for (0: tw stands)
 };
 constexpr int kMaxSlots = 4;
 
@@ -109,11 +110,12 @@ constexpr int kMaxSlots = 4;
 struct SolveJob {
     const MGFast *mp;
     double *phi;
-    int nr;
+    int nz, nr;
     SolveLayout lay;
     double tol;
     int max_cycles;
     int block0, nblocks;  // this job's blocks in the launch
+    int most;             // what it can use of a GPU with room to spare
     // host side
     int M, mixed, minb;
     size_t smem;

@@ -19,15 +19,28 @@ def reactor(mesh, prec, seed):
                              mg_tol=1e-11, mg_max_cycles=100, seed=seed), 4000)
 
 
+# few FP64 reactors of long lines, which take what the GPU has to spare, and many, with a block
+# or two each and the widest tiles
+LONG = [[(33, 1025)], [(9, 130), (17, 300)], [(129, 200)] * 2, [(65, 514)] * 3, [(9, 700)] * 90, [(257, 257)] * 6]
+
+
+@pytest.mark.parametrize("meshes", LONG, ids=lambda m: "%dx%d of %d" % (*m[0], len(m)))
+def test_batched_solves_of_long_fp64_lines(meshes):
+    check([reactor(m, "fp64", 10 + k) for k, m in enumerate(meshes)], "fp64")
+
+
 @pytest.mark.parametrize("prec", ["fp64", "mixed"])
 @pytest.mark.parametrize("copies", [1, 4])
 def test_batched_solves_of_many_shapes(prec, copies):
+    check([reactor(m, prec, 10 + c) for c in range(copies) for m in MESHES], prec)
+
+
+def check(cfgs, prec):
     torch = pytest.importorskip("torch")
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
     from paper_1001_2969_gb300 import pic
 
-    cfgs = [reactor(m, prec, 10 + c) for c in range(copies) for m in MESHES]
     hs = [pic.pic_init(c) for c in cfgs]
     b = pic.pic_batch_init(hs)
     for step in (1, 1):  # the second reads what the first left in the flagged words
