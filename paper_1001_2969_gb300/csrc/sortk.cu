@@ -664,11 +664,15 @@ void launch_birth_finish(const BirthJob &b, const PassReset *r, cudaStream_t st,
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_birth_finish, kRadixThreads, 0);
         grid = std::max(1, std::min(nsm, nsm * per));
     }
-    // no more blocks than tiles of the largest batch of births (a small
-    // reactor's numbering does not hold the whole GPU)
+    // no more blocks than tiles of the largest batch of births or 4096 nodes to
+    // clear each (a small reactor's numbering does not hold the whole GPU; with the
+    // births alone deciding, a capacity of 2048 had one block clear 257 x 1025
+    // nodes: 751 us a step against 633)
     // (max_grid: a reactor of a batch, whose numbering must not wait for
     // many co-resident blocks while the other reactors' kernels hold SMs)
-    const int g = std::max(1, std::min(std::min(grid, max_grid), (b.tmp.max_n + kRadixTile - 1) / kRadixTile));
+    const int clear = r ? (std::max(r->ng, r->ncell) + 4095) / 4096 : 1;
+    const int want = std::max((b.tmp.max_n + kRadixTile - 1) / kRadixTile, clear);
+    const int g = std::max(1, std::min(std::min(grid, max_grid), want));
     BirthJob job = b;
     PassReset rs = r ? *r : PassReset{};
     int reset = r ? 1 : 0;
