@@ -748,6 +748,7 @@ __device__ __forceinline__ void solve_body(const MGFast *__restrict__ mp, double
     }
     const MGFast &m = s_m;
     MGCtl *ctl = m.ctl;
+    const unsigned ep = *(volatile unsigned *)m.epoch;  // tags of this solve: ep + 1 + cycle
     if (ctl->skip) return;  // an earlier failure of this step
     const int n = nr - 1, nz0 = m.nz[0], L = m.nlev - 1;
     using Sh = Shape<Tv, M>;
@@ -761,7 +762,6 @@ __device__ __forceinline__ void solve_body(const MGFast *__restrict__ mp, double
     using Fv = Flag<Tv>;
     using Wv = typename Fv::W;
     constexpr bool mixed = sizeof(Tv) == 4;  // flexible GCR(1) around the V-cycle; else the plain V(0,1) iteration
-    const unsigned ep = *(volatile unsigned *)m.epoch;  // tags of this solve: ep + 1 + cycle
     __shared__ unsigned long long s_max[2][2][nt / 32];
     __shared__ double s_dot[2][4][nt / 32];
     __shared__ double s_ab[4];  // the GCR step's beta, alpha, |q|^2 and the inverse of that

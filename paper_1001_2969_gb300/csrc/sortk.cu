@@ -567,7 +567,18 @@ __device__ bool radix_births(const uint64_t *key, uint64_t *id, int nb, StepCtl 
 __global__ void __launch_bounds__(kRadixThreads) k_birth_finish(BirthJob b, PassReset r, int reset) {
     const int tid = threadIdx.x, t = blockIdx.x * blockDim.x + tid, all = gridDim.x * blockDim.x;
     StepCtl *ctl = b.ctl;
-    if (reset && !ctl->halt) {
+    // (read at once, ahead of the stores: the pass waits for this launch.)
+    // Every block reads the counts and the bases before the first barrier;
+    // block 0 moves the bases on at the end
+    const bool halt = ctl->halt != 0, skip = sort_skip(ctl);
+    int nb[2], first[2];
+    uint64_t base[2];
+    for (int s = 0; s < 2; ++s) {
+        first[s] = *b.nb0[s];
+        nb[s] = first[s] < 0 ? 0 : *b.nb[s] - first[s];
+        base[s] = ctl->next_id[s];
+    }
+    if (reset && !halt) {
         for (int s = 0; s < 2; ++s) {
             if (r.N[s])
                 for (int k = t; k < r.ng; k += all) r.N[s][k] = 0.0;
@@ -584,18 +595,9 @@ __global__ void __launch_bounds__(kRadixThreads) k_birth_finish(BirthJob b, Pass
             for (int s = 0; s < 2; ++s)
                 if (r.nbirths[s]) *r.nbirths[s] = 0;
     };
-    if (sort_skip(ctl)) {
+    if (skip) {
         drop_births();
         return;
-    }
-    // every block reads the counts and the bases before the first barrier;
-    // block 0 moves the bases on at the end
-    int nb[2], first[2];
-    uint64_t base[2];
-    for (int s = 0; s < 2; ++s) {
-        first[s] = *b.nb0[s];
-        nb[s] = first[s] < 0 ? 0 : *b.nb[s] - first[s];
-        base[s] = ctl->next_id[s];
     }
     const bool large = nb[0] > kRankBirths || nb[1] > kRankBirths;
     if (!large && blockIdx.x != 0) return;
