@@ -270,15 +270,10 @@ __global__ void __launch_bounds__(kSetupThreads)
         if (i + 1 < nz) hi = face(c, chi[j + nr], gz);
         if (j + 1 < nr) right = face(c, chi[j + 1], m.gr[l][j]);
         const size_t k = (size_t)i * nr + j;
-        if (mixed) {
-            m.cz32[l][k] = (float)hi;
-            m.cr32[l][k] = (float)right;
-        }
-        if (!mixed || l == 0) {  // (the mixed path's coarse levels are FP32)
-            m.cz[l][k] = hi;
-            m.cr[l][k] = right;
-        }
+        if (mixed) m.cz32[l][k] = (float)hi;
+        if (!mixed || l == 0) m.cz[l][k] = hi;  // (the mixed path's coarse levels are FP32)
         if (l == 0) {
+            m.cr[k] = right;
             const double left = j > 0 ? face(chi[j - 1], c, m.gr[0][j - 1]) : 0.0;
             rhs_node(m, a, V, nz, nr, i, j, lo + hi + left + right);
         }
@@ -674,7 +669,7 @@ __device__ __noinline__ void solve_row(const MGFast &m, double *phi, int nr, dou
     __shared__ unsigned long long s_max[2][kSolveThreads / 32];
     __shared__ double s_x[256];
     const int tid = threadIdx.x, n = nr - 1;
-    const double *cz = m.cz[0], *cr = m.cr[0];
+    const double *cz = m.cz[0], *cr = m.cr;
     for (int k = tid; k < Sh::elems; k += kSolveThreads) F[k] = m.facc[k];
     double bn = 0.0;
     for (int cyc = 0;; ++cyc) {
@@ -825,7 +820,7 @@ __device__ __forceinline__ void solve_body(const MGFast *__restrict__ mp, double
         // maxima as bit patterns of |x| (ordered like the values; a NaN
         // compares above every number), so the reductions are integer work
         unsigned long long rmax = 0ull, bmax = 0ull;
-        const double *cz = m.cz[0], *cr = m.cr[0];
+        const double *cz = m.cz[0], *cr = m.cr;
         // the level-0 correction of the cycle before at the tile's nodes and
         // its neighbour columns' (zero on the boundary), a batch per thread
         auto delta_batch = [&](int e0, int j0, Tv (&dv)[kU]) {
@@ -1342,8 +1337,6 @@ size_t mg_tile_elems(int nz, int nr, bool with_neighbours) {
     return with_neighbours ? (size_t)nz * (nr + kWideTile) * 3 : (size_t)nz * (nr + 8);
 }
 
-int mg_line_chunk(int nr) { return line_chunk(nr - 1); }
-
 namespace {
 
 template <typename Tv, int M>
@@ -1524,7 +1517,6 @@ bool solve_job(const FieldDims &fd, MGFast &m, double *phi, bool mixed, double t
     job.most = lay.tw_max ? std::max(most, grid) : grid;
     job.M = M;
     job.mixed = mixed ? 1 : 0;
-    job.minb = minb;
     job.smem = sp;
     job.fn = fn;
     fit_tiles(job);

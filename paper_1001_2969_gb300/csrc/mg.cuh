@@ -52,8 +52,11 @@ struct MGFast {
     int nlev;
     int nz[kMaxLevels];
     double dz[kMaxLevels];
-    double *chi[kMaxLevels], *cz[kMaxLevels], *cr[kMaxLevels];
-    float *cz32[kMaxLevels], *cr32[kMaxLevels];
+    double *chi[kMaxLevels];
+    // face coefficients: in z per level (mixed path: FP64 on the fine level
+    // alone, FP32 on all), in r of the fine level (the line factors hold the rest)
+    double *cz[kMaxLevels], *cr;
+    float *cz32[kMaxLevels];
     // face geometry per level, by column j (filled once by mg_fast_geometry):
     // gz = pi (r_{j+1/2}^2 - r_{j-1/2}^2) / dz_l, gr = 2 pi r_{j+1/2} dz_l / dr;
     // ga = pi (r_{j+1/2}^2 - r_{j-1/2}^2) dz / eps0 (level 0's right-hand side)
@@ -94,7 +97,7 @@ struct FieldSource {
 
 // Shared-memory layout of the one-launch solve (byte offsets), set on the host.
 struct SolveLayout {
-    // from 0 in the line phases: three line buffers, M * 33 values each
+    // from 0 in the line phases: three line buffers (line_buffer values each)
     int offT;   // from 0 in the residual phase: the tile with its neighbour columns; at offT: two restriction buffers
     int offF;   // factor slots: each two red lines and the black line
     int offC;   // factors of the coarsest row
@@ -117,7 +120,7 @@ struct SolveJob {
     int block0, nblocks;  // this job's blocks in the launch
     int most;             // what it can use of a GPU with room to spare
     // host side
-    int M, mixed, minb;
+    int M, mixed;
     size_t smem;
     void *fn;
 };
@@ -144,8 +147,9 @@ void mg_fast_geometry(const MGFast &m, int nr, double dr, std::vector<double> &o
 // once sctl->halt is set, reports cycles, residual and failures to sctl, and
 // returns 0 (or kSolveNoLaunch).  at_solve (optional) is recorded on st just
 // before the one-launch solve, after the set-up: work that waits for it runs
-// beside the solve.  wide: two blocks per black line (a reactor alone on the
-// GPU); else one (many reactors solving side by side).
+// beside the solve.  wide: a block per SM, as many as there are line units or
+// residual tiles (a reactor alone on the GPU); else one per two rows (many
+// reactors solving side by side).
 // defer (narrow solves of a batch): the set-up is enqueued, the solve itself
 // is described in *defer and left to mg_multi_launch; the report to sctl is
 // then the caller's.

@@ -123,7 +123,6 @@ struct pic_handle {
     cudaEvent_t ev_in = nullptr, ev_out = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_fork2 = nullptr, ev_join2 = nullptr;
     StepGraph graphs[8];       // per (cur, cur_i, the pass moves the ions)
-    StepGraph sort_graphs[4];  // the last pass's cell sort at the end of a call, per (cur, cur_i)
     bool sort_deferred = false;  // the last pass's rank and births numbering are still to run
     bool in_batch = false;     // stepped with other reactors (pic_batch): narrow solves
     double ngas = 0.0, nu_max[2] = {0, 0}, p_null[2] = {0, 0};
@@ -646,12 +645,9 @@ void setup_device(pic_handle *h) {
         const size_t g = (size_t)z * h->nr;
         // (level 0: the caller's chi)
         if (l > 0) m.chi[l] = (double *)dalloc(h, g * sizeof(double));
-        m.cz[l] = (double *)dalloc(h, g * sizeof(double));
-        m.cr[l] = (double *)dalloc(h, g * sizeof(double));
-        if (h->mixed) {
-            m.cz32[l] = (float *)dalloc(h, g * sizeof(float));
-            m.cr32[l] = (float *)dalloc(h, g * sizeof(float));
-        }
+        if (l == 0) m.cr = (double *)dalloc(h, g * sizeof(double));
+        if (l == 0 || !h->mixed) m.cz[l] = (double *)dalloc(h, g * sizeof(double));
+        if (h->mixed) m.cz32[l] = (float *)dalloc(h, g * sizeof(float));
         const size_t fe = (size_t)(z - 2) * line_fe;
         if (z == 3) {
             m.facc = (double *)dalloc(h, mg_line_factor_elems(h->nr, true) * sizeof(double));
@@ -680,7 +676,7 @@ void setup_device(pic_handle *h) {
     const size_t tb = mg_tile_elems(h->nz, h->nr, !h->mixed) * sizeof(double);
     if (h->mixed) {
         for (double **z : {&m.kr, &m.kw, &m.kzp, &m.kwp}) *z = (double *)dalloc(h, tb);
-        // (read, times zero, by a solve's first GCR step)
+        // (read by a solve's first GCR step, which drops its products with it)
         cudaMemsetAsync(m.kwp, 0, tb, h->st);
     } else {
         m.ps = (double *)dalloc(h, tb);
@@ -1085,10 +1081,6 @@ void drop_graphs(pic_handle *h) {
         if (g.exec) cudaGraphExecDestroy(g.exec);
         g = StepGraph();
     }
-    for (StepGraph &g : h->sort_graphs) {
-        if (g.exec) cudaGraphExecDestroy(g.exec);
-        g = StepGraph();
-    }
 }
 
 void destroy_streams(pic_handle *h) {
@@ -1127,53 +1119,6 @@ void capture_step(pic_handle *h, StepGraph &g, bool mv) {
         g.failed = true;
         cudaGetLastError();
     }
-}
-
-// capture the pending sort of the current parity
-template <typename T>
-void capture_sort(pic_handle *h, StepGraph &g) {
-    const int64_t L0 = h->launches;
-    cudaStream_t keep = h->st;
-    h->st = h->gst;
-    cudaGraph_t graph = nullptr;
-    cudaError_t e = cudaStreamBeginCapture(h->gst, cudaStreamCaptureModeThreadLocal);
-    if (e == cudaSuccess) {
-        sort_tail<T>(h);
-        e = cudaStreamEndCapture(h->gst, &graph);
-    }
-    h->st = keep;
-    g.launches = h->launches - L0;
-    h->launches = L0;
-    if (e == cudaSuccess && graph) e = cudaGraphInstantiate(&g.exec, graph, 0);
-    if (graph) cudaGraphDestroy(graph);
-    if (e != cudaSuccess || !g.exec) {
-        g.exec = nullptr;
-        g.failed = true;
-        cudaGetLastError();
-    }
-}
-
-// enqueue the pending sort on stream `on` (private stream: as a graph)
-void enqueue_sort_tail(pic_handle *h, cudaStream_t on) {
-    StepGraph &g = h->sort_graphs[h->cur + 2 * h->cur_i];
-    if (on == h->gst && !g.exec && !g.failed) {
-        if (h->mixed)
-            capture_sort<float>(h, g);
-        else
-            capture_sort<double>(h, g);
-    }
-    if (on == h->gst && g.exec) {
-        cudaGraphLaunch(g.exec, h->gst);
-        h->launches += g.launches;
-        return;
-    }
-    cudaStream_t keep = h->st;
-    h->st = on;
-    if (h->mixed)
-        sort_tail<float>(h);
-    else
-        sort_tail<double>(h);
-    h->st = keep;
 }
 
 // capture one step of every reactor of the batch as one fork-join graph
@@ -1559,7 +1504,10 @@ bool here_and_aligned(const double *p) {
 pic_status complete_sort(pic_handle *h) {
     if (!h->sort_deferred) return PIC_OK;
     h->sort_deferred = false;
-    enqueue_sort_tail(h, h->st);
+    if (h->mixed)
+        sort_tail<float>(h);
+    else
+        sort_tail<double>(h);
     return finish_call(h, h->step, h->cur, h->cur_i, 0, false);
 }
 
