@@ -580,15 +580,14 @@ __global__ void k_rhs_bc(const MGFast *__restrict__ mp, RhsArgs a, int nz, int n
 // another's look at the norms, which are kept in two sets.  A solve's tags
 // start where the one before ended (block 0 moves `epoch` on), so either all
 // of its blocks run or none does (MGCtl::skip).
-// Measured, a whole stand-alone solve (with its set-up launches) against the
-// same phases between grid barriers, which took ~1 us each and cost every
-// phase its L1: 33 x 65 mixed 216 -> 157 us, 65 x 300 mixed 326 -> 228,
-// 257 x 1025 mixed 626 -> 527, 129 x 513 FP64 886 -> 803 (FP64 line solves).
 // What is exchanged all-to-all is kept in kCopies copies (with one, 128 blocks
-// polling the same few lines of L2 took 3 us for the norms, now 1.8), sums and
+// polling the same few lines of L2 take 3 us for the norms, so 1.8), sums and
 // maxima take few FP64 and 64-bit operations, a tile's restricted levels are
-// stored by rows, and the lines' factors wait in registers: 157 -> 147 us,
-// 228 -> 202, 527 -> 508.
+// stored by rows, and FP32 lines' factors wait in registers.
+// Measured, a whole stand-alone solve with its set-up, against one whose phases
+// meet at grid barriers (~1 us each, and each costs every phase its L1): 33 x 65
+// mixed 218 -> 123 us, 65 x 300 mixed 327 -> 178, 257 x 1025 mixed 627 -> 465,
+// 129 x 513 FP64 887 -> 528 (there the line solves take the rest of the time).
 // ---------------------------------------------------------------------------
 
 // ---- factor lines into shared memory ----
@@ -1108,7 +1107,6 @@ __device__ __forceinline__ void solve_body(const MGFast *__restrict__ mp, double
                 if (t + P < ntile) __syncthreads();
             }
         }
-        // ---- decision: every block reads every block's maxima ----
         block_max2(rmax, bmax, s_max[0]);
         // (two sets in turn: a block that owns no unit may still be reading the
         // norms of the cycle before)
@@ -1550,7 +1548,7 @@ int mg_fast_solve(const FieldDims &fd, MGFast &m, const FieldSource &src, double
     MGFast *mp = m.self;  // uploaded once (mg_fast_upload)
     const RhsArgs ra{src.rho, phi, phi_zL, V, warm ? 0 : 1, v_from_ctl ? 1 : 0, warm ? phi_prev : nullptr};
     if (setup) {
-        int lc = 2;  // four columns (a 32-byte sector a row): c2's FP64 divisions on most SMs
+        int lc = 2;  // four columns: a 32-byte sector a row, and blocks for most SMs
         size_t smem = 0;
         while ((smem = (((size_t)2 * nz + kMaxLevels) * sizeof(double)) << lc) > kSolveSmemLimit && lc > 0) --lc;
         if (src.Ne || nlev > 1) {

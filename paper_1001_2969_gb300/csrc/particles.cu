@@ -369,10 +369,11 @@ constexpr int kEedfCopies = 8;
 // a time, ahead of their use (for latency-bound passes)
 // PPT: particles per thread in a unit (32 * PPT particles per warp)
 // XYZ: the global X-Y-Z pusher (a_theta carried; a.xyz set)
-// S: 1 the ions (charge exchange alone: fewer registers, no spills, c2 230 -> 221
-// us), 0 the electrons.  Fixing the species at compile time for the electrons
-// too gave 2 %, but the compiler then contracts the scattering differently and
-// one electron in a thousand moves by an FP32 rounding: not done.
+// S: 1 the ions (charge exchange alone: fewer registers, no spills in the shape
+// they take, c2 230 -> 221 us), 0 the electrons.  That one keeps the species at run
+// time, and with it branches of the ions that it never takes: without them the
+// pass is 2 % faster, but the compiler contracts the scattering differently and
+// one electron in a thousand moves by an FP32 rounding.
 template <typename T, bool PF, int kPPT, bool XYZ, int S>
 __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 4 : 2) k_step(StepArgs<T> a) {
     constexpr int kChunk = kThreads * kPPT;  // the block's staging slots
@@ -748,8 +749,8 @@ void launch_variant(const StepArgs<T> &a, int grid, cudaStream_t st) {
 // variant: bit 0 = prefetch the chunk into shared memory, bit 1 = 8
 // particles per thread (else 4); -1 = the default for the species, the
 // faster shape on GB300 at 1e7 particles per species: ions prefetch 4 per
-// thread (their pass is latency-bound), electrons load directly, 8 per
-// thread (theirs is bound by issue)
+// thread, electrons load directly, 8 per thread (the prefetch's shared memory
+// would leave their field gather and cross-section table too little L1)
 template <typename T>
 void launch_step(const StepArgs<T> &a, int grid, int variant, cudaStream_t st) {
     const int v = variant >= 0 ? (variant & 3) : (a.s == 1 ? 1 : 2);

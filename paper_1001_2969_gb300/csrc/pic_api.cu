@@ -1480,7 +1480,7 @@ pic_status finish_call(pic_handle *h, int64_t step0, int cur0, int cur_i0, int32
             return fail(h, PIC_ERR_CAPACITY, (why & ST_CAPACITY) ? "particle capacity exceeded"
                                                                  : "births capacity exceeded");
         return fail(h, PIC_ERR_TIMEOUT, c.sort_fail ? "births numbering: grid barrier timed out"
-                                                    : "multigrid grid barrier timed out");
+                                                    : "multigrid wait timed out");
     }
     cudaStreamSynchronize(h->st);
     return result;
@@ -1852,7 +1852,7 @@ pic_status pic_field_solve(pic_handle *h, const double *rho, const double *chi, 
                                 nullptr, true, nullptr, nullptr, true, nullptr,
                                 h->host_ctl ? &h->host_ctl->mg : nullptr);
     h->launches += L;
-    if (r == kSolveTimeout) return fail(h, PIC_ERR_TIMEOUT, "multigrid grid barrier timed out");
+    if (r == kSolveTimeout) return fail(h, PIC_ERR_TIMEOUT, "multigrid wait timed out");
     if (r == kSolveNoLaunch) return fail(h, PIC_ERR_CUDA, "multigrid solve could not be launched");
     cudaMemcpyAsync(phi, h->tmp_grid[2], gb, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, h->st);
     cudaStreamSynchronize(h->st);

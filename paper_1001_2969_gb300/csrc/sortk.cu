@@ -192,8 +192,8 @@ void launch_step_check(const DevScalars *ds, StepCtl *ctl, cudaStream_t st) {
 
 // The end of a call: the capacity check of the last pass's pending sort and
 // the call's report, in one launch.  The sort's totals are the sums of the
-// cell counts (its scans, run here before, took seven launches, 15-40 us at
-// the end of every call); blocks of both species add their parts, the last
+// cell counts (the scans themselves would be seven launches, 15-40 us at the
+// end of every call); blocks of both species add their parts, the last
 // block to finish checks the totals against the capacities, fails the sort if
 // one is over, and writes the step control and the status word to `report`
 // (pinned host memory; null: none).
@@ -397,11 +397,9 @@ constexpr int kRadixTile = kRadixThreads * kRadixPer;
 // and passes all keys through shared memory.  No block waits for another, so
 // it runs as an ordinary kernel beside the field solve (ids are first read
 // by the next particle pass).  Bound by issue: the n^2 comparisons are spread
-// over the grid.  One block per species, which made the same comparisons
-// before, held up the pass after the solve for 105 us per species in the
-// first steps of c2 (many births) and 4 us with few; with this kernel beside
-// the solve c2 went from 1107 to 1092 us a step, c1 from 314 to 298, eight
-// batched reactors from 1739 to 1667.  The line to the radix sort is where
+// over the grid.  (One block per species after the solve takes 105 us a species
+// for the same comparisons in the first steps of c2, with many births, and 4 us
+// with few.)  The line to the radix sort is where
 // the comparisons (67M: some 9 us of the whole GPU's issue slots, mostly
 // hidden by the solve) still cost less than its ~20 grid barriers (~1 us
 // each, after the solve).
@@ -561,8 +559,7 @@ __device__ bool radix_births(const uint64_t *key, uint64_t *id, int nb, StepCtl 
 // The end of the pending sort and the start of the pass that reads it: the
 // births k_birth_rank left are numbered, the ids move on, the sorted counts
 // take effect, and (reset) what the coming pass accumulates into is cleared.
-// One launch for what were seven nodes in a row between the field and the
-// pass (two births numberings with their counters' clears, sort end, reset).
+// One launch between the field and the pass, which waits for it.
 // Cooperative when it has more than one block (the radix sort's barriers).
 __global__ void __launch_bounds__(kRadixThreads) k_birth_finish(BirthJob b, PassReset r, int reset) {
     const int tid = threadIdx.x, t = blockIdx.x * blockDim.x + tid, all = gridDim.x * blockDim.x;

@@ -637,7 +637,7 @@ int window_run(const WindowIn<T> &in, int K, int ckpt, const double *w_host, dou
         }
         if (c.halt) {
             status = PIC_ERR_TIMEOUT;
-            err = "window: multigrid grid barrier timed out";
+            err = "window: multigrid wait timed out";
         } else if (c.mg_flags & 1) {
             status = PIC_ERR_NOT_CONVERGED;
             err = "window: multigrid stopped before the tolerance";
