@@ -588,7 +588,7 @@ __global__ void __launch_bounds__(kRadixThreads) k_birth_finish(BirthJob b, Pass
     // sorted here: they are the state's until this sort is done, and stay
     // where it failed
     auto drop_births = [&]() {
-        if (reset && t == 0 && !*(const volatile int32_t *)&ctl->halt)
+        if (reset && t == 0 && !halt)
             for (int s = 0; s < 2; ++s)
                 if (r.nbirths[s]) *r.nbirths[s] = 0;
     };
