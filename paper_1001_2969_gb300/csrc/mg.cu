@@ -586,8 +586,8 @@ __global__ void k_rhs_bc(const MGFast *__restrict__ mp, RhsArgs a, int nz, int n
 // stored by rows, and FP32 lines' factors wait in registers.
 // Measured, a whole stand-alone solve with its set-up, against one whose phases
 // meet at grid barriers (~1 us each, and each costs every phase its L1): 33 x 65
-// mixed 218 -> 123 us, 65 x 300 mixed 327 -> 178, 257 x 1025 mixed 627 -> 465,
-// 129 x 513 FP64 887 -> 528 (there the line solves take the rest of the time).
+// mixed 218 -> 117 us, 65 x 300 mixed 327 -> 178, 257 x 1025 mixed 627 -> 460,
+// 129 x 513 FP64 887 -> 527 (there the line solves take the rest of the time).
 // ---------------------------------------------------------------------------
 
 // ---- factor lines into shared memory ----

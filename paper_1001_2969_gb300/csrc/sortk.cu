@@ -666,7 +666,7 @@ void launch_birth_finish(const BirthJob &b, const PassReset *r, cudaStream_t st,
     // no more blocks than tiles of the largest batch of births or 4096 nodes to
     // clear each (a small reactor's numbering does not hold the whole GPU; with the
     // births alone deciding, a capacity of 2048 had one block clear 257 x 1025
-    // nodes: 751 us a step against 633)
+    // nodes: 744 us a step against 659)
     // (max_grid: a reactor of a batch, whose numbering must not wait for
     // many co-resident blocks while the other reactors' kernels hold SMs)
     const int clear = r ? (std::max(r->ng, r->ncell) + 4095) / 4096 : 1;
